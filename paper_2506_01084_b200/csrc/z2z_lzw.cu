@@ -1,12 +1,12 @@
 // LZW codebook kernels: session reset, prompt compression, online update.
 //
-// One warp owns one sequence.  The codebook of a sequence is an open-addressing hash table in
-// global memory keyed by (prefix code, next base token), probed linearly from an even slot; a warp
-// probe is one coalesced 256-byte load of 32 consecutive slots followed by a ballot.  Entries are
+// The codebook of a sequence is an open-addressing hash table in global memory keyed by (prefix
+// code, next base token), probed linearly from an even slot; the online update probes it with one
+// warp (one coalesced 256-byte load of 32 consecutive slots followed by a ballot).  Entries are
 // never deleted and an insert always takes the first empty slot in probe order, so an empty slot
 // proves absence.
-// The parse itself is a dependent chain (each token's lookup needs the previous match), which is
-// why the unit of parallelism is the sequence (paper Section 2.4: compression is per document).
+// Prompt compression gives every sequence a block (paper Section 2.4: compression is per document)
+// that parses a window of positions at a time.
 #include "z2z_common.cuh"
 #include "z2z_internal.h"
 #include "z2z_lzw_dev.cuh"
@@ -27,187 +27,147 @@ __global__ void k_codebook_clear(CbView cb) {
   }
 }
 
-// Prompt compression (Section 2.1; Section 2.3 step 2).  grid = ceil(B / warps per block).
-__global__ void __launch_bounds__(128) k_lzw_encode(CbView cb, const int32_t* __restrict__ tokens,
-                                                    const int32_t* __restrict__ lens, int T_max,
-                                                    int32_t* __restrict__ codes,
-                                                    int32_t* __restrict__ code_lens,
-                                                    int32_t* __restrict__ entries_after) {
-  const int lane = threadIdx.x & 31;
-  const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (b >= cb.B) return;
-  unsigned long long* table = cb.hash + (size_t)b * cb.n_slots;
-  int T = lens ? lens[b] : T_max;
-  T = T < 0 ? 0 : (T > T_max ? T_max : T);
-  const int32_t* x = tokens + (size_t)b * T_max;
-  int32_t* out = codes + (size_t)b * T_max;
-  int32_t* aft = entries_after ? entries_after + (size_t)b * T_max : nullptr;
-  int n = cb.n[b];
-  int st = 0;
-  int w = -1, wlen = 0, n_out = 0;
-  for (int base = 0; base < T; base += 32) {
-    int mine = (base + lane < T) ? x[base + lane] : 0;
-    int cnt = T - base < 32 ? T - base : 32;
-    for (int i = 0; i < cnt; ++i) {
-      int c = __shfl_sync(0xffffffffu, mine, i);
-      if ((unsigned)c >= (unsigned)cb.V) { st |= Z2Z_ST_BAD_TOKEN; c = 0; }   // not a base token
-      if (wlen == 0) { w = c; wlen = 1; continue; }
-      Probe p{-1, -1};
-      if (wlen < cb.M) {
-        p = warp_probe(table, cb.n_slots, (uint32_t)w, (uint32_t)c);
-        if (p.found >= 0) { w = cb.V + p.found; ++wlen; continue; }      // match grows
-      }
-      // longest match ends: emit it, then remember (w ++ c) if allowed
-      if (lane == 0) out[n_out] = w;
-      if (wlen < cb.M && n < cb.cap) {
-        if (p.slot >= 0) {
-          if (lane == 0) table[p.slot] = pack_slot((uint32_t)w, (uint32_t)c, (uint32_t)n);
-          warp_write_entry(cb, b, n, w, wlen, c);
-          ++n;
-          if (n >= cb.cap) st |= Z2Z_ST_CAP_FROZEN;
-          __syncwarp();                     // the new slot and entry are visible to later probes
-        } else {
-          st |= Z2Z_ST_TABLE_FULL;
-        }
-      }
-      if (aft && lane == 0) aft[n_out] = n;
-      ++n_out;
-      w = c; wlen = 1;
-    }
-  }
-  if (wlen > 0) {                             // final flush creates no entry
-    if (lane == 0) { out[n_out] = w; if (aft) aft[n_out] = n; }
-    ++n_out;
-  }
-  if (lane == 0) {
-    code_lens[b] = n_out;
-    cb.n[b] = n;
-    if (n_out > 0) cb.prev[b] = w;
-    if (st) atomicOr(&cb.status[b], st);
-  }
-}
-
-// The same parse with the sequence's hash table held in shared memory for the duration of the
-// kernel (codebooks of up to 12800 entries: at most 25600 slots, 200 KB).  The parse is a
-// dependent chain of one probe per token, and a chain that a single warp executes is paced by the
-// number of instructions it issues per token (about one every four to five cycles), not by memory.
-// A warp-wide probe spends most of them on warp primitives (broadcast, ballot, shuffle: about
-// 240 ns per token with the table in shared memory, 290 with the table in global memory); here
-// ONE thread walks the probe sequence two slots (one 16-byte shared-memory load) at a time, which
-// at a load factor of at most one half ends after one or two loads: 165-195 ns per token.  The
-// rest of warp 0 stages the tokens (the batch after the one being parsed is already in flight)
-// and the other warps move the table in and out.  A new entry is the last wlen + 1 input tokens,
-// so the chain only records where the phrase starts and how long it is (one word in the first
-// constituent slot, one length byte); all threads expand the records into constituent rows from
-// the token array after the parse.
-constexpr int kEncodeSmemThreads = 128;
-constexpr size_t kEncodeSmemMaxBytes = 200 * 1024;
-
-__global__ void __launch_bounds__(kEncodeSmemThreads) k_lzw_encode_smem(CbView cb, const int32_t* __restrict__ tokens,
-                                                                        const int32_t* __restrict__ lens, int T_max,
-                                                                        int32_t* __restrict__ codes,
-                                                                        int32_t* __restrict__ code_lens,
-                                                                        int32_t* __restrict__ entries_after) {
-  extern __shared__ __align__(16) unsigned long long s_table[];
-  __shared__ int4 s_tok[64];                         // two batches of 32 tokens: {c, hash part, c >> 16, c & 0xffff}
-  __shared__ int s_n0, s_n1;                         // entries before / after this call
-  const int lane = threadIdx.x & 31;
+// Prompt compression (Section 2.1; Section 2.3 step 2).  One block per sequence; a window of
+// kParseLanes input positions at a time (z2z_lzw_dev.cuh).
+//
+// Each lane follows the longest match from its own position (at most M - 1 dependent lookups).
+// Which positions start a phrase is a walk position -> position + match length: inside a warp by
+// pointer doubling (five rounds carry the set of visited lanes and the exit), across the four
+// warps by looking up the exit of one as the entry of the next (a match is at most kMaxM long, so
+// only the first kMaxM lanes of a warp can be entered).
+//
+// Bound by the latency of one window (a few dependent shared-memory lookups, ten shuffles, four
+// barriers).  The chain used to be walked token by token by one thread: 180 ns per token with the
+// table in shared memory, 220 with it in global memory.  Four texts of 32768 tokens (cap 16384), to
+// codes and back with both session resets: 9.62 ms before, 1.00 ms with windows here and in the replay.
+template <bool SMEM>
+__global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const int32_t* __restrict__ tokens,
+                                                              const int32_t* __restrict__ lens, int T_max,
+                                                              int32_t* __restrict__ codes,
+                                                              int32_t* __restrict__ code_lens,
+                                                              int32_t* __restrict__ entries_after) {
+  extern __shared__ __align__(16) unsigned char s_parse[];
+  __shared__ int s_tok[4 * kParseLanes];             // four chunks of tokens, position p at p mod 512
+  __shared__ int2 s_walk[4][kMaxM];                  // per warp and entry lane: lanes visited, exit
+  __shared__ ParseVotes s_votes;
+  __shared__ int s_prev, s_n1, s_st;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
-  unsigned long long* table = cb.hash + (size_t)b * cb.n_slots;
-  for (int i = threadIdx.x; i < cb.n_slots; i += blockDim.x) s_table[i] = table[i];
+  const int V = cb.V, M = cb.M, cap = cb.cap;
+  const int n0 = cb.n[b];
   int T = lens ? lens[b] : T_max;
   T = T < 0 ? 0 : (T > T_max ? T_max : T);
   const int32_t* x = tokens + (size_t)b * T_max;
-  int32_t* const cons = cb.cons + (size_t)b * cb.cap * cb.M;
-  uint8_t* const len = cb.len + (size_t)b * cb.cap;
+  ParseTable<SMEM> table;
+  table.open(cb, b, n0, s_parse);
+  if (tid == 0) { s_prev = -1; s_st = 0; s_n1 = n0; }
   __syncthreads();
-  if (threadIdx.x < 32) {
+  if (tid < kParseLanes) {
     int32_t* out = codes + (size_t)b * T_max;
     int32_t* aft = entries_after ? entries_after + (size_t)b * T_max : nullptr;
-    const int V = cb.V, M = cb.M, cap = cb.cap;
-    const uint32_t pair_mask = (uint32_t)(cb.n_slots - 1) & ~1u;
-    // a slot as two words: hi = prefix << 8 | token >> 16, lo = token << 16 | entry (all-ones hi = empty)
-    const uint2* const slots = reinterpret_cast<const uint2*>(s_table);
-    int n = cb.n[b];
-    if (lane == 0) s_n0 = n;
-    int st = 0;
-    int w = -1, wlen = 0, n_out = 0;
-    int ahead = lane < T ? x[lane] : 0;              // tokens of the batch after the current one
-    for (int base = 0; base < T; base += 32) {
-      int mine = ahead;
-      ahead = base + 32 + lane < T ? x[base + 32 + lane] : 0;
-      if ((unsigned)mine >= (unsigned)V) { if (base + lane < T) st |= Z2Z_ST_BAD_TOKEN; mine = 0; }   // not a base token
-      s_tok[(base & 32) + lane] = make_int4(mine, (int)hash_token_part((uint32_t)mine), mine >> 16, mine & 0xffff);
-      __syncwarp();
-      if (lane == 0) {
-        const int cnt = T - base < 32 ? T - base : 32;
-        int4 t_next = s_tok[base & 63];
-        for (int i = 0; i < cnt; ++i) {
-          const int4 t = t_next;
-          t_next = s_tok[(base + i + 1) & 63];         // off the chain: ready before the next probe needs it
-          const int c = t.x;
-          if (wlen == 0) { w = c; wlen = 1; continue; }
-          int slot = -1;
-          const uint32_t key_hi = ((uint32_t)w << 8) | (uint32_t)t.z;
-          if (wlen < M) {
-            uint32_t at = hash_join((uint32_t)w, (uint32_t)t.y) & pair_mask;
-            int found = -1;
-            for (int it = 0; it < cb.n_slots; it += 2) {   // bounded: at most the whole table
-              const uint4 pr = *reinterpret_cast<const uint4*>(&slots[at]);      // slots at, at + 1: {lo, hi, lo, hi}
-              if (pr.y == key_hi && (pr.x >> 16) == (uint32_t)t.w) { found = (int)(pr.x & 0xffffu); break; }
-              if (pr.y == 0xffffffffu) { slot = (int)at; break; }              // (no prefix is 2^24 - 1)
-              if (pr.w == key_hi && (pr.z >> 16) == (uint32_t)t.w) { found = (int)(pr.z & 0xffffu); break; }
-              if (pr.w == 0xffffffffu) { slot = (int)at + 1; break; }
-              at = (at + 2) & pair_mask;
-            }
-            if (found >= 0) { w = V + found; ++wlen; continue; }          // match grows
-          }
-          // longest match ends: emit it, then remember (w ++ c) if allowed
-          out[n_out] = w;
-          if (wlen < M && n < cap) {
-            if (slot >= 0) {
-              reinterpret_cast<uint2*>(s_table)[slot] = make_uint2(((uint32_t)t.w << 16) | (uint32_t)n, key_hi);
-              cons[(size_t)n * M] = base + i - wlen;                       // where the phrase starts
-              len[n] = (uint8_t)(wlen + 1);
-              ++n;
-              if (n >= cap) st |= Z2Z_ST_CAP_FROZEN;
-            } else {
-              st |= Z2Z_ST_TABLE_FULL;
-            }
-          }
-          if (aft) aft[n_out] = n;
-          ++n_out;
-          w = c; wlen = 1;
+    int n = n0, n_out = 0, st = 0;
+    int chunks = 0;                                  // token chunks already in s_tok
+    int ahead = tid < T ? x[tid] : 0;                // this thread's token of the next chunk
+    for (int p0 = 0; p0 < T;) {                      // p0: a phrase starts here
+      // positions below p0 + kParseLanes + kMaxM are looked at.  Nothing is fetched earlier than that: a
+      // window moves p0 by less than kParseLanes + kMaxM, so that a chunk is overwritten only once no
+      // warp can still be busy with the window that needed it.
+      while (chunks <= (p0 + kParseLanes + kMaxM - 1) / kParseLanes && chunks * kParseLanes < T) {
+        const int at = chunks * kParseLanes + tid;
+        int c = ahead;
+        if ((unsigned)c >= (unsigned)V) { if (at < T) st |= Z2Z_ST_BAD_TOKEN; c = 0; }     // not a base token
+        s_tok[at & (4 * kParseLanes - 1)] = c;
+        ++chunks;
+        ahead = at + kParseLanes < T ? x[at + kParseLanes] : 0;
+      }
+      parse_sync();
+      // ---- longest match from every position of the window
+      const int q = p0 + tid;
+      const bool live = q < T;
+      int w = -1, len = 1, slot = -1, c = 0;
+      bool miss = false;
+      if (live) {
+        w = s_tok[q & (4 * kParseLanes - 1)];
+        while (len < M && q + len < T) {
+          c = s_tok[(q + len) & (4 * kParseLanes - 1)];
+          const int e = table.probe((uint32_t)w, (uint32_t)c, slot);
+          if (e < 0) { miss = true; break; }
+          w = V + e; ++len;
         }
       }
-      __syncwarp();                                  // the other half of s_tok may be rewritten
-    }
-    if (lane == 0) {
-      if (wlen > 0) {                                // final flush creates no entry
-        out[n_out] = w;
-        if (aft) aft[n_out] = n;
-        ++n_out;
+      // ---- positions on the chain
+      uint32_t visited = live ? 1u << lane : 0u;
+      int to = live ? lane + len : lane;
+#pragma unroll
+      for (int r = 0; r < 5; ++r) {
+        const uint32_t v2 = __shfl_sync(0xffffffffu, visited, to & 31);
+        const int t2 = __shfl_sync(0xffffffffu, to, to & 31);
+        if (to < 32) { visited |= v2; to = t2; }
       }
-      code_lens[b] = n_out;
-      cb.n[b] = n;
-      if (n_out > 0) cb.prev[b] = w;
-      s_n1 = n;
+      if (lane < kMaxM) s_walk[warp][lane] = make_int2((int)visited, warp * 32 + to);
+      parse_sync();
+      uint32_t mine = 0;
+      int at = 0;                                    // entry into warp k, then the window's exit
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if ((at >> 5) == k) {                        // (a walk that reached the end of the input stays where it is)
+          const int2 wk = s_walk[k][at & 31];
+          if (k == warp) mine = (uint32_t)wk.x;
+          at = wk.y;
+        }
+      }
+      const bool on = (mine >> lane) & 1u;
+      // ---- new phrases of the chain bid for their slots
+      const bool ins = on && miss && n < cap && slot >= 0;
+      if (on && miss && n < cap && slot < 0) st |= Z2Z_ST_TABLE_FULL;
+      if (ins) table.bid(slot, tid);
+      parse_sync();
+      const bool own = ins && table.owns(slot, tid);
+      const uint32_t v_on = __ballot_sync(0xffffffffu, on), v_ins = __ballot_sync(0xffffffffu, ins);
+      const uint32_t v_lost = __ballot_sync(0xffffffffu, ins && !own);
+      if (lane == 0) { s_votes.on[warp] = v_on; s_votes.ins[warp] = v_ins; s_votes.lost[warp] = v_lost; }
+      parse_sync();
+      const ParseVotes votes = s_votes;
+      const int stop = parse_first_lost(votes);      // lanes below it are final
+      const int room = cap - n;
+      const int new_before = parse_count_below(votes.ins, tid);
+      if (own) {
+        const int entry = tid < stop && new_before < room ? n + new_before : -1;
+        table.settle(slot, (uint32_t)w, (uint32_t)c, entry);
+        if (entry >= 0) {                            // the phrase and its next token, -1 padded
+          int32_t* row = cb.cons + ((size_t)b * cap + entry) * M;
+          for (int j = 0; j < M; ++j) row[j] = j <= len ? s_tok[(q + j) & (4 * kParseLanes - 1)] : -1;
+          cb.len[(size_t)b * cap + entry] = (uint8_t)(len + 1);
+        }
+      }
+      const int emitted = parse_count_below(votes.on, stop);
+      if (on && tid < stop) {
+        const int pos = n_out + parse_count_below(votes.on, tid);
+        out[pos] = w;
+        const int made = new_before + (ins ? 1 : 0);
+        if (aft) aft[pos] = n + (made < room ? made : room);
+        if (pos == n_out + emitted - 1) s_prev = w;
+      }
+      const int made = parse_count_below(votes.ins, stop);
+      if (made > 0) {
+        n += made < room ? made : room;
+        if (n >= cap) st |= Z2Z_ST_CAP_FROZEN;
+      }
+      n_out += emitted;
+      p0 += stop < kParseLanes ? stop : at;
+      // (the barrier at the head of the next window orders these writes before its lookups; s_votes
+      // and s_walk are rewritten behind further barriers)
     }
-    st = __reduce_or_sync(0xffffffffu, st);           // BAD_TOKEN is found per lane
-    if (lane == 0 && st) atomicOr(&cb.status[b], st);
+    if (st) atomicOr(&s_st, st);
+    if (tid == 0) { code_lens[b] = n_out; s_n1 = n; }
   }
   __syncthreads();
-  // constituent rows of the entries created here: tokens [start, start + len), -1 padded
-  for (int e = s_n0 + threadIdx.x; e < s_n1; e += blockDim.x) {
-    const int start = cons[(size_t)e * cb.M];
-    const int L = len[e];
-    for (int j = 0; j < cb.M; ++j) {
-      int v = -1;
-      if (j < L) { v = x[start + j]; if ((unsigned)v >= (unsigned)cb.V) v = 0; }
-      cons[(size_t)e * cb.M + j] = v;
-    }
+  if (tid == 0) {
+    cb.n[b] = s_n1;
+    if (s_prev >= 0) cb.prev[b] = s_prev;
+    if (s_st) atomicOr(&cb.status[b], s_st);
   }
-  for (int i = threadIdx.x; i < cb.n_slots; i += blockDim.x) table[i] = s_table[i];
+  table.close(n0, s_n1);
 }
 
 // Online update with one new code per sequence (Figure 1; Section 2.3 step 10).
@@ -238,18 +198,16 @@ cudaError_t launch_codebook_clear(const CbView& cb, cudaStream_t s) {
 cudaError_t launch_lzw_encode(const CbView& cb, const int32_t* tokens, const int32_t* lens,
                               int T_max, int32_t* codes, int32_t* code_lens,
                               int32_t* entries_after, cudaStream_t s) {
-  const size_t table_bytes = (size_t)cb.n_slots * sizeof(unsigned long long);
-  if (table_bytes <= kEncodeSmemMaxBytes) {
-    cudaError_t e = cudaFuncSetAttribute(k_lzw_encode_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)table_bytes);
+  // Shared memory holds codebooks of up to 16384 entries (224 KB); a larger table stays in global
+  // memory and every lookup of a window costs a round trip to L2 instead.
+  if (cb.cap <= kParseSmemMaxCap) {
+    const size_t smem = parse_smem_bytes(cb.n_slots, cb.cap);
+    cudaError_t e = cudaFuncSetAttribute(k_lzw_encode<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k_lzw_encode_smem<<<cb.B, kEncodeSmemThreads, table_bytes, s>>>(cb, tokens, lens, T_max, codes, code_lens,
-                                                                     entries_after);
-    return cudaGetLastError();
+    k_lzw_encode<true><<<cb.B, kParseThreads, smem, s>>>(cb, tokens, lens, T_max, codes, code_lens, entries_after);
+  } else {
+    k_lzw_encode<false><<<cb.B, kParseThreads, 0, s>>>(cb, tokens, lens, T_max, codes, code_lens, entries_after);
   }
-  // larger codebooks keep the table in global memory.  One warp per block: every sequence gets
-  // its own SM while B <= 148, which keeps each dependent probe chain at the lowest latency the
-  // memory system gives
-  k_lzw_encode<<<cb.B, 32, 0, s>>>(cb, tokens, lens, T_max, codes, code_lens, entries_after);
   return cudaGetLastError();
 }
 

@@ -3,12 +3,8 @@
 // back into base tokens).
 //
 // Two kernels:
-//   k_lzw_replay  (k_lzw_replay_smem while the table fits shared memory) rebuilds (or continues)
-//                 each sequence's codebook from the code stream alone by
-//                 replaying the online update once per code.  A dependent chain per sequence, so
-//                 one warp owns one sequence, keeps the running state in registers and prefetches
-//                 (first token, length) of the next 32 codes in one coalesced pass; an entry that
-//                 was created inside the current batch of 32 is re-read when its code comes up.
+//   k_lzw_replay  rebuilds (or continues) each sequence's codebook from the code stream alone by
+//                 replaying the online update once per code, a window of codes at a time.
 //   k_lzw_expand  turns codes into base tokens with the codebook that is resident: an exclusive
 //                 scan of phrase lengths gives every code its output offset, each thread then
 //                 copies one phrase.  Blocks are (sequence, chunk of codes); a block finds its
@@ -36,211 +32,156 @@ __device__ __forceinline__ int entry_len(const CbView& cb, int b, int code) {
 // Replays the online update (Figure 1; Section 2.3 step 10) for codes[b][0 .. code_lens[b]).
 // n_valid[b] = number of codes accepted; replay of a sequence stops at the first code that names
 // no hypertoken (BAD_TOKEN; the state is the one after the last accepted code).
-__global__ void __launch_bounds__(32) k_lzw_replay(CbView cb, const int32_t* __restrict__ codes,
-                                                   const int32_t* __restrict__ code_lens,
-                                                   int Tc_max, int32_t* __restrict__ n_valid) {
-  const int lane = threadIdx.x & 31;
-  const int b = blockIdx.x;
-  if (b >= cb.B) return;
-  unsigned long long* table = cb.hash + (size_t)b * cb.n_slots;
-  int Tc = code_lens ? code_lens[b] : Tc_max;
-  Tc = Tc < 0 ? 0 : (Tc > Tc_max ? Tc_max : Tc);
-  const int32_t* zs = codes + (size_t)b * Tc_max;
-  int n = cb.n[b];
-  int prev = cb.prev[b];
-  int plen = 0, pfirst = -1;
-  if (prev >= 0) { plen = entry_len(cb, b, prev); pfirst = entry_first(cb, b, prev); }
-  int st = 0, valid = 0;
-  bool bad = false;
-  for (int base = 0; base < Tc && !bad; base += 32) {
-    const int cnt = Tc - base < 32 ? Tc - base : 32;
-    const int n_batch = n;                       // entries below this index exist for the whole batch
-    int z_mine = -1, f_mine = -1, l_mine = 0;
-    if (lane < cnt) {
-      z_mine = zs[base + lane];
-      if (z_mine >= 0 && z_mine < cb.V + n_batch) {
-        f_mine = entry_first(cb, b, z_mine);
-        l_mine = entry_len(cb, b, z_mine);
-      }
-    }
-    for (int i = 0; i < cnt; ++i) {
-      const int z = __shfl_sync(0xffffffffu, z_mine, i);
-      int f = __shfl_sync(0xffffffffu, f_mine, i);
-      int l = __shfl_sync(0xffffffffu, l_mine, i);
-      if (z < 0 || z > cb.V + n) { bad = true; break; }
-      const bool self_ref = (z == cb.V + n);     // the entry this very code creates
-      const bool can = prev >= 0 && plen < cb.M && n < cb.cap;
-      if (self_ref) {
-        if (!can) { bad = true; break; }
-        f = pfirst; l = plen + 1;
-      } else if (z >= cb.V + n_batch) {          // created earlier in this batch: read it now
-        f = entry_first(cb, b, z);
-        l = entry_len(cb, b, z);
-      }
-      if (can) {
-        Probe p = warp_probe(table, cb.n_slots, (uint32_t)prev, (uint32_t)f);
-        if (p.found < 0) {
-          if (p.slot >= 0) {
-            if (lane == 0) table[p.slot] = pack_slot((uint32_t)prev, (uint32_t)f, (uint32_t)n);
-            warp_write_entry(cb, b, n, prev, plen, f);
-            ++n;
-            if (n >= cb.cap) st |= Z2Z_ST_CAP_FROZEN;
-            __syncwarp();                        // slot and entry visible to the probes that follow
-          } else {
-            st |= Z2Z_ST_TABLE_FULL;
-          }
-        } else if (self_ref) {                   // that phrase already has another id
-          bad = true; break;
-        }
-      }
-      prev = z; plen = l; pfirst = f;
-      ++valid;
-    }
-  }
-  if (bad) st |= Z2Z_ST_BAD_TOKEN;
-  if (lane == 0) {
-    cb.n[b] = n;
-    if (valid > 0) cb.prev[b] = prev;
-    n_valid[b] = valid;
-    if (st) atomicOr(&cb.status[b], st);
-  }
-}
-
-// The same replay with the sequence's hash table in shared memory and ONE thread walking the
-// probe sequences (as the prompt parse does: a chain that a single warp executes is paced by the
-// instructions it issues, and a warp-wide probe of a table in global memory costs a round trip to
-// L2 per code).  Beside the table the CTA keeps (first token, length) of every entry and the slot
-// each new entry went to: the slot holds (prefix code, last token), which is all that is needed
-// to write the entry's constituent row afterwards, by all threads, walking back through the
-// prefixes (at most M - 1 steps).
-constexpr int kReplaySmemThreads = 128;
-constexpr size_t kReplaySmemMaxBytes = 200 * 1024;
-__host__ __device__ inline size_t replay_smem_bytes(int n_slots, int cap) {
-  return (size_t)n_slots * 8 + (size_t)cap * 4 + (size_t)cap * 2 + 16;
-}
-
-__global__ void __launch_bounds__(kReplaySmemThreads) k_lzw_replay_smem(CbView cb, const int32_t* __restrict__ codes,
-                                                                        const int32_t* __restrict__ code_lens,
-                                                                        int Tc_max, int32_t* __restrict__ n_valid) {
-  extern __shared__ __align__(16) unsigned long long s_table[];
-  uint32_t* const s_fl = reinterpret_cast<uint32_t*>(s_table + cb.n_slots);          // first token << 8 | length
-  uint16_t* const s_slot = reinterpret_cast<uint16_t*>(s_fl + cb.cap);               // slot of each new entry
-  __shared__ int s_code[64];
-  __shared__ int s_n0, s_n1;
-  const int lane = threadIdx.x & 31;
+//
+// One block per sequence; a window of kParseLanes codes at a time (z2z_lzw_dev.cuh).  Code i asks
+// for the entry (code i - 1, first token of code i), which depends on no other code of the window
+// as long as both name entries from before it: the window ends before the first code that does not
+// (the entry it names is known once the codes before it are in), and before the first lane whose bid
+// for a slot lost.  The code that names the very entry it creates can only be the window's first.
+//
+// Bound by the latency of one window (the codes' first tokens and lengths from L2, one lookup, three
+// barriers); one thread that replayed code by code took 170 ns per code with the table in shared
+// memory and 260 with it in global memory.
+template <bool SMEM>
+__global__ void __launch_bounds__(kParseThreads) k_lzw_replay(CbView cb, const int32_t* __restrict__ codes,
+                                                              const int32_t* __restrict__ code_lens, int Tc_max,
+                                                              int32_t* __restrict__ n_valid) {
+  extern __shared__ __align__(16) unsigned char s_parse[];
+  __shared__ int s_code[kParseLanes + 1], s_first[kParseLanes + 1];   // [0]: the code before the window
+  __shared__ uint8_t s_len[kParseLanes + 4];
+  __shared__ uint32_t s_known[4];
+  __shared__ ParseVotes s_votes;
+  __shared__ int s_n1, s_bad0;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
   const int V = cb.V, M = cb.M, cap = cb.cap;
-  unsigned long long* table = cb.hash + (size_t)b * cb.n_slots;
   int32_t* const cons = cb.cons + (size_t)b * cap * M;
-  uint8_t* const len = cb.len + (size_t)b * cap;
-  const int n_start = cb.n[b];
-  for (int i = threadIdx.x; i < cb.n_slots; i += blockDim.x) s_table[i] = table[i];
-  for (int k = threadIdx.x; k < n_start; k += blockDim.x) s_fl[k] = ((uint32_t)cons[(size_t)k * M] << 8) | len[k];
+  uint8_t* const elen = cb.len + (size_t)b * cap;
+  const int n0 = cb.n[b];
   int Tc = code_lens ? code_lens[b] : Tc_max;
   Tc = Tc < 0 ? 0 : (Tc > Tc_max ? Tc_max : Tc);
   const int32_t* zs = codes + (size_t)b * Tc_max;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    const uint32_t pair_mask = (uint32_t)(cb.n_slots - 1) & ~1u;
-    const uint2* const slots = reinterpret_cast<const uint2*>(s_table);
-    int n = n_start;
-    int prev = cb.prev[b];
-    int plen = 0, pfirst = -1;
-    if (prev >= 0) {
-      if (prev < V) { plen = 1; pfirst = prev; }
-      else { const uint32_t fl = s_fl[prev - V]; plen = (int)(fl & 255u); pfirst = (int)(fl >> 8); }
-    }
-    int st = 0, valid = 0;
-    bool bad = false;
-    int ahead = lane < Tc ? zs[lane] : -1;           // codes of the batch after the current one
-    for (int base = 0; base < Tc && !bad; base += 32) {
-      s_code[(base & 32) + lane] = ahead;
-      ahead = base + 32 + lane < Tc ? zs[base + 32 + lane] : -1;
-      __syncwarp();
-      if (lane == 0) {
-        const int cnt = Tc - base < 32 ? Tc - base : 32;
-        for (int i = 0; i < cnt; ++i) {
-          const int z = s_code[(base + i) & 63];
-          if (z < 0 || z > V + n) { bad = true; break; }
-          const bool self_ref = (z == V + n);        // the entry this very code creates
-          const bool can = prev >= 0 && plen < M && n < cap;
-          int f, l;
-          if (self_ref) {
-            if (!can) { bad = true; break; }
-            f = pfirst; l = plen + 1;
-          } else if (z < V) {
-            f = z; l = 1;
-          } else {
-            const uint32_t fl = s_fl[z - V];
-            f = (int)(fl >> 8); l = (int)(fl & 255u);
-          }
-          if (can) {
-            const uint32_t key_hi = ((uint32_t)prev << 8) | ((uint32_t)f >> 16), key_lo = (uint32_t)f & 0xffffu;
-            uint32_t at = hash_pair((uint32_t)prev, (uint32_t)f) & pair_mask;
-            int found = -1, slot = -1;
-            for (int it = 0; it < cb.n_slots; it += 2) {   // bounded: at most the whole table
-              const uint4 pr = *reinterpret_cast<const uint4*>(&slots[at]);      // slots at, at + 1: {lo, hi, lo, hi}
-              if (pr.y == key_hi && (pr.x >> 16) == key_lo) { found = (int)(pr.x & 0xffffu); break; }
-              if (pr.y == 0xffffffffu) { slot = (int)at; break; }
-              if (pr.w == key_hi && (pr.z >> 16) == key_lo) { found = (int)(pr.z & 0xffffu); break; }
-              if (pr.w == 0xffffffffu) { slot = (int)at + 1; break; }
-              at = (at + 2) & pair_mask;
-            }
-            if (found < 0) {
-              if (slot >= 0) {
-                reinterpret_cast<uint2*>(s_table)[slot] = make_uint2((key_lo << 16) | (uint32_t)n, key_hi);
-                s_fl[n] = ((uint32_t)pfirst << 8) | (uint32_t)(plen + 1);
-                s_slot[n] = (uint16_t)slot;
-                ++n;
-                if (n >= cap) st |= Z2Z_ST_CAP_FROZEN;
-              } else {
-                st |= Z2Z_ST_TABLE_FULL;
-              }
-            } else if (self_ref) {                   // that phrase already has another id
-              bad = true; break;
-            }
-          }
-          prev = z; plen = l; pfirst = f;
-          ++valid;
-        }
-      }
-      bad = __shfl_sync(0xffffffffu, bad ? 1 : 0, 0) != 0;
-    }
-    if (lane == 0) {
-      if (bad) st |= Z2Z_ST_BAD_TOKEN;
-      cb.n[b] = n;
-      if (valid > 0) cb.prev[b] = prev;
-      n_valid[b] = valid;
-      if (st) atomicOr(&cb.status[b], st);
-      s_n0 = n_start; s_n1 = n;
-    }
+  ParseTable<SMEM> table;
+  table.open(cb, b, n0, s_parse);
+  if (tid == 0) {
+    const int prev = cb.prev[b];
+    s_code[0] = prev;
+    s_first[0] = prev >= 0 ? entry_first(cb, b, prev) : -1;
+    s_len[0] = (uint8_t)(prev >= 0 ? entry_len(cb, b, prev) : 0);
+    s_n1 = n0;
+    s_bad0 = 0;
   }
   __syncthreads();
-  // constituent rows and lengths of the entries created here
-  for (int e = s_n0 + threadIdx.x; e < s_n1; e += blockDim.x) {
+  if (tid < kParseLanes) {
+    int n = n0, st = 0, base = 0;
+    int z = tid < Tc ? zs[tid] : -1;
+    while (base < Tc) {
+      const int z_ahead = base + kParseLanes + tid < Tc ? zs[base + kParseLanes + tid] : -1;
+      const int i = base + tid;
+      // ---- first token and length of every code, as far as known
+      bool known = i < Tc && z >= 0 && z < V + n;
+      int f = -1, l = 0;
+      if (known) { f = entry_first(cb, b, z); l = entry_len(cb, b, z); }
+      const int prev0 = s_code[0], plen0 = s_len[0];
+      const bool self_ref = tid == 0 && z == V + n && prev0 >= 0 && plen0 < M && n < cap;   // the entry this code creates
+      if (self_ref) { known = true; f = s_first[0]; l = plen0 + 1; }
+      s_code[tid + 1] = z; s_first[tid + 1] = f; s_len[tid + 1] = (uint8_t)l;
+      const uint32_t v_known = __ballot_sync(0xffffffffu, known);
+      if (lane == 0) s_known[warp] = v_known;
+      parse_sync();
+      int limit = kParseLanes;                       // first lane that is not known
+#pragma unroll
+      for (int k = 3; k >= 0; --k)
+        if (~s_known[k]) limit = k * 32 + __ffs((int)~s_known[k]) - 1;
+      // the table in global memory keeps no keys to rebuild a row from later: a row is written at once,
+      // which needs the previous code's row to be there
+      if (!SMEM && limit > 1 && s_code[1] == V + n) limit = 1;
+      const int pz = s_code[tid], pf = s_first[tid], pl = s_len[tid];
+      bool want = tid < limit && pz >= 0 && pl < M && n < cap;
+      int slot = -1;
+      if (want) {
+        const bool found = table.probe((uint32_t)pz, (uint32_t)f, slot) >= 0;
+        if (found && self_ref) s_bad0 = 1;           // that phrase already has another id
+        if (!found && slot < 0) st |= Z2Z_ST_TABLE_FULL;
+        want = !found && slot >= 0;
+      }
+      parse_sync();
+      if (want) table.bid(slot, tid);
+      parse_sync();
+      const bool own = want && table.owns(slot, tid);
+      const uint32_t v_ins = __ballot_sync(0xffffffffu, want), v_lost = __ballot_sync(0xffffffffu, want && !own);
+      if (lane == 0) { s_votes.ins[warp] = v_ins; s_votes.lost[warp] = v_lost; }
+      parse_sync();
+      const ParseVotes votes = s_votes;
+      int stop = parse_first_lost(votes);
+      if (stop > limit) stop = limit;
+      if (s_bad0) stop = 0;
+      const int room = cap - n;
+      const int new_before = parse_count_below(votes.ins, tid);
+      if (own) {
+        const int entry = tid < stop && new_before < room ? n + new_before : -1;
+        table.settle(slot, (uint32_t)pz, (uint32_t)f, entry);
+        if (entry >= 0) {
+          int32_t* row = cons + (size_t)entry * M;
+          row[0] = pf;                               // what later windows ask for; SMEM: the rest follows below
+          if (!SMEM) {
+            const int32_t* from = pz < V ? nullptr : cons + (size_t)(pz - V) * M;
+            for (int j = 1; j < M; ++j) row[j] = j < pl ? from[j] : (j == pl ? f : -1);
+          }
+          elen[entry] = (uint8_t)(pl + 1);
+        }
+      }
+      const int made = parse_count_below(votes.ins, stop);
+      if (made > 0) {
+        n += made < room ? made : room;
+        if (n >= cap) st |= Z2Z_ST_CAP_FROZEN;
+      }
+      if (stop == 0) { st |= Z2Z_ST_BAD_TOKEN; break; }        // the window's first code names no hypertoken
+      const int lz = s_code[stop], lf = s_first[stop], ll = s_len[stop];
+      base += stop;
+      z = stop == kParseLanes ? z_ahead : (base + tid < Tc ? zs[base + tid] : -1);
+      parse_sync();                                  // everybody has read the window's last code
+      if (tid == 0) { s_code[0] = lz; s_first[0] = lf; s_len[0] = (uint8_t)ll; }
+      parse_sync();
+    }
+    if (tid == 0) {
+      s_n1 = n;
+      cb.n[b] = n;
+      if (base > 0) cb.prev[b] = s_code[0];
+      n_valid[b] = base;
+    }
+    if (st) atomicOr(&cb.status[b], st);
+  }
+  __syncthreads();
+  const int n1 = s_n1;
+  table.close(n0, n1);
+  if (!SMEM) return;
+  // constituent rows of the entries created here: walk back through the prefixes (each at most
+  // M - 1 steps); only rows from before this call are read
+  for (int e = n0 + tid; e < n1; e += blockDim.x) {
     int tok[kMaxM];
 #pragma unroll
     for (int j = 0; j < kMaxM; ++j) tok[j] = -1;
-    const int L = (int)(s_fl[e] & 255u);
-    int pos = L - 1, cur = e;
-    for (int hop = 0; hop < kMaxM && pos >= 0; ++hop) {          // bounded: a phrase has at most M tokens
-      const unsigned long long slot = s_table[s_slot[cur]];
-      const int last = (int)((slot >> 16) & 0xffffffu), p = (int)(slot >> 40);
-      tok[pos--] = last;
-      if (pos < 0) break;                                        // (cannot happen: a prefix remains)
-      if (p < V) { tok[pos--] = p; break; }
-      const int k = p - V;
-      if (k < s_n0) {                                            // an entry from before this call: its row is final
-        for (int j = 0; j <= pos; ++j) tok[j] = cons[(size_t)k * M + j];
-        pos = -1;
+    int pos = (int)elen[e] - 1, cur = e;
+    for (int hop = 0; hop < kMaxM && pos > 0; ++hop) {
+      const int p = (int)table.prefix_of(cur);
+#pragma unroll
+      for (int j = 0; j < kMaxM; ++j) if (j == pos) tok[j] = (int)table.token_of(cur);
+      --pos;
+      if (p < V) {
+        if (pos == 0) tok[0] = p;
         break;
       }
-      cur = k;
+      if (p - V < n0) {
+#pragma unroll
+        for (int j = 0; j < kMaxM; ++j) if (j <= pos) tok[j] = cons[(size_t)(p - V) * M + j];
+        break;
+      }
+      cur = p - V;
     }
-    for (int j = 0; j < M; ++j) cons[(size_t)e * M + j] = tok[j];
-    len[e] = (uint8_t)L;
+#pragma unroll
+    for (int j = 0; j < kMaxM; ++j) if (j < M) cons[(size_t)e * M + j] = tok[j];
   }
-  for (int i = threadIdx.x; i < cb.n_slots; i += blockDim.x) table[i] = s_table[i];
 }
 
 // Block-wide exclusive scan of one int per thread (kExpandThreads threads); returns the
@@ -348,14 +289,14 @@ cudaError_t launch_lzw_decode(const CbView& cb, const int32_t* codes, const int3
                               int Tc_max, int replay, int32_t* n_valid, int32_t* tokens,
                               int32_t* token_lens, int T_out_max, cudaStream_t s) {
   if (replay) {
-    const size_t smem = replay_smem_bytes(cb.n_slots, cb.cap);
     cudaError_t e;
-    if (smem <= kReplaySmemMaxBytes && cb.n_slots <= 65536) {    // (a slot number fits 16 bits)
-      e = cudaFuncSetAttribute(k_lzw_replay_smem, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (cb.cap <= kParseSmemMaxCap) {                // as for prompt compression
+      const size_t smem = parse_smem_bytes(cb.n_slots, cb.cap);
+      e = cudaFuncSetAttribute(k_lzw_replay<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
       if (e != cudaSuccess) return e;
-      k_lzw_replay_smem<<<cb.B, kReplaySmemThreads, smem, s>>>(cb, codes, code_lens, Tc_max, n_valid);
+      k_lzw_replay<true><<<cb.B, kParseThreads, smem, s>>>(cb, codes, code_lens, Tc_max, n_valid);
     } else {
-      k_lzw_replay<<<cb.B, 32, 0, s>>>(cb, codes, code_lens, Tc_max, n_valid);
+      k_lzw_replay<false><<<cb.B, kParseThreads, 0, s>>>(cb, codes, code_lens, Tc_max, n_valid);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;

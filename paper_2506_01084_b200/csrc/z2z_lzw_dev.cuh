@@ -147,4 +147,166 @@ __device__ __forceinline__ int warp_lzw_step(const CbView& cb, int b, int z) {
   return warp_lzw_step(cb, b, z, warp_lzw_load(cb, b));
 }
 
+// ---------------------------------------------------------------------------------------------
+// Windowed parsing, shared by prompt compression and by replay of a code stream.
+//
+// Both are defined as a chain of one dictionary lookup per token or code, but the dictionary
+// changes little while 128 of them are looked at: kParseLanes threads look up kParseLanes starting
+// points at once in the dictionary as it was before the window, the results that lie on the chain
+// are picked out, and only the new phrases of the chain are inserted.  A lookup is invalid only if
+// an earlier phrase of the same window inserted exactly the key that it missed; such a lane shares
+// its first empty slot with the earlier lane, so one atomicMin of the lane number per new phrase on
+// that slot finds it (a loser may also be a different key whose probe sequence ends in the same
+// slot; it is treated the same).  The window then ends before the first loser, which is looked up
+// again; the lowest lane never loses, so every window makes progress.
+//
+// ParseTable holds the dictionary during the parse.
+//   SMEM  (codebooks of at most kParseSmemMaxCap entries): the slot array lies in shared memory as
+//         4-byte words (15-bit tag << 16 | entry, four slots per 16-byte load) with the full keys
+//         beside it (6 bytes per entry): 224 KB at 16384 entries, where the 8-byte slots of the
+//         codebook itself would take 256.  New entries go to the codebook's own hash table at the end.
+//   else  the codebook's hash table in global memory is used in place (two slots per 16-byte load).
+// ---------------------------------------------------------------------------------------------
+constexpr int kParseLanes = 128;          // starting points looked up at once (four warps)
+constexpr int kParseThreads = 512;        // the other warps only help to fill and to write back
+constexpr int kParseSmemMaxCap = 16384;
+
+inline size_t parse_smem_bytes(int n_slots, int cap) { return (size_t)n_slots * 4 + (size_t)(cap + (cap & 1)) * 6; }
+
+// Barrier among the kParseLanes parsing threads only.
+__device__ __forceinline__ void parse_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kParseLanes) : "memory"); }
+
+template <bool SMEM>
+struct ParseTable {
+  unsigned long long* hash;   // this sequence's table of the codebook
+  int n_slots;
+  uint32_t* tab;              // SMEM: [n_slots], all-ones = empty
+  uint32_t* key0;             // SMEM: [cap] prefix | (token & 0xff) << 24
+  uint16_t* key1;             // SMEM: [cap] token >> 8
+
+  static __device__ __forceinline__ uint32_t mix(uint32_t prefix, uint32_t token) {
+    return prefix * 0x9E3779B1u ^ hash_token_part(token);
+  }
+  // The slot index takes bits 13 and up of the mix, the tag the 13 bits below and the top two.
+  static __device__ __forceinline__ uint32_t tag_of(uint32_t h) { return (h & 0x1fffu) | ((h >> 30) << 13); }
+
+  // Entry of (prefix, token), or -1 and the first empty slot of its probe sequence (-1: table full).
+  __device__ __forceinline__ int probe(uint32_t prefix, uint32_t token, int& slot) const {
+    slot = -1;
+    if (SMEM) {
+      const uint32_t h = mix(prefix, token), tag = tag_of(h);
+      const uint32_t k0 = prefix | (token << 24), k1 = token >> 8;
+      uint32_t at = (h >> 13) & (uint32_t)(n_slots - 4);
+      for (int it = 0; it < n_slots; it += 4) {                    // bounded: at most the whole table
+        const uint4 g = *reinterpret_cast<const uint4*>(tab + at);
+        const uint32_t v[4] = {g.x, g.y, g.z, g.w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (v[j] == 0xffffffffu) { slot = (int)at + j; return -1; }
+          if ((v[j] >> 16) == tag) {
+            const int e = (int)(v[j] & 0xffffu);
+            if (key0[e] == k0 && key1[e] == (uint16_t)k1) return e;
+          }
+        }
+        at = (at + 4) & (uint32_t)(n_slots - 1);
+      }
+    } else {
+      const unsigned long long key = pack_slot(prefix, token, 0) >> 16;
+      int at = probe_start(n_slots, prefix, token);
+      for (int it = 0; it < n_slots; it += 2) {
+        const ulonglong2 g = __ldcg(reinterpret_cast<const ulonglong2*>(hash + at));
+        if (g.x == kEmptySlot) { slot = at; return -1; }
+        if ((g.x >> 16) == key) return (int)(g.x & 0xffffu);
+        if (g.y == kEmptySlot) { slot = at + 1; return -1; }
+        if ((g.y >> 16) == key) return (int)(g.y & 0xffffu);
+        at = (at + 2) & (n_slots - 1);
+      }
+    }
+    return -1;
+  }
+  // A lane bids for its empty slot; after a barrier the lowest lane among the bidders owns it.
+  __device__ __forceinline__ void bid(int slot, int lane) {
+    if (SMEM) atomicMin(tab + slot, (uint32_t)lane);
+    else atomicMin(hash + slot, (unsigned long long)lane);
+  }
+  __device__ __forceinline__ bool owns(int slot, int lane) const {
+    if (SMEM) return *reinterpret_cast<volatile uint32_t*>(tab + slot) == (uint32_t)lane;
+    return __ldcg(hash + slot) == (unsigned long long)lane;
+  }
+  // The owner turns its bid into the entry, or back into an empty slot.
+  __device__ __forceinline__ void settle(int slot, uint32_t prefix, uint32_t token, int entry) {
+    if (SMEM) {
+      tab[slot] = entry < 0 ? 0xffffffffu : (tag_of(mix(prefix, token)) << 16) | (uint32_t)entry;
+      if (entry >= 0) { key0[entry] = prefix | (token << 24); key1[entry] = (uint16_t)(token >> 8); }
+    } else {
+      hash[slot] = entry < 0 ? kEmptySlot : pack_slot(prefix, token, (uint32_t)entry);
+    }
+  }
+  __device__ __forceinline__ uint32_t prefix_of(int e) const { return key0[e] & 0xffffffu; }
+  __device__ __forceinline__ uint32_t token_of(int e) const { return (key0[e] >> 24) | ((uint32_t)key1[e] << 8); }
+
+  // All threads of the block: carve the shared memory and take over the codebook's n entries.
+  __device__ void open(const CbView& cb, int b, int n, unsigned char* smem) {
+    hash = cb.hash + (size_t)b * cb.n_slots;
+    n_slots = cb.n_slots;
+    if (!SMEM) return;
+    tab = reinterpret_cast<uint32_t*>(smem);
+    key0 = tab + n_slots;
+    key1 = reinterpret_cast<uint16_t*>(key0 + (cb.cap + (cb.cap & 1)));
+    for (int i = threadIdx.x; i < n_slots / 4; i += blockDim.x)
+      reinterpret_cast<uint4*>(tab)[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    if (n <= 0) return;                                   // (the caller synchronises the block)
+    __syncthreads();
+    for (int i = threadIdx.x; i < n_slots; i += blockDim.x) {
+      const unsigned long long s = hash[i];
+      if (s == kEmptySlot) continue;
+      const uint32_t prefix = (uint32_t)(s >> 40), token = (uint32_t)(s >> 16) & 0xffffffu, e = (uint32_t)s & 0xffffu;
+      key0[e] = prefix | (token << 24);
+      key1[e] = (uint16_t)(token >> 8);
+      const uint32_t h = mix(prefix, token), word = (tag_of(h) << 16) | e;
+      uint32_t at = (h >> 13) & (uint32_t)(n_slots - 4);
+      for (int it = 0; it < n_slots; ++it) {
+        if (atomicCAS(tab + at, 0xffffffffu, word) == 0xffffffffu) break;
+        at = (at + 1) & (uint32_t)(n_slots - 1);
+      }
+    }
+  }
+  // All threads of the block: entries [n0, n1) go to the codebook's hash table.
+  __device__ void close(int n0, int n1) {
+    if (!SMEM) return;
+    for (int e = n0 + (int)threadIdx.x; e < n1; e += blockDim.x) {
+      const uint32_t prefix = prefix_of(e), token = token_of(e);
+      int at = probe_start(n_slots, prefix, token);
+      for (int it = 0; it < n_slots; ++it) {
+        if (atomicCAS(hash + at, kEmptySlot, pack_slot(prefix, token, (uint32_t)e)) == kEmptySlot) break;
+        at = (at + 1) & (n_slots - 1);
+      }
+    }
+  }
+};
+
+// What the four parsing warps tell each other inside a window: per warp a mask of lanes on the
+// chain, of those that want a new entry, and of those whose bid lost.
+struct ParseVotes { uint32_t on[4], ins[4], lost[4]; };
+
+// First losing lane of the window (kParseLanes if none).
+__device__ __forceinline__ int parse_first_lost(const ParseVotes& v) {
+  int f = kParseLanes;
+#pragma unroll
+  for (int k = 3; k >= 0; --k)
+    if (v.lost[k]) f = k * 32 + __ffs((int)v.lost[k]) - 1;
+  return f;
+}
+// Bits of m[0..3] below lane `at` of the window.
+__device__ __forceinline__ int parse_count_below(const uint32_t (&m)[4], int at) {
+  int c = 0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int left = at - k * 32;
+    const uint32_t keep = left >= 32 ? 0xffffffffu : (left <= 0 ? 0u : (1u << left) - 1u);
+    c += __popc(m[k] & keep);
+  }
+  return c;
+}
+
 }  // namespace z2z
