@@ -20,6 +20,7 @@ struct z2z_codebook {
   int prefill_strips;        // > 0: fixed number of column strips in the prompt-scoring kernel
   int* h_frozen;             // pinned host word the decode-update kernel writes once every codebook is full
   int epoch;                 // session number: incremented by every z2z_codebook_init
+  size_t part_clean;         // bytes of the stream GEMM's result matrix known to be zero in this session
   void* half_scratch;        // caller's memory for fp16 copies of one encoder's linear-layer weights, or NULL
   size_t half_bytes;
   std::vector<const void*> half_ptrs;   // device addresses of the copies, ABI tensor order
@@ -95,6 +96,7 @@ z2z::EncoderArgs encoder_args(z2z_codebook* cb, const void* table, const z2z_enc
   }
   a.part = reinterpret_cast<float*>(cb->ws + cb->plan.off_part);
   a.part_bytes = cb->plan.part_bytes;
+  a.part_clean = &cb->part_clean;
   a.entries = entries;
   a.err = reinterpret_cast<int*>(cb->ws + cb->plan.off_words);
   return a;
@@ -226,8 +228,10 @@ int32_t z2z_codebook_init(z2z_codebook** cb, const z2z_config* cfg, void* d_ws, 
   v.n_emb = reinterpret_cast<int32_t*>(h->ws + plan.off_n_emb);
   *cb = h;
   Z2Z_CUDA(cudaMemsetAsync(h->ws + plan.off_words, 0, 256, reinterpret_cast<cudaStream_t>(stream)), "codebook_init");
-  // the GEMM result matrix of the hyper-encoder passes is all zero between GEMMs; establish that once
-  Z2Z_CUDA(cudaMemsetAsync(h->ws + plan.off_part, 0, plan.part_bytes, reinterpret_cast<cudaStream_t>(stream)), "codebook_init");
+  // the stream GEMM's result matrix is all zero between GEMMs; the first pass of the session that needs
+  // it clears what it needs (the whole matrix is 280-440 MB at d = 3072 / 4096 and took 28-70 us to clear
+  // here, a decode step uses 1-10 MB of it and a prompt-sized pass none)
+  h->part_clean = 0;
   z2z::ProfScope ps(&h->prof, z2z::kProfLzw, 1, reinterpret_cast<cudaStream_t>(stream));
   Z2Z_CUDA(z2z::launch_codebook_clear(v, reinterpret_cast<cudaStream_t>(stream)), "codebook_init");
   return Z2Z_OK;

@@ -27,7 +27,7 @@
 // whenever no GEMM result is pending.  The element-wise kernel after a GEMM reads each element of
 // that GEMM's result exactly once and stores zero back ("consume and clear"), for every live row
 // of the pass (the GEMM adds nothing to rows beyond them), which restores the invariant for the
-// next GEMM.  The session start clears Y once.
+// next GEMM.  The first pass of a session that needs it clears Y.
 //
 // Launches per layer: GEMM(qkv) -> [+ bias, attention] -> GEMM(o) -> [+ bias + residual,
 // LayerNorm 2] -> GEMM(1) -> [+ bias, GELU] -> GEMM(2) -> [+ bias + residual, LayerNorm 1 of the
@@ -793,7 +793,17 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   auto rlk = narrow ? k_tc_reduce_resid_ln<kNarrowVec4> : k_tc_reduce_resid_ln<kMaxVec4>;
   float* Y = a0.part;                                  // GEMM results, all zero between GEMMs
   const size_t wide = (size_t)(3 * d > dff ? 3 * d : dff);
-  if ((size_t)ng * Rt * wide * sizeof(float) > a0.part_bytes) return cudaErrorMemoryAllocation;
+  const size_t y_bytes = (size_t)ng * Rt * wide * sizeof(float);
+  if (y_bytes > a0.part_bytes) return cudaErrorMemoryAllocation;
+  if (a0.layers > 0 && y_bytes > *a0.part_clean) {
+    // a clear that is only captured into a graph leaves nothing cleared for calls outside of it
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t ce = cudaStreamIsCapturing(s, &cap);
+    if (ce == cudaSuccess)
+      ce = cudaMemsetAsync(reinterpret_cast<char*>(Y) + *a0.part_clean, 0, y_bytes - *a0.part_clean, s);
+    if (ce != cudaSuccess) return ce;
+    if (cap == cudaStreamCaptureStatusNone) *a0.part_clean = y_bytes;
+  }
   auto P2 = [&](auto f) { Ptr2 p; p.p[0] = f(grp[0]); p.p[1] = ng > 1 ? f(grp[1]) : f(grp[0]); return p; };
   auto M2 = [&](auto f) { MPtr2 p; p.p[0] = f(grp[0]); p.p[1] = ng > 1 ? f(grp[1]) : f(grp[0]); return p; };
   auto W = [&](int i) { return P2([&](const EncoderArgs& a) { return a.w[i]; }); };

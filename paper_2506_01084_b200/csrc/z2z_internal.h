@@ -66,6 +66,7 @@ struct EncoderArgs {
   __nv_bfloat16 *Ahl, *Hhl;     // bf16 hi/lo scratch for the tensor-core path
   float* part;                  // fp32 GEMM results [groups][rows][J], zero between GEMMs
   size_t part_bytes;
+  size_t* part_clean;           // host word of the session: leading bytes of `part` known to be zero
   int entries;                  // host bound on the entries of this pass (<= chunk)
   int* err;                     // device error word of the tensor-core kernels
 };
