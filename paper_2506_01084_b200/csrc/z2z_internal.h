@@ -93,6 +93,12 @@ cudaError_t launch_mark_embedded(const CbView& cb, int which, cudaStream_t s);
 cudaError_t run_encoder_pass(const CbView& cb, const EncoderArgs& a, const EntryList& el,
                              bool use_tensor_cores, Prof* prof, cudaStream_t s);
 
+// ---- z2z_encoder_entry.cu --------------------------------------------------------------------
+// Narrow models on the CUDA cores: the whole pass of one or two encoders in one launch.
+bool encoder_entry_applies(int d, int dff, int layers);
+cudaError_t run_encoder_entries(const CbView& cb, const EncoderArgs* groups, int n_groups, const EntryList& el,
+                                Prof* prof, cudaStream_t s);
+
 // ---- z2z_logits.cu ---------------------------------------------------------------------------
 struct LogitsArgs {
   int d, dtype, N;
