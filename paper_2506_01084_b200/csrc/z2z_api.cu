@@ -113,24 +113,25 @@ int check_encoder(z2z_codebook* cb, const z2z_encoder_weights* enc) {
   return Z2Z_OK;
 }
 
-// Rows at or above which the prompt-scoring kernel (CTA pairs, 256 x 256 tiles) takes over from
-// the weight-streaming kernel: enough row tiles to give every cluster work.
-constexpr int kPrefillMinRows = 2048;
-
 int logits_call(z2z_codebook* cb, z2z::LogitsArgs a, cudaStream_t s, z2z::LogitsPartInfo* info = nullptr) {
   // rows are processed in blocks so that the partial-reduction scratch stays bounded
   const int N = a.N;
   const size_t esz = cb->cfg.dtype == Z2Z_DTYPE_FP32 ? 4 : 2;
   const size_t ldbg = (size_t)cb->cfg.V + cb->cfg.cap;
   const bool tc = cb->use_tensor_cores && z2z::logits_tc_supported(cb->cfg.d, cb->cfg.dtype);
-  const bool prefill = tc && info == nullptr && z2z::prefill_logits_supported(cb->cfg.d, cb->cfg.dtype) &&
-                       (cb->use_tensor_cores == 2 || N >= kPrefillMinRows);
+  // By rows: up to 32 the decode kernel; up to 128 rows of a batch (every row another sequence) the
+  // single-CTA stream, whose 128-row tiles and narrow hypertoken granules waste less than pairs with 256
+  // (V = 12000, d = 2176, 128 sequences: 54 against 69 us); more rows, or positions of few sequences, the
+  // CTA pairs (V = 32064, d = 3072, 128 positions of 5 sequences: 82 against 115 us).
+  const bool decode = tc && z2z::decode_logits_applies(a);
+  const bool batch = info != nullptr || (N <= 128 && a.row_seq == nullptr);
+  const bool prefill = tc && info == nullptr && (cb->use_tensor_cores == 2 || !(decode || batch));
   long long chunk = z2z::kLogitRowChunk;
   int prefill_strips = cb->prefill_strips;
   if (prefill) {
     // the number of column strips is fixed for the whole call; when the partial-reduction scratch
     // cannot take all rows at that split, the rows go out in launches of equal size
-    if (prefill_strips <= 0) prefill_strips = z2z::prefill_logits_strips(N, cb->cfg.d);
+    if (prefill_strips <= 0) prefill_strips = z2z::prefill_logits_strips(N, cb->cfg.d, cb->cfg.V);
     const long long cap_rows = z2z::prefill_logits_max_rows(cb->plan.lpart_bytes, cb->plan.plan_bytes, prefill_strips);
     if (cap_rows < 256) return fail(Z2Z_ERR_WORKSPACE_TOO_SMALL, "logits scratch too small for one row tile");
     chunk = cap_rows;
@@ -158,9 +159,11 @@ int logits_call(z2z_codebook* cb, z2z::LogitsArgs a, cudaStream_t s, z2z::Logits
     int* words = reinterpret_cast<int*>(cb->ws + cb->plan.off_words);
     if (prefill) {
       Z2Z_CUDA(z2z::run_logits_prefill(cb->view, c, reinterpret_cast<int32_t*>(cb->ws + cb->plan.off_plan), words,
-                                       prefill_strips, &cb->prof, s), "logits (prompt scoring)");
+                                       prefill_strips, &cb->prof, s), "logits (CTA pairs)");
+    } else if (decode) {
+      Z2Z_CUDA(z2z::run_logits_decode(cb->view, c, words + 2, words, info, &cb->prof, s), "logits (decode batch)");
     } else if (tc) {
-      Z2Z_CUDA(z2z::run_logits_tc(cb->view, c, words + 1, words, info, &cb->prof, s), "logits (tensor cores)");
+      Z2Z_CUDA(z2z::run_logits_stream(cb->view, c, words + 1, words, info, &cb->prof, s), "logits (batch)");
     } else {
       Z2Z_CUDA(z2z::run_logits_simt(cb->view, c, info, &cb->prof, s), "logits");
     }

@@ -205,4 +205,76 @@ struct RowRed {
   }
 };
 
+// Folds 32 consecutive logits of one hidden row into its running reduction; those at or beyond `limit`
+// do not exist for the row.  The maximum of the 32 first, then one exp2 per logit against it: a
+// column costs about five instructions, where RowRed::add takes both of its branches in a warp whose
+// rows reach new maxima at different columns (250 cycles per column measured, which made a 256 x 256
+// tile's epilogue take 34 us, twice its MMAs at d = 4096).
+__device__ __forceinline__ void fold_row32(uint32_t (&v)[32], int limit, int col, RowRed& red) {
+  if (limit <= 0) return;
+  if (limit < 32) {
+#pragma unroll
+    for (int x = 0; x < 32; ++x) if (x >= limit) v[x] = 0xff800000u;          // -inf adds nothing
+  }
+  float cm = __uint_as_float(v[0]);
+#pragma unroll
+  for (int x = 1; x < 32; ++x) cm = fmaxf(cm, __uint_as_float(v[x]));
+  if (cm == INFINITY || red.m == INFINITY) {      // an overflowed logit: differences to it are not numbers
+#pragma unroll
+    for (int x = 0; x < 32; ++x) if (x < limit) red.add(__uint_as_float(v[x]), col + x);
+    return;
+  }
+  constexpr float kLog2e = 1.4426950408889634f;
+  if (cm > red.m) {                               // a new maximum: its first occurrence wins ties
+    int at = 31;
+#pragma unroll
+    for (int x = 30; x >= 0; --x) at = __uint_as_float(v[x]) == cm ? x : at;
+    red.idx = col + at;
+    red.s *= exp2f((red.m - cm) * kLog2e);
+    red.m = cm;
+  }
+  float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+  auto ex = [&](uint32_t w) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"((__uint_as_float(w) - red.m) * kLog2e));
+    return y;
+  };
+#pragma unroll
+  for (int x = 0; x < 32; x += 4) { a0 += ex(v[x]); a1 += ex(v[x + 1]); a2 += ex(v[x + 2]); a3 += ex(v[x + 3]); }
+  red.s += (a0 + a1) + (a2 + a3);
+}
+// v[i] for a lane-dependent i in [0, 32), without indexing registers.
+__device__ __forceinline__ float pick32(const uint32_t (&v)[32], int i) {
+  uint32_t r = v[0];
+#pragma unroll
+  for (int x = 1; x < 32; ++x) r = i == x ? v[x] : r;
+  return __uint_as_float(r);
+}
+
+// Gumbel-max over 32 consecutive logits of one hidden row (those at or beyond `limit` do not exist).
+// Nearly every column loses, and that is seen without its two logarithms: its noise g = -log(-log u) can
+// beat the running best only if g > t = best - l / T, and -log u >= 1 - u, so that 1 - u > exp(-t) rules it
+// out.  The margin of 1e-3 is far above the rounding of either side (a few 1e-6): whatever the comparison
+// of the scores themselves would let through is computed in full.
+__device__ __forceinline__ void sample_row32(const uint32_t (&v)[32], int limit, int col0, float inv_t, uint32_t row,
+                                             uint32_t c2, uint32_t c3, uint32_t k0, uint32_t k1, RowRed& red) {
+  Philox4 px{0, 0, 0, 0};
+  int blk = -1;
+#pragma unroll
+  for (int x = 0; x < 32; ++x) {
+    if (x < limit) {
+      const int col = col0 + x;
+      if ((col >> 2) != blk) {
+        blk = col >> 2;
+        px = philox4x32_10((uint32_t)blk, row, c2, c3, k0, k1);
+      }
+      const uint32_t w = philox_word(px, col & 3);
+      const float l = __uint_as_float(v[x]);
+      const float t = fmaf(l, -inv_t, red.gm);
+      const float left = ((float)(8388608u - (w >> 9)) - 0.5f) * 1.1920928955078125e-07f;          // 1 - u, exact
+      if (!(left > 1.001f * __expf(-t))) red.add_score(fmaf(l, inv_t, gumbel_from_word(w)), col);
+    }
+  }
+}
+
 }  // namespace z2z

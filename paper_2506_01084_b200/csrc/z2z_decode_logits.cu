@@ -406,10 +406,7 @@ __global__ void __launch_bounds__(128) k_decode_logits_merge(LogitsArgs a, int s
   if (r >= a.N) return;
   const LogitPartial* lp = reinterpret_cast<const LogitPartial*>(a.lpart) + (size_t)r * stride;
   RowRed red; red.init();
-  for (int g = lane; g < count; g += 32) {
-    RowRed o; o.m = lp[g].m; o.s = lp[g].s; o.idx = lp[g].idx; o.gm = lp[g].gm; o.gidx = lp[g].gidx;
-    red.merge(o);
-  }
+  for (int g = lane; g < count; g += 32) red.merge(load_partial(lp + g));
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     RowRed o;
@@ -435,9 +432,10 @@ __global__ void k_decode_fill_nan(float* p, int n) {
 
 }  // namespace
 
-// Decode batches: at most 32 hidden rows, with any outputs; d a multiple of 256.
+// Decode batches: at most 32 hidden rows, with any outputs; d a multiple of 128 (a 64-row job's stage
+// holds two k-blocks).
 bool decode_logits_applies(const LogitsArgs& a) {
-  return a.dtype == Z2Z_DTYPE_BF16 && a.d % 256 == 0 && a.N <= 32;
+  return a.dtype == Z2Z_DTYPE_BF16 && a.d % 128 == 0 && a.N <= 32;
 }
 
 template <int NB, bool GENERIC>
@@ -476,8 +474,8 @@ cudaError_t run_logits_decode(const CbView& cb, const LogitsArgs& a, int* counte
   p.counters = counters; p.err = err_word;
   // hidden rows stay resident in shared memory when they take at most 64 KB
   const bool resident = (size_t)p.ksteps * p.hid_rows * 128 <= 64 * 1024;
-  p.hid_box_kb = 4;
-  for (int k = 16; k >= 4; --k) if (p.ksteps % k == 0) { p.hid_box_kb = k; break; }
+  p.hid_box_kb = 2;
+  for (int k = 16; k >= 2; --k) if (p.ksteps % k == 0) { p.hid_box_kb = k; break; }
   const int gs = (cb.V + kGran - 1) / kGran;
   const int grid = gs < n_sm ? gs : n_sm;
   // fixed share: nine tenths of W_U; the rest and all of U_h are pooled

@@ -27,10 +27,7 @@ __global__ void __launch_bounds__(1024) k_decode_update(CbView cb, DecodeUpdateA
     // ---- merge the partial reductions of hidden row b
     const LogitPartial* lp = a.lpart + (size_t)b * a.part_stride;
     RowRed red; red.init();
-    for (int g = lane; g < a.part_count; g += 32) {
-      RowRed o; o.m = lp[g].m; o.s = lp[g].s; o.idx = lp[g].idx; o.gm = lp[g].gm; o.gidx = lp[g].gidx;
-      red.merge(o);
-    }
+    for (int g = lane; g < a.part_count; g += 32) red.merge(load_partial(lp + g));
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
       RowRed o;

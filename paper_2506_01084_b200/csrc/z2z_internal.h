@@ -116,22 +116,27 @@ struct LogitsArgs {
 };
 // Partial reduction of one hidden row over a subset of the columns.
 struct __align__(32) LogitPartial { float m, s; int idx; float gm; int gidx; int pad[3]; };
+__device__ __forceinline__ RowRed load_partial(const LogitPartial* p) {      // two loads instead of five
+  const float4 a = *reinterpret_cast<const float4*>(p);
+  RowRed r;
+  r.m = a.x; r.s = a.y; r.idx = __float_as_int(a.z); r.gm = a.w; r.gidx = p->gidx;
+  return r;
+}
 // Where a logits kernel left its partials when the caller merges them itself (decode step).
 struct LogitsPartInfo { int stride, count; };
 // When `info` is given the merge kernel is skipped and the layout of the partials is returned.
 cudaError_t run_logits_simt(const CbView& cb, const LogitsArgs& a, LogitsPartInfo* info, Prof* prof,
                             cudaStream_t s);
-// Tensor-core (tcgen05) version for bf16 (d % 64 == 0).
-cudaError_t run_logits_tc(const CbView& cb, const LogitsArgs& a, int* vt_word, int* err_word,
-                          LogitsPartInfo* info, Prof* prof, cudaStream_t s);
+// Batches of 33 .. 128 rows of different sequences (bf16, d % 64 == 0).
+cudaError_t run_logits_stream(const CbView& cb, const LogitsArgs& a, int* vt_word, int* err_word,
+                              LogitsPartInfo* info, Prof* prof, cudaStream_t s);
 
 // ---- z2z_prefill_logits.cu -------------------------------------------------------------------
-// Same outputs as run_logits_tc, for many hidden rows (bf16, d % 64 == 0).  `plan` is scratch for
-// 3 int32 per 256-row tile.  strips_override > 0 fixes the number of column strips (tests).
-bool prefill_logits_supported(int d, int dtype);
+// Many hidden rows, or positions of few sequences (bf16, d % 64 == 0).  `plan` is scratch for 3 int32 per 256-row tile.
+// strips_override > 0 fixes the number of column strips (tests).
 // Rows one launch can take with the given scratch when `strips` partials per row are needed.
 long long prefill_logits_max_rows(size_t lpart_bytes, size_t plan_bytes, int strips);
-int prefill_logits_strips(int N, int d);
+int prefill_logits_strips(int N, int d, int V);
 cudaError_t run_logits_prefill(const CbView& cb, const LogitsArgs& a, int32_t* plan, int* err_word,
                                int strips_override, Prof* prof, cudaStream_t s);
 

@@ -11,7 +11,7 @@
 //     N operand, as wide as the rows that exist; work is cut stream-K style, every CTA gets the
 //     same number of (tile, k-step) units and adds its accumulators into one fp32 result matrix
 //     with reductions in global memory (sums of two or three partial tiles in arrival order);
-//   * joint logits for 33 .. 2047 hidden rows (k_stream_logits; paper Section 2.3 steps 7-9):
+//   * joint logits for 33 .. 128 hidden rows of a batch (k_stream_logits; paper Section 2.3 steps 7-9):
 //     the hidden rows are the 128-row M operand, tiles run over W_U and then over the visible
 //     rows of each sequence's U_h; the epilogue keeps max / sum-exp / argmax / best perturbed
 //     score per hidden row in registers, so the logits are never written.  Only the hidden rows
@@ -488,25 +488,16 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
           uint32_t v[32];
           tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + buf * NT + c0, v);
           tmem_ld_wait();
-          Philox4 px{0, 0, 0, 0};
-          int px_blk = -1;
+          const int col0 = j.col0 + c0;
+          if (a.select == Z2Z_SELECT_GUMBEL) sample_row32(v, limit - c0, col0, a.inv_temperature, (uint32_t)(a.row_base + r), c2, c3, k0, k1, red);
+          if (a.logits_debug) {
 #pragma unroll
-          for (int x = 0; x < 32; ++x) {
-            if (c0 + x < limit) {
-              const float l = __uint_as_float(v[x]);
-              const int col = j.col0 + c0 + x;
-              red.add(l, col);
-              if (a.select == Z2Z_SELECT_GUMBEL) {
-                if ((col >> 2) != px_blk) {
-                  px_blk = col >> 2;
-                  px = philox4x32_10((uint32_t)px_blk, (uint32_t)(a.row_base + r), c2, c3, k0, k1);
-                }
-                red.add_score(fmaf(l, a.inv_temperature, gumbel_from_word(philox_word(px, col & 3))), col);
-              }
-              if (a.logits_debug) a.logits_debug[(size_t)r * ldbg + col] = l;
-              if (col == my_tgt && a.target_logit) a.target_logit[r] = l;
-            }
+            for (int x = 0; x < 32; ++x)
+              if (c0 + x < limit) a.logits_debug[(size_t)r * ldbg + col0 + x] = __uint_as_float(v[x]);
           }
+          const int at = my_tgt - col0;                 // the row's target column, if it lies here and exists
+          if (at >= 0 && at < 32 && at < limit - c0 && a.target_logit) a.target_logit[r] = pick32(v, at);
+          fold_row32(v, limit - c0, col0, red);
         }
       }
       tc_fence_before();
@@ -534,8 +525,7 @@ __global__ void __launch_bounds__(128) k_stream_logits_merge(StreamLogitsParams 
   const LogitPartial* lp = reinterpret_cast<const LogitPartial*>(a.lpart) + (size_t)r * p.part_stride;
   RowRed red; red.init();
   for (int g = lane; g <= (int)(last - first); g += 32) {
-    RowRed o; o.m = lp[g].m; o.s = lp[g].s; o.idx = lp[g].idx; o.gm = lp[g].gm; o.gidx = lp[g].gidx;
-    red.merge(o);
+    red.merge(load_partial(lp + g));
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
@@ -705,11 +695,8 @@ static cudaError_t launch_logits_t(const StreamLogitsParams& p, const LogitMaps*
   return cudaGetLastError();
 }
 
-bool logits_tc_supported(int d, int dtype) { return dtype == Z2Z_DTYPE_BF16 && d % 64 == 0; }
-
-cudaError_t run_logits_tc(const CbView& cb, const LogitsArgs& a, int* vt_word, int* err_word,
-                          LogitsPartInfo* info, Prof* prof, cudaStream_t s) {
-  if (decode_logits_applies(a)) return run_logits_decode(cb, a, vt_word + 1, err_word, info, prof, s);
+cudaError_t run_logits_stream(const CbView& cb, const LogitsArgs& a, int* vt_word, int* err_word,
+                              LogitsPartInfo* info, Prof* prof, cudaStream_t s) {
   static int n_sm = 0;
   if (!n_sm) {
     int dev = 0;

@@ -10,6 +10,7 @@ namespace z2z {
 
 constexpr int kMaxStages = 8;
 constexpr int kGemmNT = 128;                    // weight rows per tile of the stream-K GEMM
+
 constexpr int kLogitNT = 128, kLogitKSB = 1;
 constexpr int kLogitGran = 32;                  // scheduling granule of the logits kernel, in weight rows (TMA boxes of
                                                 // fewer rows stream several times slower)
@@ -32,7 +33,7 @@ struct DecodeLogitMaps {
 struct DecodeLogitsParams {
   CbView cb;
   LogitsArgs la;
-  int ksteps;            // d / 64 (a multiple of 4)
+  int ksteps;            // d / 64 (a multiple of 2)
   int hid_rows;          // hidden rows held per k-block in shared memory (N rounded up to 8)
   int hid_box_kb;        // k-blocks per TMA box of the resident hidden rows
   int stages;            // stages of the load ring
@@ -83,18 +84,20 @@ struct StreamLogitsParams {
   int* err;
 };
 
-// Prompt-scoring logits kernel (z2z_prefill_logits.cu): CTA pairs, 256 x 256 tiles.
-constexpr int kPrefillMaxStrips = 8;            // column strips a row tile may be cut into
+// Logits kernel for many rows (z2z_prefill_logits.cu): CTA pairs, tiles of 256 x up to 256.
+constexpr int kPrefillMaxStrips = 8;            // column strips a row tile is cut into when there are many row tiles
 struct PrefillLogitsParams {
   CbView cb;
   LogitsArgs la;
   int ksteps;            // d / 64
   int row_tiles;         // ceil(N / 256)
-  int n_static;          // ceil(V / 256)
+  int cta_rows;          // hidden rows per CTA (128, fewer when there are few rows in all)
+  int n_static;          // 64-column granules of W_U
   int strips;            // column strips per row tile = partial reductions per hidden row
+  int stages;            // of the load ring
   int32_t* tile_lo;      // [row_tiles] lowest / highest sequence owning a row of the tile
   int32_t* tile_hi;
-  int32_t* tile_nh;      // [row_tiles] hypertoken column tiles of the tile
+  int32_t* tile_nh;      // [row_tiles] cost of the tile's hypertoken columns
   int* err;
 };
 
@@ -117,8 +120,8 @@ cudaError_t launch_pair_gemm(const PairGemmParams& p, const void* act, const voi
 
 bool make_tmap_bf16(CUtensorMap* m, const void* base, long long rows, long long cols, int box_rows);
 int stream_gemm_stages(int ksb, int a_box_rows);
-cudaError_t launch_stream_gemm(const StreamGemmParams& p, const CUtensorMap* maps, int grid, cudaStream_t s);
 cudaError_t launch_stream_logits(const StreamLogitsParams& p, const LogitMaps* maps, int grid, bool merge,
                                  Prof* prof, cudaStream_t s);
+cudaError_t launch_stream_gemm(const StreamGemmParams& p, const CUtensorMap* maps, int grid, cudaStream_t s);
 
 }  // namespace z2z

@@ -1,0 +1,113 @@
+"""Joint logits at the sizes where the CTA-pair kernel's split can go wrong: every number of rows around a
+change of the rows per CTA or of the row tiles, vocabularies that end inside a granule of 64, widths that
+are no multiple of 256 (also for decode batches of up to 32 rows), sequences with 0, 1, 63 .. 65 and 300
+visible entries, rows without an owner, targets in and outside of what a row sees.  Against fp64 sums."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2506_01084_b200 import binding as zb
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _session(V, d, B, cap, counts, seed):
+    """Codebooks of exactly the given sizes: runs of distinct pairs compressed as prompts."""
+    cb = zb.Codebook(zb.make_config(V, d, 2, cap, B, "bf16", 0, 1, 8), DEV)
+    T = 2 * max(max(counts), 1) + 2
+    tok = np.zeros((B, T), dtype=np.int32)
+    lens = []
+    for b, n in enumerate(counts):
+        seen, row = set(), [b % V]
+        rng = np.random.default_rng(seed + b)
+        while len(seen) < n:                             # a walk whose every step is a pair not seen before
+            c = int(rng.integers(0, V))
+            if (row[-1], c) not in seen:
+                seen.add((row[-1], c))
+                row.append(c)
+        tok[b, :len(row)] = row
+        lens.append(len(row))
+    codes = torch.zeros(B, T, dtype=torch.int32, device=DEV)
+    clen = torch.zeros(B, dtype=torch.int32, device=DEV)
+    zb.z2z_lzw_encode(cb, torch.from_numpy(tok).to(DEV), torch.tensor(lens, dtype=torch.int32, device=DEV), codes, clen, None)
+    _, n = zb.z2z_status(cb)
+    assert [int(x) for x in n] == list(counts)
+    return cb
+
+
+@pytest.mark.parametrize("B", [33, 90, 128, 200])
+@pytest.mark.parametrize("V,d", [(1003, 192), (4097, 1152)])
+def test_sampled_batch_of_one_row_per_sequence(V, d, B):
+    """Gumbel-max over every column, in and beyond the batch kernel's 128 rows: the sample has to be the
+    argmax of the perturbed scores, which the oracle draws column by column."""
+    from oracle import logits as olg
+    counts = [(7 * b) % 70 for b in range(B)]
+    cap, T, seed, step = 80, 0.9, 77, 5
+    cb = _session(V, d, B, cap, counts, 4)
+    g = torch.Generator(device=DEV)
+    g.manual_seed(B + V)
+    rnd = lambda *s, std: (torch.randn(*s, generator=g, device=DEV) * std).to(torch.bfloat16)
+    hid, WU, Uh = rnd(B, d, std=1.0), rnd(V, d, std=0.05), rnd(B, cap, d, std=0.05)
+    lse, mx = torch.zeros(B, device=DEV), torch.zeros(B, device=DEV)
+    am, sm = torch.zeros(B, dtype=torch.int32, device=DEV), torch.zeros(B, dtype=torch.int32, device=DEV)
+    zb.z2z_dynamic_logits(cb, hid, None, None, WU, Uh, zb.SELECT_GUMBEL, T, seed, step, None, lse, am, mx, sm)
+    h, w, u = hid.double().cpu().numpy(), WU.double().cpu().numpy(), Uh.double().cpu().numpy()
+    for r in range(B):
+        l = np.concatenate([w @ h[r], u[r, :counts[r]] @ h[r]])
+        choice, scores, gap = olg.select(l, 1, T, seed, step, r)
+        # a score is a logit (error below 1e-4 here) plus noise in fp32 (error below 1e-5 at |g| < 20)
+        assert scores[int(sm[r])] >= scores[choice] - 5e-4
+        assert abs(float(lse[r]) - (l.max() + np.log(np.exp(l - l.max()).sum()))) < 1e-4
+
+
+@pytest.mark.parametrize("N", [1, 31, 32, 33, 64, 65, 96, 128, 129, 192, 193, 256, 257, 511, 700])
+@pytest.mark.parametrize("V,d", [(4097, 192), (1000, 1152), (130, 2176)])
+def test_joint_logits_against_fp64(V, d, N):
+    counts = [0, 1, 63, 64, 65, 300]
+    B, cap = len(counts), 320
+    cb = _session(V, d, B, cap, counts, 3)
+    g = torch.Generator(device=DEV)
+    g.manual_seed(N * 7 + V)
+    rnd = lambda *s, std: (torch.randn(*s, generator=g, device=DEV) * std).to(torch.bfloat16)
+    hid, WU, Uh = rnd(N, d, std=1.0), rnd(V, d, std=0.05), rnd(B, cap, d, std=0.05)
+    seq = torch.randint(0, B, (N,), generator=g, device=DEV, dtype=torch.int32).sort().values
+    nvis = torch.randint(0, cap, (N,), generator=g, device=DEV, dtype=torch.int32)
+    if N > 40:
+        seq[N // 2] = -1                                  # a row without an owner sees nothing
+    tgt = torch.randint(0, V + cap, (N,), generator=g, device=DEV, dtype=torch.int32)
+    out = dict(lse=torch.zeros(N, device=DEV), am=torch.zeros(N, dtype=torch.int32, device=DEV),
+               mx=torch.zeros(N, device=DEV), tl=torch.zeros(N, device=DEV))
+    zb.z2z_dynamic_logits(cb, hid, seq, nvis, WU, Uh, zb.SELECT_ARGMAX, 1.0, 0, 0, tgt, out["lse"], out["am"], out["mx"],
+                          None, out["tl"])
+    st, _ = zb.z2z_status(cb)
+    assert all(int(s) & zb.ST_WAIT_TIMEOUT == 0 for s in st)
+    h, w, u = hid.double(), WU.double(), Uh.double()
+    for r in range(N):
+        s = int(seq[r])
+        if s < 0:
+            continue
+        vis = min(int(nvis[r]), counts[s])
+        l = torch.cat([w @ h[r], u[s, :vis] @ h[r]])
+        # fp32 sums of d products of size std 0.05: relative 2^-24 sqrt(d) of their 2-norm, well under 2e-5
+        assert abs(float(out["lse"][r]) - float(torch.logsumexp(l, 0))) < 2e-5 * (1 + float(l.abs().max()))
+        assert abs(float(out["mx"][r]) - float(l.max())) < 2e-5 * (1 + float(l.abs().max()))
+        assert float(l.max() - l[int(out["am"][r])]) < 4e-5 * (1 + float(l.abs().max()))
+        t = int(tgt[r])
+        if t < V + vis:
+            assert abs(float(out["tl"][r]) - float(l[t])) < 2e-5 * (1 + float(l.abs().max()))
+        else:
+            assert torch.isnan(out["tl"][r])
+
+
+def test_overflowed_logit_keeps_its_row_a_number():
+    N = 100
+    cb = _session(300, 256, N, 8, [1] * N, 5)
+    hid = torch.ones(N, 256, dtype=torch.bfloat16, device=DEV)
+    WU = torch.zeros(300, 256, dtype=torch.bfloat16, device=DEV)
+    WU[77] = 3e38                                         # one column of +inf, the others 0
+    Uh = torch.zeros(N, 8, 256, dtype=torch.bfloat16, device=DEV)
+    lse, mx = torch.zeros(N, device=DEV), torch.zeros(N, device=DEV)
+    am = torch.zeros(N, dtype=torch.int32, device=DEV)
+    zb.z2z_dynamic_logits(cb, hid, None, None, WU, Uh, zb.SELECT_ARGMAX, 1.0, 0, 0, None, lse, am, mx)
+    assert torch.all(torch.isposinf(lse)) and torch.all(torch.isposinf(mx)) and torch.all(am == 77)
