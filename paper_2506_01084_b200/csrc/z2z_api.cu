@@ -342,6 +342,10 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
     a.w_half = cb->half_ptrs.data();
   }
   for (int c = 0; c < n_chunks; ++c) {
+    // a short call, and the rest of a long one, is sized for what it can hold: 16 entries at d = 4096 took
+    // 0.86 ms per encoder when every pass was sized for 1024, and take 0.22
+    const long long left = bound - (long long)c * el.chunk;
+    a.entries = left < el.chunk ? (int)left : el.chunk;
     {
       z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 1, s);
       Z2Z_CUDA(z2z::launch_entry_fill(cb->view, which, d_first, nullptr, el, c, s), "hyper_embed");

@@ -1,5 +1,5 @@
 // Hyper-encoder pass on the tensor cores (bf16 weights): the linear layers run in the stream-K
-// tcgen05 kernel of z2z_stream.cu; this file holds the element-wise kernels between them and the
+// tcgen05 kernels of z2z_stream.cu and z2z_stream_pair.cu (prompt-sized passes: z2z_pair_gemm.cu); this file holds the element-wise kernels between them and the
 // host-side sequencing.  Both encoders (embedding side and unembedding side, paper Section 2.2)
 // go through the same launches as two "groups".
 //
@@ -52,7 +52,13 @@ constexpr int kNT = kGemmNT;
 constexpr int kRowThreads = 256;
 constexpr int kMaxVec4 = 8;            // float4 per thread in the row kernels: d <= 8192
 constexpr int kNarrowVec4 = 4;         // ... and for d <= 4096, where half the registers do
-constexpr int kPairPassMinRows = 1024; // passes of at least this many rows use the CTA-pair GEMM
+// Which linear-layer kernel a pass takes, by its row capacity.  Up to 128 rows one CTA per weight tile streams
+// best (24 rows, d = 3072, both encoders: 249 us a step against 272 with pairs; 96 rows, d = 4096: equal);
+// beyond, CTA pairs carry up to 256 rows on one stream (270 rows, one encoder: 486 -> 327 us a step).  From 900
+// rows on whole output tiles beat the stream (one encoder, d = 3072, 900 rows: 767 against 749 us, 1023 rows:
+// 860 against 949; d = 4096, 800 rows: 1116 against 1085, 1024 rows: 1138 against 1197).
+constexpr int kStreamSingleRows = 128;
+constexpr int kPairPassMinRows = 900;
 
 struct Ptr2 { const void* p[2]; };
 struct MPtr2 { void* p[2]; };
@@ -786,7 +792,6 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   const int R = E * M;                                 // row capacity of this pass
   if (ng == 1 && R >= kPairPassMinRows) return run_encoder_pass_pair(cb, a0, el, E, prof, s);
   const int Rt = (R + 7) / 8 * 8;                      // rows of the result matrix per group
-  const int row_tiles = (Rt + 127) / 128;
   const int* total = el.row_off + E;                   // packed rows of this pass (device word)
   const int n_sm = sm_count();
   const bool narrow = d <= 4 * kRowThreads * kNarrowVec4;      // a row fits four float4 per thread
@@ -816,25 +821,22 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
 
   // one GEMM: activations (hi/lo of packed row r in operand rows 2r, 2r + 1; K columns) x weight
   // [J, K], added into Y[group][Rt][J]
+  const bool paired = R > kStreamSingleRows;
+  const int ksb = paired ? stream_pair_ksb(R) : stream_gemm_ksb(R);
+  StreamGemmMaps maps;
   auto gemm = [&](const MPtr2& act, int K, int widx, int J) -> cudaError_t {
-    StreamGemmParams p{};
-    p.row_tiles = row_tiles; p.groups = ng; p.tiles_per_group = J / kNT;
-    p.a_box_rows = row_tiles == 1 ? 2 * Rt : 256;      // one box per stage: all operand rows of a row tile
-    // two k-blocks per stage (fewer TMA operations per byte) while at least four stages still fit
-    p.ksb = (K % 128 == 0 && stream_gemm_stages(2, p.a_box_rows) >= 4) ? 2 : 1;
-    p.ksteps = (K / 64 + p.ksb - 1) / p.ksb;
-    p.out = Y; p.J = J; p.Rt = Rt; p.rows_dev = total;
-    p.err = a0.err;
-    const long long tiles = (long long)row_tiles * ng * p.tiles_per_group;
-    const int G = tiles * p.ksteps < n_sm ? (int)(tiles * p.ksteps) : n_sm;     // every CTA owns >= 1 unit
-    CUtensorMap maps[4];
-    for (int g = 0; g < 2; ++g) {
-      const int gg = g < ng ? g : 0;
-      if (!make_tmap_bf16_kblocks(&maps[g], act.p[gg], 2ll * Rt, K, p.a_box_rows, p.ksb)) return cudaErrorInvalidValue;
-      if (!make_tmap_bf16_kblocks(&maps[2 + g], grp[gg].w[widx], J, K, kNT, p.ksb)) return cudaErrorInvalidValue;
+    for (int g = 0; g < ng; ++g) {
+      if (!(paired ? stream_pair_act_maps : stream_gemm_act_maps)(maps.a[g], act.p[g], Rt, K, R)) return cudaErrorInvalidValue;
+      if (!make_tmap_bf16_kblocks(&maps.w[g], grp[g].w[widx], J, K, kNT, ksb)) return cudaErrorInvalidValue;
     }
+    if (ng == 1) { maps.w[1] = maps.w[0]; for (int i = 0; i < 8; ++i) maps.a[1][i] = maps.a[0][i]; }
+    auto fill = [&](auto p) {
+      p.groups = ng; p.ksteps = K / (64 * ksb); p.R = R; p.out = Y; p.J = J; p.Rt = Rt; p.rows_dev = total; p.err = a0.err;
+      return p;
+    };
     ProfScope ps(prof, kProfEncGemm, 1, s);
-    return launch_stream_gemm(p, maps, G, s);
+    if (paired) return launch_stream_pair(fill(StreamPairParams{}), maps, n_sm, s);
+    return launch_stream_gemm(fill(StreamGemmParams{}), maps, n_sm, s);
   };
 
   if (!rows_mapped) {

@@ -215,12 +215,12 @@ __device__ __forceinline__ void setup_barriers(Ctrl* ctrl) {
 // =================================================================================================
 // GEMM kernel: weights as the M operand, activation rows (hi | lo) as the N operand
 // =================================================================================================
-struct GemmJob { int g, arow, wrow, kb0, kb1; };
+struct GemmJob { int g, wrow, kb0, kb1; };
 struct GemmWalk {
   const StreamGemmParams& p;
   long long u, u1;
   __device__ GemmWalk(const StreamGemmParams& pp) : p(pp) {
-    const long long U = (long long)p.row_tiles * p.groups * p.tiles_per_group * p.ksteps, G = gridDim.x, c = blockIdx.x;
+    const long long U = (long long)p.groups * p.tiles_per_group * p.ksteps, G = gridDim.x, c = blockIdx.x;
     u = c * U / G;
     u1 = (c + 1) * U / G;
   }
@@ -230,12 +230,8 @@ struct GemmWalk {
     j.kb0 = (int)(u - tile * p.ksteps);
     const long long left = u1 - u;
     j.kb1 = (int)((p.ksteps - j.kb0) < left ? p.ksteps : j.kb0 + left);
-    const int per_rt = p.groups * p.tiles_per_group;
-    const int rt = (int)(tile / per_rt);
-    const int rem = (int)(tile - (long long)rt * per_rt);
-    j.g = rem / p.tiles_per_group;
-    j.arow = rt * 128;
-    j.wrow = (rem - j.g * p.tiles_per_group) * kGemmNT;
+    j.g = (int)tile / p.tiles_per_group;
+    j.wrow = ((int)tile - j.g * p.tiles_per_group) * kGemmNT;
     u += j.kb1 - j.kb0;
     return true;
   }
@@ -245,20 +241,15 @@ __host__ __device__ constexpr uint32_t gemm_tmem_cols(int n_act) {
   return 2 * n_act <= 32 ? 32u : (2 * n_act <= 64 ? 64u : (2 * n_act <= 128 ? 128u : (2 * n_act <= 256 ? 256u : 512u)));
 }
 
-// Live packed rows of row tile `arow / 128`, rounded up to 8 (at least 8, at most half a box).
-__device__ __forceinline__ int gemm_tile_rows8(const StreamGemmParams& p, int live, int arow) {
-  int rows = live - arow;
-  rows = rows < 1 ? 1 : rows;
-  rows = (rows + 7) & ~7;
-  const int cap = p.a_box_rows / 2;
-  return rows > cap ? cap : rows;
+// Operand rows (hi and lo) of `live` packed rows, up to a multiple of `step`; at least one step.
+__device__ __forceinline__ int gemm_op_rows(const StreamGemmParams& p, int live, int step) {
+  const int n = ((live < 1 ? 2 : 2 * live) + step - 1) / step * step;
+  return n < p.a_box_rows ? n : p.a_box_rows;
 }
 
 template <int KSB, int STAGES>
 __global__ void __launch_bounds__(kThreads, 1)
-k_stream_gemm(const StreamGemmParams p, const __grid_constant__ CUtensorMap tmA0,
-              const __grid_constant__ CUtensorMap tmA1, const __grid_constant__ CUtensorMap tmW0,
-              const __grid_constant__ CUtensorMap tmW1) {
+k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps tm) {
   constexpr int NT = kGemmNT;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -267,10 +258,9 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ CUtensorMap tmA0
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t a_bytes = (uint32_t)KSB * p.a_box_rows * 128;
   const uint32_t stage_bytes = a_bytes + (uint32_t)KSB * NT * 128;
-  const bool narrow_n = p.row_tiles == 1;          // one row tile: the MMA's N follows the live rows
   pdl_trigger();                                   // the next kernel may get resident behind this one
   setup_barriers<STAGES>(ctrl);
-  if (warp == 0 && lane == 0) { prefetch_tmap(&tmA0); prefetch_tmap(&tmW0); if (p.groups > 1) { prefetch_tmap(&tmA1); prefetch_tmap(&tmW1); } }
+  if (warp == 0 && lane == 0) { prefetch_tmap(&tm.w[0]); if (p.groups > 1) prefetch_tmap(&tm.w[1]); }
   __syncthreads();
   if (warp == 2) { tmem_alloc(smem_u32(&ctrl->tmem_base), gemm_tmem_cols(p.a_box_rows)); tmem_relinquish(); }
   tc_fence_before();
@@ -280,22 +270,31 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ CUtensorMap tmA0
 
   if (warp == 0) {
     if (lane == 0) {
-      // ---- TMA producer.  The weight tiles depend on no earlier kernel, the activation tiles do:
-      // during the first pass over the ring only the weight boxes are issued and the activation
-      // boxes are noted; once the ring is full (or the work ends) the producer waits for the
-      // preceding kernel and issues them.  With an ordinary launch the wait returns at once.
-      const CUtensorMap* amaps[2] = {&tmA0, &tmA1};
-      const CUtensorMap* wmaps[2] = {&tmW0, &tmW1};
+      // ---- TMA producer.  The weight tiles depend on no earlier kernel, the activation rows and their
+      // count do: during the first pass over the ring only the weight boxes are issued and the
+      // activation boxes are noted; once the ring is full (or the work ends) the producer waits for the
+      // preceding kernel, picks the box that covers the live rows and issues them.  (A box of the pass's
+      // capacity brought 1.5 bytes of activations per byte of weights at 96 rows of which 55 were live,
+      // and what an SM takes in from L2 bounds a batch of this size, not HBM: 546 -> 511 us per step of
+      // 32 sequences at d = 4096, 251 -> 244 of 8 at d = 3072.)  With an ordinary launch the wait
+      // returns at once.
       const uint64_t pol_w = policy_evict_first(), pol_a = policy_evict_last();
-      struct Deferred { uint32_t dst, bar; int map, arow, kb; };
-      Deferred def[kMaxStages];
-      int n_def = 0, issued = 0;
+      struct Deferred { int g, kb; };
+      Deferred def[kMaxStages];                       // load i of the first pass uses stage i
+      int n_def = 0, issued = 0, box = 0;
+      uint32_t box_bytes = 0;
       bool deps = false, ok = true;
       auto need_deps = [&]() {
         if (deps) return;
         pdl_wait();
-        for (int i = 0; i < n_def; ++i)
-          tma_load_3d(def[i].dst, amaps[def[i].map], 0, 2 * def[i].arow, def[i].kb, def[i].bar, pol_a);
+        const int rows = gemm_op_rows(p, *p.rows_dev, p.box_step);
+        box = rows / p.box_step - 1;
+        box_bytes = (uint32_t)KSB * rows * 128;
+        for (int i = 0; i < n_def; ++i) {
+          const uint32_t full = smem_u32(&ctrl->full[i]);
+          mbar_expect_tx(full, box_bytes);
+          tma_load_3d(stage_base + (uint32_t)i * stage_bytes, &tm.a[def[i].g][box], 0, 0, def[i].kb, full, pol_a);
+        }
         deps = true;
       };
       int stage = 0; uint32_t phase = 0;
@@ -306,11 +305,12 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ CUtensorMap tmA0
           if (issued == STAGES) need_deps();
           if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) { ok = false; break; }
           const uint32_t full = smem_u32(&ctrl->full[stage]);
-          mbar_expect_tx(full, stage_bytes);        // rows of a box outside the tensor are zero-filled and counted
           const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
-          tma_load_3d(sb + a_bytes, wmaps[j.g], 0, j.wrow, ks * KSB, full, pol_w);
-          if (deps) tma_load_3d(sb, amaps[j.g], 0, 2 * j.arow, ks * KSB, full, pol_a);
-          else { def[n_def].dst = sb; def[n_def].bar = full; def[n_def].map = j.g; def[n_def].arow = j.arow; def[n_def].kb = ks * KSB; ++n_def; }
+          if (deps) mbar_expect_tx(full, KSB * NT * 128 + box_bytes);   // rows outside the tensor are zero-filled and counted
+          else mbar_expect_only(full, KSB * NT * 128);
+          tma_load_3d(sb + a_bytes, &tm.w[j.g], 0, j.wrow, ks * KSB, full, pol_w);
+          if (deps) tma_load_3d(sb, &tm.a[j.g][box], 0, 0, ks * KSB, full, pol_a);
+          else { def[n_def].g = j.g; def[n_def].kb = ks * KSB; ++n_def; }
           ++issued;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
@@ -322,6 +322,8 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ CUtensorMap tmA0
       // ---- MMA issue: D[128 weight rows][n] += W tile (M operand) x live activation rows (N operand)
       pdl_wait();                                      // the live-row count comes from an earlier kernel
       const int live = *p.rows_dev;
+      const uint32_t box_kb = (uint32_t)gemm_op_rows(p, live, p.box_step) * 128;    // one k-block of the activation box
+      const uint32_t idesc = idesc_bf16_f32(128, gemm_op_rows(p, live, 16));
       int stage = 0; uint32_t phase = 0, job_i = 0;
       bool ok = true;
       GemmWalk walk(p);
@@ -330,9 +332,6 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ CUtensorMap tmA0
         const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
         if (!mbar_wait(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) break;
         tc_fence_after();
-        // N covers the live operand rows, which sit at the start of the box (a multiple of 16)
-        const int n_rows = narrow_n ? 2 * gemm_tile_rows8(p, live, j.arow) : p.a_box_rows;
-        const uint32_t idesc = idesc_bf16_f32(128, n_rows);
         const uint32_t d = tmem_base + buf * (uint32_t)p.a_box_rows;
         uint32_t acc = 0;
         for (int ks = j.kb0; ks < j.kb1; ++ks) {
@@ -341,7 +340,7 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ CUtensorMap tmA0
           const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
 #pragma unroll
           for (int i = 0; i < KSB; ++i) {
-            const uint32_t ab = sb + (uint32_t)i * p.a_box_rows * 128;
+            const uint32_t ab = sb + (uint32_t)i * box_kb;
             const uint32_t wb = sb + a_bytes + (uint32_t)i * NT * 128;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -362,7 +361,8 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ CUtensorMap tmA0
     // live activation rows (pairs of TMEM columns): hi + lo in registers, one reduction per
     // (row, feature)
     pdl_wait();                                      // the result matrix may still be read by the kernel before
-    const int live = *p.rows_dev;
+    int rows = *p.rows_dev;
+    rows = rows < p.a_box_rows / 2 ? rows : p.a_box_rows / 2;
     const int q = warp & 3;                          // TMEM lane quarter this warp may read
     const int feature = q * 32 + lane;
     uint32_t job_i = 0;
@@ -372,9 +372,7 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ CUtensorMap tmA0
       const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
       if (!mbar_wait(smem_u32(&ctrl->acc_full[buf]), aph, &ctrl->abort)) break;
       tc_fence_after();
-      int rows = live - j.arow;                      // live activation rows of this row tile
-      rows = rows > 128 ? 128 : rows;
-      float* dst = p.out + ((size_t)j.g * p.Rt + j.arow) * p.J + j.wrow + feature;
+      float* dst = p.out + (size_t)j.g * p.Rt * p.J + j.wrow + feature;
       const uint32_t t0 = tmem_base + ((uint32_t)(q * 32) << 16) + buf * (uint32_t)p.a_box_rows;
 #pragma unroll 1
       for (int r0 = 0; r0 < rows; r0 += 8) {
@@ -645,43 +643,57 @@ static int pick_stages(int a_parts, int a_box_rows, int extra) {
   return s > kMaxStages ? kMaxStages : s;
 }
 
+// Capacity of the activation box (hi and lo rows of R packed rows) and the step of its heights: eight
+// heights cover it.
+static int gemm_box_step(int R) { return 2 * R <= 128 ? 16 : 32; }
+static int gemm_box_rows(int R) { return (2 * R + gemm_box_step(R) - 1) / gemm_box_step(R) * gemm_box_step(R); }
+
 // Stages of the GEMM ring that fit beside the control block (every operand row an MMA reads is
 // loaded or zero-filled, so no readable padding is needed behind the ring).
-int stream_gemm_stages(int ksb, int a_box_rows) {
+static int gemm_stages(int ksb, int a_box_rows) {
   const int stage = ksb * a_box_rows * 128 + ksb * kGemmNT * 128;
   const int s = (227 * 1024 - 2048) / stage;
   return s > kMaxStages ? kMaxStages : s;
 }
+// Two k-blocks per stage (fewer TMA operations per byte) while at least four stages still fit.
+int stream_gemm_ksb(int R) { return gemm_stages(2, gemm_box_rows(R)) >= 4 ? 2 : 1; }
+
+// Tensor maps of one activation operand ([2 Rt, K], hi and lo rows interleaved): one per box height.
+bool stream_gemm_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int R) {
+  const int step = gemm_box_step(R), n = gemm_box_rows(R) / step, ksb = stream_gemm_ksb(R);
+  for (int i = 0; i < 8; ++i) {
+    if (i >= n) { maps[i] = maps[n - 1]; continue; }
+    if (!make_tmap_bf16_kblocks(&maps[i], act, 2ll * Rt, K, step * (i + 1), ksb)) return false;
+  }
+  return true;
+}
 
 template <int KSB, int STAGES>
-static cudaError_t launch_gemm_t(const StreamGemmParams& p, const CUtensorMap* maps, int grid, cudaStream_t s) {
+static cudaError_t launch_gemm_t(const StreamGemmParams& p, const StreamGemmMaps& maps, int grid, cudaStream_t s) {
   const size_t stage = (size_t)KSB * p.a_box_rows * 128 + (size_t)KSB * kGemmNT * 128;
   const size_t smem = 1024 + 1024 + STAGES * stage;
   auto kern = k_stream_gemm<KSB, STAGES>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(grid), dim3(kThreads), smem, s, p, maps[0], maps[1], maps[2], maps[3]);
+  return launch_pdl(kern, dim3(grid), dim3(kThreads), smem, s, p, maps);
 }
 
-// Launches the stream-K GEMM.  maps = {A group 0, A group 1, W group 0, W group 1}, built for
-// p.ksb k-blocks per box.
 template <int KSB>
-static cudaError_t launch_stream_gemm_k(const StreamGemmParams& p, const CUtensorMap* maps, int grid, cudaStream_t s) {
-  const int st = stream_gemm_stages(KSB, p.a_box_rows);
+static cudaError_t launch_stream_gemm_k(const StreamGemmParams& p, const StreamGemmMaps& maps, int grid, cudaStream_t s) {
+  const int st = gemm_stages(KSB, p.a_box_rows);
   if (st >= 8) return launch_gemm_t<KSB, 8>(p, maps, grid, s);
   if (st >= 6) return launch_gemm_t<KSB, 6>(p, maps, grid, s);
   if (st >= 5) return launch_gemm_t<KSB, 5>(p, maps, grid, s);
-  if (st >= 4) return launch_gemm_t<KSB, 4>(p, maps, grid, s);
-  if (st >= 3) return launch_gemm_t<KSB, 3>(p, maps, grid, s);
-  return cudaErrorInvalidConfiguration;
+  return launch_gemm_t<KSB, 4>(p, maps, grid, s);
 }
-cudaError_t launch_stream_gemm(const StreamGemmParams& p, const CUtensorMap* maps, int grid, cudaStream_t s) {
-  if (!p.out || !p.err || !p.rows_dev || p.a_box_rows % 16 || p.a_box_rows < 16 || p.a_box_rows > 256 ||
-      (p.row_tiles > 1 && p.a_box_rows != 256))
-    return cudaErrorInvalidValue;
-  if (p.ksb == 2) return launch_stream_gemm_k<2>(p, maps, grid, s);
-  if (p.ksb == 1) return launch_stream_gemm_k<1>(p, maps, grid, s);
-  return cudaErrorInvalidValue;
+cudaError_t launch_stream_gemm(StreamGemmParams p, const StreamGemmMaps& maps, int n_sm, cudaStream_t s) {
+  if (!p.out || !p.err || !p.rows_dev || p.R < 1 || p.R > 128) return cudaErrorInvalidValue;
+  p.box_step = gemm_box_step(p.R);
+  p.a_box_rows = gemm_box_rows(p.R);
+  p.tiles_per_group = p.J / kGemmNT;
+  const long long units = (long long)p.groups * p.tiles_per_group * p.ksteps;
+  const int grid = units < n_sm ? (int)units : n_sm;           // every CTA owns >= 1 unit
+  return stream_gemm_ksb(p.R) == 2 ? launch_stream_gemm_k<2>(p, maps, grid, s) : launch_stream_gemm_k<1>(p, maps, grid, s);
 }
 
 template <int NT, int KSB, int STAGES>

@@ -49,7 +49,7 @@ cudaError_t run_logits_decode(const CbView& cb, const LogitsArgs& a, int* counte
                               LogitsPartInfo* info, Prof* prof, cudaStream_t s);
 
 // Stream-K GEMM over `groups` independent problems of identical shape (the two hyper-encoders).
-// The unit space is (row tile, group, weight tile, k-step); CTA c of G owns units
+// The unit space is (group, weight tile, k-step); CTA c of G owns units
 // [floor(cU/G), floor((c+1)U/G)).  Every maximal run of units inside one tile and one CTA is one
 // accumulator.  Operands are swapped with respect to the result's orientation: the 128 weight rows
 // of a tile are the MMA's M, the activation rows its N, and a thread of the epilogue owns one
@@ -57,21 +57,49 @@ cudaError_t run_logits_decode(const CbView& cb, const LogitsArgs& a, int* counte
 //
 // The activation operand holds the hi part and the lo part of PACKED row r in rows 2r and 2r + 1
 // (bf16 [2 * Rt, K]); only the first *rows_dev packed rows carry data, a count that only the device
-// knows.  One TMA box of a_box_rows (= 2 * min(Rt, 128)) operand rows is loaded per stage; with a
-// single row tile the MMA's N is 2 * P8 (P8 = live rows rounded up to 8): the tensor-core work
-// and the epilogue's reductions follow the number of rows that exist, not the capacity of the
-// pass.  The epilogue adds the hi and lo columns of a row in registers and reduces the sums into
-// the fp32 result matrix out[group][Rt][J] (lanes = consecutive features = consecutive addresses).
+// knows.  The TMA box and the MMA's N follow it: loads, tensor-core work and the epilogue's
+// reductions grow with the number of rows that exist, not with the capacity of the pass.  The
+// epilogue adds the hi and lo columns of a row in registers and reduces the sums into the fp32
+// result matrix out[group][Rt][J] (lanes = consecutive features = consecutive addresses).
+// The caller fills the first block of fields, the launch the second.
 struct StreamGemmParams {
-  int row_tiles;         // 128-row tiles of the packed activation rows (outermost dimension of the unit space)
-  int groups, tiles_per_group, ksteps;
-  int ksb;               // 64-column k-blocks per stage and TMA box: 2 when the stages stay small, else 1
-  int a_box_rows;        // operand rows per TMA box (multiple of 16, <= 256): the MMA's largest N
+  int groups, ksteps;    // ksteps = K / (64 * ksb), ksb = 64-column k-blocks per stage and TMA box
+  int R;                 // row capacity of the pass
   float* out;            // [groups][Rt][J] fp32, zero before the first add
   int J, Rt;
-  const int* rows_dev;   // device word: packed rows that carry data (<= Rt)
+  const int* rows_dev;   // device word: packed rows that carry data (<= R)
   int* err;
+
+  int tiles_per_group;
+  int a_box_rows, box_step;   // most operand rows of a box; boxes are multiples of box_step rows
 };
+struct StreamGemmMaps {
+  CUtensorMap a[2][8];   // activation operand of each group, boxes of 1 .. 8 steps
+  CUtensorMap w[2];      // weights of each group, 128 rows
+};
+int stream_gemm_ksb(int R);
+bool stream_gemm_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int R);
+// At most 128 rows, one CTA per tile of 128 weight rows.
+cudaError_t launch_stream_gemm(StreamGemmParams p, const StreamGemmMaps& maps, int n_sm, cudaStream_t s);
+
+// The same product on CTA pairs (z2z_stream_pair.cu): up to 256 packed rows ride on one stream of the
+// weights, and more run as blocks of 256.
+struct StreamPairParams {
+  int groups, ksteps;
+  int R;
+  float* out;
+  int J, Rt;
+  const int* rows_dev;
+  int* err;
+
+  int tiles_per_group;   // tiles of 256 weight rows
+  int blocks;            // blocks of 256 packed rows the capacity asks for
+  int act_bytes;         // activation part of a stage
+  int stages, acc_bufs, acc_stride, tmem_cols;
+};
+int stream_pair_ksb(int R);
+bool stream_pair_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int R);     // boxes of 16, 32, .. 128 rows
+cudaError_t launch_stream_pair(StreamPairParams p, const StreamGemmMaps& maps, int n_sm, cudaStream_t s);
 
 struct StreamLogitsParams {
   CbView cb;
@@ -119,9 +147,7 @@ cudaError_t launch_pair_gemm(const PairGemmParams& p, const void* act, const voi
                              cudaStream_t s);
 
 bool make_tmap_bf16(CUtensorMap* m, const void* base, long long rows, long long cols, int box_rows);
-int stream_gemm_stages(int ksb, int a_box_rows);
 cudaError_t launch_stream_logits(const StreamLogitsParams& p, const LogitMaps* maps, int grid, bool merge,
                                  Prof* prof, cudaStream_t s);
-cudaError_t launch_stream_gemm(const StreamGemmParams& p, const CUtensorMap* maps, int grid, cudaStream_t s);
 
 }  // namespace z2z

@@ -1,0 +1,314 @@
+// Weight-streaming skinny GEMM on CTA pairs, for hyper-encoder passes of a large decode batch or of a short
+// prompt (hundreds of activation rows):
+//
+//   out[group][r][j] += sum_k A[group][r][k] * W[group][j][k]
+//
+// A weight byte crosses HBM once, but the activation rows have to be brought from L2 into every SM
+// for every weight tile it streams, and that ingest is what bounds a batch of this size.  One CTA per
+// weight tile and row tile of 128 rows brought the weights again for every row tile, also for tiles
+// without a live row.  Here
+//   * two CTAs share a tile of 256 weight rows (tcgen05.mma.cta_group::2, M = 256): each loads its own
+//     128 weight rows and HALF of the activation rows;
+//   * the activation box follows the LIVE rows, a count that only the device knows: one tensor map
+//     per box height (16, 32, .. 128 rows), picked once the preceding kernel is done.  The weight
+//     boxes of the first pass over the ring are issued before that;
+//   * up to 256 packed rows (hi and lo part: 512 operand rows) ride on one stream of the weights: two
+//     accumulators of 256 columns fill tensor memory.  More rows run as several such blocks, the
+//     same weight tile one after the other, so that it comes from L2 the second time.
+// A decode step of 90 sequences (d = 3072, one encoder, 270 rows of capacity, about 150 live) went from
+// 486 to 327 us, the 240 rows of a short prompt's entries (both encoders) from 1.49 to 0.94 ms.
+//
+// Work is cut stream-K style: cluster c of C owns units [floor(c U / C), floor((c + 1) U / C)) of the
+// (group, weight tile, row block, k-step) space and adds its accumulators into the fp32 result with
+// reductions in global memory, like k_stream_gemm.
+//
+// Operand layout: packed row r of the activations is rows 2 r (bf16 hi) and 2 r + 1 (lo) of
+// [2 Rt, K]; an epilogue thread owns one output feature and adds the two columns of a row.
+//
+// Roles per CTA: warp 0 lane 0 TMA producer, warp 1 lane 0 MMA issuer (leader CTA only), warps 2-5
+// epilogue.  Every mbarrier wait is bounded.
+#include "z2z_common.cuh"
+#include "z2z_internal.h"
+#include "z2z_sm100.cuh"
+#include "z2z_stream.h"
+
+namespace z2z {
+using namespace sm100;
+
+namespace {
+
+constexpr int kThreads = 192;
+constexpr int kSpMaxStages = 8;
+constexpr int kSpBlockRows = 256;        // packed rows that share one stream of the weights
+constexpr int kSpSmem = 227 * 1024;
+
+struct SpCtrl {
+  unsigned long long full[kSpMaxStages], empty[kSpMaxStages], acc_full[2], acc_empty[2];
+  uint32_t tmem_base;
+  int abort;
+};
+
+struct SpJob { int g, wrow, block, kb0, kb1; };
+struct SpWalk {
+  const StreamPairParams& p;
+  int blocks;
+  long long u, u1;
+  __device__ SpWalk(const StreamPairParams& pp, int live_blocks) : p(pp), blocks(live_blocks) {
+    const long long U = (long long)p.groups * p.tiles_per_group * blocks * p.ksteps, C = gridDim.x >> 1, c = blockIdx.x >> 1;
+    u = c * U / C;
+    u1 = (c + 1) * U / C;
+  }
+  __device__ bool next(SpJob& j) {
+    if (u >= u1) return false;
+    const long long job = u / p.ksteps;
+    j.kb0 = (int)(u - job * p.ksteps);
+    const long long left = u1 - u;
+    j.kb1 = (int)((p.ksteps - j.kb0) < left ? p.ksteps : j.kb0 + left);
+    const long long tile = job / blocks;
+    j.block = (int)(job - tile * blocks);
+    j.g = (int)(tile / p.tiles_per_group);
+    j.wrow = ((int)tile - j.g * p.tiles_per_group) * 256;
+    u += j.kb1 - j.kb0;
+    return true;
+  }
+};
+
+// Operand rows (hi and lo) of half `h` of a row block that the MMA covers: a multiple of 32 (the pair's
+// N), 0 if the half has no live row; the first half of a block always counts as having one.
+__device__ __forceinline__ int sp_cols(int live, int block, int h) {
+  int rows = live - block * kSpBlockRows - h * 128;
+  if (rows < 1) rows = (h == 0) ? 1 : 0;
+  if (rows > 128) rows = 128;
+  return (2 * rows + 31) & ~31;
+}
+// Row blocks with a live row (at least one).  A pass whose capacity is one block does not need the count.
+__device__ __forceinline__ int sp_live_blocks(const StreamPairParams& p, int live) {
+  return p.blocks > 1 && live > kSpBlockRows ? (live + kSpBlockRows - 1) / kSpBlockRows : 1;
+}
+
+template <int KSB>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps tm) {
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  SpCtrl* ctrl = reinterpret_cast<SpCtrl*>(sm);
+  const uint32_t stage_base = smem_u32(sm + 1024);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();          // 0: leader (issues the MMAs), 1: peer
+  const uint32_t stage_bytes = (uint32_t)p.act_bytes + KSB * 16384u;
+  const int STAGES = p.stages;
+  pdl_trigger();                                    // the next kernel may get resident behind this one
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(smem_u32(&ctrl->full[s]), 1);        // leader: its producer's arrive + bytes of both CTAs
+      mbar_init(smem_u32(&ctrl->empty[s]), 1);       // one multicast commit
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_u32(&ctrl->acc_full[b]), 1);    // one multicast commit
+      mbar_init(smem_u32(&ctrl->acc_empty[b]), 8);   // leader: 4 epilogue warps of each CTA
+    }
+    ctrl->abort = 0;
+    mbar_init_fence();
+    prefetch_tmap(&tm.w[0]);
+    if (p.groups > 1) prefetch_tmap(&tm.w[1]);
+  }
+  __syncthreads();
+  if (warp == 2) { tmem_alloc_pair(smem_u32(&ctrl->tmem_base), p.tmem_cols); tmem_relinquish_pair(); }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();                               // both CTAs' barriers exist before any remote signal
+  tc_fence_after();
+  const uint32_t tmem_base = ctrl->tmem_base;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      // ---------------- TMA producer (both CTAs) ---------------------------------------------------
+      const uint64_t pol_a = policy_evict_last();
+      const uint64_t pol_w = p.blocks > 1 ? policy_evict_last() : policy_evict_first();
+      uint32_t full_leader[kSpMaxStages];
+      for (int s = 0; s < STAGES; ++s) full_leader[s] = map_to_cta(smem_u32(&ctrl->full[s]), 0);
+      // Weight tiles depend on no earlier kernel, activations and their row count do: during the first
+      // pass over the ring only the weight boxes are issued and the activation boxes are noted.
+      SpJob def[kSpMaxStages];                        // load i of the first pass uses stage i; kb0 = its k-step
+      int n_def = 0, issued = 0, live = 0;
+      bool deps = false, ok = true;
+      auto act_bytes = [&](int block) { return (uint32_t)(sp_cols(live, block, 0) + sp_cols(live, block, 1)) * (KSB * 64u); };
+      auto load_act = [&](int st, const SpJob& j, int ks) {
+        const uint32_t sb = stage_base + (uint32_t)st * stage_bytes;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int n = sp_cols(live, j.block, h);
+          if (n == 0) continue;
+          const int row = 2 * (j.block * kSpBlockRows + h * 128) + (int)rank * (n >> 1);
+          tma_load_3d_pair(sb + h * (KSB * 16384u), &tm.a[j.g][(n >> 5) - 1], 0, row, ks * KSB, full_leader[st], pol_a);
+        }
+      };
+      auto need_deps = [&]() {
+        if (deps) return;
+        pdl_wait();
+        live = *p.rows_dev;
+        live = live < p.R ? live : p.R;
+        for (int i = 0; i < n_def; ++i) {
+          if (rank == 0) mbar_expect_tx(smem_u32(&ctrl->full[i]), 2 * act_bytes(def[i].block));
+          load_act(i, def[i], def[i].kb0);
+        }
+        deps = true;
+      };
+      if (p.blocks > 1) need_deps();                   // the walk itself depends on the row count
+      int stage = 0; uint32_t phase = 0;
+      SpWalk walk(p, sp_live_blocks(p, live));
+      SpJob j;
+      while (ok && walk.next(j)) {
+        for (int ks = j.kb0; ks < j.kb1; ++ks) {
+          if (issued == STAGES) need_deps();
+          if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) { ok = false; break; }
+          if (rank == 0) {
+            const uint32_t full = smem_u32(&ctrl->full[stage]);
+            if (deps) mbar_expect_tx(full, 2 * (KSB * 16384u + act_bytes(j.block)));
+            else mbar_expect_only(full, 2 * KSB * 16384u);
+          }
+          const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
+          tma_load_3d_pair(sb + p.act_bytes, &tm.w[j.g], 0, j.wrow + (int)rank * 128, ks * KSB, full_leader[stage], pol_w);
+          if (deps) load_act(stage, j, ks);
+          else { def[n_def] = j; def[n_def].kb0 = ks; ++n_def; }
+          ++issued;
+          if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+        }
+      }
+      need_deps();
+    }
+  } else {
+    pdl_wait();                                       // the row count and the result matrix belong to earlier kernels
+    int live = *p.rows_dev;
+    live = live < p.R ? live : p.R;
+    const int n_blocks = sp_live_blocks(p, live);
+    const uint32_t nbuf = (uint32_t)p.acc_bufs;
+    if (warp == 1) {
+      if (lane == 0 && rank == 0) {
+        // ---------------- MMA issuer (leader only): D[256 weight rows][n] += W tile x activation rows -----
+        int stage = 0; uint32_t phase = 0, job_i = 0;
+        bool ok = true;
+        SpWalk walk(p, n_blocks);
+        SpJob j;
+        while (ok && walk.next(j)) {
+          const uint32_t buf = job_i % nbuf, aph = (job_i / nbuf) & 1u;
+          if (!mbar_wait(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) break;
+          tc_fence_after();
+          const int n0 = sp_cols(live, j.block, 0), n1 = sp_cols(live, j.block, 1);
+          const uint32_t id0 = idesc_bf16_f32(256, n0), id1 = idesc_bf16_f32(256, n1 ? n1 : 32);
+          const uint32_t d = tmem_base + buf * (uint32_t)p.acc_stride;
+          uint32_t acc = 0;
+          for (int ks = j.kb0; ks < j.kb1; ++ks) {
+            if (!mbar_wait(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
+            tc_fence_after();
+            const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
+#pragma unroll
+            for (int i = 0; i < KSB; ++i) {
+              const uint32_t wb = sb + p.act_bytes + i * 16384u;
+              const uint32_t a0 = sb + (uint32_t)i * n0 * 64u, a1 = sb + KSB * 16384u + (uint32_t)i * n1 * 64u;
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                umma_bf16_pair(d, smem_desc_sw128(wb + k * 32), smem_desc_sw128(a0 + k * 32), id0, acc);
+                if (n1) umma_bf16_pair(d + 256, smem_desc_sw128(wb + k * 32), smem_desc_sw128(a1 + k * 32), id1, acc);
+                acc = 1;
+              }
+            }
+            umma_commit_pair(smem_u32(&ctrl->empty[stage]));      // frees the stage in both CTAs
+            if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+          }
+          if (!ok) break;
+          umma_commit_pair(smem_u32(&ctrl->acc_full[buf]));       // wakes the epilogues of both CTAs
+          ++job_i;
+        }
+      }
+    } else {
+      // ---------------- epilogue (both CTAs): thread = output feature -----------------------------------
+      const int q = warp & 3;                          // TMEM lane quarter this warp may read
+      uint32_t acc_empty_leader[2];
+      acc_empty_leader[0] = map_to_cta(smem_u32(&ctrl->acc_empty[0]), 0);
+      acc_empty_leader[1] = map_to_cta(smem_u32(&ctrl->acc_empty[1]), 0);
+      uint32_t job_i = 0;
+      SpWalk walk(p, n_blocks);
+      SpJob j;
+      while (walk.next(j)) {
+        const uint32_t buf = job_i % nbuf, aph = (job_i / nbuf) & 1u;
+        if (!mbar_wait(smem_u32(&ctrl->acc_full[buf]), aph, &ctrl->abort)) break;
+        tc_fence_after();
+        const int feature0 = j.wrow + (int)rank * 128;
+        if (feature0 < p.J) {                          // the last tile may be half outside (J is a multiple of 128)
+#pragma unroll 1
+          for (int h = 0; h < 2; ++h) {
+            const int row0 = j.block * kSpBlockRows + h * 128;
+            int rows = live - row0;
+            rows = rows > 128 ? 128 : rows;
+            float* dst = p.out + ((size_t)j.g * p.Rt + row0) * p.J + feature0 + q * 32 + lane;
+            const uint32_t t0 = tmem_base + ((uint32_t)(q * 32) << 16) + buf * (uint32_t)p.acc_stride + h * 256u;
+#pragma unroll 1
+            for (int r0 = 0; r0 < rows; r0 += 8) {
+              uint32_t v[16];
+              tmem_ld16(t0 + 2 * r0, v);
+              tmem_ld_wait();
+#pragma unroll
+              for (int x = 0; x < 8; ++x)
+                if (r0 + x < rows) red_add_f32(dst + (size_t)(r0 + x) * p.J, __uint_as_float(v[2 * x]) + __uint_as_float(v[2 * x + 1]));
+            }
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(acc_empty_leader[buf]);
+        ++job_i;
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (threadIdx.x == 0 && ctrl->abort) atomicOr(p.err, 1);
+  cluster_sync_all();                               // nobody leaves while the pair's MMAs may read its memory
+  if (warp == 2) tmem_dealloc_pair(tmem_base, p.tmem_cols);
+}
+
+int cols32(int rows) { return (2 * (rows < 128 ? rows : 128) + 31) / 32 * 32; }
+
+// Shared memory of one stage's activation boxes per CTA and k-block, for a pass of at most R rows.
+int pair_act_bytes(int R) { return R > 128 ? 16384 + cols32(R - 128) * 64 : cols32(R) * 64; }
+
+}  // namespace
+
+// Two k-blocks per stage (fewer TMA operations per byte) while at least four stages still fit.
+int stream_pair_ksb(int R) { return (kSpSmem - 2048) / (2 * (16384 + pair_act_bytes(R))) >= 4 ? 2 : 1; }
+
+// Tensor maps of one activation operand ([2 Rt, K], hi and lo rows interleaved): one per box height.
+bool stream_pair_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int R) {
+  const int n = cols32(R) / 32, ksb = stream_pair_ksb(R);
+  for (int i = 0; i < 8; ++i) {
+    if (i >= n) { maps[i] = maps[n - 1]; continue; }
+    if (!make_tmap_bf16_kblocks(&maps[i], act, 2ll * Rt, K, 16 * (i + 1), ksb)) return false;
+  }
+  return true;
+}
+
+cudaError_t launch_stream_pair(StreamPairParams p, const StreamGemmMaps& maps, int n_sm, cudaStream_t s) {
+  if (!p.out || !p.err || !p.rows_dev || p.R < 1) return cudaErrorInvalidValue;
+  const int ksb = stream_pair_ksb(p.R);
+  p.tiles_per_group = (p.J + 255) / 256;
+  p.blocks = (p.R + kSpBlockRows - 1) / kSpBlockRows;
+  p.act_bytes = ksb * pair_act_bytes(p.R);
+  p.acc_bufs = p.R > 128 ? 1 : 2;                   // two accumulators in turn, or one with two halves
+  p.acc_stride = p.R > 128 ? 0 : cols32(p.R);
+  int cols = 32;
+  while (cols < (p.R > 128 ? 512 : 2 * p.acc_stride)) cols <<= 1;
+  p.tmem_cols = cols;
+  const int stage = p.act_bytes + ksb * 16384;
+  p.stages = (kSpSmem - 2048) / stage;
+  if (p.stages > kSpMaxStages) p.stages = kSpMaxStages;
+  const size_t smem = 2048 + (size_t)p.stages * stage;
+  const long long units = (long long)p.groups * p.tiles_per_group * p.ksteps;      // every cluster owns >= 1 unit
+  const int clusters = units < n_sm / 2 ? (int)units : n_sm / 2;
+  auto kern = ksb == 2 ? k_stream_pair<2> : k_stream_pair<1>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(kern, dim3(2 * clusters), dim3(kThreads), smem, s, p, maps);
+}
+
+}  // namespace z2z

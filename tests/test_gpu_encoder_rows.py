@@ -1,0 +1,83 @@
+"""Hyper-encoder passes at the row counts where the linear-layer kernel, its activation box or its row blocks
+change: one entry, capacities around 128 and 256 packed rows (also with few of them live), the switch
+to whole output tiles, a rest behind full passes; odd multiples of 128 as width (half a tile of 256 weight
+rows); a session whose very first pass is captured into a graph.  Against the fp64 oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import hyper_encoder as ohe
+from paper_2506_01084_b200 import binding as zb
+from paper_2506_01084_b200 import synth_inputs as si
+from tests._harness import Pair, TOL, f64
+
+pytestmark = pytest.mark.gpu
+
+
+def _pair(d, dff, M, B, T, cap, seed, tied=0):
+    w = si.Workload("rows", V=2000, d=d, dtype="bf16", B=B, T=T, M=M, cap=cap, zipf_s=1.0, copy_p=0.5, seg_min=4,
+                    seg_max=14, steps=2, tied=tied, enc_layers=2, enc_heads=d // 128, enc_dff=dff)
+    p = Pair(w, seed)
+    p.gpu_encode()
+    for b in range(w.B):
+        p.oracle.books[b].encode(p.tokens[b].tolist())
+    return w, p
+
+
+def _check(w, p, got, first, count):
+    enc = [f64(t) for t in p.enc_E]
+    table = f64(p.W_E)
+    for b in range(w.B):
+        for k in {first[b], first[b] + count[b] - 1, first[b] + count[b] // 2} if count[b] else ():
+            want = ohe.hyper_embed([p.oracle.books[b].entries[k]], table, enc, w.heads)[0]
+            assert np.abs(got[b, k].double().cpu().numpy() - want).max() <= TOL
+        mask = torch.ones(w.cap, dtype=torch.bool)
+        mask[first[b]:first[b] + count[b]] = False
+        assert torch.all(got[b].cpu()[mask] == -5)            # no other row is touched
+
+
+@pytest.mark.parametrize("bound", ["exact", "count", "loose"])
+@pytest.mark.parametrize("d,dff,M,total", [(128, 384, 3, 1), (256, 512, 3, 42), (256, 512, 3, 43), (384, 640, 8, 16),
+                                           (128, 256, 3, 85), (384, 1152, 3, 86), (256, 512, 3, 171), (256, 256, 4, 224),
+                                           (256, 256, 4, 225), (128, 384, 2, 512), (128, 128, 3, 1050)])
+def test_embedding_a_range_of_entries(d, dff, M, total, bound):
+    B = 3
+    w, p = _pair(d, dff, M, B, T=max(400, 6 * total), cap=1400, seed=total)
+    n = [p.oracle.books[b].n() for b in range(B)]
+    count = [total - 2 * (total // 3), total // 3, total // 3]
+    first = [1, 0, 2]
+    assert all(n[b] >= first[b] + count[b] for b in range(B))
+    i32 = lambda x: torch.tensor(x, dtype=torch.int32, device=p.dev)
+    got = torch.full((B, w.cap, d), -5.0, dtype=torch.bfloat16, device=p.dev)
+    f32 = torch.full((B, w.cap, d), -5.0, dtype=torch.float32, device=p.dev)
+    lim = {"exact": -1, "count": total, "loose": total + 300}[bound]
+    zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, i32(first), i32(count), lim, got, f32)
+    st, _ = zb.z2z_status(p.cb)
+    assert all(int(s) & zb.ST_WAIT_TIMEOUT == 0 for s in st)
+    _check(w, p, f32, first, count)
+    assert torch.equal(got[0, first[0]].cpu(), f32[0, first[0]].cpu().bfloat16())
+
+
+@pytest.mark.parametrize("B,tied", [(43, 0), (90, 1), (128, 0)])
+def test_decode_step_of_a_large_batch_captured_first(B, tied):
+    w, p = _pair(256, 512, 3, B, T=64, cap=64, seed=B, tied=tied)
+    hid = si.make_hidden(w, B, 3).to(p.dev)
+    nxt, new = (torch.zeros(B, dtype=torch.int32, device=p.dev) for _ in range(2))
+    lse = torch.zeros(B, device=p.dev)
+    forced = torch.tensor([(31 * b + 7) % w.V for b in range(B)], dtype=torch.int32, device=p.dev)
+    forced[::5] = zb.CODE_NONE
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()                     # nothing of this session has run an encoder pass yet
+    with torch.cuda.graph(graph):
+        zb.z2z_decode_step(p.cb, hid, p.g_WE, p.g_WU, p.g_encE, p.g_encU, p.E_h, p.U_h, zb.SELECT_ARGMAX, 1.0, 0, 0,
+                           forced, nxt, None, lse, new, p.E_f32, p.U_f32)
+    graph.replay()
+    torch.cuda.synchronize()
+    enc = [f64(t) for t in p.enc_E]
+    table = f64(p.W_E)
+    for b in range(B):
+        want = -1 if b % 5 == 0 else p.oracle.books[b].step(int(forced[b]))
+        assert int(new[b]) == want
+        if want >= 0 and b % 7 < 2:
+            row = ohe.hyper_embed([p.oracle.books[b].entries[want]], table, enc, w.heads)[0]
+            assert np.abs(p.E_f32[b, want].double().cpu().numpy() - row).max() <= TOL
