@@ -73,6 +73,7 @@ z2z::EntryList entry_list(z2z_codebook* cb) {
   el.row_tok = reinterpret_cast<int32_t*>(cb->ws + cb->plan.off_row_tok);
   el.off = reinterpret_cast<int32_t*>(cb->ws + cb->plan.off_entry_off);
   el.chunk = cb->plan.enc_chunk_entries;
+  el.list = cb->plan.enc_list;
   return el;
 }
 
@@ -317,17 +318,23 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
     z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 1, s);
     Z2Z_CUDA(z2z::launch_entry_offsets(cb->view, which, d_first, d_count, el, s), "hyper_embed");
   }
-  long long bound = (long long)cb->cfg.B * cb->cfg.cap;
+  long long bound = (long long)cb->cfg.B * cb->cfg.cap, rows = 0;
   if (max_entries > 0 && max_entries < bound) bound = max_entries;
   if (max_entries < 0) {
-    // exact: read the number of entries this call has to embed back from the device (the one
-    // place where an enqueueing call waits for the stream), so that no pass is launched for nothing
-    int32_t total = 0;
-    int32_t* land = cb->h_frozen ? cb->h_frozen + 8 : &total;      // pinned host word when there is one
-    Z2Z_CUDA(cudaMemcpyAsync(land, el.off + cb->cfg.B, 4, cudaMemcpyDeviceToHost, s), "hyper_embed (entry count)");
+    // exact: read the number of entries this call has to embed, and of their rows, back from the device
+    // (the one place where an enqueueing call waits for the stream), so that no pass is launched for
+    // nothing
+    if (tc) {
+      z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 1, s);
+      Z2Z_CUDA(z2z::launch_entry_rows(cb->view, which, d_first, el, s), "hyper_embed");
+    }
+    int32_t host[2] = {0, 0};
+    int32_t* land = cb->h_frozen ? cb->h_frozen + 8 : host;        // pinned host words when there are any
+    Z2Z_CUDA(cudaMemcpyAsync(land, el.off + cb->cfg.B, 8, cudaMemcpyDeviceToHost, s), "hyper_embed (entry count)");
     Z2Z_CUDA(cudaStreamSynchronize(s), "hyper_embed (entry count)");
-    total = *reinterpret_cast<volatile int32_t*>(land);
+    const int32_t total = reinterpret_cast<volatile int32_t*>(land)[0];
     if (total >= 0 && total < bound) bound = total;
+    if (tc) rows = reinterpret_cast<volatile int32_t*>(land)[1];
   }
   const int n_chunks = (int)((bound + el.chunk - 1) / el.chunk);
   // Single-pass fp16 form of the prompt-sized passes: when the caller has lent memory for the
@@ -341,7 +348,31 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
                                                   cb->half_ptrs.data(), a.err, &cb->prof, s), "hyper_embed (fp16 weight copies)");
     a.w_half = cb->half_ptrs.data();
   }
-  for (int c = 0; c < n_chunks; ++c) {
+  // The rows of all entries are known (exact mode, tensor cores): passes are cut by rows, so that the tiles
+  // of the linear layers fill their waves, and the rest is sized by what is left.
+  int32_t* pass_first = reinterpret_cast<int32_t*>(cb->ws + cb->plan.off_plan);
+  const int pass_rows = rows > 0 ? z2z::encoder_pass_rows(rows, cb->plan.enc_rows < 256 ? 256 : cb->plan.enc_rows, cb->cfg.M, cb->cfg.d, cb->dff) : 0;
+  const int per = pass_rows - (cb->cfg.M - 1);
+  const long long n_passes = rows > 0 ? (rows + per - 1) / per : 0;
+  if (n_passes > 0 && pass_rows <= cb->plan.enc_rows && (size_t)(n_passes + 1) * 4 <= cb->plan.plan_bytes) {
+    {
+      z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 1, s);
+      Z2Z_CUDA(z2z::launch_entry_passes(cb->view, which, d_first, el, pass_rows, (int)n_passes, pass_first, s), "hyper_embed");
+    }
+    for (int c = 0; c < (int)n_passes; ++c) {
+      // a pass holds the entries whose first row is one of its `per` rows: up to M - 1 rows more, and no
+      // more than half as many entries, as an entry has two rows or more
+      const long long left = rows - (long long)c * per;
+      a.rows = left < pass_rows ? (int)left : pass_rows;
+      a.entries = (a.rows + 1) / 2;
+      if (a.entries > bound) a.entries = (int)bound;
+      {
+        z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 1, s);
+        Z2Z_CUDA(z2z::launch_entry_fill_pass(cb->view, which, d_first, el, c, pass_first, a.entries, s), "hyper_embed");
+      }
+      Z2Z_CUDA(z2z::run_encoder_pass_tc(cb->view, &a, 1, el, false, &cb->prof, s), "hyper_embed (tensor cores)");
+    }
+  } else for (int c = 0; c < n_chunks; ++c) {
     // a short call, and the rest of a long one, is sized for what it can hold: 16 entries at d = 4096 took
     // 0.86 ms per encoder when every pass was sized for 1024, and take 0.22
     const long long left = bound - (long long)c * el.chunk;

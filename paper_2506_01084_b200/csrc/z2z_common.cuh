@@ -67,6 +67,8 @@ struct WsPlan {
   int n_slots;
   int enc_chunk_entries;      // entries the encoder processes per pass
   int enc_rows;               // = enc_chunk_entries * M (rows padded to M per entry)
+  int enc_list;               // entries the work list of a pass can hold: passes cut by rows may hold more
+                              // entries than enc_chunk_entries, at two rows or more each
   size_t off_hash, off_cons, off_len, off_n, off_prev, off_status, off_n_emb, state_end;
   size_t off_entry_seq, off_entry_idx, off_entry_len, off_entry_tok, off_row_off, off_row_src, off_row_tok, off_entry_off, off_new_entry, off_sel;
   size_t off_X, off_A, off_QKV, off_H;            // fp32 encoder activations
@@ -97,6 +99,8 @@ inline WsPlan plan_workspace(const z2z_config& c) {
   if (chunk < 1) chunk = 1;
   p.enc_chunk_entries = chunk;
   p.enc_rows = chunk * c.M;
+  p.enc_list = chunk * c.M / 2 > chunk ? chunk * c.M / 2 : chunk;
+  const size_t list = (size_t)p.enc_list;
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
   p.off_hash = take((size_t)c.B * ns * 8);
@@ -107,11 +111,11 @@ inline WsPlan plan_workspace(const z2z_config& c) {
   p.off_status = take((size_t)c.B * 4);
   p.off_n_emb = take((size_t)2 * c.B * 4);
   p.state_end = o;
-  p.off_entry_seq = take((size_t)chunk * 4);
-  p.off_entry_idx = take((size_t)chunk * 4);
-  p.off_entry_len = take((size_t)chunk * 4);
-  p.off_entry_tok = take((size_t)chunk * c.M * 4);
-  p.off_row_off = take((size_t)(chunk + 1) * 4);
+  p.off_entry_seq = take(list * 4);
+  p.off_entry_idx = take(list * 4);
+  p.off_entry_len = take(list * 4);
+  p.off_entry_tok = take(list * c.M * 4);
+  p.off_row_off = take((list + 1) * 4);
   p.off_row_src = take((size_t)chunk * c.M * 4);
   p.off_row_tok = take((size_t)chunk * c.M * 4);
   p.off_entry_off = take((size_t)(c.B + 2) * 4);

@@ -52,30 +52,18 @@ __global__ void __launch_bounds__(1024) k_entry_offsets(CbView cb, int which, in
   int excl, total;
   block_exclusive_scan_1024(c, sm, excl, total);
   if (b < cb.B) off[b] = excl;
-  if (b == 0) off[cb.B] = total;
+  if (b == 0) { off[cb.B] = total; off[cb.B + 1] = 0; }
 }
 
-__global__ void k_entry_fill(CbView cb, int which, int mode, const int32_t* __restrict__ first,
-                             const int32_t* __restrict__ new_entry, EntryList el, int chunk_index) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  const int total = el.off[cb.B];
-  if (e == 0) {
-    long long left = (long long)total - (long long)chunk_index * el.chunk;
-    el.off[cb.B + 1] = (int)(left < 0 ? 0 : (left > el.chunk ? el.chunk : left));
-  }
-  if (e >= el.chunk) return;
-  const long long g = (long long)chunk_index * el.chunk + e;
-  if (g >= total) {
-    el.seq[e] = -1; el.idx[e] = 0; el.len[e] = 0;
-    for (int i = 0; i < cb.M; ++i) el.tok[(size_t)e * cb.M + i] = -1;
-    return;
-  }
+// Entry g of the call: its sequence and number within it.
+__device__ __forceinline__ void entry_of(const CbView& cb, int which, int mode, const int32_t* first,
+                                         const int32_t* new_entry, const EntryList& el, long long g, int& b, int& k) {
   int lo = 0, hi = cb.B - 1;                     // last b with off[b] <= g
   while (lo < hi) {
     int mid = (lo + hi + 1) >> 1;
     if (el.off[mid] <= g) lo = mid; else hi = mid - 1;
   }
-  const int b = lo;
+  b = lo;
   int f;
   if (mode == 1) f = new_entry[b];
   else {
@@ -83,13 +71,77 @@ __global__ void k_entry_fill(CbView cb, int which, int mode, const int32_t* __re
     const int n = cb.n[b];
     f = f < 0 ? 0 : (f > n ? n : f);
   }
-  const int k = f + (int)(g - el.off[b]);
+  k = f + (int)(g - el.off[b]);
+}
+
+// Work list of a pass: entries [g0, g0 + slots) of the call, or those of one pass of pass_first.
+__global__ void k_entry_fill(CbView cb, int which, int mode, const int32_t* __restrict__ first,
+                             const int32_t* __restrict__ new_entry, EntryList el, long long g0, int slots,
+                             const int32_t* __restrict__ pass_first) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  long long end = el.off[cb.B];
+  if (pass_first) { g0 = pass_first[0]; end = pass_first[1]; }
+  if (e == 0) {
+    const long long left = end - g0;
+    el.off[cb.B + 1] = (int)(left < 0 ? 0 : (left > slots ? slots : left));
+  }
+  if (e >= slots) return;
+  const long long g = g0 + e;
+  if (g >= end) {
+    el.seq[e] = -1; el.idx[e] = 0; el.len[e] = 0;
+    for (int i = 0; i < cb.M; ++i) el.tok[(size_t)e * cb.M + i] = -1;
+    return;
+  }
+  int b, k;
+  entry_of(cb, which, mode, first, new_entry, el, g, b, k);
   el.seq[e] = b;
   el.idx[e] = k;
   const bool in_book = k >= 0 && k < cb.cap;
   el.len[e] = in_book ? (int)cb.len[(size_t)b * cb.cap + k] : 0;
   for (int i = 0; i < cb.M; ++i)                       // constituents are -1 padded behind the entry's length
     el.tok[(size_t)e * cb.M + i] = in_book ? cb.cons[((size_t)b * cb.cap + k) * cb.M + i] : -1;
+}
+
+// Packed rows (base tokens) of all entries of the call, added up in el.off[B + 1] (zero before).
+__global__ void __launch_bounds__(256) k_entry_rows(CbView cb, int which, const int32_t* __restrict__ first, EntryList el) {
+  const int b = blockIdx.x;
+  const int count = el.off[b + 1] - el.off[b];
+  int f = first ? first[b] : cb.n_emb[which * cb.B + b];
+  const int n = cb.n[b];
+  f = f < 0 ? 0 : (f > n ? n : f);
+  int sum = 0;
+  for (int i = threadIdx.x; i < count; i += blockDim.x) sum += (int)cb.len[(size_t)b * cb.cap + f + i];
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  if ((threadIdx.x & 31) == 0 && sum) atomicAdd(&el.off[cb.B + 1], sum);
+}
+
+// First entry of every pass: the entry whose first row is row r of the call belongs to pass r / rows_per, so
+// that a pass holds at most rows_per + M - 1 rows.  One block walks the entries 1024 at a time.
+__global__ void __launch_bounds__(1024) k_entry_passes(CbView cb, int which, const int32_t* __restrict__ first, EntryList el,
+                                                       int rows_per, int n_passes, int32_t* __restrict__ pass_first) {
+  __shared__ int sm[1024];
+  const int total = el.off[cb.B];
+  long long before = 0;                          // rows ahead of this batch of entries
+  for (int g0 = 0; g0 < total; g0 += 1024) {
+    const int g = g0 + (int)threadIdx.x;
+    int len = 0;
+    if (g < total) {
+      int b, k;
+      entry_of(cb, which, 0, first, nullptr, el, g, b, k);
+      if (k < cb.cap) len = (int)cb.len[(size_t)b * cb.cap + k];
+    }
+    int excl, rows;
+    block_exclusive_scan_1024(len, sm, excl, rows);
+    if (g < total) {
+      const long long r0 = before + excl;
+      const int pass = (int)(r0 / rows_per);
+      const int next = (int)((r0 + len) / rows_per);       // pass of the entry that follows
+      if (g == 0) pass_first[0] = 0;
+      if (next != pass && next <= n_passes && g + 1 < total) pass_first[next] = g + 1;
+      if (g + 1 == total) for (int q = pass + 1; q <= n_passes; ++q) pass_first[q] = total;
+    }
+    before += rows;
+  }
 }
 
 __global__ void k_mark_embedded(CbView cb, int which) {
@@ -286,8 +338,22 @@ cudaError_t launch_entry_offsets_from_new(const CbView& cb, const int32_t* new_e
 cudaError_t launch_entry_fill(const CbView& cb, int which, const int32_t* first,
                               const int32_t* new_entry, const EntryList& el, int chunk_index,
                               cudaStream_t s) {
-  k_entry_fill<<<(el.chunk + 255) / 256, 256, 0, s>>>(cb, which, new_entry ? 1 : 0, first,
-                                                      new_entry, el, chunk_index);
+  k_entry_fill<<<(el.chunk + 255) / 256, 256, 0, s>>>(cb, which, new_entry ? 1 : 0, first, new_entry, el,
+                                                      (long long)chunk_index * el.chunk, el.chunk, nullptr);
+  return cudaGetLastError();
+}
+cudaError_t launch_entry_rows(const CbView& cb, int which, const int32_t* first, const EntryList& el, cudaStream_t s) {
+  k_entry_rows<<<cb.B, 256, 0, s>>>(cb, which, first, el);
+  return cudaGetLastError();
+}
+cudaError_t launch_entry_passes(const CbView& cb, int which, const int32_t* first, const EntryList& el, int rows,
+                                int n_passes, int32_t* pass_first, cudaStream_t s) {
+  k_entry_passes<<<1, 1024, 0, s>>>(cb, which, first, el, rows - (cb.M - 1), n_passes, pass_first);
+  return cudaGetLastError();
+}
+cudaError_t launch_entry_fill_pass(const CbView& cb, int which, const int32_t* first, const EntryList& el, int pass,
+                                   const int32_t* pass_first, int slots, cudaStream_t s) {
+  k_entry_fill<<<(slots + 255) / 256, 256, 0, s>>>(cb, which, 0, first, nullptr, el, 0, slots, pass_first + pass);
   return cudaGetLastError();
 }
 cudaError_t launch_mark_embedded(const CbView& cb, int which, cudaStream_t s) {

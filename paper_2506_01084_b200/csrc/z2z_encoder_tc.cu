@@ -413,12 +413,20 @@ __global__ void k_tc_qkv_attention(CbView cb, EntryList el, float* Y, Ptr2 bias,
 //
 // One block: first packed row of every entry (exclusive scan of the lengths), the total behind the
 // last entry slot, the way back from a packed row to (entry, position) and the row's base token.
-// E <= 1024 entries.  (The decode step's update kernel writes the same map itself.)
+// E <= 1024 * kMapPerThread entries, neighbouring ones per thread.  (The decode step's update kernel
+// writes the same map itself.)
+constexpr int kMapPerThread = kMaxM / 2;
 __global__ void __launch_bounds__(1024) k_tc_row_map(CbView cb, EntryList el, int E) {
   __shared__ int warp_sums[32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int len = tid < E ? entry_len_tc(cb, el, tid) : 0;
-  int inc = len;
+  const int per = (E + 1023) / 1024, e0 = tid * per;
+  int len[kMapPerThread], mine = 0;
+#pragma unroll
+  for (int q = 0; q < kMapPerThread; ++q) {
+    len[q] = q < per && e0 + q < E ? entry_len_tc(cb, el, e0 + q) : 0;
+    mine += len[q];
+  }
+  int inc = mine;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int x = __shfl_up_sync(0xffffffffu, inc, o);
@@ -436,13 +444,16 @@ __global__ void __launch_bounds__(1024) k_tc_row_map(CbView cb, EntryList el, in
     warp_sums[lane] = w;
   }
   __syncthreads();
-  const int excl = inc - len + (warp > 0 ? warp_sums[warp - 1] : 0);
-  if (tid < E) {
-    el.row_off[tid] = excl;
-    for (int i = 0; i < len; ++i) {
-      el.row_src[excl + i] = tid * cb.M + i;
-      el.row_tok[excl + i] = el.tok[tid * cb.M + i];
+  int row = inc - mine + (warp > 0 ? warp_sums[warp - 1] : 0);
+#pragma unroll
+  for (int q = 0; q < kMapPerThread; ++q) {
+    if (q >= per || e0 + q >= E) break;
+    el.row_off[e0 + q] = row;
+    for (int i = 0; i < len[q]; ++i) {
+      el.row_src[row + i] = (e0 + q) * cb.M + i;
+      el.row_tok[row + i] = el.tok[(size_t)(e0 + q) * cb.M + i];
     }
+    row += len[q];
   }
   if (tid == 0) el.row_off[E] = warp_sums[31];
 }
@@ -689,10 +700,10 @@ bool encoder_tc_supported(int d, int dff, int dtype, int heads, int M) {
 // Prompt-sized pass of ONE encoder (thousands of rows): the linear layers run as CTA-pair GEMMs
 // that own whole output tiles, so bias, residual and GELU are applied in their epilogues; only
 // attention, LayerNorm and pooling remain as separate kernels.
-static cudaError_t run_encoder_pass_pair(const CbView& cb, const EncoderArgs& a, const EntryList& el, int E,
+static cudaError_t run_encoder_pass_pair(const CbView& cb, const EncoderArgs& a, const EntryList& el, int E, int R,
                                          Prof* prof, cudaStream_t s) {
   const int d = a.d, dff = a.dff, M = cb.M;
-  const int R = E * M, Rt = (R + 7) / 8 * 8;
+  const int Rt = (R + 7) / 8 * 8;
   const bool half = a.w_half != nullptr;               // fp16 copies of the linear-layer weights exist
   auto Wp = [&](int i) { return reinterpret_cast<const bf16*>(a.w[i]); };
   const int* total = el.row_off + E;                   // packed rows of this pass (device word)
@@ -784,13 +795,37 @@ cudaError_t convert_encoder_weights_to_half(const void* const* w, int d, int dff
   return cudaGetLastError();
 }
 
+// A GEMM of the prompt-sized passes costs ceil(row tiles x column tiles / CTA pairs) waves of its K, so that the
+// number of rows in a pass decides how full the last wave is: with d = 3072 passes of 1024 entries (about
+// 2400 rows, ten row tiles) left a fifth of the tile slots empty, passes of six or twelve row tiles a
+// thirtieth; with d = 4096 nine row tiles fit.
+int encoder_pass_rows(long long total, int max_rows, int M, int d, int dff) {
+  const int nc = sm_count() / 2;
+  const int J[4] = {3 * d, d, dff, d}, K[4] = {d, d, d, dff};
+  auto cost = [&](long long rows) {                    // of one pass, in columns of K; the kernels between count too
+    const long long t = (rows + 255) / 256;
+    long long c = rows > 0 ? 2 * d : 0;
+    for (int i = 0; i < (dff > 0 ? 4 : 2); ++i) c += (t * ((J[i] + 255) / 256) + nc - 1) / nc * K[i];
+    return c;
+  };
+  int best = 256;
+  long long best_cost = -1;
+  for (int rows = 256; rows <= max_rows; rows += 256) {
+    const int per = rows - (M - 1);
+    const long long c = total / per * cost(rows) + cost(total % per);
+    if (best_cost < 0 || c <= best_cost) { best_cost = c; best = rows; }
+  }
+  return best;
+}
+
 cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng, const EntryList& el,
                                 bool rows_mapped, Prof* prof, cudaStream_t s) {
   const EncoderArgs& a0 = grp[0];
   const int d = a0.d, dff = a0.dff, M = cb.M;
-  const int E = a0.entries < el.chunk ? a0.entries : el.chunk;
-  const int R = E * M;                                 // row capacity of this pass
-  if (ng == 1 && R >= kPairPassMinRows) return run_encoder_pass_pair(cb, a0, el, E, prof, s);
+  const int E = a0.entries;
+  if (E > el.list || E > 1024 * kMapPerThread) return cudaErrorInvalidValue;
+  const int R = a0.rows > 0 ? a0.rows : E * M;         // row capacity of this pass
+  if (ng == 1 && R >= kPairPassMinRows) return run_encoder_pass_pair(cb, a0, el, E, R, prof, s);
   const int Rt = (R + 7) / 8 * 8;                      // rows of the result matrix per group
   const int* total = el.row_off + E;                   // packed rows of this pass (device word)
   const int n_sm = sm_count();

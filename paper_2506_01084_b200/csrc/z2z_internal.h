@@ -52,7 +52,8 @@ struct EntryList {
   int32_t* row_src;   // [chunk * M]  tensor-core passes: packed row -> entry * M + position
   int32_t* row_tok;   // [chunk * M]  tensor-core passes: base token of each packed row
   int32_t* off;       // [B + 2]  exclusive prefix sum of per-sequence counts, then the total
-  int chunk;
+  int chunk;          // entries of a pass cut by entries
+  int list;           // entries the work list can hold
 };
 struct EncoderArgs {
   int d, dff, heads, layers, M;
@@ -67,7 +68,8 @@ struct EncoderArgs {
   float* part;                  // fp32 GEMM results [groups][rows][J], zero between GEMMs
   size_t part_bytes;
   size_t* part_clean;           // host word of the session: leading bytes of `part` known to be zero
-  int entries;                  // host bound on the entries of this pass (<= chunk)
+  int entries;                  // host bound on the entries of this pass (<= the work list's capacity)
+  int rows;                     // host bound on its packed rows, 0 = entries * M
   int* err;                     // device error word of the tensor-core kernels
 };
 bool encoder_tc_supported(int d, int dff, int dtype, int heads, int M);
@@ -89,6 +91,18 @@ cudaError_t launch_entry_offsets_from_new(const CbView& cb, const int32_t* new_e
 cudaError_t launch_entry_fill(const CbView& cb, int which, const int32_t* first,
                               const int32_t* new_entry, const EntryList& el, int chunk_index,
                               cudaStream_t s);
+// Passes cut by packed rows instead of entries.  launch_entry_rows leaves the rows of all entries of the
+// call in el.off[B + 1] (behind their number in el.off[B]); launch_entry_passes writes the first entry of
+// every pass of at most `rows` rows to pass_first[0 .. n_passes]; launch_entry_fill_pass fills the work
+// list of one of them (`slots` entries at most).
+cudaError_t launch_entry_rows(const CbView& cb, int which, const int32_t* first, const EntryList& el, cudaStream_t s);
+cudaError_t launch_entry_passes(const CbView& cb, int which, const int32_t* first, const EntryList& el, int rows,
+                                int n_passes, int32_t* pass_first, cudaStream_t s);
+cudaError_t launch_entry_fill_pass(const CbView& cb, int which, const int32_t* first, const EntryList& el, int pass,
+                                   const int32_t* pass_first, int slots, cudaStream_t s);
+// Rows per pass (a multiple of 256, at most max_rows) that take the linear layers of `total` rows the fewest
+// waves of output tiles.
+int encoder_pass_rows(long long total, int max_rows, int M, int d, int dff);
 cudaError_t launch_mark_embedded(const CbView& cb, int which, cudaStream_t s);
 cudaError_t run_encoder_pass(const CbView& cb, const EncoderArgs& a, const EntryList& el,
                              bool use_tensor_cores, Prof* prof, cudaStream_t s);

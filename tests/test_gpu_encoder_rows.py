@@ -81,3 +81,17 @@ def test_decode_step_of_a_large_batch_captured_first(B, tied):
         if want >= 0 and b % 7 < 2:
             row = ohe.hyper_embed([p.oracle.books[b].entries[want]], table, enc, w.heads)[0]
             assert np.abs(p.E_f32[b, want].double().cpu().numpy() - row).max() <= TOL
+
+
+@pytest.mark.parametrize("M,d,dff", [(2, 128, 256), (3, 384, 384), (5, 128, 128)])
+def test_whole_prompts_in_passes_cut_by_rows(M, d, dff):
+    """Every entry of a call of several passes, so that those on both sides of a cut are among them."""
+    w, p = _pair(d, dff, M, B=3, T=9000, cap=3000, seed=M)
+    n = [p.oracle.books[b].n() for b in range(w.B)]
+    assert sum(len(e) for b in range(w.B) for e in p.oracle.books[b].entries) > 2 * 1024 * M       # more than one pass holds
+    zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, None, None, -1, p.E_h, p.E_f32)
+    enc = [f64(t) for t in p.enc_E]
+    for b in range(w.B):
+        want = ohe.hyper_embed(p.oracle.books[b].entries, f64(p.W_E), enc, w.heads)
+        assert np.abs(p.E_f32[b, :n[b]].double().cpu().numpy() - want).max() <= TOL
+        assert torch.all(p.E_f32[b, n[b]:] == 0)
