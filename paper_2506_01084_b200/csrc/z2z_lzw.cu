@@ -32,7 +32,7 @@ __global__ void k_codebook_clear(CbView cb) {
 //
 // Each lane follows the longest match from its own position (at most M - 1 dependent lookups).
 // Which positions start a phrase is a walk position -> position + match length: inside a warp by
-// pointer doubling (five rounds carry the set of visited lanes and the exit), across the four
+// pointer doubling (five rounds carry the set of visited lanes and the exit), across the
 // warps by looking up the exit of one as the entry of the next (a match is at most kMaxM long, so
 // only the first kMaxM lanes of a warp can be entered).
 //
@@ -40,6 +40,9 @@ __global__ void k_codebook_clear(CbView cb) {
 // barriers).  The chain used to be walked token by token by one thread: 180 ns per token with the
 // table in shared memory, 220 with it in global memory.  Four texts of 32768 tokens (cap 16384), to
 // codes and back with both session resets: 9.62 ms before, 1.00 ms with windows here and in the replay.
+constexpr int kTokRing = 512;
+static_assert(kTokRing >= kParseLanes + kMaxM, "a window's tokens fit the ring");
+
 template <bool SMEM>
 __global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const int32_t* __restrict__ tokens,
                                                               const int32_t* __restrict__ lens, int T_max,
@@ -47,8 +50,8 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const i
                                                               int32_t* __restrict__ code_lens,
                                                               int32_t* __restrict__ entries_after) {
   extern __shared__ __align__(16) unsigned char s_parse[];
-  __shared__ int s_tok[4 * kParseLanes];             // four chunks of tokens, position p at p mod 512
-  __shared__ int2 s_walk[4][kMaxM];                  // per warp and entry lane: lanes visited, exit
+  __shared__ int s_tok[kTokRing];                    // token of position p at p mod kTokRing
+  __shared__ int2 s_walk[kParseWarps][kMaxM];        // per warp and entry lane: lanes visited, exit
   __shared__ ParseVotes s_votes;
   __shared__ int s_prev, s_n1, s_st;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -66,19 +69,21 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const i
     int32_t* out = codes + (size_t)b * T_max;
     int32_t* aft = entries_after ? entries_after + (size_t)b * T_max : nullptr;
     int n = n0, n_out = 0, st = 0;
-    int chunks = 0;                                  // token chunks already in s_tok
-    int ahead = tid < T ? x[tid] : 0;                // this thread's token of the next chunk
+    int loaded = 0;                                  // tokens already in s_tok
+    int ahead = tid < T ? x[tid] : 0;                // token loaded + tid
     for (int p0 = 0; p0 < T;) {                      // p0: a phrase starts here
-      // positions below p0 + kParseLanes + kMaxM are looked at.  Nothing is fetched earlier than that: a
-      // window moves p0 by less than kParseLanes + kMaxM, so that a chunk is overwritten only once no
-      // warp can still be busy with the window that needed it.
-      while (chunks <= (p0 + kParseLanes + kMaxM - 1) / kParseLanes && chunks * kParseLanes < T) {
-        const int at = chunks * kParseLanes + tid;
+      // positions below p0 + kParseLanes + kMaxM are looked at.  (s_tok is only read ahead of a window's
+      // second barrier, so that the tokens of the last window may be overwritten here.)
+      const int need = p0 + kParseLanes + kMaxM < T ? p0 + kParseLanes + kMaxM : T;
+      while (loaded < need) {
+        const int at = loaded + tid;
         int c = ahead;
-        if ((unsigned)c >= (unsigned)V) { if (at < T) st |= Z2Z_ST_BAD_TOKEN; c = 0; }     // not a base token
-        s_tok[at & (4 * kParseLanes - 1)] = c;
-        ++chunks;
-        ahead = at + kParseLanes < T ? x[at + kParseLanes] : 0;
+        if (at < need) {
+          if ((unsigned)c >= (unsigned)V) { st |= Z2Z_ST_BAD_TOKEN; c = 0; }     // not a base token
+          s_tok[at & (kTokRing - 1)] = c;
+        }
+        loaded = loaded + kParseLanes < need ? loaded + kParseLanes : need;
+        ahead = loaded + tid < T ? x[loaded + tid] : 0;
       }
       parse_sync();
       // ---- longest match from every position of the window
@@ -87,9 +92,9 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const i
       int w = -1, len = 1, slot = -1, c = 0;
       bool miss = false;
       if (live) {
-        w = s_tok[q & (4 * kParseLanes - 1)];
+        w = s_tok[q & (kTokRing - 1)];
         while (len < M && q + len < T) {
-          c = s_tok[(q + len) & (4 * kParseLanes - 1)];
+          c = s_tok[(q + len) & (kTokRing - 1)];
           const int e = table.probe((uint32_t)w, (uint32_t)c, slot);
           if (e < 0) { miss = true; break; }
           w = V + e; ++len;
@@ -109,7 +114,7 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const i
       uint32_t mine = 0;
       int at = 0;                                    // entry into warp k, then the window's exit
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
+      for (int k = 0; k < kParseWarps; ++k) {
         if ((at >> 5) == k) {                        // (a walk that reached the end of the input stays where it is)
           const int2 wk = s_walk[k][at & 31];
           if (k == warp) mine = (uint32_t)wk.x;
@@ -128,27 +133,26 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const i
       if (lane == 0) { s_votes.on[warp] = v_on; s_votes.ins[warp] = v_ins; s_votes.lost[warp] = v_lost; }
       parse_sync();
       const ParseVotes votes = s_votes;
-      const int stop = parse_first_lost(votes);      // lanes below it are final
+      const int stop = parse_first_lost(votes.lost); // lanes below it are final
       const int room = cap - n;
-      const int new_before = parse_count_below(votes.ins, tid);
+      int made, emitted;
+      const int new_before = parse_rank(votes.ins, warp, lane, made), on_before = parse_rank(votes.on, warp, lane, emitted);
+      if (stop < kParseLanes) { made = parse_count_below(votes.ins, stop); emitted = parse_count_below(votes.on, stop); }
       if (own) {
         const int entry = tid < stop && new_before < room ? n + new_before : -1;
         table.settle(slot, (uint32_t)w, (uint32_t)c, entry);
-        if (entry >= 0) {                            // the phrase and its next token, -1 padded
-          int32_t* row = cb.cons + ((size_t)b * cap + entry) * M;
-          for (int j = 0; j < M; ++j) row[j] = j <= len ? s_tok[(q + j) & (4 * kParseLanes - 1)] : -1;
+        if (entry >= 0) {                            // the phrase and its next token: input from q on (expanded below)
+          cb.cons[((size_t)b * cap + entry) * M] = q;
           cb.len[(size_t)b * cap + entry] = (uint8_t)(len + 1);
         }
       }
-      const int emitted = parse_count_below(votes.on, stop);
       if (on && tid < stop) {
-        const int pos = n_out + parse_count_below(votes.on, tid);
+        const int pos = n_out + on_before;
         out[pos] = w;
-        const int made = new_before + (ins ? 1 : 0);
-        if (aft) aft[pos] = n + (made < room ? made : room);
-        if (pos == n_out + emitted - 1) s_prev = w;
+        const int mine_too = new_before + (ins ? 1 : 0);
+        if (aft) aft[pos] = n + (mine_too < room ? mine_too : room);
+        if (on_before == emitted - 1) s_prev = w;
       }
-      const int made = parse_count_below(votes.ins, stop);
       if (made > 0) {
         n += made < room ? made : room;
         if (n >= cap) st |= Z2Z_ST_CAP_FROZEN;
@@ -168,6 +172,16 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const i
     if (s_st) atomicOr(&cb.status[b], s_st);
   }
   table.close(n0, s_n1);
+  // constituent rows of the entries created here: tokens [start, start + len), -1 padded
+  for (int e = n0 + tid; e < s_n1; e += blockDim.x) {
+    int32_t* row = cb.cons + ((size_t)b * cap + e) * M;
+    const int start = row[0], L = cb.len[(size_t)b * cap + e];
+    for (int j = 0; j < M; ++j) {
+      int v = -1;
+      if (j < L) { v = x[start + j]; if ((unsigned)v >= (unsigned)V) v = 0; }
+      row[j] = v;
+    }
+  }
 }
 
 // Online update with one new code per sequence (Figure 1; Section 2.3 step 10).

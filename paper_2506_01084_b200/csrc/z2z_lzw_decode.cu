@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_replay(CbView cb, const i
   extern __shared__ __align__(16) unsigned char s_parse[];
   __shared__ int s_code[kParseLanes + 1], s_first[kParseLanes + 1];   // [0]: the code before the window
   __shared__ uint8_t s_len[kParseLanes + 4];
-  __shared__ uint32_t s_known[4];
+  __shared__ uint32_t s_known[kParseWarps];
   __shared__ ParseVotes s_votes;
   __shared__ int s_n1, s_bad0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_replay(CbView cb, const i
       parse_sync();
       int limit = kParseLanes;                       // first lane that is not known
 #pragma unroll
-      for (int k = 3; k >= 0; --k)
+      for (int k = kParseWarps - 1; k >= 0; --k)
         if (~s_known[k]) limit = k * 32 + __ffs((int)~s_known[k]) - 1;
       // the table in global memory keeps no keys to rebuild a row from later: a row is written at once,
       // which needs the previous code's row to be there
@@ -113,11 +113,13 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_replay(CbView cb, const i
       if (lane == 0) { s_votes.ins[warp] = v_ins; s_votes.lost[warp] = v_lost; }
       parse_sync();
       const ParseVotes votes = s_votes;
-      int stop = parse_first_lost(votes);
+      int stop = parse_first_lost(votes.lost);
       if (stop > limit) stop = limit;
       if (s_bad0) stop = 0;
       const int room = cap - n;
-      const int new_before = parse_count_below(votes.ins, tid);
+      int made;
+      const int new_before = parse_rank(votes.ins, warp, lane, made);
+      if (stop < kParseLanes) made = parse_count_below(votes.ins, stop);
       if (own) {
         const int entry = tid < stop && new_before < room ? n + new_before : -1;
         table.settle(slot, (uint32_t)pz, (uint32_t)f, entry);
@@ -131,7 +133,6 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_replay(CbView cb, const i
           elen[entry] = (uint8_t)(pl + 1);
         }
       }
-      const int made = parse_count_below(votes.ins, stop);
       if (made > 0) {
         n += made < room ? made : room;
         if (n >= cap) st |= Z2Z_ST_CAP_FROZEN;

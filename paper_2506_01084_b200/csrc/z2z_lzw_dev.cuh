@@ -151,7 +151,7 @@ __device__ __forceinline__ int warp_lzw_step(const CbView& cb, int b, int z) {
 // Windowed parsing, shared by prompt compression and by replay of a code stream.
 //
 // Both are defined as a chain of one dictionary lookup per token or code, but the dictionary
-// changes little while 128 of them are looked at: kParseLanes threads look up kParseLanes starting
+// changes little while 256 of them are looked at: kParseLanes threads look up kParseLanes starting
 // points at once in the dictionary as it was before the window, the results that lie on the chain
 // are picked out, and only the new phrases of the chain are inserted.  A lookup is invalid only if
 // an earlier phrase of the same window inserted exactly the key that it missed; such a lane shares
@@ -167,7 +167,11 @@ __device__ __forceinline__ int warp_lzw_step(const CbView& cb, int b, int z) {
 //         codebook itself would take 256.  New entries go to the codebook's own hash table at the end.
 //   else  the codebook's hash table in global memory is used in place (two slots per 16-byte load).
 // ---------------------------------------------------------------------------------------------
-constexpr int kParseLanes = 128;          // starting points looked up at once (four warps)
+// A window of 256 costs little more than one of 128 (two warps per scheduler hide each other's latencies)
+// and moves 216 tokens on in long repetitive text where 128 moved 122; 512 would gain there and lose
+// where phrases repeat sooner (vocabulary 32064: 93 tokens either way).
+constexpr int kParseLanes = 256;          // starting points looked up at once
+constexpr int kParseWarps = kParseLanes / 32;
 constexpr int kParseThreads = 512;        // the other warps only help to fill and to write back
 constexpr int kParseSmemMaxCap = 16384;
 
@@ -188,7 +192,7 @@ struct ParseTable {
     return prefix * 0x9E3779B1u ^ hash_token_part(token);
   }
   // The slot index takes bits 13 and up of the mix, the tag the 13 bits below and the top two.
-  static __device__ __forceinline__ uint32_t tag_of(uint32_t h) { return (h & 0x1fffu) | ((h >> 30) << 13); }
+  static __device__ __forceinline__ uint32_t tag_of(uint32_t h) { return (h & 0x1fffu) | ((h >> 30) << 13); }       // below 2^15
 
   // Entry of (prefix, token), or -1 and the first empty slot of its probe sequence (-1: table full).
   __device__ __forceinline__ int probe(uint32_t prefix, uint32_t token, int& slot) const {
@@ -198,16 +202,18 @@ struct ParseTable {
       const uint32_t k0 = prefix | (token << 24), k1 = token >> 8;
       uint32_t at = (h >> 13) & (uint32_t)(n_slots - 4);
       for (int it = 0; it < n_slots; it += 4) {                    // bounded: at most the whole table
+        // all four slots at once, as bit masks: lanes of a warp differ in where their key or their gap lies
         const uint4 g = *reinterpret_cast<const uint4*>(tab + at);
-        const uint32_t v[4] = {g.x, g.y, g.z, g.w};
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (v[j] == 0xffffffffu) { slot = (int)at + j; return -1; }
-          if ((v[j] >> 16) == tag) {
-            const int e = (int)(v[j] & 0xffffu);
-            if (key0[e] == k0 && key1[e] == (uint16_t)k1) return e;
-          }
+        const uint32_t gap = (g.x == ~0u ? 1u : 0u) | (g.y == ~0u ? 2u : 0u) | (g.z == ~0u ? 4u : 0u) | (g.w == ~0u ? 8u : 0u);
+        uint32_t hit = (g.x >> 16 == tag ? 1u : 0u) | (g.y >> 16 == tag ? 2u : 0u) | (g.z >> 16 == tag ? 4u : 0u) |
+                       (g.w >> 16 == tag ? 8u : 0u);               // (an empty slot's tag is never one of a key's)
+        while (hit) {
+          const uint32_t v = (hit & 1u) ? g.x : (hit & 2u) ? g.y : (hit & 4u) ? g.z : g.w;
+          const int e = (int)(v & 0xffffu);
+          if (key0[e] == k0 && key1[e] == (uint16_t)k1) return e;
+          hit &= hit - 1;
         }
+        if (gap) { slot = (int)at + __ffs((int)gap) - 1; return -1; }
         at = (at + 4) & (uint32_t)(n_slots - 1);
       }
     } else {
@@ -285,28 +291,39 @@ struct ParseTable {
   }
 };
 
-// What the four parsing warps tell each other inside a window: per warp a mask of lanes on the
-// chain, of those that want a new entry, and of those whose bid lost.
-struct ParseVotes { uint32_t on[4], ins[4], lost[4]; };
+// What the parsing warps tell each other inside a window: per warp a mask of lanes on the chain, of
+// those that want a new entry, and of those whose bid lost.
+struct ParseVotes { uint32_t on[kParseWarps], ins[kParseWarps], lost[kParseWarps]; };
 
 // First losing lane of the window (kParseLanes if none).
-__device__ __forceinline__ int parse_first_lost(const ParseVotes& v) {
+__device__ __forceinline__ int parse_first_lost(const uint32_t (&lost)[kParseWarps]) {
   int f = kParseLanes;
 #pragma unroll
-  for (int k = 3; k >= 0; --k)
-    if (v.lost[k]) f = k * 32 + __ffs((int)v.lost[k]) - 1;
+  for (int k = kParseWarps - 1; k >= 0; --k)
+    if (lost[k]) f = k * 32 + __ffs((int)lost[k]) - 1;
   return f;
 }
-// Bits of m[0..3] below lane `at` of the window.
-__device__ __forceinline__ int parse_count_below(const uint32_t (&m)[4], int at) {
+// Bits of m below lane `at` of the window.
+__device__ __forceinline__ int parse_count_below(const uint32_t (&m)[kParseWarps], int at) {
   int c = 0;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
+  for (int k = 0; k < kParseWarps; ++k) {
     const int left = at - k * 32;
     const uint32_t keep = left >= 32 ? 0xffffffffu : (left <= 0 ? 0u : (1u << left) - 1u);
     c += __popc(m[k] & keep);
   }
   return c;
+}
+// The same for this thread's own lane, and the number of all bits.
+__device__ __forceinline__ int parse_rank(const uint32_t (&m)[kParseWarps], int warp, int lane, int& total) {
+  int below = 0;
+  total = 0;
+#pragma unroll
+  for (int k = 0; k < kParseWarps; ++k) {
+    if (k == warp) below = total + __popc(m[k] & ((1u << lane) - 1u));
+    total += __popc(m[k]);
+  }
+  return below;
 }
 
 }  // namespace z2z
