@@ -82,7 +82,7 @@ bool stream_gemm_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int
 // At most 128 rows, one CTA per tile of 128 weight rows.
 cudaError_t launch_stream_gemm(StreamGemmParams p, const StreamGemmMaps& maps, int n_sm, cudaStream_t s);
 
-// The same product on CTA pairs (z2z_stream_pair.cu): up to 256 packed rows ride on one stream of the
+// The same product for more than 128 rows on CTA pairs (z2z_stream_pair.cu): up to 256 packed rows ride on one stream of the
 // weights, and more run as blocks of 256.
 struct StreamPairParams {
   int groups, ksteps;
@@ -95,7 +95,7 @@ struct StreamPairParams {
   int tiles_per_group;   // tiles of 256 weight rows
   int blocks;            // blocks of 256 packed rows the capacity asks for
   int act_bytes;         // activation part of a stage
-  int stages, acc_bufs, acc_stride, tmem_cols;
+  int stages;
 };
 int stream_pair_ksb(int R);
 bool stream_pair_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int R);     // boxes of 16, 32, .. 128 rows

@@ -25,7 +25,7 @@
 // Operand layout: packed row r of the activations is rows 2 r (bf16 hi) and 2 r + 1 (lo) of
 // [2 Rt, K]; an epilogue thread owns one output feature and adds the two columns of a row.
 //
-// Roles per CTA: warp 0 lane 0 TMA producer, warp 1 lane 0 MMA issuer (leader CTA only), warps 2-5
+// Roles per CTA: warp 0 lane 0 TMA producer, warp 1 lane 0 MMA issuer (leader CTA only), warps 2-9
 // epilogue.  Every mbarrier wait is bounded.
 #include "z2z_common.cuh"
 #include "z2z_internal.h"
@@ -37,13 +37,14 @@ using namespace sm100;
 
 namespace {
 
-constexpr int kThreads = 192;
+constexpr int kEpiWarps = 8;             // two per tensor-memory lane quarter, one for each half of a row block
+constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kSpMaxStages = 8;
 constexpr int kSpBlockRows = 256;        // packed rows that share one stream of the weights
 constexpr int kSpSmem = 227 * 1024;
 
 struct SpCtrl {
-  unsigned long long full[kSpMaxStages], empty[kSpMaxStages], acc_full[2], acc_empty[2];
+  unsigned long long full[kSpMaxStages], empty[kSpMaxStages], acc_full, acc_empty;
   uint32_t tmem_base;
   int abort;
 };
@@ -86,6 +87,18 @@ __device__ __forceinline__ int sp_live_blocks(const StreamPairParams& p, int liv
   return p.blocks > 1 && live > kSpBlockRows ? (live + kSpBlockRows - 1) / kSpBlockRows : 1;
 }
 
+// 4 x 4 transpose among four neighbouring lanes: f[x] of lane t becomes f[t] of lane x.
+__device__ __forceinline__ void transpose4(float (&f)[4], int lane) {
+  float s0 = (lane & 1) ? f[0] : f[1], s1 = (lane & 1) ? f[2] : f[3];
+  s0 = __shfl_xor_sync(0xffffffffu, s0, 1);
+  s1 = __shfl_xor_sync(0xffffffffu, s1, 1);
+  if (lane & 1) { f[0] = s0; f[2] = s1; } else { f[1] = s0; f[3] = s1; }
+  s0 = (lane & 2) ? f[0] : f[2]; s1 = (lane & 2) ? f[1] : f[3];
+  s0 = __shfl_xor_sync(0xffffffffu, s0, 2);
+  s1 = __shfl_xor_sync(0xffffffffu, s1, 2);
+  if (lane & 2) { f[0] = s0; f[1] = s1; } else { f[2] = s0; f[3] = s1; }
+}
+
 template <int KSB>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps tm) {
@@ -103,17 +116,15 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps t
       mbar_init(smem_u32(&ctrl->full[s]), 1);        // leader: its producer's arrive + bytes of both CTAs
       mbar_init(smem_u32(&ctrl->empty[s]), 1);       // one multicast commit
     }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(smem_u32(&ctrl->acc_full[b]), 1);    // one multicast commit
-      mbar_init(smem_u32(&ctrl->acc_empty[b]), 8);   // leader: 4 epilogue warps of each CTA
-    }
+    mbar_init(smem_u32(&ctrl->acc_full), 1);         // one multicast commit
+    mbar_init(smem_u32(&ctrl->acc_empty), 2 * kEpiWarps);        // leader: epilogue warps of both CTAs
     ctrl->abort = 0;
     mbar_init_fence();
     prefetch_tmap(&tm.w[0]);
     if (p.groups > 1) prefetch_tmap(&tm.w[1]);
   }
   __syncthreads();
-  if (warp == 2) { tmem_alloc_pair(smem_u32(&ctrl->tmem_base), p.tmem_cols); tmem_relinquish_pair(); }
+  if (warp == 2) { tmem_alloc_pair(smem_u32(&ctrl->tmem_base), 512); tmem_relinquish_pair(); }
   tc_fence_before();
   __syncthreads();
   cluster_sync_all();                               // both CTAs' barriers exist before any remote signal
@@ -182,7 +193,6 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps t
     int live = *p.rows_dev;
     live = live < p.R ? live : p.R;
     const int n_blocks = sp_live_blocks(p, live);
-    const uint32_t nbuf = (uint32_t)p.acc_bufs;
     if (warp == 1) {
       if (lane == 0 && rank == 0) {
         // ---------------- MMA issuer (leader only): D[256 weight rows][n] += W tile x activation rows -----
@@ -191,12 +201,12 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps t
         SpWalk walk(p, n_blocks);
         SpJob j;
         while (ok && walk.next(j)) {
-          const uint32_t buf = job_i % nbuf, aph = (job_i / nbuf) & 1u;
-          if (!mbar_wait(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) break;
+          const uint32_t aph = job_i & 1u;
+          if (!mbar_wait(smem_u32(&ctrl->acc_empty), aph ^ 1u, &ctrl->abort)) break;
           tc_fence_after();
           const int n0 = sp_cols(live, j.block, 0), n1 = sp_cols(live, j.block, 1);
           const uint32_t id0 = idesc_bf16_f32(256, n0), id1 = idesc_bf16_f32(256, n1 ? n1 : 32);
-          const uint32_t d = tmem_base + buf * (uint32_t)p.acc_stride;
+          const uint32_t d = tmem_base;
           uint32_t acc = 0;
           for (int ks = j.kb0; ks < j.kb1; ++ks) {
             if (!mbar_wait(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
@@ -217,46 +227,53 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps t
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
           }
           if (!ok) break;
-          umma_commit_pair(smem_u32(&ctrl->acc_full[buf]));       // wakes the epilogues of both CTAs
+          umma_commit_pair(smem_u32(&ctrl->acc_full));       // wakes the epilogues of both CTAs
           ++job_i;
         }
       }
     } else {
       // ---------------- epilogue (both CTAs): thread = output feature -----------------------------------
+      // With two halves in tensor memory nothing overlaps the epilogue, and one reduction instruction per
+      // row and feature is what it costs: four lanes transpose four rows x four features among
+      // themselves and add 16 bytes each.  (217 rows, d = 3072, both encoders: 859 us a request start
+      // with single words on four warps, 805 with 16 bytes, 714 with the split below, 654 on eight warps.)
       const int q = warp & 3;                          // TMEM lane quarter this warp may read
-      uint32_t acc_empty_leader[2];
-      acc_empty_leader[0] = map_to_cta(smem_u32(&ctrl->acc_empty[0]), 0);
-      acc_empty_leader[1] = map_to_cta(smem_u32(&ctrl->acc_empty[1]), 0);
+      const int h = (warp - 2) >> 2;                   // half of the row block it takes
+      const uint32_t acc_empty_leader = map_to_cta(smem_u32(&ctrl->acc_empty), 0);
       uint32_t job_i = 0;
       SpWalk walk(p, n_blocks);
       SpJob j;
       while (walk.next(j)) {
-        const uint32_t buf = job_i % nbuf, aph = (job_i / nbuf) & 1u;
-        if (!mbar_wait(smem_u32(&ctrl->acc_full[buf]), aph, &ctrl->abort)) break;
+        const uint32_t aph = job_i & 1u;
+        if (!mbar_wait(smem_u32(&ctrl->acc_full), aph, &ctrl->abort)) break;
         tc_fence_after();
         const int feature0 = j.wrow + (int)rank * 128;
         if (feature0 < p.J) {                          // the last tile may be half outside (J is a multiple of 128)
+          const int row0 = j.block * kSpBlockRows + h * 128;
+          int rows = live - row0;
+          rows = rows > 128 ? 128 : rows;
+          // this lane's row of every four, and the first of the four features it adds
+          float* dst = p.out + ((size_t)j.g * p.Rt + row0 + (lane & 3)) * p.J + feature0 + q * 32 + (lane & ~3);
+          const uint32_t t0 = tmem_base + ((uint32_t)(q * 32) << 16) + h * 256u;
 #pragma unroll 1
-          for (int h = 0; h < 2; ++h) {
-            const int row0 = j.block * kSpBlockRows + h * 128;
-            int rows = live - row0;
-            rows = rows > 128 ? 128 : rows;
-            float* dst = p.out + ((size_t)j.g * p.Rt + row0) * p.J + feature0 + q * 32 + lane;
-            const uint32_t t0 = tmem_base + ((uint32_t)(q * 32) << 16) + buf * (uint32_t)p.acc_stride + h * 256u;
-#pragma unroll 1
-            for (int r0 = 0; r0 < rows; r0 += 8) {
-              uint32_t v[16];
-              tmem_ld16(t0 + 2 * r0, v);
-              tmem_ld_wait();
+          for (int r0 = 0; r0 < rows; r0 += 16) {
+            uint32_t v[32];
+            tmem_ld32(t0 + 2 * r0, v);
+            tmem_ld_wait();
 #pragma unroll
-              for (int x = 0; x < 8; ++x)
-                if (r0 + x < rows) red_add_f32(dst + (size_t)(r0 + x) * p.J, __uint_as_float(v[2 * x]) + __uint_as_float(v[2 * x + 1]));
+            for (int y = 0; y < 4; ++y) {
+              float f[4];
+#pragma unroll
+              for (int x = 0; x < 4; ++x) f[x] = __uint_as_float(v[8 * y + 2 * x]) + __uint_as_float(v[8 * y + 2 * x + 1]);
+              transpose4(f, lane);
+              const int r = r0 + 4 * y;
+              if (r + (lane & 3) < rows) red_add_f32x4(dst + (size_t)r * p.J, f[0], f[1], f[2], f[3]);
             }
           }
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(acc_empty_leader[buf]);
+        if (lane == 0) mbar_arrive_cluster(acc_empty_leader);
         ++job_i;
       }
     }
@@ -265,13 +282,13 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps t
   __syncthreads();
   if (threadIdx.x == 0 && ctrl->abort) atomicOr(p.err, 1);
   cluster_sync_all();                               // nobody leaves while the pair's MMAs may read its memory
-  if (warp == 2) tmem_dealloc_pair(tmem_base, p.tmem_cols);
+  if (warp == 2) tmem_dealloc_pair(tmem_base, 512);
 }
 
 int cols32(int rows) { return (2 * (rows < 128 ? rows : 128) + 31) / 32 * 32; }
 
-// Shared memory of one stage's activation boxes per CTA and k-block, for a pass of at most R rows.
-int pair_act_bytes(int R) { return R > 128 ? 16384 + cols32(R - 128) * 64 : cols32(R) * 64; }
+// Shared memory of one stage's activation boxes per CTA and k-block, for a pass of at most R > 128 rows.
+int pair_act_bytes(int R) { return 16384 + cols32(R - 128) * 64; }
 
 }  // namespace
 
@@ -289,22 +306,22 @@ bool stream_pair_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int
 }
 
 cudaError_t launch_stream_pair(StreamPairParams p, const StreamGemmMaps& maps, int n_sm, cudaStream_t s) {
-  if (!p.out || !p.err || !p.rows_dev || p.R < 1) return cudaErrorInvalidValue;
+  if (!p.out || !p.err || !p.rows_dev || p.R <= 128) return cudaErrorInvalidValue;
   const int ksb = stream_pair_ksb(p.R);
   p.tiles_per_group = (p.J + 255) / 256;
   p.blocks = (p.R + kSpBlockRows - 1) / kSpBlockRows;
   p.act_bytes = ksb * pair_act_bytes(p.R);
-  p.acc_bufs = p.R > 128 ? 1 : 2;                   // two accumulators in turn, or one with two halves
-  p.acc_stride = p.R > 128 ? 0 : cols32(p.R);
-  int cols = 32;
-  while (cols < (p.R > 128 ? 512 : 2 * p.acc_stride)) cols <<= 1;
-  p.tmem_cols = cols;
   const int stage = p.act_bytes + ksb * 16384;
   p.stages = (kSpSmem - 2048) / stage;
   if (p.stages > kSpMaxStages) p.stages = kSpMaxStages;
   const size_t smem = 2048 + (size_t)p.stages * stage;
   const long long units = (long long)p.groups * p.tiles_per_group * p.ksteps;      // every cluster owns >= 1 unit
-  const int clusters = units < n_sm / 2 ? (int)units : n_sm / 2;
+  int clusters = units < n_sm / 2 ? (int)units : n_sm / 2;
+  // A whole number of clusters per tile leaves every cluster with one piece of one tile, and so with one
+  // epilogue instead of two; worth up to a seventh of the clusters (217 rows, d = 3072: 859 -> 750 us a
+  // request start with 72 of 74).
+  const int tiles = p.groups * p.tiles_per_group, whole = clusters / tiles * tiles;
+  if (7 * whole >= 6 * clusters) clusters = whole;
   auto kern = ksb == 2 ? k_stream_pair<2> : k_stream_pair<1>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
