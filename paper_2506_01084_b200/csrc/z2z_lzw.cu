@@ -72,19 +72,23 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const i
     int loaded = 0;                                  // tokens already in s_tok
     int ahead = tid < T ? x[tid] : 0;                // token loaded + tid
     for (int p0 = 0; p0 < T;) {                      // p0: a phrase starts here
-      // positions below p0 + kParseLanes + kMaxM are looked at.  (s_tok is only read ahead of a window's
-      // second barrier, so that the tokens of the last window may be overwritten here.)
+      // Positions below p0 + kParseLanes + kMaxM are looked at; the ring is filled as far as it goes, so
+      // that a token has been on its way for a window before it is stored.  (A window moves p0 by 257 on
+      // average where no phrase repeats in it: with nothing in reserve every other window would wait for
+      // the last few tokens.  s_tok is only read ahead of a window's second barrier, so that the tokens
+      // of the last window may be overwritten here.)
       const int need = p0 + kParseLanes + kMaxM < T ? p0 + kParseLanes + kMaxM : T;
-      while (loaded < need) {
-        const int at = loaded + tid;
-        int c = ahead;
-        if (at < need) {
+      const int room_end = p0 + kTokRing < T ? p0 + kTokRing : T;
+      do {
+        const int cnt = room_end - loaded < kParseLanes ? room_end - loaded : kParseLanes;
+        if (tid < cnt) {
+          int c = ahead;
           if ((unsigned)c >= (unsigned)V) { st |= Z2Z_ST_BAD_TOKEN; c = 0; }     // not a base token
-          s_tok[at & (kTokRing - 1)] = c;
+          s_tok[(loaded + tid) & (kTokRing - 1)] = c;
         }
-        loaded = loaded + kParseLanes < need ? loaded + kParseLanes : need;
+        loaded += cnt;
         ahead = loaded + tid < T ? x[loaded + tid] : 0;
-      }
+      } while (loaded < need);
       parse_sync();
       // ---- longest match from every position of the window
       const int q = p0 + tid;
