@@ -4,19 +4,25 @@
 // they can be stored once (z2z_dynamic_logits with its full-logit output) and filtered here; the
 // fused argmax / Gumbel-max path of the logits kernels needs no stored logits.
 //
-// A cluster of 1 to 8 CTAs per row (as many as keep all rows within one wave of the SMs); every
-// pass reads the row from L2 (16-byte loads, two in flight per thread), each CTA its share of the
-// columns, and the CTAs add up their maxima, sums and digit histograms through distributed shared
-// memory between two cluster barriers:
+// A cluster of 1 to 8 CTAs per row (as many as keep all rows within one wave of the SMs); each CTA
+// reads its share of the columns once, keeps it in shared memory (up to 160 KB; a longer share is read
+// from L2 again by every pass), and the CTAs add up their maxima, sums and digit histograms through
+// distributed shared memory, one cluster barrier per pass:
 //   1. m = max l,  Z = sum exp((l - m) / T), in one pass and only when a nucleus is asked for;
 //   2. top-k: radix select (4 passes of 8 bits over order-preserving keys of the logits) of the
 //      k-th largest logit; everything >= it is kept (ties stay together);
 //   3. top-p: the same descent weighted by probability mass: the largest logit v with
-//      mass{l >= v} >= p Z; everything >= v is kept;
+//      mass{l >= v} >= p Z; everything >= v is kept.  After a top-k filter only its columns can matter:
+//      if they hold less than p Z the nucleus is the wider set and is not looked for, else the descent
+//      runs over them alone;
 //   4. Gumbel-max over the kept columns with the noise the fused sampler uses
 //      (Philox4x32-10 keyed by the seed, counter (column / 4, row, step), word column % 4).
 // The thresholds are found on the logits themselves, not on l / T: a positive scale preserves the
 // order, and equal logits stay exactly equal.
+//
+// Bound by the passes' barriers and dependent round trips, not by bytes.  (16 rows of 128 k columns, k = 50,
+// p = 0.9: 100 us when every pass read its columns from L2, took two cluster barriers and the nucleus was
+// always looked for; a whole step of 16 sequences went from 716 to 679 us.)
 #include <cooperative_groups.h>
 
 #include "z2z_common.cuh"
@@ -27,6 +33,7 @@ namespace z2z {
 namespace {
 
 constexpr int kSfThreads = 1024;
+constexpr int kSfHold = 40960;         // columns a CTA can keep in shared memory
 
 __device__ __forceinline__ uint32_t order_key(float x) {          // larger float <-> larger key
   const uint32_t u = __float_as_uint(x);
@@ -44,11 +51,13 @@ struct SfShared {
   } lanes;
   float red_f[32];
   int red_i[32];
-  unsigned int hist[256];       // per digit, this CTA's columns: count (top-k pass) or "occupied" flag (nucleus pass)
-  float mass[256];              // per digit, this CTA's columns: probability mass
+  // per digit, this CTA's columns: count (top-k pass) or "occupied" flag (nucleus pass), and probability mass.
+  // Two sets in turn: a pass may write its own while other CTAs still read the last one's.
+  unsigned int hist[2][256];
+  float mass[2][256];
   unsigned int tot_hist[256];   // the same over all CTAs that share the row
   float tot_mass[256];
-  float xf[3];                  // what a CTA shows the others: max, partition sum, best score
+  float xf[4];                  // what a CTA shows the others: max, partition sum, best score, mass of the k largest
   int xi[2];                    // best column, kept columns
   float m, Z;
   unsigned int prefix;
@@ -79,30 +88,22 @@ __device__ __forceinline__ float block_sum_f(float v, SfShared* sh) {
   return t;
 }
 
-// Calls f(logit, column) for every column of a row, each thread its share.  A row is read from L2
-// seven to eleven times by one CTA, so what counts is the bytes a thread keeps in flight: 16-byte
-// loads, two per thread at a time, when the row starts on a 16-byte boundary.
-// `t` is the thread's index among the `nt` threads that share the row (all CTAs of the cluster).
+// Calls f(logit, column) for the n columns from c0 on that lie at l (shared or global memory), each
+// thread its share: 16-byte loads when l starts on a 16-byte boundary.
 template <typename F>
-__device__ __forceinline__ void for_each_logit(const float* __restrict__ l, int C, int t, int nt, F f) {
+__device__ __forceinline__ void for_each_logit(const float* l, int c0, int n, F f) {
+  const int t = threadIdx.x;
   if ((reinterpret_cast<uintptr_t>(l) & 15u) == 0) {
     const float4* l4 = reinterpret_cast<const float4*>(l);
-    const int C4 = C >> 2;
-    int i = t;
-    for (; i + nt < C4; i += 2 * nt) {
-      const float4 a = l4[i], b = l4[i + nt];
-      const int ca = 4 * i, cb = 4 * (i + nt);
-      f(a.x, ca); f(a.y, ca + 1); f(a.z, ca + 2); f(a.w, ca + 3);
-      f(b.x, cb); f(b.y, cb + 1); f(b.z, cb + 2); f(b.w, cb + 3);
-    }
-    for (; i < C4; i += nt) {
+    const int n4 = n >> 2;
+    for (int i = t; i < n4; i += kSfThreads) {
       const float4 a = l4[i];
-      const int ca = 4 * i;
-      f(a.x, ca); f(a.y, ca + 1); f(a.z, ca + 2); f(a.w, ca + 3);
+      const int c = c0 + 4 * i;
+      f(a.x, c); f(a.y, c + 1); f(a.z, c + 2); f(a.w, c + 3);
     }
-    for (int c = (C4 << 2) + t; c < C; c += nt) f(l[c], c);
+    for (int i = (n4 << 2) + t; i < n; i += kSfThreads) f(l[i], c0 + i);
   } else {
-    for (int c = t; c < C; c += nt) f(l[c], c);
+    for (int i = t; i < n; i += kSfThreads) f(l[i], c0 + i);
   }
 }
 
@@ -111,29 +112,42 @@ __device__ __forceinline__ void for_each_logit(const float* __restrict__ l, int 
 __global__ void __launch_bounds__(kSfThreads) k_sample_filtered(const float* __restrict__ logits, long long ld,
                                                                 const int32_t* __restrict__ n_cols, int top_k,
                                                                 float top_p, float inv_t, uint32_t k0, uint32_t k1,
-                                                                uint32_t c2, uint32_t c3, int row_base,
+                                                                uint32_t c2, uint32_t c3, int row_base, int hold,
                                                                 int32_t* __restrict__ choice, int32_t* __restrict__ kept) {
+  extern __shared__ __align__(16) float s_hold[];                // this CTA's columns, if `hold` floats take them
   __shared__ SfShared sh;
   namespace cg = cooperative_groups;
   cg::cluster_group cluster = cg::this_cluster();
   const int G = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();     // CTAs that share the row
   const int r = blockIdx.x / G, tid = threadIdx.x;
-  const int gt = rank * kSfThreads + tid, gnt = G * kSfThreads;
   const int C = n_cols[r];
   const float* l = logits + (size_t)r * ld;
   if (C <= 0) { if (tid == 0 && rank == 0) { choice[r] = -1; if (kept) kept[r] = 0; } return; }   // (the whole cluster returns)
-  // ---- 1. max and partition sum in one pass (running maximum, sum rescaled when it moves); only
-  //         the nucleus filter needs them
+  // this CTA's columns [c0, c0 + n), c0 a multiple of 4
+  const int share = ((C + G - 1) / G + 3) & ~3;
+  const int c0 = rank * share < C ? rank * share : C;
+  const int n = C - c0 < share ? C - c0 : share;
+  const bool held = share <= hold;
+  const float* mine = held ? s_hold : l + c0;
+  float m = -INFINITY;
+  if (held) {
+    for_each_logit(l + c0, 0, n, [&](float x, int i) { s_hold[i] = x; m = fmaxf(m, x); });
+    __syncthreads();
+  } else if (top_p < 1.0f) {
+    for_each_logit(mine, c0, n, [&](float x, int) { m = fmaxf(m, x); });
+  }
+  auto each = [&](auto f) {
+    if (held) for_each_logit(static_cast<const float*>(s_hold), c0, n, f);
+    else for_each_logit(mine, c0, n, f);
+  };
+  // ---- 1. max and partition sum; only the nucleus filter needs them
   float mx = 0.f, z = 0.f;
   if (top_p < 1.0f) {
-    float m = -INFINITY, sum = 0.f;
-    for_each_logit(l, C, gt, gnt, [&](float x, int) {
-      if (x > m) { sum = sum * expf((m - x) * inv_t) + 1.f; m = x; }
-      else if (m > -INFINITY) sum += expf((x - m) * inv_t);     // (-inf logits before any finite one add nothing)
-    });
     const float m_cta = block_max(m, &sh);
-    // (a thread, or further down a CTA, without columns has m = -inf and adds nothing)
-    const float s_cta = block_sum_f(m > -INFINITY ? sum * expf((m - m_cta) * inv_t) : 0.f, &sh);
+    float sum = 0.f;
+    // (a CTA without columns, or with nothing but -inf, has m_cta = -inf and adds nothing)
+    if (m_cta > -INFINITY) each([&](float x, int) { sum += x == m_cta ? 1.f : expf((x - m_cta) * inv_t); });
+    const float s_cta = block_sum_f(sum, &sh);
     if (tid == 0) { sh.xf[0] = m_cta; sh.xf[1] = s_cta; }
     cluster.sync();
     mx = m_cta;
@@ -152,22 +166,22 @@ __global__ void __launch_bounds__(kSfThreads) k_sample_filtered(const float* __r
       for (int i = tid; i < 256 * 32; i += kSfThreads) sh.lanes.cnt[i] = 0u;
       __syncthreads();
       const unsigned int prefix = sh.prefix;
-      for_each_logit(l, C, gt, gnt, [&](float x, int) {
+      each([&](float x, int) {
         const uint32_t k = order_key(x);
         if (pass == 0 || (k >> (shift + 8)) == prefix) atomicAdd(&sh.lanes.cnt[((k >> shift) & 255u) * 32 + (tid & 31)], 1u);
       });
       __syncthreads();
       for (int d = tid >> 5; d < 256; d += kSfThreads / 32) {          // a warp sums the 32 copies of a digit
         const unsigned int v = __reduce_add_sync(0xffffffffu, sh.lanes.cnt[d * 32 + (tid & 31)]);
-        if ((tid & 31) == 0) sh.hist[d] = v;
+        if ((tid & 31) == 0) sh.hist[pass & 1][d] = v;
       }
       cluster.sync();                                    // every CTA's digit counts are in place
       if (tid < 256) {
         unsigned int v = 0u;
-        for (int g = 0; g < G; ++g) v += *cluster.map_shared_rank(&sh.hist[tid], g);
+        for (int g = 0; g < G; ++g) v += *cluster.map_shared_rank(&sh.hist[pass & 1][tid], g);
         sh.tot_hist[tid] = v;
       }
-      cluster.sync();                                    // ... and have been read by everyone
+      __syncthreads();
       if (tid < 32) {
         // from the largest digit down: lane L holds digits 255 - 8 L .. 248 - 8 L; the digit in which
         // the running count reaches what is left is the next digit of the k-th largest key (every
@@ -200,21 +214,32 @@ __global__ void __launch_bounds__(kSfThreads) k_sample_filtered(const float* __r
     key_k = sh.prefix;
   }
   // ---- 3. nucleus threshold by radix descent on probability mass
-  if (top_p < 1.0f) {
+  bool nucleus = top_p < 1.0f;
+  if (nucleus && key_k > 0u) {
+    float in_k = 0.f;
+    each([&](float x, int) { if (order_key(x) >= key_k) in_k += expf((x - mx) * inv_t); });
+    in_k = block_sum_f(in_k, &sh);
+    if (tid == 0) sh.xf[3] = in_k;
+    cluster.sync();
+    float mass_k = 0.f;
+    for (int g = 0; g < G; ++g) mass_k += *cluster.map_shared_rank(&sh.xf[3], g);
+    nucleus = !(mass_k < top_p * z);                       // the same sums and the same decision in every CTA
+  }
+  if (nucleus) {
     __syncthreads();
     if (tid == 0) { sh.prefix = 0u; sh.p_left = top_p * z; }
     for (int pass = 0; pass < 4; ++pass) {
       const int shift = 24 - 8 * pass;
       for (int i = tid; i < 256 * 32; i += kSfThreads) sh.lanes.mass[i] = 0.f;
-      if (tid < 256) sh.hist[tid] = 0u;
+      if (tid < 256) sh.hist[pass & 1][tid] = 0u;
       __syncthreads();
       const unsigned int prefix = sh.prefix;
-      for_each_logit(l, C, gt, gnt, [&](float x, int) {
+      each([&](float x, int) {
         const uint32_t k = order_key(x);
-        if (pass == 0 || (k >> (shift + 8)) == prefix) {
+        if (k >= key_k && (pass == 0 || (k >> (shift + 8)) == prefix)) {
           const unsigned int d = (k >> shift) & 255u;
           atomicAdd(&sh.lanes.mass[d * 32 + (tid & 31)], expf((x - mx) * inv_t));
-          sh.hist[d] = 1u;                                         // occupied (every writer stores 1)
+          sh.hist[pass & 1][d] = 1u;                                         // occupied (every writer stores 1)
         }
       });
       __syncthreads();
@@ -222,19 +247,19 @@ __global__ void __launch_bounds__(kSfThreads) k_sample_filtered(const float* __r
         float v = sh.lanes.mass[d * 32 + (tid & 31)];
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if ((tid & 31) == 0) sh.mass[d] = v;
+        if ((tid & 31) == 0) sh.mass[pass & 1][d] = v;
       }
       cluster.sync();                                    // every CTA's digit masses are in place
       if (tid < 256) {
         float v = 0.f;
         unsigned int occ = 0u;
         for (int g = 0; g < G; ++g) {
-          v += *cluster.map_shared_rank(&sh.mass[tid], g);
-          occ |= *cluster.map_shared_rank(&sh.hist[tid], g);
+          v += *cluster.map_shared_rank(&sh.mass[pass & 1][tid], g);
+          occ |= *cluster.map_shared_rank(&sh.hist[pass & 1][tid], g);
         }
         sh.tot_mass[tid] = v; sh.tot_hist[tid] = occ;
       }
-      cluster.sync();                                    // ... and have been read by everyone
+      __syncthreads();
       if (tid < 32) {
         // the same descent on probability mass (unoccupied digits hold none)
         float h[8], mine = 0.f;
@@ -281,7 +306,7 @@ __global__ void __launch_bounds__(kSfThreads) k_sample_filtered(const float* __r
   // ---- 4. Gumbel-max over the kept columns (lowest index on ties)
   float best = -INFINITY;
   int best_c = 0x7fffffff, n_kept = 0;
-  for_each_logit(l, C, gt, gnt, [&](float x, int c) {
+  each([&](float x, int c) {
     if (order_key(x) < key_t) return;
     ++n_kept;
     const Philox4 px = philox4x32_10((uint32_t)(c >> 2), (uint32_t)(row_base + r), c2, c3, k0, k1);
@@ -296,10 +321,10 @@ __global__ void __launch_bounds__(kSfThreads) k_sample_filtered(const float* __r
     if (ob > best || (ob == best && oc < best_c)) { best = ob; best_c = oc; }
   }
   __syncthreads();
-  if ((tid & 31) == 0) { sh.red_f[tid >> 5] = best; sh.red_i[tid >> 5] = best_c; sh.hist[tid >> 5] = (unsigned)n_kept; }
+  if ((tid & 31) == 0) { sh.red_f[tid >> 5] = best; sh.red_i[tid >> 5] = best_c; sh.tot_hist[tid >> 5] = (unsigned)n_kept; }
   __syncthreads();
   if (tid < 32) {
-    best = sh.red_f[tid]; best_c = sh.red_i[tid]; n_kept = (int)sh.hist[tid];
+    best = sh.red_f[tid]; best_c = sh.red_i[tid]; n_kept = (int)sh.tot_hist[tid];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const float ob = __shfl_xor_sync(0xffffffffu, best, o);
@@ -341,18 +366,22 @@ extern "C" int32_t z2z_sample_filtered(const float* d_logits, int32_t N, int64_t
   // within one wave of the 148 SMs)
   int G = 1;
   while (G < 8 && (long long)N * (2 * G) <= 148) G *= 2;
+  const long long share = ((ld + G - 1) / G + 3) & ~3ll;
+  const int hold = share <= z2z::kSfHold ? (int)share : 0;
+  cudaError_t e = cudaFuncSetAttribute(z2z::k_sample_filtered, cudaFuncAttributeMaxDynamicSharedMemorySize, z2z::kSfHold * 4);
+  if (e != cudaSuccess) { z2z::set_last_error(cudaGetErrorString(e)); return Z2Z_ERR_CUDA; }
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)N * (unsigned)G);
   lc.blockDim = dim3(z2z::kSfThreads);
-  lc.dynamicSmemBytes = 0;
+  lc.dynamicSmemBytes = (size_t)hold * 4;
   lc.stream = reinterpret_cast<cudaStream_t>(stream);
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)G; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   lc.attrs = at; lc.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&lc, z2z::k_sample_filtered, d_logits, (long long)ld, d_n_cols, top_k, top_p,
+  e = cudaLaunchKernelEx(&lc, z2z::k_sample_filtered, d_logits, (long long)ld, d_n_cols, top_k, top_p,
                                      1.0f / temperature, (uint32_t)seed, (uint32_t)(seed >> 32), (uint32_t)step,
-                                     (uint32_t)(step >> 32), row_base, d_choice, d_kept);
+                                     (uint32_t)(step >> 32), row_base, hold, d_choice, d_kept);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) { z2z::set_last_error(cudaGetErrorString(e)); return Z2Z_ERR_CUDA; }
   return Z2Z_OK;
