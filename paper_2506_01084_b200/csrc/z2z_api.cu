@@ -469,6 +469,8 @@ int32_t z2z_decode_step(z2z_codebook* cb, const void* d_hidden, const void* d_WE
     u.part_stride = info.stride; u.part_count = info.count; u.select = select; u.forced = d_forced;
     u.next_codes = d_next_codes; u.selected = d_selected; u.lse = a.lse; u.new_entry = w_new;
     u.frozen_flag = cb->h_frozen; u.epoch = cb->epoch;
+    u.records = cb->ws + cb->plan.off_step_out;
+    u.done = reinterpret_cast<unsigned*>(cb->ws + cb->plan.off_words) + 4;
     z2z::ProfScope ps(&cb->prof, z2z::kProfLzw, 1, s);
     Z2Z_CUDA(z2z::launch_decode_update(cb->view, u, el, s), "decode_step");
   } else {

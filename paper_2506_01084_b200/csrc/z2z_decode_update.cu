@@ -2,8 +2,13 @@
 // softmax reductions of every sequence from the per-CTA partials of the logits kernel, select the
 // token (argmax or Gumbel-max sample, or the caller's forced code; a sequence may sit out), apply the online LZW update,
 // and build the work list of new codebook entries for the hyper-encoder pass that follows.
-// One warp per sequence; a single block, so that the list can be compacted without a second
-// launch.
+// One block per sequence: its four warps merge the partials, the first one does the rest, and the block
+// that finishes last compacts the work list from the records that all of them left.
+//
+// Latency is all that counts here (a chain of dependent loads between two streams of weights): as one
+// block of 32 warps the kernel pulled the partials of the whole batch (148 per row, 32 bytes each)
+// through one SM and took 7.8 us at 8 sequences, 13 at 32 and 23 at 90; its 42 KB of shared memory also
+// kept it from being resident before the logits kernel had ended.
 #include "z2z_common.cuh"
 #include "z2z_internal.h"
 #include "z2z_lzw_dev.cuh"
@@ -11,33 +16,49 @@
 
 namespace z2z {
 
-__global__ void __launch_bounds__(1024) k_decode_update(CbView cb, DecodeUpdateArgs a, EntryList el) {
-  __shared__ int s_cnt[1024];
-  __shared__ int s_n[1024];                 // hypertokens of the sequence after this step
-  __shared__ signed char s_len[1024];       // base tokens of the entry it created
-  __shared__ int s_tok[1024][kMaxM];        // ... and the tokens themselves: the work list needs no reload
-  __shared__ int s_warp[32];
+namespace {
+
+constexpr int kUpdateThreads = 128;         // also the most sequences a fused step takes
+
+// What a block leaves for the last one: entry number + 1 (0: none), base tokens of the entry, hypertokens
+// of the sequence after the step, then the entry's tokens.
+struct StepRecord { int created, len, n, pad, tok[kMaxM]; };
+static_assert(sizeof(StepRecord) <= 64, "64 bytes per sequence are set aside");
+
+__device__ __forceinline__ RowRed shfl_xor_red(const RowRed& r, int off) {
+  RowRed o;
+  o.m = __shfl_xor_sync(0xffffffffu, r.m, off);
+  o.s = __shfl_xor_sync(0xffffffffu, r.s, off);
+  o.idx = __shfl_xor_sync(0xffffffffu, r.idx, off);
+  o.gm = __shfl_xor_sync(0xffffffffu, r.gm, off);
+  o.gidx = __shfl_xor_sync(0xffffffffu, r.gidx, off);
+  return o;
+}
+
+}  // namespace
+
+__global__ void __launch_bounds__(kUpdateThreads) k_decode_update(CbView cb, DecodeUpdateArgs a, EntryList el) {
+  __shared__ RowRed s_red[kUpdateThreads / 32];
+  __shared__ int s_warp[kUpdateThreads / 32], s_last;
   sm100::pdl_trigger();
   sm100::pdl_wait();               // the logits partials and the codebook state come from earlier kernels
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  for (int b = tid; b < 1024; b += blockDim.x) s_cnt[b] = 0;
-  __syncthreads();
-  for (int b = warp; b < cb.B; b += 32) {
-    const LzwPrev state = warp_lzw_load(cb, b);            // independent of the selection: loaded ahead of it
-    // ---- merge the partial reductions of hidden row b
-    const LogitPartial* lp = a.lpart + (size_t)b * a.part_stride;
-    RowRed red; red.init();
-    for (int g = lane; g < a.part_count; g += 32) red.merge(load_partial(lp + g));
+  const int b = blockIdx.x;
+  LzwPrev state{};
+  if (warp == 0) state = warp_lzw_load(cb, b);               // independent of the selection: loaded ahead of it
+  // ---- merge the partial reductions of hidden row b
+  const LogitPartial* lp = a.lpart + (size_t)b * a.part_stride;
+  RowRed red; red.init();
+  for (int g = tid; g < a.part_count; g += kUpdateThreads) red.merge(load_partial(lp + g));
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      RowRed o;
-      o.m = __shfl_xor_sync(0xffffffffu, red.m, off);
-      o.s = __shfl_xor_sync(0xffffffffu, red.s, off);
-      o.idx = __shfl_xor_sync(0xffffffffu, red.idx, off);
-      o.gm = __shfl_xor_sync(0xffffffffu, red.gm, off);
-      o.gidx = __shfl_xor_sync(0xffffffffu, red.gidx, off);
-      red.merge(o);
-    }
+  for (int off = 16; off > 0; off >>= 1) red.merge(shfl_xor_red(red, off));
+  if (lane == 0) s_red[warp] = red;
+  __syncthreads();
+  StepRecord* rec = reinterpret_cast<StepRecord*>(reinterpret_cast<char*>(a.records) + (size_t)b * 64);
+  if (warp == 0) {
+    red = s_red[0];
+#pragma unroll
+    for (int w = 1; w < kUpdateThreads / 32; ++w) red.merge(s_red[w]);
     const int amax = red.idx == 0x7fffffff ? -1 : red.idx;
     const int smp = red.gidx == 0x7fffffff ? -1 : red.gidx;
     const int sel = a.select == Z2Z_SELECT_GUMBEL ? smp : amax;
@@ -52,22 +73,36 @@ __global__ void __launch_bounds__(1024) k_decode_update(CbView cb, DecodeUpdateA
     // ---- online LZW update with the applied code
     int new_tok = -1;
     const int created = sits_out ? -1 : warp_lzw_step(cb, b, code, state, &new_tok);
-    if (lane < cb.M) s_tok[b][lane] = new_tok;
+    if (lane < cb.M) rec->tok[lane] = new_tok;
     if (lane == 0) {
       if (a.new_entry) a.new_entry[b] = created;
-      s_cnt[b] = created >= 0 ? created + 1 : 0;         // 0: none, else entry number + 1
-      s_len[b] = (signed char)(created >= 0 ? state.plen + 1 : 0);
-      s_n[b] = state.n + (created >= 0 ? 1 : 0);
+      rec->created = created + 1;
+      rec->len = created >= 0 ? state.plen + 1 : 0;
+      rec->n = state.n + (created >= 0 ? 1 : 0);
     }
+    __threadfence();                                         // the record is out before the block counts as done
+    __syncwarp();
+    if (lane == 0) s_last = atomicInc(a.done, gridDim.x - 1) == gridDim.x - 1;     // (returns to 0 by itself)
   }
   __syncthreads();
-  // ---- compact the new entries into the encoder's work list (exclusive scan over sequences): an
-  // entry's slot in the list, and the first of the PACKED rows that its base tokens take (the
-  // tensor-core pass keeps no padding rows).  Both sums travel in one word: entries in the low
-  // half, rows in the high half (at most 1024 entries of at most 8 rows).
-  const int mine = tid < cb.B ? s_cnt[tid] : 0;
-  const int flag = mine > 0 ? 1 : 0;
-  const int my_len = flag ? (int)s_len[tid] : 0;
+  if (!s_last) return;
+  __threadfence();
+  // ---- the last block: compact the new entries into the encoder's work list (exclusive scan over
+  // sequences): an entry's slot in the list, and the first of the PACKED rows that its base tokens
+  // take (the tensor-core pass keeps no padding rows).  Both sums travel in one word: entries in the
+  // low half, rows in the high half (at most 128 entries of at most 8 rows).
+  const StepRecord* mine_rec = reinterpret_cast<const StepRecord*>(reinterpret_cast<const char*>(a.records) + (size_t)tid * 64);
+  int4 head = make_int4(0, 0, 0, 0);
+  int tok[kMaxM];
+#pragma unroll
+  for (int i = 0; i < kMaxM; ++i) tok[i] = -1;
+  if (tid < cb.B) {
+    head = __ldcg(reinterpret_cast<const int4*>(mine_rec));
+    const int4 t0 = __ldcg(reinterpret_cast<const int4*>(mine_rec) + 1), t1 = __ldcg(reinterpret_cast<const int4*>(mine_rec) + 2);
+    tok[0] = t0.x; tok[1] = t0.y; tok[2] = t0.z; tok[3] = t0.w;
+    tok[4] = t1.x; tok[5] = t1.y; tok[6] = t1.z; tok[7] = t1.w;
+  }
+  const int mine = head.x, flag = mine > 0 ? 1 : 0, my_len = flag ? head.y : 0;
   const int val = flag | (my_len << 16);
   int incl = val;
 #pragma unroll
@@ -77,19 +112,15 @@ __global__ void __launch_bounds__(1024) k_decode_update(CbView cb, DecodeUpdateA
   }
   if (lane == 31) s_warp[warp] = incl;
   __syncthreads();
-  if (warp == 0) {
-    int w = s_warp[lane];
+  int before = 0, all = 0;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int x = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += x;
-    }
-    s_warp[lane] = w;
+  for (int w = 0; w < kUpdateThreads / 32; ++w) {
+    if (w < warp) before += s_warp[w];
+    all += s_warp[w];
   }
-  __syncthreads();
-  const int excl_both = incl - val + (warp > 0 ? s_warp[warp - 1] : 0);
+  const int excl_both = incl - val + before;
   const int excl = excl_both & 0xffff, row0 = excl_both >> 16;
-  const int total = s_warp[31] & 0xffff, total_rows = s_warp[31] >> 16;
+  const int total = all & 0xffff, total_rows = all >> 16;
   if (tid < cb.B) el.off[tid] = excl;
   if (tid == 0) {
     el.off[cb.B] = total; el.off[cb.B + 1] = total < el.chunk ? total : el.chunk;
@@ -99,20 +130,21 @@ __global__ void __launch_bounds__(1024) k_decode_update(CbView cb, DecodeUpdateA
     el.seq[excl] = tid; el.idx[excl] = mine - 1;
     el.len[excl] = my_len;
     el.row_off[excl] = row0;
-    for (int i = 0; i < cb.M; ++i) {
-      const int tok = s_tok[tid][i];
-      el.tok[(size_t)excl * cb.M + i] = tok;
-      if (i < my_len) { el.row_src[row0 + i] = excl * cb.M + i; el.row_tok[row0 + i] = tok; }
+#pragma unroll
+    for (int i = 0; i < kMaxM; ++i) {
+      if (i >= cb.M) break;
+      el.tok[(size_t)excl * cb.M + i] = tok[i];
+      if (i < my_len) { el.row_src[row0 + i] = excl * cb.M + i; el.row_tok[row0 + i] = tok[i]; }
     }
   }
-  for (int e = total + tid; e < el.chunk && e < cb.B; e += blockDim.x) {
+  for (int e = total + tid; e < el.chunk && e < cb.B; e += kUpdateThreads) {
     el.seq[e] = -1; el.idx[e] = 0; el.len[e] = 0; el.row_off[e] = total_rows;
     for (int i = 0; i < cb.M; ++i) el.tok[(size_t)e * cb.M + i] = -1;
   }
   // both caches will hold every entry once the encoder pass that follows has run
   int full = 1;
   if (tid < cb.B) {
-    const int n = s_n[tid];
+    const int n = head.z;
     cb.n_emb[tid] = n; cb.n_emb[cb.B + tid] = n;
     full = n >= cb.cap && mine == 0;             // full already when this step began: it created nothing
   }
@@ -121,7 +153,7 @@ __global__ void __launch_bounds__(1024) k_decode_update(CbView cb, DecodeUpdateA
   // against a late store from before a reset).  The word is only written by a step that found every
   // codebook full on entry: the step that creates the last entry still needs its encoder pass, and
   // the host may read the word at any time after this kernel was enqueued.
-  if (a.frozen_flag && cb.B <= (int)blockDim.x) {
+  if (a.frozen_flag) {
     const int all_full = __syncthreads_and(full);
     if (all_full && tid == 0) *reinterpret_cast<volatile int*>(a.frozen_flag) = a.epoch;
   }
@@ -129,8 +161,8 @@ __global__ void __launch_bounds__(1024) k_decode_update(CbView cb, DecodeUpdateA
 
 cudaError_t launch_decode_update(const CbView& cb, const DecodeUpdateArgs& a, const EntryList& el,
                                  cudaStream_t s) {
-  return launch_pdl(k_decode_update, dim3(1), dim3(1024), 0, s, cb, a, el);
-  return cudaGetLastError();
+  if (cb.B > kUpdateThreads) return cudaErrorInvalidValue;
+  return launch_pdl(k_decode_update, dim3(cb.B), dim3(kUpdateThreads), 0, s, cb, a, el);
 }
 
 }  // namespace z2z

@@ -162,6 +162,8 @@ struct DecodeUpdateArgs {
   int32_t* next_codes; int32_t* selected; float* lse; int32_t* new_entry;
   int* frozen_flag;   // host word mapped into the device's address space, or NULL
   int epoch;          // written there once every codebook of the session is full
+  void* records;      // 64 bytes per sequence
+  unsigned* done;     // blocks finished, zero before and after
 };
 cudaError_t launch_decode_update(const CbView& cb, const DecodeUpdateArgs& a, const EntryList& el,
                                  cudaStream_t s);
