@@ -341,7 +341,7 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
   // weight copies and the call is long enough (several passes) to repay making them.
   a.w_half = nullptr;
   if (tc && cb->half_scratch && cb->cfg.enc_layers > 0 && n_chunks >= 4 &&
-      z2z::encoder_pass_is_prompt_sized(a.entries, el.chunk, cb->cfg.M) &&
+      z2z::encoder_pass_is_prompt_sized(a.entries, el.chunk, cb->cfg.M, cb->cfg.d) &&
       cb->half_bytes >= z2z::encoder_half_bytes(cb->cfg.d, cb->dff, cb->cfg.enc_layers)) {
     cb->half_ptrs.assign((size_t)enc->n_tensors, nullptr);
     Z2Z_CUDA(z2z::convert_encoder_weights_to_half(enc->tensors, cb->cfg.d, cb->dff, cb->cfg.enc_layers, cb->half_scratch,

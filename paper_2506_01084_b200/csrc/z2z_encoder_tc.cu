@@ -54,11 +54,12 @@ constexpr int kMaxVec4 = 8;            // float4 per thread in the row kernels: 
 constexpr int kNarrowVec4 = 4;         // ... and for d <= 4096, where half the registers do
 // Which linear-layer kernel a pass takes, by its row capacity.  Up to 128 rows one CTA per weight tile streams
 // best (24 rows, d = 3072, both encoders: 249 us a step against 272 with pairs; 96 rows, d = 4096: equal);
-// beyond, CTA pairs carry up to 256 rows on one stream (270 rows, one encoder: 486 -> 327 us a step).  From 900
-// rows on whole output tiles beat the stream (one encoder, d = 3072, 900 rows: 767 against 749 us, 1023 rows:
-// 860 against 949; d = 4096, 800 rows: 1116 against 1085, 1024 rows: 1138 against 1197).
+// beyond, CTA pairs carry up to 512 rows on one stream (270 rows, one encoder: 486 -> 291 us a step).  Past that
+// the stream comes twice and whole output tiles take over, the earlier the wider the model, as a wave of
+// tiles is then fuller (one encoder: d = 3072, 768 rows 755 against 725 us, 1023 rows 860 against 949;
+// d = 4096, 680 rows 957 against 830, 800 rows 1116 against 1253).
 constexpr int kStreamSingleRows = 128;
-constexpr int kPairPassMinRows = 900;
+static int pair_pass_min_rows(int d) { return d > 3584 ? 720 : 900; }
 
 struct Ptr2 { const void* p[2]; };
 struct MPtr2 { void* p[2]; };
@@ -767,9 +768,9 @@ size_t encoder_half_bytes(int d, int dff, int layers) {
 }
 
 // Whether a pass of `entries` work-list slots is a prompt-sized one (CTA-pair GEMMs).
-bool encoder_pass_is_prompt_sized(int entries, int chunk, int M) {
+bool encoder_pass_is_prompt_sized(int entries, int chunk, int M, int d) {
   const int E = entries < chunk ? entries : chunk;
-  return E * M >= kPairPassMinRows;
+  return E * M >= pair_pass_min_rows(d);
 }
 
 // Makes fp16 copies of the linear-layer weights of one encoder in `scratch` and fills
@@ -825,7 +826,7 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   const int E = a0.entries;
   if (E > el.list || E > 1024 * kMapPerThread) return cudaErrorInvalidValue;
   const int R = a0.rows > 0 ? a0.rows : E * M;         // row capacity of this pass
-  if (ng == 1 && R >= kPairPassMinRows) return run_encoder_pass_pair(cb, a0, el, E, R, prof, s);
+  if (ng == 1 && R >= pair_pass_min_rows(d)) return run_encoder_pass_pair(cb, a0, el, E, R, prof, s);
   const int Rt = (R + 7) / 8 * 8;                      // rows of the result matrix per group
   const int* total = el.row_off + E;                   // packed rows of this pass (device word)
   const int n_sm = sm_count();
@@ -859,18 +860,26 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   const bool paired = R > kStreamSingleRows;
   const int ksb = paired ? stream_pair_ksb(R) : stream_gemm_ksb(R);
   StreamGemmMaps maps;
+  StreamPairMaps pair_maps;
   auto gemm = [&](const MPtr2& act, int K, int widx, int J) -> cudaError_t {
-    for (int g = 0; g < ng; ++g) {
-      if (!(paired ? stream_pair_act_maps : stream_gemm_act_maps)(maps.a[g], act.p[g], Rt, K, R)) return cudaErrorInvalidValue;
-      if (!make_tmap_bf16_kblocks(&maps.w[g], grp[g].w[widx], J, K, kNT, ksb)) return cudaErrorInvalidValue;
-    }
-    if (ng == 1) { maps.w[1] = maps.w[0]; for (int i = 0; i < 8; ++i) maps.a[1][i] = maps.a[0][i]; }
     auto fill = [&](auto p) {
       p.groups = ng; p.ksteps = K / (64 * ksb); p.R = R; p.out = Y; p.J = J; p.Rt = Rt; p.rows_dev = total; p.err = a0.err;
       return p;
     };
+    auto make = [&](auto& m, auto act_maps) {
+      for (int g = 0; g < ng; ++g)
+        if (!act_maps(g) || !make_tmap_bf16_kblocks(&m.w[g], grp[g].w[widx], J, K, kNT, ksb)) return false;
+      if (ng == 1) { m.w[1] = m.w[0]; for (int i = 0; i < 8; ++i) m.a[1][i] = m.a[0][i]; }
+      return true;
+    };
     ProfScope ps(prof, kProfEncGemm, 1, s);
-    if (paired) return launch_stream_pair(fill(StreamPairParams{}), maps, n_sm, s);
+    if (paired) {
+      if (!make(pair_maps, [&](int g) { return stream_pair_act_maps(pair_maps.a[g], pair_maps.wide[g], act.p[g], Rt, K, R); }))
+        return cudaErrorInvalidValue;
+      if (ng == 1) for (int i = 0; i < 8; ++i) pair_maps.wide[1][i] = pair_maps.wide[0][i];
+      return launch_stream_pair(fill(StreamPairParams{}), pair_maps, n_sm, s);
+    }
+    if (!make(maps, [&](int g) { return stream_gemm_act_maps(maps.a[g], act.p[g], Rt, K, R); })) return cudaErrorInvalidValue;
     return launch_stream_gemm(fill(StreamGemmParams{}), maps, n_sm, s);
   };
 

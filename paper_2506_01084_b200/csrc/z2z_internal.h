@@ -74,7 +74,7 @@ struct EncoderArgs {
 };
 bool encoder_tc_supported(int d, int dff, int dtype, int heads, int M);
 size_t encoder_half_bytes(int d, int dff, int layers);
-bool encoder_pass_is_prompt_sized(int entries, int chunk, int M);
+bool encoder_pass_is_prompt_sized(int entries, int chunk, int M, int d);
 cudaError_t convert_encoder_weights_to_half(const void* const* w, int d, int dff, int layers, void* scratch,
                                             const void** half_ptrs, int* err_word, Prof* prof, cudaStream_t s);
 bool logits_tc_supported(int d, int dtype);

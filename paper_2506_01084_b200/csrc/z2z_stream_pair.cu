@@ -12,18 +12,23 @@
 //   * the activation box follows the LIVE rows, a count that only the device knows: one tensor map
 //     per box height (16, 32, .. 128 rows), picked once the preceding kernel is done.  The weight
 //     boxes of the first pass over the ring are issued before that;
-//   * up to 256 packed rows (hi and lo part: 512 operand rows) ride on one stream of the weights: two
-//     accumulators of 256 columns fill tensor memory.  More rows run as several such blocks, the
-//     same weight tile one after the other, so that it comes from L2 the second time.
+//   * up to 512 packed rows ride on one stream of the weights.  NARROW, up to 256 live rows: hi and lo
+//     part of a row are two columns of tensor memory, two accumulators of 128 rows.  WIDE, more: the two
+//     parts accumulate into one column, two accumulators of 256 rows.  (At 217 rows narrow takes 654 us
+//     a request start and wide 719; rows in a second block of 256 brought the weights again: 902 against
+//     681 us on prompts of 200 to 300 rows.)  More rows run as several such blocks, the same
+//     weight tile one after the other, so that it comes from L2 the second time.
 // A decode step of 90 sequences (d = 3072, one encoder, 270 rows of capacity, about 150 live) went from
-// 486 to 327 us, the 240 rows of a short prompt's entries (both encoders) from 1.49 to 0.94 ms.
+// 486 to 291 us, the 200 to 300 rows of a short prompt's entries (both encoders) from 1.49 to 0.68 ms.
 //
 // Work is cut stream-K style: cluster c of C owns units [floor(c U / C), floor((c + 1) U / C)) of the
 // (group, weight tile, row block, k-step) space and adds its accumulators into the fp32 result with
 // reductions in global memory, like k_stream_gemm.
 //
 // Operand layout: packed row r of the activations is rows 2 r (bf16 hi) and 2 r + 1 (lo) of
-// [2 Rt, K]; an epilogue thread owns one output feature and adds the two columns of a row.
+// [2 Rt, K].  The narrow form's tensor map sees [k-block][operand row][64]; the wide form's sees
+// [k-block][part][row][64], so that one box brings the hi rows and behind them the lo rows.  An
+// epilogue thread owns one output feature.
 //
 // Roles per CTA: warp 0 lane 0 TMA producer, warp 1 lane 0 MMA issuer (leader CTA only), warps 2-9
 // epilogue.  Every mbarrier wait is bounded.
@@ -40,7 +45,8 @@ namespace {
 constexpr int kEpiWarps = 8;             // two per tensor-memory lane quarter, one for each half of a row block
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kSpMaxStages = 8;
-constexpr int kSpBlockRows = 256;        // packed rows that share one stream of the weights
+constexpr int kSpNarrowRows = 256;       // packed rows that two accumulators take with a column per part
+constexpr int kSpBlockRows = 512;        // packed rows that share one stream of the weights
 constexpr int kSpSmem = 227 * 1024;
 
 struct SpCtrl {
@@ -74,14 +80,19 @@ struct SpWalk {
   }
 };
 
-// Operand rows (hi and lo) of half `h` of a row block that the MMA covers: a multiple of 32 (the pair's
-// N), 0 if the half has no live row; the first half of a block always counts as having one.
+__device__ __forceinline__ bool sp_wide(int live) { return live > kSpNarrowRows; }
+// Columns of tensor memory (the MMA's N, a multiple of 32) that half `h` of a row block takes, 0 if it has
+// no live row; the first half of a block always counts as having one.
 __device__ __forceinline__ int sp_cols(int live, int block, int h) {
-  int rows = live - block * kSpBlockRows - h * 128;
+  const bool wide = sp_wide(live);
+  const int half = wide ? kSpBlockRows / 2 : kSpNarrowRows / 2;
+  int rows = live - block * kSpBlockRows - h * half;
   if (rows < 1) rows = (h == 0) ? 1 : 0;
-  if (rows > 128) rows = 128;
-  return (2 * rows + 31) & ~31;
+  if (rows > half) rows = half;
+  return ((wide ? rows : 2 * rows) + 31) & ~31;
 }
+// Bytes per CTA and k-block of the activation box for n columns: half of the operand rows.
+__device__ __forceinline__ uint32_t sp_box_bytes(bool wide, int n) { return (uint32_t)n * (wide ? 128u : 64u); }
 // Row blocks with a live row (at least one).  A pass whose capacity is one block does not need the count.
 __device__ __forceinline__ int sp_live_blocks(const StreamPairParams& p, int live) {
   return p.blocks > 1 && live > kSpBlockRows ? (live + kSpBlockRows - 1) / kSpBlockRows : 1;
@@ -101,7 +112,7 @@ __device__ __forceinline__ void transpose4(float (&f)[4], int lane) {
 
 template <int KSB>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps tm) {
+k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps tm) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   SpCtrl* ctrl = reinterpret_cast<SpCtrl*>(sm);
@@ -143,15 +154,19 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps t
       SpJob def[kSpMaxStages];                        // load i of the first pass uses stage i; kb0 = its k-step
       int n_def = 0, issued = 0, live = 0;
       bool deps = false, ok = true;
-      auto act_bytes = [&](int block) { return (uint32_t)(sp_cols(live, block, 0) + sp_cols(live, block, 1)) * (KSB * 64u); };
+      auto act_bytes = [&](int block) { return KSB * sp_box_bytes(sp_wide(live), sp_cols(live, block, 0) + sp_cols(live, block, 1)); };
       auto load_act = [&](int st, const SpJob& j, int ks) {
         const uint32_t sb = stage_base + (uint32_t)st * stage_bytes;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int n = sp_cols(live, j.block, h);
           if (n == 0) continue;
-          const int row = 2 * (j.block * kSpBlockRows + h * 128) + (int)rank * (n >> 1);
-          tma_load_3d_pair(sb + h * (KSB * 16384u), &tm.a[j.g][(n >> 5) - 1], 0, row, ks * KSB, full_leader[st], pol_a);
+          if (sp_wide(live))
+            tma_load_4d_pair(sb + h * (KSB * 32768u), &tm.wide[j.g][(n >> 5) - 1], 0,
+                             j.block * kSpBlockRows + h * (kSpBlockRows / 2) + (int)rank * (n >> 1), 0, ks * KSB, full_leader[st], pol_a);
+          else
+            tma_load_3d_pair(sb + h * (KSB * 16384u), &tm.a[j.g][(n >> 5) - 1], 0, h * kSpNarrowRows + (int)rank * (n >> 1), ks * KSB,
+                             full_leader[st], pol_a);
         }
       };
       auto need_deps = [&]() {
@@ -193,6 +208,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps t
     int live = *p.rows_dev;
     live = live < p.R ? live : p.R;
     const int n_blocks = sp_live_blocks(p, live);
+    const bool wide = sp_wide(live);
     if (warp == 1) {
       if (lane == 0 && rank == 0) {
         // ---------------- MMA issuer (leader only): D[256 weight rows][n] += W tile x activation rows -----
@@ -207,6 +223,9 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps t
           const int n0 = sp_cols(live, j.block, 0), n1 = sp_cols(live, j.block, 1);
           const uint32_t id0 = idesc_bf16_f32(256, n0), id1 = idesc_bf16_f32(256, n1 ? n1 : 32);
           const uint32_t d = tmem_base;
+          const uint32_t kb0 = sp_box_bytes(wide, n0), kb1 = sp_box_bytes(wide, n1);        // one k-block of a half's box
+          const uint32_t half1 = KSB * (wide ? 32768u : 16384u);
+          const int parts = wide ? 2 : 1;
           uint32_t acc = 0;
           for (int ks = j.kb0; ks < j.kb1; ++ks) {
             if (!mbar_wait(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
@@ -215,13 +234,14 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps t
 #pragma unroll
             for (int i = 0; i < KSB; ++i) {
               const uint32_t wb = sb + p.act_bytes + i * 16384u;
-              const uint32_t a0 = sb + (uint32_t)i * n0 * 64u, a1 = sb + KSB * 16384u + (uint32_t)i * n1 * 64u;
+              const uint32_t a0 = sb + (uint32_t)i * kb0, a1 = sb + half1 + (uint32_t)i * kb1;
+              for (int part = 0; part < parts; ++part)         // wide: hi rows, then lo rows, into the same columns
 #pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                umma_bf16_pair(d, smem_desc_sw128(wb + k * 32), smem_desc_sw128(a0 + k * 32), id0, acc);
-                if (n1) umma_bf16_pair(d + 256, smem_desc_sw128(wb + k * 32), smem_desc_sw128(a1 + k * 32), id1, acc);
-                acc = 1;
-              }
+                for (int k = 0; k < 4; ++k) {
+                  umma_bf16_pair(d, smem_desc_sw128(wb + k * 32), smem_desc_sw128(a0 + part * (kb0 / 2) + k * 32), id0, acc);
+                  if (n1) umma_bf16_pair(d + 256, smem_desc_sw128(wb + k * 32), smem_desc_sw128(a1 + part * (kb1 / 2) + k * 32), id1, acc);
+                  acc = 1;
+                }
             }
             umma_commit_pair(smem_u32(&ctrl->empty[stage]));      // frees the stage in both CTAs
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -233,12 +253,12 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps t
       }
     } else {
       // ---------------- epilogue (both CTAs): thread = output feature -----------------------------------
-      // With two halves in tensor memory nothing overlaps the epilogue, and one reduction instruction per
+      // Nothing overlaps the epilogue, as both accumulators are in use, and one reduction instruction per
       // row and feature is what it costs: four lanes transpose four rows x four features among
       // themselves and add 16 bytes each.  (217 rows, d = 3072, both encoders: 859 us a request start
       // with single words on four warps, 805 with 16 bytes, 714 with the split below, 654 on eight warps.)
       const int q = warp & 3;                          // TMEM lane quarter this warp may read
-      const int h = (warp - 2) >> 2;                   // half of the row block it takes
+      const int group = (warp - 2) >> 2;               // takes every other 32 columns
       const uint32_t acc_empty_leader = map_to_cta(smem_u32(&ctrl->acc_empty), 0);
       uint32_t job_i = 0;
       SpWalk walk(p, n_blocks);
@@ -249,25 +269,36 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps t
         tc_fence_after();
         const int feature0 = j.wrow + (int)rank * 128;
         if (feature0 < p.J) {                          // the last tile may be half outside (J is a multiple of 128)
-          const int row0 = j.block * kSpBlockRows + h * 128;
-          int rows = live - row0;
-          rows = rows > 128 ? 128 : rows;
+          const int row0 = j.block * kSpBlockRows;
+          const int rows = live - row0 < kSpBlockRows ? live - row0 : kSpBlockRows;
           // this lane's row of every four, and the first of the four features it adds
           float* dst = p.out + ((size_t)j.g * p.Rt + row0 + (lane & 3)) * p.J + feature0 + q * 32 + (lane & ~3);
-          const uint32_t t0 = tmem_base + ((uint32_t)(q * 32) << 16) + h * 256u;
+          const uint32_t t0 = tmem_base + ((uint32_t)(q * 32) << 16);
+          auto add4 = [&](float (&f)[4], int r) {      // rows r .. r + 3
+            transpose4(f, lane);
+            if (r + (lane & 3) < rows) red_add_f32x4(dst + (size_t)r * p.J, f[0], f[1], f[2], f[3]);
+          };
 #pragma unroll 1
-          for (int r0 = 0; r0 < rows; r0 += 16) {
+          for (int c0 = 32 * group; c0 < (wide ? rows : 2 * rows); c0 += 64) {
             uint32_t v[32];
-            tmem_ld32(t0 + 2 * r0, v);
+            tmem_ld32(t0 + c0, v);
             tmem_ld_wait();
+            if (wide) {
 #pragma unroll
-            for (int y = 0; y < 4; ++y) {
-              float f[4];
+              for (int y = 0; y < 8; ++y) {
+                float f[4];
 #pragma unroll
-              for (int x = 0; x < 4; ++x) f[x] = __uint_as_float(v[8 * y + 2 * x]) + __uint_as_float(v[8 * y + 2 * x + 1]);
-              transpose4(f, lane);
-              const int r = r0 + 4 * y;
-              if (r + (lane & 3) < rows) red_add_f32x4(dst + (size_t)r * p.J, f[0], f[1], f[2], f[3]);
+                for (int x = 0; x < 4; ++x) f[x] = __uint_as_float(v[4 * y + x]);
+                add4(f, c0 + 4 * y);
+              }
+            } else {
+#pragma unroll
+              for (int y = 0; y < 4; ++y) {
+                float f[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) f[x] = __uint_as_float(v[8 * y + 2 * x]) + __uint_as_float(v[8 * y + 2 * x + 1]);
+                add4(f, c0 / 2 + 4 * y);
+              }
             }
           }
         }
@@ -285,10 +316,14 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamGemmMaps t
   if (warp == 2) tmem_dealloc_pair(tmem_base, 512);
 }
 
-int cols32(int rows) { return (2 * (rows < 128 ? rows : 128) + 31) / 32 * 32; }
+int round32(int n) { return (n + 31) / 32 * 32; }
 
 // Shared memory of one stage's activation boxes per CTA and k-block, for a pass of at most R > 128 rows.
-int pair_act_bytes(int R) { return 16384 + cols32(R - 128) * 64; }
+int pair_act_bytes(int R) {
+  if (R <= kSpNarrowRows) return 16384 + round32(2 * (R - 128)) * 64;
+  R = R < kSpBlockRows ? R : kSpBlockRows;
+  return 32768 + round32(R - kSpBlockRows / 2) * 128;          // (the narrow form takes at most 32 KB)
+}
 
 }  // namespace
 
@@ -296,16 +331,17 @@ int pair_act_bytes(int R) { return 16384 + cols32(R - 128) * 64; }
 int stream_pair_ksb(int R) { return (kSpSmem - 2048) / (2 * (16384 + pair_act_bytes(R))) >= 4 ? 2 : 1; }
 
 // Tensor maps of one activation operand ([2 Rt, K], hi and lo rows interleaved): one per box height.
-bool stream_pair_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int R) {
-  const int n = cols32(R) / 32, ksb = stream_pair_ksb(R);
+bool stream_pair_act_maps(CUtensorMap* narrow, CUtensorMap* wide, const void* act, int Rt, int K, int R) {
+  const int ksb = stream_pair_ksb(R);
   for (int i = 0; i < 8; ++i) {
-    if (i >= n) { maps[i] = maps[n - 1]; continue; }
-    if (!make_tmap_bf16_kblocks(&maps[i], act, 2ll * Rt, K, 16 * (i + 1), ksb)) return false;
+    if (!make_tmap_bf16_kblocks(&narrow[i], act, 2ll * Rt, K, 16 * (i + 1), ksb)) return false;
+    if (R <= kSpNarrowRows) wide[i] = narrow[i];
+    else if (!make_tmap_bf16_parts(&wide[i], act, Rt, K, 16 * (i + 1), ksb)) return false;
   }
   return true;
 }
 
-cudaError_t launch_stream_pair(StreamPairParams p, const StreamGemmMaps& maps, int n_sm, cudaStream_t s) {
+cudaError_t launch_stream_pair(StreamPairParams p, const StreamPairMaps& maps, int n_sm, cudaStream_t s) {
   if (!p.out || !p.err || !p.rows_dev || p.R <= 128) return cudaErrorInvalidValue;
   const int ksb = stream_pair_ksb(p.R);
   p.tiles_per_group = (p.J + 255) / 256;

@@ -1,5 +1,5 @@
 """Hyper-encoder passes at the row counts where the linear-layer kernel, its activation box or its row blocks
-change: one entry, capacities around 128 and 256 packed rows (also with few of them live), the switch
+change: one entry, capacities around 128, 256 and 512 packed rows (also with few of them live), the switch
 to whole output tiles, a rest behind full passes; odd multiples of 128 as width (half a tile of 256 weight
 rows); a session whose very first pass is captured into a graph.  Against the fp64 oracle."""
 import numpy as np
@@ -39,7 +39,8 @@ def _check(w, p, got, first, count):
 @pytest.mark.parametrize("bound", ["exact", "count", "loose"])
 @pytest.mark.parametrize("d,dff,M,total", [(128, 384, 3, 1), (256, 512, 3, 42), (256, 512, 3, 43), (384, 640, 8, 16),
                                            (128, 256, 3, 85), (384, 1152, 3, 86), (256, 512, 3, 171), (256, 256, 4, 224),
-                                           (256, 256, 4, 225), (128, 384, 2, 512), (128, 128, 3, 1050)])
+                                           (256, 256, 4, 225), (128, 384, 2, 512), (128, 128, 3, 1050),
+                                           (256, 384, 3, 112), (384, 256, 3, 230), (128, 256, 3, 290)])
 def test_embedding_a_range_of_entries(d, dff, M, total, bound):
     B = 3
     w, p = _pair(d, dff, M, B, T=max(400, 6 * total), cap=1400, seed=total)
