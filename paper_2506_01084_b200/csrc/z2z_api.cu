@@ -355,7 +355,9 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
   const int per = pass_rows - (cb->cfg.M - 1);
   const long long n_passes = rows > 0 ? (rows + per - 1) / per : 0;
   if (n_passes > 0 && pass_rows <= cb->plan.enc_rows && (size_t)(n_passes + 1) * 4 <= cb->plan.plan_bytes) {
-    {
+    if (n_passes == 1) {
+      pass_first = nullptr;                            // all entries of the call
+    } else {
       z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 1, s);
       Z2Z_CUDA(z2z::launch_entry_passes(cb->view, which, d_first, el, pass_rows, (int)n_passes, pass_first, s), "hyper_embed");
     }

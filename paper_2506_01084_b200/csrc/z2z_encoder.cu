@@ -8,6 +8,7 @@
 #include "z2z_common.cuh"
 #include "z2z_internal.h"
 #include "z2z_simt_tile.cuh"
+#include "z2z_sm100.cuh"
 
 namespace z2z {
 
@@ -78,6 +79,8 @@ __device__ __forceinline__ void entry_of(const CbView& cb, int which, int mode, 
 __global__ void k_entry_fill(CbView cb, int which, int mode, const int32_t* __restrict__ first,
                              const int32_t* __restrict__ new_entry, EntryList el, long long g0, int slots,
                              const int32_t* __restrict__ pass_first) {
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   long long end = el.off[cb.B];
   if (pass_first) { g0 = pass_first[0]; end = pass_first[1]; }
@@ -338,9 +341,8 @@ cudaError_t launch_entry_offsets_from_new(const CbView& cb, const int32_t* new_e
 cudaError_t launch_entry_fill(const CbView& cb, int which, const int32_t* first,
                               const int32_t* new_entry, const EntryList& el, int chunk_index,
                               cudaStream_t s) {
-  k_entry_fill<<<(el.chunk + 255) / 256, 256, 0, s>>>(cb, which, new_entry ? 1 : 0, first, new_entry, el,
-                                                      (long long)chunk_index * el.chunk, el.chunk, nullptr);
-  return cudaGetLastError();
+  return launch_pdl(k_entry_fill, dim3((el.chunk + 255) / 256), dim3(256), 0, s, cb, which, new_entry ? 1 : 0, first, new_entry,
+                    el, (long long)chunk_index * el.chunk, el.chunk, nullptr);
 }
 cudaError_t launch_entry_rows(const CbView& cb, int which, const int32_t* first, const EntryList& el, cudaStream_t s) {
   k_entry_rows<<<cb.B, 256, 0, s>>>(cb, which, first, el);
@@ -353,8 +355,8 @@ cudaError_t launch_entry_passes(const CbView& cb, int which, const int32_t* firs
 }
 cudaError_t launch_entry_fill_pass(const CbView& cb, int which, const int32_t* first, const EntryList& el, int pass,
                                    const int32_t* pass_first, int slots, cudaStream_t s) {
-  k_entry_fill<<<(slots + 255) / 256, 256, 0, s>>>(cb, which, 0, first, nullptr, el, 0, slots, pass_first + pass);
-  return cudaGetLastError();
+  return launch_pdl(k_entry_fill, dim3((slots + 255) / 256), dim3(256), 0, s, cb, which, 0, first, nullptr, el, 0ll, slots,
+                    pass_first ? pass_first + pass : nullptr);
 }
 cudaError_t launch_mark_embedded(const CbView& cb, int which, cudaStream_t s) {
   k_mark_embedded<<<(cb.B + 255) / 256, 256, 0, s>>>(cb, which);

@@ -419,6 +419,8 @@ __global__ void k_tc_qkv_attention(CbView cb, EntryList el, float* Y, Ptr2 bias,
 constexpr int kMapPerThread = kMaxM / 2;
 __global__ void __launch_bounds__(1024) k_tc_row_map(CbView cb, EntryList el, int E) {
   __shared__ int warp_sums[32];
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int per = (E + 1023) / 1024, e0 = tid * per;
   int len[kMapPerThread], mine = 0;
@@ -466,6 +468,8 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_gather_ln_packed(CbView cb, 
                                                                      const bf16* ln_b, float* X, bf16* Ahl, int d, int Rt,
                                                                      int has_ln) {
   __shared__ float sm[32];
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   const int r = blockIdx.x;
   if (r >= *total) return;
   const int src = el.row_src[r];
@@ -495,6 +499,8 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_gather_ln_packed(CbView cb, 
 // ceil(d / (4 * kRowThreads))): a thread owns 4 columns and loads all rows before it adds.
 __global__ void __launch_bounds__(kRowThreads) k_tc_pool_packed(CbView cb, EntryList el, const float* X, void* cache,
                                                                 float* cache_f32, int d) {
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   const int e = blockIdx.x;
   const int col = ((int)blockIdx.y * kRowThreads + (int)threadIdx.x) * 4;
   if (col >= d) return;
@@ -523,6 +529,8 @@ template <int NV, bool HALF>
 __global__ void __launch_bounds__(kRowThreads) k_tc_ln_rows(const int* total, const float* X, const bf16* ln_w,
                                                             const bf16* ln_b, bf16* Ahl, int d, int Rt) {
   __shared__ float sm[32];
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   const int r = blockIdx.x;
   if (r >= *total) return;
   const float* x = X + (size_t)r * d;
@@ -550,6 +558,8 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_ln_rows(const int* total, co
 template <int MM, bool HALF>
 __global__ void __launch_bounds__(256) k_tc_attention_rows_warp(CbView cb, EntryList el, const float* QKV, bf16* Ohl,
                                                                 int E, int d, int heads, int Rt) {
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   const int lane = threadIdx.x & 31;
   const int item = blockIdx.x * 8 + (threadIdx.x >> 5);
   if (item >= E * heads) return;
@@ -609,6 +619,8 @@ __global__ void __launch_bounds__(256) k_tc_attention_rows_warp(CbView cb, Entry
 __global__ void k_tc_attention_rows(CbView cb, EntryList el, const float* QKV, bf16* Ohl, int d, int heads, int Rt,
                                     int half) {
   extern __shared__ float s_qkv[];
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   const int e = blockIdx.x, h = blockIdx.y, i = threadIdx.y, lane = threadIdx.x;
   const int L = entry_len_tc(cb, el, e);
   if (L <= 0) return;
@@ -719,16 +731,17 @@ static cudaError_t run_encoder_pass_pair(const CbView& cb, const EncoderArgs& a,
     ProfScope ps(prof, kProfEncGemm, 1, s);
     return launch_pair_gemm(p, act, half ? a.w_half[widx] : a.w[widx], K, epi, half, s);
   };
+  cudaError_t e;
   {
     ProfScope ps(prof, kProfEncOther, 2, s);
-    k_tc_row_map<<<1, 1024, 0, s>>>(cb, el, E);
+    if ((e = launch_pdl(k_tc_row_map, dim3(1), dim3(1024), 0, s, cb, el, E)) != cudaSuccess) return e;
     auto gk = half ? (narrow ? k_tc_gather_ln_packed<kNarrowVec4, true> : k_tc_gather_ln_packed<kMaxVec4, true>)
                    : (narrow ? k_tc_gather_ln_packed<kNarrowVec4, false> : k_tc_gather_ln_packed<kMaxVec4, false>);
-    gk<<<R, kRowThreads, 0, s>>>(cb, el, total, reinterpret_cast<const bf16*>(a.table), Wp(0), a.layers ? Wp(1) : Wp(0),
-                                 a.layers ? Wp(2) : Wp(0), a.X, a.Ahl, d, Rt, a.layers > 0 ? 1 : 0);
+    e = launch_pdl(gk, dim3(R), dim3(kRowThreads), 0, s, cb, el, total, reinterpret_cast<const bf16*>(a.table), Wp(0),
+                   a.layers ? Wp(1) : Wp(0), a.layers ? Wp(2) : Wp(0), a.X, a.Ahl, d, Rt, a.layers > 0 ? 1 : 0);
+    if (e != cudaSuccess) return e;
   }
   const int dh = d / a.heads;
-  cudaError_t e;
   for (int l = 0; l < a.layers; ++l) {
     const int o = 1 + 12 * l;
     if ((e = gemm(a.Ahl, d, o + 2, 3 * d, kEpiStore, a.QKV, nullptr)) != cudaSuccess) return e;
@@ -736,30 +749,30 @@ static cudaError_t run_encoder_pass_pair(const CbView& cb, const EncoderArgs& a,
       ProfScope ps(prof, kProfEncOther, 1, s);
       if (dh <= 128 && M <= 4) {
         auto ak = half ? k_tc_attention_rows_warp<4, true> : k_tc_attention_rows_warp<4, false>;
-        ak<<<(E * a.heads + 7) / 8, 256, 0, s>>>(cb, el, a.QKV, a.Ahl, E, d, a.heads, Rt);
+        e = launch_pdl(ak, dim3((E * a.heads + 7) / 8), dim3(256), 0, s, cb, el, a.QKV, a.Ahl, E, d, a.heads, Rt);
       } else {
-        k_tc_attention_rows<<<dim3(E, a.heads), dim3(32, M), (size_t)M * 3 * dh * 4, s>>>(cb, el, a.QKV, a.Ahl, d,
-                                                                                           a.heads, Rt, half ? 1 : 0);
+        e = launch_pdl(k_tc_attention_rows, dim3(E, a.heads), dim3(32, M), (size_t)M * 3 * dh * 4, s, cb, el, a.QKV, a.Ahl, d,
+                       a.heads, Rt, half ? 1 : 0);
       }
+      if (e != cudaSuccess) return e;
     }
     if ((e = gemm(a.Ahl, d, o + 4, d, kEpiResid, a.X, nullptr)) != cudaSuccess) return e;
     if (dff > 0) {                                     // dff == 0: attention-only layer
       {
         ProfScope ps(prof, kProfEncOther, 1, s);
-        lnk<<<R, kRowThreads, 0, s>>>(total, a.X, Wp(o + 6), Wp(o + 7), a.Ahl, d, Rt);
+        if ((e = launch_pdl(lnk, dim3(R), dim3(kRowThreads), 0, s, total, a.X, Wp(o + 6), Wp(o + 7), a.Ahl, d, Rt)) != cudaSuccess) return e;
       }
       if ((e = gemm(a.Ahl, d, o + 8, dff, kEpiGelu, nullptr, a.Hhl)) != cudaSuccess) return e;
       if ((e = gemm(a.Hhl, dff, o + 10, d, kEpiResid, a.X, nullptr)) != cudaSuccess) return e;
     }
     if (l + 1 < a.layers) {
       ProfScope ps(prof, kProfEncOther, 1, s);
-      lnk<<<R, kRowThreads, 0, s>>>(total, a.X, Wp(o + 12), Wp(o + 13), a.Ahl, d, Rt);
+      if ((e = launch_pdl(lnk, dim3(R), dim3(kRowThreads), 0, s, total, a.X, Wp(o + 12), Wp(o + 13), a.Ahl, d, Rt)) != cudaSuccess) return e;
     }
   }
   ProfScope ps(prof, kProfEncOther, 1, s);
-  k_tc_pool_packed<<<dim3(E, (d / 4 + kRowThreads - 1) / kRowThreads), kRowThreads, 0, s>>>(cb, el, a.X, a.cache,
-                                                                                        a.cache_f32, d);
-  return cudaGetLastError();
+  return launch_pdl(k_tc_pool_packed, dim3(E, (d / 4 + kRowThreads - 1) / kRowThreads), dim3(kRowThreads), 0, s, cb, el,
+                    a.X, a.cache, a.cache_f32, d);
 }
 
 // Bytes of fp16 copies of one encoder's linear-layer weights.
@@ -885,7 +898,7 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
 
   if (!rows_mapped) {
     ProfScope ps(prof, kProfEncOther, 1, s);
-    k_tc_row_map<<<1, 1024, 0, s>>>(cb, el, E);
+    launch_pdl(k_tc_row_map, dim3(1), dim3(1024), 0, s, cb, el, E);
   }
   cudaError_t e;
   {

@@ -94,7 +94,7 @@ cudaError_t launch_entry_fill(const CbView& cb, int which, const int32_t* first,
 // Passes cut by packed rows instead of entries.  launch_entry_rows leaves the rows of all entries of the
 // call in el.off[B + 1] (behind their number in el.off[B]); launch_entry_passes writes the first entry of
 // every pass of at most `rows` rows to pass_first[0 .. n_passes]; launch_entry_fill_pass fills the work
-// list of one of them (`slots` entries at most).
+// list of one of them, or of the whole call when pass_first is NULL (`slots` entries at most).
 cudaError_t launch_entry_rows(const CbView& cb, int which, const int32_t* first, const EntryList& el, cudaStream_t s);
 cudaError_t launch_entry_passes(const CbView& cb, int which, const int32_t* first, const EntryList& el, int rows,
                                 int n_passes, int32_t* pass_first, cudaStream_t s);

@@ -60,12 +60,7 @@ k_pair_gemm(const PairGemmParams p, const __grid_constant__ CUtensorMap tmA, con
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();          // 0: leader (issues the MMAs), 1: peer
   const int n_clusters = gridDim.x >> 1, cluster_id = blockIdx.x >> 1;
-  // only the row tiles that hold rows of live entries of this pass are computed (the host sizes
-  // the launch for its upper bound of entries; the count itself is device state)
-  int live_rows = *p.live_rows;                     // rows are packed: no padding rows inside entries
-  live_rows = live_rows < p.R ? live_rows : p.R;
-  const int row_tiles = (live_rows + 255) / 256;
-  const int n_tiles = row_tiles * p.col_tiles;
+  pdl_trigger();                                    // the next kernel may get resident behind this one
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kPgStages; ++s) {
@@ -87,6 +82,13 @@ k_pair_gemm(const PairGemmParams p, const __grid_constant__ CUtensorMap tmA, con
   cluster_sync_all();                               // both CTAs' barriers exist before any remote signal
   tc_fence_after();
   const uint32_t tmem_base = ctrl->tmem_base;
+  pdl_wait();                                       // operands, result matrices and the row count: all dependent
+  // only the row tiles that hold rows of live entries of this pass are computed (the host sizes
+  // the launch for its upper bound of entries; the count itself is device state)
+  int live_rows = *p.live_rows;                     // rows are packed: no padding rows inside entries
+  live_rows = live_rows < p.R ? live_rows : p.R;
+  const int row_tiles = (live_rows + 255) / 256;
+  const int n_tiles = row_tiles * p.col_tiles;
 
   // tile t -> (row tile, column tile): neighbouring clusters take different row tiles of the same
   // column tile, so that a weight tile is read from HBM once and found in L2 by the others
@@ -257,8 +259,7 @@ static cudaError_t launch_pair_gemm_t(const PairGemmParams& p, const CUtensorMap
   auto kern = k_pair_gemm<EPI, HALF>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<2 * clusters, kThreads, smem, s>>>(p, mA, mW);
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3(2 * clusters), dim3(kThreads), smem, s, p, mA, mW);
 }
 
 // D = A W^T with the epilogue `epi`, for a pass of R rows.  half == false: A = A_hi + A_lo, two bf16
