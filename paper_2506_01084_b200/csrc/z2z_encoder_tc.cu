@@ -59,6 +59,7 @@ constexpr int kNarrowVec4 = 4;         // ... and for d <= 4096, where half the 
 // tiles is then fuller (one encoder: d = 3072, 768 rows 755 against 725 us, 1023 rows 860 against 949;
 // d = 4096, 680 rows 957 against 830, 800 rows 1116 against 1253).
 constexpr int kStreamSingleRows = 128;
+constexpr int kPromptSessionRows = 1024;      // rows a pass of the session can hold from which it counts as prompt-sized
 static int pair_pass_min_rows(int d) { return d > 3584 ? 720 : 900; }
 
 struct Ptr2 { const void* p[2]; };
@@ -839,7 +840,9 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   const int E = a0.entries;
   if (E > el.list || E > 1024 * kMapPerThread) return cudaErrorInvalidValue;
   const int R = a0.rows > 0 ? a0.rows : E * M;         // row capacity of this pass
-  if (ng == 1 && R >= pair_pass_min_rows(d)) return run_encoder_pass_pair(cb, a0, el, E, R, prof, s);
+  // Passes of a call that knows its rows (a0.rows) always take whole tiles in a session of prompt size: their
+  // results are then the same bits whatever else is in the call, which stream-K sums are not.
+  if (ng == 1 && (R >= pair_pass_min_rows(d) || (a0.rows > 0 && el.chunk * M >= kPromptSessionRows))) return run_encoder_pass_pair(cb, a0, el, E, R, prof, s);
   const int Rt = (R + 7) / 8 * 8;                      // rows of the result matrix per group
   const int* total = el.row_off + E;                   // packed rows of this pass (device word)
   const int n_sm = sm_count();

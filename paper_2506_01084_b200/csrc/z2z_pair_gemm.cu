@@ -12,6 +12,11 @@
 //   kEpiStore   out[r, c]  = acc + bias                      (q, k, v for the attention kernel)
 //   kEpiResid   X[r, c]   += acc + bias                      (attention output / second MLP layer)
 //   kEpiGelu    H[r, c]    = split_hi_lo(gelu(acc + bias))   (first MLP layer)
+// With few row tiles the tiles are cut narrower (N = 128 or 64 columns): a 256-column tile keeps a CTA pair
+// for the whole K range, and one row tile has 12 of them in a d = 3072 output while there are 74 pairs.
+// Cutting K instead would be faster still, but its sums would depend on the cut: an element's products are
+// added in the same order whatever the tile, so that an entry's embedding does not change with the other
+// entries of the call.
 // Rows that are padding of their entry (or lie beyond the pass) are not written (kEpiGelu writes
 // zeros there, because the next GEMM reads them).
 //
@@ -96,6 +101,7 @@ k_pair_gemm(const PairGemmParams p, const __grid_constant__ CUtensorMap tmA, con
     if (lane == 0) {
       // ---------------- TMA producer (both CTAs) ---------------------------------------------------
       const uint64_t pol = policy_evict_last();
+      const uint32_t bytes = 2u * (kWOff + (uint32_t)p.tile_cols * 64u);        // of both CTAs
       uint32_t full_leader[kPgStages];
       for (int s = 0; s < kPgStages; ++s) full_leader[s] = map_to_cta(smem_u32(&ctrl->full[s]), 0);
       int stage = 0; uint32_t phase = 0;
@@ -103,10 +109,10 @@ k_pair_gemm(const PairGemmParams p, const __grid_constant__ CUtensorMap tmA, con
       for (int t = cluster_id; t < n_tiles && ok; t += n_clusters) {
         const int rt = t % row_tiles, ct = t / row_tiles;
         const int arow = rt * 256 + (int)rank * 128;
-        const int wrow = ct * 256 + (int)rank * 128;
+        const int wrow = ct * p.tile_cols + (int)rank * (p.tile_cols / 2);
         for (int ks = 0; ks < p.ksteps; ++ks) {
           if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) { ok = false; break; }
-          if (rank == 0) mbar_expect_tx(smem_u32(&ctrl->full[stage]), 2 * kPgStageBytes);
+          if (rank == 0) mbar_expect_tx(smem_u32(&ctrl->full[stage]), bytes);
           const uint32_t sb = stage_base + (uint32_t)stage * kPgStageBytes;
           tma_load_2d_pair(sb, &tmA, ks * 64, arow, full_leader[stage], pol);                 // hi rows (HALF: the rows)
           if (!HALF) tma_load_2d_pair(sb + 16384, &tmA, ks * 64, p.Rt + arow, full_leader[stage], pol);   // lo rows
@@ -118,7 +124,7 @@ k_pair_gemm(const PairGemmParams p, const __grid_constant__ CUtensorMap tmA, con
   } else if (warp == 1) {
     if (lane == 0 && rank == 0) {
       // ---------------- MMA issuer (leader only) ------------------------------------------------------
-      const uint32_t idesc = HALF ? idesc_f16_f32(256, 256) : idesc_bf16_f32(256, 256);
+      const uint32_t idesc = HALF ? idesc_f16_f32(256, p.tile_cols) : idesc_bf16_f32(256, p.tile_cols);
       int stage = 0; uint32_t phase = 0, job_i = 0;
       bool ok = true;
       for (int t = cluster_id; t < n_tiles && ok; t += n_clusters) {
@@ -166,8 +172,8 @@ k_pair_gemm(const PairGemmParams p, const __grid_constant__ CUtensorMap tmA, con
       if (__any_sync(0xffffffffu, writes)) {
         const uint32_t tbase = tmem_base + ((uint32_t)(q * 32) << 16) + buf * 256;
 #pragma unroll 1
-        for (int c0 = 0; c0 < 256; c0 += 32) {
-          const int col = ct * 256 + c0;
+        for (int c0 = 0; c0 < p.tile_cols; c0 += 32) {
+          const int col = ct * p.tile_cols + c0;
           if (col >= p.J) break;                       // the last column tile may be half outside
           uint32_t v[32];
           tmem_ld32(tbase + c0, v);
@@ -276,11 +282,21 @@ cudaError_t launch_pair_gemm(const PairGemmParams& p0, const void* act, const vo
   PairGemmParams p = p0;
   p.ksteps = K / 64;
   p.row_tiles = (p.R + 255) / 256;
-  p.col_tiles = (p.J + 255) / 256;
+  // The width that the busiest pair is through with first: waves of tiles x clocks of a k-step, which are
+  // those of its MMAs (2 per column and operand part) or of its loads (60 bytes a clock from L2).
+  const int parts = half ? 1 : 2;
+  long long best = -1;
+  for (int cols = 256; cols >= 64; cols /= 2) {
+    const long long tiles = (long long)p.row_tiles * ((p.J + cols - 1) / cols), waves = (tiles + n_sm / 2 - 1) / (n_sm / 2);
+    const int mma = 2 * cols * parts, load = (16384 * parts + 64 * cols) / 60;
+    const long long cost = waves * (mma > load ? mma : load);
+    if (best < 0 || cost < best) { best = cost; p.tile_cols = cols; }
+  }
+  p.col_tiles = (p.J + p.tile_cols - 1) / p.tile_cols;
   CUtensorMap mA, mW;
   // (the element type of a tensor map only fixes the element size and the fill value: bf16 and fp16 alike)
   if (!make_tmap_bf16(&mA, act, (half ? 1ll : 2ll) * p.Rt, K, 128)) return cudaErrorInvalidValue;
-  if (!make_tmap_bf16(&mW, W, p.J, K, 128)) return cudaErrorInvalidValue;
+  if (!make_tmap_bf16(&mW, W, p.J, K, p.tile_cols / 2)) return cudaErrorInvalidValue;
   const int tiles = p.row_tiles * p.col_tiles;
   const int clusters = tiles < n_sm / 2 ? tiles : n_sm / 2;
   if (half) {

@@ -145,6 +145,7 @@ struct PairGemmParams {
   float* out;            // kEpiStore / kEpiResid: fp32 [R, J]
   __nv_bfloat16* out_hl; // kEpiGelu: bf16 [2 Rt, J], hi rows then lo rows (single fp16 operand: fp16 [Rt, J])
   int ksteps, row_tiles, col_tiles;
+  int tile_cols;         // columns per tile: 256, 128 or 64
   int* err;
 };
 cudaError_t launch_pair_gemm(const PairGemmParams& p, const void* act, const void* W, int K, int epi, bool half,
