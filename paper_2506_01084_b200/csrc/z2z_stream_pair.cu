@@ -1,5 +1,5 @@
-// Weight-streaming skinny GEMM on CTA pairs, for hyper-encoder passes of a large decode batch or of a short
-// prompt (hundreds of activation rows):
+// Weight-streaming skinny GEMM on CTA pairs, for hyper-encoder passes of a large decode batch or of a call
+// bounded to some hundred activation rows:
 //
 //   out[group][r][j] += sum_k A[group][r][k] * W[group][j][k]
 //
@@ -14,12 +14,12 @@
 //     boxes of the first pass over the ring are issued before that;
 //   * up to 512 packed rows ride on one stream of the weights.  NARROW, up to 256 live rows: hi and lo
 //     part of a row are two columns of tensor memory, two accumulators of 128 rows.  WIDE, more: the two
-//     parts accumulate into one column, two accumulators of 256 rows.  (At 217 rows narrow takes 654 us
-//     a request start and wide 719; rows in a second block of 256 brought the weights again: 902 against
-//     681 us on prompts of 200 to 300 rows.)  More rows run as several such blocks, the same
+//     parts accumulate into one column, two accumulators of 256 rows.  (The 217 rows of a prompt, both
+//     encoders: narrow 654 us, wide 719; 200 to 300 rows with the rest in a second block of 256, which
+//     brings the weights again: 902 against 681 us.)  More rows run as several such blocks, the same
 //     weight tile one after the other, so that it comes from L2 the second time.
 // A decode step of 90 sequences (d = 3072, one encoder, 270 rows of capacity, about 150 live) went from
-// 486 to 291 us, the 200 to 300 rows of a short prompt's entries (both encoders) from 1.49 to 0.68 ms.
+// 486 to 291 us, 170 entries of one encoder (about 390 rows) from 500 to 428 us.
 //
 // Work is cut stream-K style: cluster c of C owns units [floor(c U / C), floor((c + 1) U / C)) of the
 // (group, weight tile, row block, k-step) space and adds its accumulators into the fp32 result with
