@@ -131,8 +131,9 @@ int32_t z2z_lzw_step(z2z_codebook* cb, const int32_t* d_new_codes, const uint8_t
  *            only selects which "embedded so far" counter is used when d_first/d_count are NULL.
  *   d_table  [V, d]; enc: that side's encoder.
  *   d_first / d_count [B] or both NULL = every entry created since the last such call.
- *   max_entries  host upper bound on sum_b count_b (<= 0: B * cap).  It bounds the launch count:
- *            entries are processed in passes of 1024, and a pass is about ten launches per layer
+ *   max_entries  host upper bound on sum_b count_b (<= 0: B * cap).  It bounds the launch count
+ *            and sizes the passes (entries beyond it are not embedded): entries are processed in
+ *            passes of at most 1024, the last one sized for the rest, and a pass is about ten launches per layer
  *            whether or not it finds entries (the counts are device state).  After z2z_lzw_encode
  *            pass the number of prompt tokens (or the sum of the code lengths, if known on the
  *            host): a prompt of T tokens creates fewer than T entries.  With 0 a large session
@@ -140,6 +141,7 @@ int32_t z2z_lzw_step(z2z_codebook* cb, const int32_t* d_new_codes, const uint8_t
  *            max_entries < 0: exact.  The call reads the number of entries it has to embed back
  *            from the device - it waits for the stream once, the only enqueueing call that does,
  *            and therefore cannot be captured into a graph - and launches no pass without work.
+ *            In prompt-sized bf16 sessions the rows are then the same bits whatever else is in the call.
  *            Meant for whole prompts, where hundreds of empty passes would cost more than the wait.
  *   d_cache  [B, cap, d] in the configured dtype (row k of sequence b = hypertoken V + k).
  *   d_cache_f32 [B, cap, d] fp32 or NULL: the same rows before rounding to the cache dtype.    */
