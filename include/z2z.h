@@ -132,7 +132,7 @@ int32_t z2z_lzw_step(z2z_codebook* cb, const int32_t* d_new_codes, const uint8_t
  *   d_table  [V, d]; enc: that side's encoder.
  *   d_first / d_count [B] or both NULL = every entry created since the last such call.
  *   max_entries  host upper bound on sum_b count_b (<= 0: B * cap).  It bounds the launch count
- *            and sizes the passes (entries beyond it are not embedded): entries are processed in
+ *            and sizes the passes (entries beyond it stay due for the next call): entries are processed in
  *            passes of at most 1024, the last one sized for the rest, and a pass is about ten launches per layer
  *            whether or not it finds entries (the counts are device state).  After z2z_lzw_encode
  *            pass the number of prompt tokens (or the sum of the code lengths, if known on the

@@ -389,7 +389,7 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
   }
   if (!d_first) {
     z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 1, s);
-    Z2Z_CUDA(z2z::launch_mark_embedded(cb->view, which, s), "hyper_embed");
+    Z2Z_CUDA(z2z::launch_mark_embedded(cb->view, which, el.off, bound, s), "hyper_embed");
   }
   return Z2Z_OK;
 }
@@ -491,8 +491,8 @@ int32_t z2z_decode_step(z2z_codebook* cb, const void* d_hidden, const void* d_WE
       z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 4, s);
       Z2Z_CUDA(z2z::launch_entry_offsets_from_new(cb->view, w_new, el, s), "decode_step");
       Z2Z_CUDA(z2z::launch_entry_fill(cb->view, 0, nullptr, w_new, el, 0, s), "decode_step");
-      Z2Z_CUDA(z2z::launch_mark_embedded(cb->view, 0, s), "decode_step");
-      Z2Z_CUDA(z2z::launch_mark_embedded(cb->view, 1, s), "decode_step");
+      Z2Z_CUDA(z2z::launch_mark_embedded(cb->view, 0, nullptr, 0, s), "decode_step");
+      Z2Z_CUDA(z2z::launch_mark_embedded(cb->view, 1, nullptr, 0, s), "decode_step");
     }
   }
   // cache update: the at most one new entry per sequence, on both sides.  Once an earlier step has

@@ -147,9 +147,18 @@ __global__ void __launch_bounds__(1024) k_entry_passes(CbView cb, int which, con
   }
 }
 
-__global__ void k_mark_embedded(CbView cb, int which) {
+// off == NULL: every entry is embedded; else those among the first `bound` of the call (off: offsets of the
+// sequences' entries in it), so that what a bound left out is still due for the next call.
+__global__ void k_mark_embedded(CbView cb, int which, const int32_t* off, long long bound) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < cb.B) cb.n_emb[which * cb.B + b] = cb.n[b];
+  if (b >= cb.B) return;
+  int left_out = 0;
+  if (off) {
+    const long long beyond = (long long)off[b + 1] - bound;
+    const int count = off[b + 1] - off[b];
+    left_out = beyond <= 0 ? 0 : (beyond < count ? (int)beyond : count);
+  }
+  cb.n_emb[which * cb.B + b] = cb.n[b] - left_out;
 }
 
 __device__ __forceinline__ int entry_len(const CbView& cb, const EntryList& el, int e) {
@@ -358,8 +367,8 @@ cudaError_t launch_entry_fill_pass(const CbView& cb, int which, const int32_t* f
   return launch_pdl(k_entry_fill, dim3((slots + 255) / 256), dim3(256), 0, s, cb, which, 0, first, nullptr, el, 0ll, slots,
                     pass_first ? pass_first + pass : nullptr);
 }
-cudaError_t launch_mark_embedded(const CbView& cb, int which, cudaStream_t s) {
-  k_mark_embedded<<<(cb.B + 255) / 256, 256, 0, s>>>(cb, which);
+cudaError_t launch_mark_embedded(const CbView& cb, int which, const int32_t* off, long long bound, cudaStream_t s) {
+  k_mark_embedded<<<(cb.B + 255) / 256, 256, 0, s>>>(cb, which, off, bound);
   return cudaGetLastError();
 }
 

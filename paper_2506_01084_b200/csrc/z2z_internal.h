@@ -103,7 +103,7 @@ cudaError_t launch_entry_fill_pass(const CbView& cb, int which, const int32_t* f
 // Rows per pass (a multiple of 256, at most max_rows) that take the linear layers of `total` rows the fewest
 // waves of output tiles.
 int encoder_pass_rows(long long total, int max_rows, int M, int d, int dff);
-cudaError_t launch_mark_embedded(const CbView& cb, int which, cudaStream_t s);
+cudaError_t launch_mark_embedded(const CbView& cb, int which, const int32_t* off, long long bound, cudaStream_t s);
 cudaError_t run_encoder_pass(const CbView& cb, const EncoderArgs& a, const EntryList& el,
                              bool use_tensor_cores, Prof* prof, cudaStream_t s);
 

@@ -96,3 +96,14 @@ def test_whole_prompts_in_passes_cut_by_rows(M, d, dff):
         want = ohe.hyper_embed(p.oracle.books[b].entries, f64(p.W_E), enc, w.heads)
         assert np.abs(p.E_f32[b, :n[b]].double().cpu().numpy() - want).max() <= TOL
         assert torch.all(p.E_f32[b, n[b]:] == 0)
+
+
+def test_entries_beyond_the_bound_stay_due():
+    w, p = _pair(256, 512, 3, B=3, T=500, cap=400, seed=8)
+    n = [p.oracle.books[b].n() for b in range(w.B)]
+    for bound in (20, n[0] + n[1] // 2 - 20, sum(n)):          # inside the first and second sequence, then the rest
+        zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, None, None, bound, p.E_h, p.E_f32)
+    enc = [f64(t) for t in p.enc_E]
+    for b in range(w.B):
+        want = ohe.hyper_embed(p.oracle.books[b].entries, f64(p.W_E), enc, w.heads)
+        assert np.abs(p.E_f32[b, :n[b]].double().cpu().numpy() - want).max() <= TOL
