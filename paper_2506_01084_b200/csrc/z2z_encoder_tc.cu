@@ -54,7 +54,7 @@ constexpr int kMaxVec4 = 8;            // float4 per thread in the row kernels: 
 constexpr int kNarrowVec4 = 4;         // ... and for d <= 4096, where half the registers do
 // Which linear-layer kernel a pass takes, by its row capacity.  Up to 128 rows one CTA per weight tile streams
 // best (24 rows, d = 3072, both encoders: 249 us a step against 272 with pairs; 96 rows, d = 4096: equal);
-// beyond, CTA pairs carry up to 512 rows on one stream (270 rows, one encoder: 486 -> 291 us a step).  Past that
+// beyond, CTA pairs carry up to 256 rows on one stream (270 rows, one encoder: 486 -> 291 us a step).  Past that
 // the stream comes twice and whole output tiles take over, the earlier the wider the model, as a wave of
 // tiles is then fuller (one encoder: d = 3072, 768 rows 755 against 725 us, 1023 rows 860 against 949;
 // d = 4096, 680 rows 957 against 830, 800 rows 1116 against 1253).
@@ -890,9 +890,7 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
     };
     ProfScope ps(prof, kProfEncGemm, 1, s);
     if (paired) {
-      if (!make(pair_maps, [&](int g) { return stream_pair_act_maps(pair_maps.a[g], pair_maps.wide[g], act.p[g], Rt, K, R); }))
-        return cudaErrorInvalidValue;
-      if (ng == 1) for (int i = 0; i < 8; ++i) pair_maps.wide[1][i] = pair_maps.wide[0][i];
+      if (!make(pair_maps, [&](int g) { return stream_pair_act_maps(pair_maps.a[g], act.p[g], Rt, K, R); })) return cudaErrorInvalidValue;
       return launch_stream_pair(fill(StreamPairParams{}), pair_maps, n_sm, s);
     }
     if (!make(maps, [&](int g) { return stream_gemm_act_maps(maps.a[g], act.p[g], Rt, K, R); })) return cudaErrorInvalidValue;

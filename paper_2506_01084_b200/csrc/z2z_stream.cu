@@ -591,17 +591,16 @@ bool make_tmap_bf16(CUtensorMap* m, const void* base, long long rows, long long 
 // step, whose operands sit at the same addresses step after step, encodes none in steady state.
 namespace {
 struct TmapKey {
-  const void* base; long long rows, cols; int box_rows, box_kb, parts;
+  const void* base; long long rows, cols; int box_rows, box_kb;
   bool operator==(const TmapKey& o) const {
-    return base == o.base && rows == o.rows && cols == o.cols && box_rows == o.box_rows && box_kb == o.box_kb &&
-           parts == o.parts;
+    return base == o.base && rows == o.rows && cols == o.cols && box_rows == o.box_rows && box_kb == o.box_kb;
   }
 };
 struct TmapKeyHash {
   size_t operator()(const TmapKey& k) const {
     size_t h = reinterpret_cast<uintptr_t>(k.base) * 0x9E3779B97F4A7C15ull;
     h ^= (size_t)k.rows * 0xC2B2AE3D27D4EB4Full + (size_t)k.cols * 0x165667B19E3779F9ull;
-    h ^= ((size_t)k.box_rows << 20) ^ (size_t)k.box_kb ^ ((size_t)k.parts << 40);
+    h ^= ((size_t)k.box_rows << 20) ^ (size_t)k.box_kb;
     return h;
   }
 };
@@ -610,49 +609,32 @@ std::unordered_map<TmapKey, CUtensorMap, TmapKeyHash> g_tmap_cache;
 std::mutex g_tmap_mu;
 }  // namespace
 
-static bool make_tmap_cached(CUtensorMap* m, const void* base, long long rows, long long cols, int box_rows, int box_kb,
-                             int parts) {
+bool make_tmap_bf16_kblocks(CUtensorMap* m, const void* base, long long rows, long long cols, int box_rows,
+                            int box_kb) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
   if ((reinterpret_cast<uintptr_t>(base) & 15) || (cols % 64) || box_rows < 1 || box_rows > 256 || box_kb < 1 ||
       box_kb > 256 || rows < 1)
     return false;
-  const TmapKey key{base, rows, cols, box_rows, box_kb, parts};
+  const TmapKey key{base, rows, cols, box_rows, box_kb};
   {
     std::lock_guard<std::mutex> lock(g_tmap_mu);
     auto it = g_tmap_cache.find(key);
     if (it != g_tmap_cache.end()) { *m = it->second; return true; }
   }
-  cuuint32_t es[4] = {1, 1, 1, 1};
-  CUresult r;
-  if (parts == 1) {
-    cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)(cols / 64)};
-    cuuint64_t strides[2] = {(cuuint64_t)cols * 2, 128};
-    cuuint32_t box[3] = {64, (cuuint32_t)box_rows, (cuuint32_t)box_kb};
-    r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  } else {
-    cuuint64_t dims[4] = {64, (cuuint64_t)rows, 2, (cuuint64_t)(cols / 64)};
-    cuuint64_t strides[3] = {(cuuint64_t)cols * 4, (cuuint64_t)cols * 2, 128};
-    cuuint32_t box[4] = {64, (cuuint32_t)box_rows, 2, (cuuint32_t)box_kb};
-    r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, strides, box, es,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  }
-  if (r != CUDA_SUCCESS) return false;
+  cuuint64_t dims[3] = {64, (cuuint64_t)rows, (cuuint64_t)(cols / 64)};
+  cuuint64_t strides[2] = {(cuuint64_t)cols * 2, 128};
+  cuuint32_t box[3] = {64, (cuuint32_t)box_rows, (cuuint32_t)box_kb};
+  cuuint32_t es[3] = {1, 1, 1};
+  if (fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, es,
+         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+    return false;
   std::lock_guard<std::mutex> lock(g_tmap_mu);
   if (g_tmap_cache.size() >= kTmapCacheMax) g_tmap_cache.clear();
   g_tmap_cache.emplace(key, *m);
   return true;
 }
-bool make_tmap_bf16_kblocks(CUtensorMap* m, const void* base, long long rows, long long cols, int box_rows, int box_kb) {
-  return make_tmap_cached(m, base, rows, cols, box_rows, box_kb, 1);
-}
-bool make_tmap_bf16_parts(CUtensorMap* m, const void* base, long long rows, long long cols, int box_rows, int box_kb) {
-  return make_tmap_cached(m, base, rows, cols, box_rows, box_kb, 2);
-}
-
 template <int NT, int KSB>
 static int pick_stages(int a_parts, int a_box_rows, int extra) {
   const int stage = a_parts * KSB * a_box_rows * 128 + KSB * NT * 128;

@@ -82,8 +82,8 @@ bool stream_gemm_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int
 // At most 128 rows, one CTA per tile of 128 weight rows.
 cudaError_t launch_stream_gemm(StreamGemmParams p, const StreamGemmMaps& maps, int n_sm, cudaStream_t s);
 
-// The same product for more than 128 rows on CTA pairs (z2z_stream_pair.cu): up to 512 packed rows ride on one stream of the
-// weights, and more run as blocks of 512.
+// The same product for more than 128 rows on CTA pairs (z2z_stream_pair.cu): up to 256 packed rows ride on one stream of the
+// weights, and more run as blocks of 256.
 struct StreamPairParams {
   int groups, ksteps;
   int R;
@@ -93,16 +93,16 @@ struct StreamPairParams {
   int* err;
 
   int tiles_per_group;   // tiles of 256 weight rows
-  int blocks;            // blocks of 512 packed rows the capacity asks for
+  int blocks;            // blocks of 256 packed rows the capacity asks for
   int act_bytes;         // activation part of a stage
   int stages;
 };
 struct StreamPairMaps {
-  CUtensorMap a[2][8], wide[2][8];     // activation operand of each group in both forms, boxes of 16, 32, .. 128 rows
-  CUtensorMap w[2];                    // weights of each group, 128 rows
+  CUtensorMap a[2][8];   // activation operand of each group, boxes of 16, 32, .. 128 rows
+  CUtensorMap w[2];      // weights of each group, 128 rows
 };
 int stream_pair_ksb(int R);
-bool stream_pair_act_maps(CUtensorMap* narrow, CUtensorMap* wide, const void* act, int Rt, int K, int R);
+bool stream_pair_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int R);
 cudaError_t launch_stream_pair(StreamPairParams p, const StreamPairMaps& maps, int n_sm, cudaStream_t s);
 
 struct StreamLogitsParams {
@@ -151,8 +151,6 @@ struct PairGemmParams {
 cudaError_t launch_pair_gemm(const PairGemmParams& p, const void* act, const void* W, int K, int epi, bool half,
                              cudaStream_t s);
 
-// The hi / lo operand [2 rows, cols] (row r: hi in row 2 r, lo in 2 r + 1) seen as [k-block][part][row][64].
-bool make_tmap_bf16_parts(CUtensorMap* m, const void* base, long long rows, long long cols, int box_rows, int box_kb);
 bool make_tmap_bf16(CUtensorMap* m, const void* base, long long rows, long long cols, int box_rows);
 cudaError_t launch_stream_logits(const StreamLogitsParams& p, const LogitMaps* maps, int grid, bool merge,
                                  Prof* prof, cudaStream_t s);

@@ -12,23 +12,23 @@
 //   * the activation box follows the LIVE rows, a count that only the device knows: one tensor map
 //     per box height (16, 32, .. 128 rows), picked once the preceding kernel is done.  The weight
 //     boxes of the first pass over the ring are issued before that;
-//   * up to 512 packed rows ride on one stream of the weights.  NARROW, up to 256 live rows: hi and lo
-//     part of a row are two columns of tensor memory, two accumulators of 128 rows.  WIDE, more: the two
-//     parts accumulate into one column, two accumulators of 256 rows.  (The 217 rows of a prompt, both
-//     encoders: narrow 654 us, wide 719; 200 to 300 rows with the rest in a second block of 256, which
-//     brings the weights again: 902 against 681 us.)  More rows run as several such blocks, the same
-//     weight tile one after the other, so that it comes from L2 the second time.
+//   * up to 256 packed rows ride on one stream of the weights: hi and lo part of a row are two columns
+//     of tensor memory, two accumulators of 128 rows.  More live rows run as several such blocks, the same
+//     weight tile one after the other, so that it comes from L2 the second time;
+//   * an accumulator takes in one product per weight, hi and lo in columns of their own, and at most 8192
+//     weights before it is drained: tensor-core sums lose low bits with every product added.  (Both parts
+//     in one column would let 512 rows ride on one stream - 384 rows of both encoders, d = 3072: 687
+//     instead of 787 us a step, 640 rows 1392 against 1173 - but the error against fp64, in units of the
+//     rows' rms, is then 2.5e-5 instead of 1.35e-5 at d = 4096 and 2.1e-5 instead of 1.1e-5 at d = 3072.)
 // A decode step of 90 sequences (d = 3072, one encoder, 270 rows of capacity, about 150 live) went from
-// 486 to 291 us, 170 entries of one encoder (about 390 rows) from 500 to 428 us.
+// 486 to 291 us against one CTA per weight tile and 128 rows.
 //
 // Work is cut stream-K style: cluster c of C owns units [floor(c U / C), floor((c + 1) U / C)) of the
 // (group, weight tile, row block, k-step) space and adds its accumulators into the fp32 result with
 // reductions in global memory, like k_stream_gemm.
 //
 // Operand layout: packed row r of the activations is rows 2 r (bf16 hi) and 2 r + 1 (lo) of
-// [2 Rt, K].  The narrow form's tensor map sees [k-block][operand row][64]; the wide form's sees
-// [k-block][part][row][64], so that one box brings the hi rows and behind them the lo rows.  An
-// epilogue thread owns one output feature.
+// [2 Rt, K], seen as [k-block][operand row][64].  An epilogue thread owns one output feature.
 //
 // Roles per CTA: warp 0 lane 0 TMA producer, warp 1 lane 0 MMA issuer (leader CTA only), warps 2-9
 // epilogue.  Every mbarrier wait is bounded.
@@ -45,8 +45,9 @@ namespace {
 constexpr int kEpiWarps = 8;             // two per tensor-memory lane quarter, one for each half of a row block
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kSpMaxStages = 8;
-constexpr int kSpNarrowRows = 256;       // packed rows that two accumulators take with a column per part
-constexpr int kSpBlockRows = 512;        // packed rows that share one stream of the weights
+constexpr int kSpBlockRows = 256;        // packed rows that share one stream of the weights
+constexpr int kSpHalfRows = kSpBlockRows / 2;                     // ... of one accumulator
+constexpr int kSpChain = 128;            // k-blocks of 64 columns an accumulator takes in
 constexpr int kSpSmem = 227 * 1024;
 
 struct SpCtrl {
@@ -58,9 +59,9 @@ struct SpCtrl {
 struct SpJob { int g, wrow, block, kb0, kb1; };
 struct SpWalk {
   const StreamPairParams& p;
-  int blocks;
+  int blocks, chain;                     // a job takes at most `chain` k-steps
   long long u, u1;
-  __device__ SpWalk(const StreamPairParams& pp, int live_blocks) : p(pp), blocks(live_blocks) {
+  __device__ SpWalk(const StreamPairParams& pp, int live_blocks, int chain_) : p(pp), blocks(live_blocks), chain(chain_) {
     const long long U = (long long)p.groups * p.tiles_per_group * blocks * p.ksteps, C = gridDim.x >> 1, c = blockIdx.x >> 1;
     u = c * U / C;
     u1 = (c + 1) * U / C;
@@ -70,7 +71,9 @@ struct SpWalk {
     const long long job = u / p.ksteps;
     j.kb0 = (int)(u - job * p.ksteps);
     const long long left = u1 - u;
-    j.kb1 = (int)((p.ksteps - j.kb0) < left ? p.ksteps : j.kb0 + left);
+    int end = (j.kb0 / chain + 1) * chain;
+    end = end < p.ksteps ? end : p.ksteps;
+    j.kb1 = (int)((end - j.kb0) < left ? end : j.kb0 + left);
     const long long tile = job / blocks;
     j.block = (int)(job - tile * blocks);
     j.g = (int)(tile / p.tiles_per_group);
@@ -80,19 +83,16 @@ struct SpWalk {
   }
 };
 
-__device__ __forceinline__ bool sp_wide(int live) { return live > kSpNarrowRows; }
 // Columns of tensor memory (the MMA's N, a multiple of 32) that half `h` of a row block takes, 0 if it has
 // no live row; the first half of a block always counts as having one.
 __device__ __forceinline__ int sp_cols(int live, int block, int h) {
-  const bool wide = sp_wide(live);
-  const int half = wide ? kSpBlockRows / 2 : kSpNarrowRows / 2;
-  int rows = live - block * kSpBlockRows - h * half;
+  int rows = live - block * kSpBlockRows - h * kSpHalfRows;
   if (rows < 1) rows = (h == 0) ? 1 : 0;
-  if (rows > half) rows = half;
-  return ((wide ? rows : 2 * rows) + 31) & ~31;
+  if (rows > kSpHalfRows) rows = kSpHalfRows;
+  return (2 * rows + 31) & ~31;
 }
 // Bytes per CTA and k-block of the activation box for n columns: half of the operand rows.
-__device__ __forceinline__ uint32_t sp_box_bytes(bool wide, int n) { return (uint32_t)n * (wide ? 128u : 64u); }
+__device__ __forceinline__ uint32_t sp_box_bytes(int n) { return (uint32_t)n * 64u; }
 // Row blocks with a live row (at least one).  A pass whose capacity is one block does not need the count.
 __device__ __forceinline__ int sp_live_blocks(const StreamPairParams& p, int live) {
   return p.blocks > 1 && live > kSpBlockRows ? (live + kSpBlockRows - 1) / kSpBlockRows : 1;
@@ -154,19 +154,15 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
       SpJob def[kSpMaxStages];                        // load i of the first pass uses stage i; kb0 = its k-step
       int n_def = 0, issued = 0, live = 0;
       bool deps = false, ok = true;
-      auto act_bytes = [&](int block) { return KSB * sp_box_bytes(sp_wide(live), sp_cols(live, block, 0) + sp_cols(live, block, 1)); };
+      auto act_bytes = [&](int block) { return KSB * sp_box_bytes(sp_cols(live, block, 0) + sp_cols(live, block, 1)); };
       auto load_act = [&](int st, const SpJob& j, int ks) {
         const uint32_t sb = stage_base + (uint32_t)st * stage_bytes;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int n = sp_cols(live, j.block, h);
           if (n == 0) continue;
-          if (sp_wide(live))
-            tma_load_4d_pair(sb + h * (KSB * 32768u), &tm.wide[j.g][(n >> 5) - 1], 0,
-                             j.block * kSpBlockRows + h * (kSpBlockRows / 2) + (int)rank * (n >> 1), 0, ks * KSB, full_leader[st], pol_a);
-          else
-            tma_load_3d_pair(sb + h * (KSB * 16384u), &tm.a[j.g][(n >> 5) - 1], 0, h * kSpNarrowRows + (int)rank * (n >> 1), ks * KSB,
-                             full_leader[st], pol_a);
+          tma_load_3d_pair(sb + h * (KSB * 16384u), &tm.a[j.g][(n >> 5) - 1], 0,
+                           2 * (j.block * kSpBlockRows + h * kSpHalfRows) + (int)rank * (n >> 1), ks * KSB, full_leader[st], pol_a);
         }
       };
       auto need_deps = [&]() {
@@ -182,7 +178,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
       };
       if (p.blocks > 1) need_deps();                   // the walk itself depends on the row count
       int stage = 0; uint32_t phase = 0;
-      SpWalk walk(p, sp_live_blocks(p, live));
+      SpWalk walk(p, sp_live_blocks(p, live), p.ksteps);      // (where an accumulator ends does not matter to the loads)
       SpJob j;
       while (ok && walk.next(j)) {
         for (int ks = j.kb0; ks < j.kb1; ++ks) {
@@ -208,13 +204,12 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
     int live = *p.rows_dev;
     live = live < p.R ? live : p.R;
     const int n_blocks = sp_live_blocks(p, live);
-    const bool wide = sp_wide(live);
     if (warp == 1) {
       if (lane == 0 && rank == 0) {
         // ---------------- MMA issuer (leader only): D[256 weight rows][n] += W tile x activation rows -----
         int stage = 0; uint32_t phase = 0, job_i = 0;
         bool ok = true;
-        SpWalk walk(p, n_blocks);
+        SpWalk walk(p, n_blocks, kSpChain / KSB);
         SpJob j;
         while (ok && walk.next(j)) {
           const uint32_t aph = job_i & 1u;
@@ -223,9 +218,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
           const int n0 = sp_cols(live, j.block, 0), n1 = sp_cols(live, j.block, 1);
           const uint32_t id0 = idesc_bf16_f32(256, n0), id1 = idesc_bf16_f32(256, n1 ? n1 : 32);
           const uint32_t d = tmem_base;
-          const uint32_t kb0 = sp_box_bytes(wide, n0), kb1 = sp_box_bytes(wide, n1);        // one k-block of a half's box
-          const uint32_t half1 = KSB * (wide ? 32768u : 16384u);
-          const int parts = wide ? 2 : 1;
+          const uint32_t kb0 = sp_box_bytes(n0), kb1 = sp_box_bytes(n1);                    // one k-block of a half's box
           uint32_t acc = 0;
           for (int ks = j.kb0; ks < j.kb1; ++ks) {
             if (!mbar_wait(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
@@ -234,14 +227,13 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
 #pragma unroll
             for (int i = 0; i < KSB; ++i) {
               const uint32_t wb = sb + p.act_bytes + i * 16384u;
-              const uint32_t a0 = sb + (uint32_t)i * kb0, a1 = sb + half1 + (uint32_t)i * kb1;
-              for (int part = 0; part < parts; ++part)         // wide: hi rows, then lo rows, into the same columns
+              const uint32_t a0 = sb + (uint32_t)i * kb0, a1 = sb + KSB * 16384u + (uint32_t)i * kb1;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                  umma_bf16_pair(d, smem_desc_sw128(wb + k * 32), smem_desc_sw128(a0 + part * (kb0 / 2) + k * 32), id0, acc);
-                  if (n1) umma_bf16_pair(d + 256, smem_desc_sw128(wb + k * 32), smem_desc_sw128(a1 + part * (kb1 / 2) + k * 32), id1, acc);
-                  acc = 1;
-                }
+              for (int k = 0; k < 4; ++k) {
+                umma_bf16_pair(d, smem_desc_sw128(wb + k * 32), smem_desc_sw128(a0 + k * 32), id0, acc);
+                if (n1) umma_bf16_pair(d + 256, smem_desc_sw128(wb + k * 32), smem_desc_sw128(a1 + k * 32), id1, acc);
+                acc = 1;
+              }
             }
             umma_commit_pair(smem_u32(&ctrl->empty[stage]));      // frees the stage in both CTAs
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -261,7 +253,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
       const int group = (warp - 2) >> 2;               // takes every other 32 columns
       const uint32_t acc_empty_leader = map_to_cta(smem_u32(&ctrl->acc_empty), 0);
       uint32_t job_i = 0;
-      SpWalk walk(p, n_blocks);
+      SpWalk walk(p, n_blocks, kSpChain / KSB);
       SpJob j;
       while (walk.next(j)) {
         const uint32_t aph = job_i & 1u;
@@ -279,26 +271,16 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
             if (r + (lane & 3) < rows) red_add_f32x4(dst + (size_t)r * p.J, f[0], f[1], f[2], f[3]);
           };
 #pragma unroll 1
-          for (int c0 = 32 * group; c0 < (wide ? rows : 2 * rows); c0 += 64) {
+          for (int c0 = 32 * group; c0 < 2 * rows; c0 += 64) {
             uint32_t v[32];
             tmem_ld32(t0 + c0, v);
             tmem_ld_wait();
-            if (wide) {
 #pragma unroll
-              for (int y = 0; y < 8; ++y) {
-                float f[4];
+            for (int y = 0; y < 4; ++y) {
+              float f[4];
 #pragma unroll
-                for (int x = 0; x < 4; ++x) f[x] = __uint_as_float(v[4 * y + x]);
-                add4(f, c0 + 4 * y);
-              }
-            } else {
-#pragma unroll
-              for (int y = 0; y < 4; ++y) {
-                float f[4];
-#pragma unroll
-                for (int x = 0; x < 4; ++x) f[x] = __uint_as_float(v[8 * y + 2 * x]) + __uint_as_float(v[8 * y + 2 * x + 1]);
-                add4(f, c0 / 2 + 4 * y);
-              }
+              for (int x = 0; x < 4; ++x) f[x] = __uint_as_float(v[8 * y + 2 * x]) + __uint_as_float(v[8 * y + 2 * x + 1]);
+              add4(f, c0 / 2 + 4 * y);
             }
           }
         }
@@ -320,9 +302,7 @@ int round32(int n) { return (n + 31) / 32 * 32; }
 
 // Shared memory of one stage's activation boxes per CTA and k-block, for a pass of at most R > 128 rows.
 int pair_act_bytes(int R) {
-  if (R <= kSpNarrowRows) return 16384 + round32(2 * (R - 128)) * 64;
-  R = R < kSpBlockRows ? R : kSpBlockRows;
-  return 32768 + round32(R - kSpBlockRows / 2) * 128;          // (the narrow form takes at most 32 KB)
+  return 16384 + (R < kSpBlockRows ? round32(2 * (R - kSpHalfRows)) * 64 : 16384);
 }
 
 }  // namespace
@@ -331,13 +311,10 @@ int pair_act_bytes(int R) {
 int stream_pair_ksb(int R) { return (kSpSmem - 2048) / (2 * (16384 + pair_act_bytes(R))) >= 4 ? 2 : 1; }
 
 // Tensor maps of one activation operand ([2 Rt, K], hi and lo rows interleaved): one per box height.
-bool stream_pair_act_maps(CUtensorMap* narrow, CUtensorMap* wide, const void* act, int Rt, int K, int R) {
+bool stream_pair_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int R) {
   const int ksb = stream_pair_ksb(R);
-  for (int i = 0; i < 8; ++i) {
-    if (!make_tmap_bf16_kblocks(&narrow[i], act, 2ll * Rt, K, 16 * (i + 1), ksb)) return false;
-    if (R <= kSpNarrowRows) wide[i] = narrow[i];
-    else if (!make_tmap_bf16_parts(&wide[i], act, Rt, K, 16 * (i + 1), ksb)) return false;
-  }
+  for (int i = 0; i < 8; ++i)
+    if (!make_tmap_bf16_kblocks(&maps[i], act, 2ll * Rt, K, 16 * (i + 1), ksb)) return false;
   return true;
 }
 

@@ -1,7 +1,8 @@
 """Hyper-encoder passes at the row counts where the linear-layer kernel, its activation box or its row blocks
 change: one entry, capacities around 128, 256 and 512 packed rows (also with few of them live), the switch
 to whole output tiles, a rest behind full passes; odd multiples of 128 as width (half a tile of 256 weight
-rows); a session whose very first pass is captured into a graph.  Against the fp64 oracle."""
+rows); a session whose very first pass is captured into a graph.  Against the fp64 oracle.  Full-size decode
+passes of some hundred rows are held to the rounding of their sums, against fp64 on the GPU."""
 import numpy as np
 import pytest
 import torch
@@ -107,3 +108,65 @@ def test_entries_beyond_the_bound_stay_due():
     for b in range(w.B):
         want = ohe.hyper_embed(p.oracle.books[b].entries, f64(p.W_E), enc, w.heads)
         assert np.abs(p.E_f32[b, :n[b]].double().cpu().numpy() - want).max() <= TOL
+
+
+def _encode64(t, table, tok, heads, layers):
+    """Hyper-embedding of one phrase in fp64 on the GPU (tensors in ABI order, fp64)."""
+    d, L = table.shape[1], len(tok)
+    ln = lambda z, i: torch.nn.functional.layer_norm(z, (d,), t[i], t[i + 1], 1e-5)
+    x = table[tok].double() + t[0][:L]
+    for o in range(1, 1 + 12 * layers, 12):
+        q, k, v = (ln(x, o) @ t[o + 2].T + t[o + 3]).view(L, 3, heads, d // heads).unbind(1)
+        a = torch.softmax(torch.einsum("ihc,jhc->hij", q, k) / (d // heads) ** 0.5, -1)
+        x = x + torch.einsum("hij,jhc->ihc", a, v).reshape(L, d) @ t[o + 4].T + t[o + 5]
+        x = x + torch.nn.functional.gelu(ln(x, o + 6) @ t[o + 8].T + t[o + 9]) @ t[o + 10].T + t[o + 11]
+    return x.mean(0)
+
+
+@pytest.mark.parametrize("d,M,B,tied,bound", [(4096, 3, 128, 0, 2.0e-5), (3072, 5, 128, 0, 1.6e-5)])
+def test_sums_of_a_decode_pass_of_some_hundred_rows(d, M, B, tied, bound):
+    """Every row of the pass's capacity is live.  The tensor cores add 16 products to a sum at a time and lose
+    low bits each time, so that the error grows with the additions an accumulator takes: with one product per
+    weight and a chain over all of K = 4 d the rows were off by 1.8e-5 of their rms at d = 4096 and by 1.4e-5 at
+    d = 3072, with both operand parts in one chain by 2.5e-5 and 2.1e-5.  Bound: the former and an
+    eighth for other inputs."""
+    V, layers, cap, heads, dev = 2000, 2, 16, d // 128, "cuda:0"
+    g = torch.Generator(device=dev)
+    g.manual_seed(d + M)
+
+    def normal(shape, std, mean=0.0):
+        return (torch.randn(shape, generator=g, device=dev) * std + mean).bfloat16()
+
+    def encoder():
+        t = [normal((M, d), 0.02)]
+        for _ in range(layers):
+            t += [normal((d,), 0.1, 1.0), normal((d,), 0.05), normal((3 * d, d), 0.02), normal((3 * d,), 0.05)]
+            t += [normal((d, d), 0.02), normal((d,), 0.05), normal((d,), 0.1, 1.0), normal((d,), 0.05)]
+            t += [normal((4 * d, d), 0.02), normal((4 * d,), 0.05), normal((d, 4 * d), 0.02), normal((d,), 0.05)]
+        return t
+
+    sides = 1 if tied else 2
+    W = [normal((V, d), 0.02) for _ in range(sides)]
+    enc = [encoder() for _ in range(sides)]
+    ew = [zb.encoder_weights(t) for t in enc]
+    cache = [torch.zeros(B, cap, d, dtype=torch.bfloat16, device=dev) for _ in range(sides)]
+    f32 = [torch.zeros(B, cap, d, device=dev) for _ in range(2)]
+    cb = zb.Codebook(zb.make_config(V, d, M, cap, B, "bf16", layers, heads, 4 * d, tied), dev)
+    codes = lambda f: torch.tensor([f(b) for b in range(B)], dtype=torch.int32, device=dev)
+    zb.z2z_lzw_step(cb, codes(lambda b: b), None, None)
+    for k in range(M - 2):                               # a, a a, a a a: the previous phrase grows to M - 1 tokens
+        zb.z2z_lzw_step(cb, codes(lambda b: V + k), None, None)
+    nxt, new = (torch.zeros(B, dtype=torch.int32, device=dev) for _ in range(2))
+    lse = torch.zeros(B, device=dev)
+    zb.z2z_decode_step(cb, normal((B, d), 1.0), W[0], W[-1], ew[0], ew[-1], cache[0], cache[-1], zb.SELECT_ARGMAX, 1.0, 0, 0,
+                       codes(lambda b: 1000 + b), nxt, None, lse, new, f32[0], f32[1])
+    assert new.cpu().tolist() == [M - 2] * B             # B * M rows: every entry is M tokens long
+    for side in range(sides):
+        t = [x.double() for x in enc[side]]
+        err, ref = [], []
+        for b in range(0, B, 8):
+            want = _encode64(t, W[side], [b] * (M - 1) + [1000 + b], heads, layers)
+            ref.append(want)
+            err.append(f32[side][b, M - 2].double() - want)
+        err, ref = torch.stack(err), torch.stack(ref)
+        assert float(err.pow(2).mean().sqrt() / ref.pow(2).mean().sqrt()) <= bound
