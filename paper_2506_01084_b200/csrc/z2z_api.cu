@@ -313,6 +313,7 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
   z2z::EncoderArgs a = encoder_args(cb, d_table, enc, d_cache, d_cache_f32, el.chunk);
   const bool tc = cb->use_tensor_cores && cb->cfg.enc_layers >= 0 &&
                   z2z::encoder_tc_supported(cb->cfg.d, cb->dff, cb->cfg.dtype, cb->heads, cb->cfg.M);
+  a.prompt = z2z::encoder_rows_are_prompt_sized(el.chunk * cb->cfg.M);
   const bool entry = z2z::encoder_entry_applies(cb->cfg.d, cb->dff, cb->cfg.enc_layers);
   {
     z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 1, s);
@@ -341,7 +342,7 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
   // weight copies and the call is long enough (several passes) to repay making them.
   a.w_half = nullptr;
   if (tc && cb->half_scratch && cb->cfg.enc_layers > 0 && n_chunks >= 4 &&
-      z2z::encoder_pass_is_prompt_sized(a.entries, el.chunk, cb->cfg.M, cb->cfg.d) &&
+      a.prompt &&
       cb->half_bytes >= z2z::encoder_half_bytes(cb->cfg.d, cb->dff, cb->cfg.enc_layers)) {
     cb->half_ptrs.assign((size_t)enc->n_tensors, nullptr);
     Z2Z_CUDA(z2z::convert_encoder_weights_to_half(enc->tensors, cb->cfg.d, cb->dff, cb->cfg.enc_layers, cb->half_scratch,

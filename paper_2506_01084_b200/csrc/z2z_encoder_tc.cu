@@ -54,13 +54,17 @@ constexpr int kMaxVec4 = 8;            // float4 per thread in the row kernels: 
 constexpr int kNarrowVec4 = 4;         // ... and for d <= 4096, where half the registers do
 // Which linear-layer kernel a pass takes, by its row capacity.  Up to 128 rows one CTA per weight tile streams
 // best (24 rows, d = 3072, both encoders: 249 us a step against 272 with pairs; 96 rows, d = 4096: equal);
-// beyond, CTA pairs carry up to 256 rows on one stream (270 rows, one encoder: 486 -> 291 us a step).  Past that
-// the stream comes twice and whole output tiles take over, the earlier the wider the model, as a wave of
-// tiles is then fuller (one encoder: d = 3072, 768 rows 755 against 725 us, 1023 rows 860 against 949;
-// d = 4096, 680 rows 957 against 830, 800 rows 1116 against 1253).
+// beyond, CTA pairs carry up to 256 rows on one stream (270 rows, one encoder: 486 -> 291 us a step).  Passes
+// of 1024 rows take whole output tiles.  Those put both operand parts of all of K into one accumulator, which
+// costs accuracy (error against fp64 in units of the rows' rms, d = 4096: 4.3e-5, streamed 1.35e-5), so that
+// smaller decode steps stay with the stream also where whole tiles would be quicker (one encoder, all rows
+// live: d = 4096, 768 rows 1266 against 1188 us a step, 900 rows 1536 against 1446; d = 3072, 930 rows 991 against
+// 1012).  The calls of a session of prompt size are used to the accuracy of whole tiles and take them
+// where they are quicker, the earlier the wider the model, as a wave of tiles is then fuller (d = 4096, a call
+// bounded to 639 rows 971 against 1105 us, 768 rows 1250 against 1118; d = 3072, 768 rows 605 against 642).
 constexpr int kStreamSingleRows = 128;
-constexpr int kPromptSessionRows = 1024;      // rows a pass of the session can hold from which it counts as prompt-sized
-static int pair_pass_min_rows(int d) { return d > 3584 ? 720 : 900; }
+constexpr int kPromptPassRows = 1024;         // rows of a pass, or that a pass of the session can hold, from which it is prompt-sized
+static int prompt_call_min_rows(int d) { return d > 3584 ? 720 : 900; }
 
 struct Ptr2 { const void* p[2]; };
 struct MPtr2 { void* p[2]; };
@@ -781,11 +785,7 @@ size_t encoder_half_bytes(int d, int dff, int layers) {
   return (size_t)layers * ((size_t)4 * d * d + (size_t)2 * d * dff) * 2;
 }
 
-// Whether a pass of `entries` work-list slots is a prompt-sized one (CTA-pair GEMMs).
-bool encoder_pass_is_prompt_sized(int entries, int chunk, int M, int d) {
-  const int E = entries < chunk ? entries : chunk;
-  return E * M >= pair_pass_min_rows(d);
-}
+bool encoder_rows_are_prompt_sized(int rows) { return rows >= kPromptPassRows; }
 
 // Makes fp16 copies of the linear-layer weights of one encoder in `scratch` and fills
 // half_ptrs[i] (host array, ABI tensor order) with their device addresses (nullptr elsewhere).
@@ -842,7 +842,8 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   const int R = a0.rows > 0 ? a0.rows : E * M;         // row capacity of this pass
   // Passes of a call that knows its rows (a0.rows) always take whole tiles in a session of prompt size: their
   // results are then the same bits whatever else is in the call, which stream-K sums are not.
-  if (ng == 1 && (R >= pair_pass_min_rows(d) || (a0.rows > 0 && el.chunk * M >= kPromptSessionRows))) return run_encoder_pass_pair(cb, a0, el, E, R, prof, s);
+  const bool whole_tiles = R >= kPromptPassRows || (a0.prompt && (a0.rows > 0 || R >= prompt_call_min_rows(d)));
+  if (ng == 1 && whole_tiles) return run_encoder_pass_pair(cb, a0, el, E, R, prof, s);
   const int Rt = (R + 7) / 8 * 8;                      // rows of the result matrix per group
   const int* total = el.row_off + E;                   // packed rows of this pass (device word)
   const int n_sm = sm_count();

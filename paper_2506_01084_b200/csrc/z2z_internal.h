@@ -70,11 +70,12 @@ struct EncoderArgs {
   size_t* part_clean;           // host word of the session: leading bytes of `part` known to be zero
   int entries;                  // host bound on the entries of this pass (<= the work list's capacity)
   int rows;                     // host bound on its packed rows, 0 = entries * M
+  bool prompt;                  // a call's pass (not a decode step's) in a session whose passes are prompt-sized
   int* err;                     // device error word of the tensor-core kernels
 };
 bool encoder_tc_supported(int d, int dff, int dtype, int heads, int M);
 size_t encoder_half_bytes(int d, int dff, int layers);
-bool encoder_pass_is_prompt_sized(int entries, int chunk, int M, int d);
+bool encoder_rows_are_prompt_sized(int rows);
 cudaError_t convert_encoder_weights_to_half(const void* const* w, int d, int dff, int layers, void* scratch,
                                             const void** half_ptrs, int* err_word, Prof* prof, cudaStream_t s);
 bool logits_tc_supported(int d, int dtype);
