@@ -141,7 +141,8 @@ int32_t z2z_lzw_step(z2z_codebook* cb, const int32_t* d_new_codes, const uint8_t
  *            max_entries < 0: exact.  The call reads the number of entries it has to embed back
  *            from the device - it waits for the stream once, the only enqueueing call that does,
  *            and therefore cannot be captured into a graph - and launches no pass without work.
- *            In prompt-sized bf16 sessions the rows are then the same bits whatever else is in the call.
+ *            In prompt-sized bf16 sessions (min(max(B * cap, B), 1024) * M >= 1024) the rows are then the same
+ *            bits whatever else is in the call; with max_entries >= 0 they are the same bits for the same call.
  *            Meant for whole prompts, where hundreds of empty passes would cost more than the wait.
  *   d_cache  [B, cap, d] in the configured dtype (row k of sequence b = hypertoken V + k).
  *   d_cache_f32 [B, cap, d] fp32 or NULL: the same rows before rounding to the cache dtype.    */

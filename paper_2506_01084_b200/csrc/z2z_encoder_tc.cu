@@ -27,7 +27,9 @@
 // whenever no GEMM result is pending.  The element-wise kernel after a GEMM reads each element of
 // that GEMM's result exactly once and stores zero back ("consume and clear"), for every live row
 // of the pass (the GEMM adds nothing to rows beyond them), which restores the invariant for the
-// next GEMM.  The first pass of a session that needs it clears Y.
+// next GEMM.  The first pass of a session that needs it clears Y.  Sums of three or more partials depend on
+// the order in which they arrive: calls whose bits must not (z2z_hyper_embed in a session of prompt size)
+// use a matrix for each half of K (StreamGemmParams::half_stride), and the kernel after the GEMM adds the two.
 //
 // Launches per layer: GEMM(qkv) -> [+ bias, attention] -> GEMM(o) -> [+ bias + residual,
 // LayerNorm 2] -> GEMM(1) -> [+ bias, GELU] -> GEMM(2) -> [+ bias + residual, LayerNorm 1 of the
@@ -59,9 +61,11 @@ constexpr int kNarrowVec4 = 4;         // ... and for d <= 4096, where half the 
 // costs accuracy (error against fp64 in units of the rows' rms, d = 4096: 4.3e-5, streamed 1.35e-5), so that
 // smaller decode steps stay with the stream also where whole tiles would be quicker (one encoder, all rows
 // live: d = 4096, 768 rows 1266 against 1188 us a step, 900 rows 1536 against 1446; d = 3072, 930 rows 991 against
-// 1012).  The calls of a session of prompt size are used to the accuracy of whole tiles and take them
-// where they are quicker, the earlier the wider the model, as a wave of tiles is then fuller (d = 4096, a call
-// bounded to 639 rows 971 against 1105 us, 768 rows 1250 against 1118; d = 3072, 768 rows 605 against 642).
+// 1012).  Bounded calls in a session of prompt size stream too, with a matrix for each half of K, up to the
+// capacity below; beyond they take whole tiles, as every call of such a session did before (us for 510, 639 and
+// 768 rows, streamed / whole tiles: d = 1024 205 286 298 / 198 224 231, d = 2048 348 466 486 / 358 397 408, d = 3072
+// 501 706 748 / 540 609 618, d = 4096 708 1013 - / 755 1088 1026; the error 4.6e-6 / 1.1e-5, 6.4e-6 / 2.2e-5,
+// 8.5e-6 / 3.2e-5, 1.1e-5 / 4.3e-5: between 512 rows and the line accuracy is what speaks for the stream).
 constexpr int kStreamSingleRows = 128;
 constexpr int kPromptPassRows = 1024;         // rows of a pass, or that a pass of the session can hold, from which it is prompt-sized
 static int prompt_call_min_rows(int d) { return d > 3584 ? 720 : 900; }
@@ -108,6 +112,9 @@ __device__ __forceinline__ int entry_len_tc(const CbView& cb, const EntryList& e
 __device__ __forceinline__ float4 unpack_bf16x4(uint2 u) {
   return make_float4(bf_lo(u.x), bf_hi(u.x), bf_lo(u.y), bf_hi(u.y));
 }
+
+// A result that lies in two matrices (StreamGemmParams::half_stride): always first half + second half.
+__device__ __forceinline__ void add_half(float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; }
 
 __device__ __forceinline__ float block_sum(float v, float* sm) {
 #pragma unroll
@@ -197,8 +204,8 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_gather_ln(CbView cb, EntryLi
 // x = X[r] + Y[r] + bias for a live packed row (Y consumed and cleared); then LayerNorm -> hi/lo
 // for the next GEMM.  grid (rows, groups).  All loads (row count, Y, X, bias, gamma, beta) are
 // issued together; whether the row is live only decides what is stored.
-template <int NV>
-__global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_ln(const int* total, float* Y, Ptr2 bias,
+template <int NV, bool HALVES>
+__global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_ln(const int* total, float* Y, size_t half_stride, Ptr2 bias,
                                                                     MPtr2 X, Ptr2 ln_w, Ptr2 ln_b, MPtr2 Ahl,
                                                                     int d, int Rt) {
   __shared__ float sm[32];
@@ -212,13 +219,14 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_ln(const int* t
   const uint2* lw = reinterpret_cast<const uint2*>(ln_w.p[g]);
   const uint2* lb = reinterpret_cast<const uint2*>(ln_b.p[g]);
   const int nvec = d / 4;
-  float4 xv[NV], yv[NV];
+  float4 xv[NV], yv[NV], zv[HALVES ? NV : 1];
   uint2 bv[NV], gw[NV], gb[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     const int idx = (int)threadIdx.x + v * kRowThreads;
     if (idx < nvec) {
       yv[v] = *reinterpret_cast<const float4*>(y + idx * 4);
+      if (HALVES) zv[HALVES ? v : 0] = *reinterpret_cast<const float4*>(y + half_stride + idx * 4);
       xv[v] = *reinterpret_cast<const float4*>(x + idx * 4);
       bv[v] = bs[idx]; gw[v] = lw[idx]; gb[v] = lb[idx];
     }
@@ -229,6 +237,10 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_ln(const int* t
     const int idx = (int)threadIdx.x + v * kRowThreads;
     if (idx < nvec) {
       *reinterpret_cast<float4*>(y + idx * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (HALVES) {
+        *reinterpret_cast<float4*>(y + half_stride + idx * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
+        add_half(yv[v], zv[HALVES ? v : 0]);
+      }
       const float4 b = unpack_bf16x4(bv[v]);
       xv[v] = make_float4(xv[v].x + yv[v].x + b.x, xv[v].y + yv[v].y + b.y, xv[v].z + yv[v].z + b.z,
                           xv[v].w + yv[v].w + b.w);
@@ -242,9 +254,10 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_ln(const int* t
 // Last layer: x_i = X[r_i] + Y[r_i] + bias for the entry's rows, cache row = mean_i x_i.
 // grid (entries, groups, ceil(d / (4 * kRowThreads))): a thread owns 4 columns of the entry and
 // issues the loads of all its rows before it adds.
-__global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_pool(CbView cb, EntryList el, float* Y, Ptr2 bias,
-                                                                      MPtr2 X, MPtr2 cache, MPtr2 cache_f32, int d,
-                                                                      int Rt) {
+template <bool HALVES>
+__global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_pool(CbView cb, EntryList el, float* Y, size_t half_stride,
+                                                                      Ptr2 bias, MPtr2 X, MPtr2 cache, MPtr2 cache_f32,
+                                                                      int d, int Rt) {
   sm100::pdl_trigger();
   sm100::pdl_wait();
   const int e = blockIdx.x, g = blockIdx.y;
@@ -255,12 +268,13 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_pool(CbView cb,
   const int seq = el.seq[e], idx = el.idx[e];
   const float4 b = load_bf16x4(reinterpret_cast<const bf16*>(bias.p[g]) + col);
   if (L <= 0) return;
-  float4 yv[kMaxM], xv[kMaxM];
+  float4 yv[kMaxM], xv[kMaxM], zv[HALVES ? kMaxM : 1];
 #pragma unroll
   for (int i = 0; i < kMaxM; ++i)
     if (i < L) {
       const size_t r = (size_t)r0 + i;
       yv[i] = *reinterpret_cast<const float4*>(Y + ((size_t)g * Rt + r) * d + col);
+      if (HALVES) zv[HALVES ? i : 0] = *reinterpret_cast<const float4*>(Y + half_stride + ((size_t)g * Rt + r) * d + col);
       xv[i] = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(X.p[g]) + r * d + col);
     }
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -269,6 +283,10 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_pool(CbView cb,
     if (i < L) {
       const size_t r = (size_t)r0 + i;
       *reinterpret_cast<float4*>(Y + ((size_t)g * Rt + r) * d + col) = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (HALVES) {
+        *reinterpret_cast<float4*>(Y + half_stride + ((size_t)g * Rt + r) * d + col) = make_float4(0.f, 0.f, 0.f, 0.f);
+        add_half(yv[i], zv[HALVES ? i : 0]);
+      }
       acc.x += xv[i].x + yv[i].x + b.x; acc.y += xv[i].y + yv[i].y + b.y;
       acc.z += xv[i].z + yv[i].z + b.z; acc.w += xv[i].w + yv[i].w + b.w;
     }
@@ -308,15 +326,16 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_pool(CbView cb, EntryList el
 // kGeluThreads apart, and issues all of its loads before it computes.
 // grid = ceil(groups * R * J / 4 / (kGeluThreads * kGeluPerThread)), R = row capacity of the pass.
 constexpr int kGeluThreads = 256, kGeluPerThread = 4;
-__global__ void __launch_bounds__(kGeluThreads) k_tc_reduce_gelu(const int* total_rows, float* Y, Ptr2 bias, MPtr2 Hhl,
-                                                                 int J, int R, int Rt, int ng) {
+template <bool HALVES>
+__global__ void __launch_bounds__(kGeluThreads) k_tc_reduce_gelu(const int* total_rows, float* Y, size_t half_stride, Ptr2 bias,
+                                                                 MPtr2 Hhl, int J, int R, int Rt, int ng) {
   sm100::pdl_trigger();
   sm100::pdl_wait();
   const int J4 = J / 4;
   const long long total = (long long)ng * R * J4;
   const long long base = (long long)blockIdx.x * (kGeluThreads * kGeluPerThread) + threadIdx.x;
   const int live = *total_rows;
-  float4 q[kGeluPerThread], bs[kGeluPerThread];
+  float4 q[kGeluPerThread], bs[kGeluPerThread], q2[HALVES ? kGeluPerThread : 1];
   int row[kGeluPerThread], jj[kGeluPerThread];
 #pragma unroll
   for (int k = 0; k < kGeluPerThread; ++k) {
@@ -327,6 +346,7 @@ __global__ void __launch_bounds__(kGeluThreads) k_tc_reduce_gelu(const int* tota
       jj[k] = (int)(f - (long long)row[k] * J4) * 4;
       const int g = row[k] / R, r = row[k] - g * R;
       q[k] = *reinterpret_cast<const float4*>(Y + ((size_t)g * Rt + r) * J + jj[k]);
+      if (HALVES) q2[HALVES ? k : 0] = *reinterpret_cast<const float4*>(Y + half_stride + ((size_t)g * Rt + r) * J + jj[k]);
       bs[k] = load_bf16x4(reinterpret_cast<const bf16*>(bias.p[g]) + jj[k]);
     }
   }
@@ -336,6 +356,10 @@ __global__ void __launch_bounds__(kGeluThreads) k_tc_reduce_gelu(const int* tota
     const int g = row[k] / R, r = row[k] - g * R;
     if (r >= live) continue;                       // no row there: Y is still zero, nothing reads the operand row
     *reinterpret_cast<float4*>(Y + ((size_t)g * Rt + r) * J + jj[k]) = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (HALVES) {
+      *reinterpret_cast<float4*>(Y + half_stride + ((size_t)g * Rt + r) * J + jj[k]) = make_float4(0.f, 0.f, 0.f, 0.f);
+      add_half(q[k], q2[HALVES ? k : 0]);
+    }
     float4 v = make_float4(q[k].x + bs[k].x, q[k].y + bs[k].y, q[k].z + bs[k].z, q[k].w + bs[k].w);
     v.x = 0.5f * v.x * (1.0f + erff(v.x * 0.70710678118654752440f));
     v.y = 0.5f * v.y * (1.0f + erff(v.y * 0.70710678118654752440f));
@@ -349,8 +373,9 @@ __global__ void __launch_bounds__(kGeluThreads) k_tc_reduce_gelu(const int* tota
 // q, k, v = Y + bias for one head of one entry (consumed, cleared, staged in shared memory), then
 // bidirectional attention over the entry's rows; output as hi/lo.
 // grid (entries, heads, groups), block (32, M), dynamic smem M * 3 * dh floats; dh % 4 == 0.
-__global__ void k_tc_qkv_attention(CbView cb, EntryList el, float* Y, Ptr2 bias, MPtr2 Ohl, int d, int heads,
-                                   int Rt) {
+template <bool HALVES>
+__global__ void k_tc_qkv_attention(CbView cb, EntryList el, float* Y, size_t half_stride, Ptr2 bias, MPtr2 Ohl, int d,
+                                   int heads, int Rt) {
   extern __shared__ float s_qkv[];
   sm100::pdl_trigger();
   sm100::pdl_wait();
@@ -362,16 +387,21 @@ __global__ void k_tc_qkv_attention(CbView cb, EntryList el, float* Y, Ptr2 bias,
     const bf16* bs = reinterpret_cast<const bf16*>(bias.p[g]);
     float* y = Y + ((size_t)g * Rt + r) * 3 * d;
     for (int c = lane * 4; c < dh; c += 128) {
-      float4 p[3], b[3];
+      float4 p[3], b[3], p2[HALVES ? 3 : 1];
 #pragma unroll
-      for (int w = 0; w < 3; ++w) {                // the six loads are independent of one another
+      for (int w = 0; w < 3; ++w) {                // the loads are independent of one another
         const int col = w * d + h * dh + c;
         p[w] = *reinterpret_cast<const float4*>(y + col);
+        if (HALVES) p2[HALVES ? w : 0] = *reinterpret_cast<const float4*>(y + half_stride + col);
         b[w] = load_bf16x4(bs + col);
       }
 #pragma unroll
       for (int w = 0; w < 3; ++w) {
         *reinterpret_cast<float4*>(y + w * d + h * dh + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (HALVES) {
+          *reinterpret_cast<float4*>(y + half_stride + w * d + h * dh + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+          add_half(p[w], p2[HALVES ? w : 0]);
+        }
         *reinterpret_cast<float4*>(&s_qkv[(i * 3 + w) * dh + c]) =
             make_float4(p[w].x + b[w].x, p[w].y + b[w].y, p[w].z + b[w].z, p[w].w + b[w].w);
       }
@@ -848,10 +878,13 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   const int* total = el.row_off + E;                   // packed rows of this pass (device word)
   const int n_sm = sm_count();
   const bool narrow = d <= 4 * kRowThreads * kNarrowVec4;      // a row fits four float4 per thread
-  auto rlk = narrow ? k_tc_reduce_resid_ln<kNarrowVec4> : k_tc_reduce_resid_ln<kMaxVec4>;
+  const bool halves = a0.prompt;                       // the call's bits must not depend on who adds first
+  auto rlk = halves ? (narrow ? k_tc_reduce_resid_ln<kNarrowVec4, true> : k_tc_reduce_resid_ln<kMaxVec4, true>)
+                    : (narrow ? k_tc_reduce_resid_ln<kNarrowVec4, false> : k_tc_reduce_resid_ln<kMaxVec4, false>);
   float* Y = a0.part;                                  // GEMM results, all zero between GEMMs
   const size_t wide = (size_t)(3 * d > dff ? 3 * d : dff);
-  const size_t y_bytes = (size_t)ng * Rt * wide * sizeof(float);
+  const size_t hs = halves ? (size_t)ng * Rt * wide : 0;
+  const size_t y_bytes = (size_t)(halves ? 2 : 1) * ng * Rt * wide * sizeof(float);
   if (y_bytes > a0.part_bytes) return cudaErrorMemoryAllocation;
   if (a0.layers > 0 && y_bytes > *a0.part_clean) {
     // a clear that is only captured into a graph leaves nothing cleared for calls outside of it
@@ -880,7 +913,8 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   StreamPairMaps pair_maps;
   auto gemm = [&](const MPtr2& act, int K, int widx, int J) -> cudaError_t {
     auto fill = [&](auto p) {
-      p.groups = ng; p.ksteps = K / (64 * ksb); p.R = R; p.out = Y; p.J = J; p.Rt = Rt; p.rows_dev = total; p.err = a0.err;
+      p.groups = ng; p.ksteps = K / (64 * ksb); p.R = R; p.out = Y; p.J = J; p.Rt = Rt; p.half_stride = hs;
+      p.rows_dev = total; p.err = a0.err;
       return p;
     };
     auto make = [&](auto& m, auto act_maps) {
@@ -919,15 +953,15 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
     if ((e = gemm(Ahl, d, o + 2, 3 * d)) != cudaSuccess) return e;
     {
       ProfScope ps(prof, kProfEncOther, 1, s);
-      launch_pdl(k_tc_qkv_attention, dim3(E, a0.heads, ng), dim3(32, M), (size_t)M * 3 * dh * 4, s, cb, el, Y,
-                 W(o + 3), Ahl, d, a0.heads, Rt);
+      launch_pdl(halves ? k_tc_qkv_attention<true> : k_tc_qkv_attention<false>, dim3(E, a0.heads, ng), dim3(32, M),
+                 (size_t)M * 3 * dh * 4, s, cb, el, Y, hs, W(o + 3), Ahl, d, a0.heads, Rt);
     }
     if ((e = gemm(Ahl, d, o + 4, d)) != cudaSuccess) return e;
     int last_bias = o + 5;                             // bias of the layer's last linear map
     if (dff > 0) {                                     // dff == 0: attention-only layer
       {
         ProfScope ps(prof, kProfEncOther, 1, s);
-        launch_pdl(rlk, dim3(R, ng), dim3(kRowThreads), 0, s, total, Y, W(o + 5), X, W(o + 6),
+        launch_pdl(rlk, dim3(R, ng), dim3(kRowThreads), 0, s, total, Y, hs, W(o + 5), X, W(o + 6),
                    W(o + 7), Ahl, d, Rt);
       }
       if ((e = gemm(Ahl, d, o + 8, dff)) != cudaSuccess) return e;
@@ -935,8 +969,8 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
         ProfScope ps(prof, kProfEncOther, 1, s);
         const long long f4 = (long long)ng * R * (dff / 4);
         const int per_cta = kGeluThreads * kGeluPerThread;
-        launch_pdl(k_tc_reduce_gelu, dim3((unsigned)((f4 + per_cta - 1) / per_cta)), dim3(kGeluThreads), 0, s, total, Y,
-                   W(o + 9), Hhl, dff, R, Rt, ng);
+        launch_pdl(halves ? k_tc_reduce_gelu<true> : k_tc_reduce_gelu<false>, dim3((unsigned)((f4 + per_cta - 1) / per_cta)),
+                   dim3(kGeluThreads), 0, s, total, Y, hs, W(o + 9), Hhl, dff, R, Rt, ng);
       }
       if ((e = gemm(Hhl, dff, o + 10, d)) != cudaSuccess) return e;
       last_bias = o + 11;
@@ -944,10 +978,10 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
     {
       ProfScope ps(prof, kProfEncOther, 1, s);
       if (last)
-        launch_pdl(k_tc_reduce_resid_pool, dim3(E, ng, (d / 4 + kRowThreads - 1) / kRowThreads), dim3(kRowThreads), 0,
-                   s, cb, el, Y, W(last_bias), X, cache, c32, d, Rt);
+        launch_pdl(halves ? k_tc_reduce_resid_pool<true> : k_tc_reduce_resid_pool<false>,
+                   dim3(E, ng, (d / 4 + kRowThreads - 1) / kRowThreads), dim3(kRowThreads), 0, s, cb, el, Y, hs, W(last_bias), X, cache, c32, d, Rt);
       else
-        launch_pdl(rlk, dim3(R, ng), dim3(kRowThreads), 0, s, total, Y, W(last_bias), X, W(o + 12),
+        launch_pdl(rlk, dim3(R, ng), dim3(kRowThreads), 0, s, total, Y, hs, W(last_bias), X, W(o + 12),
                    W(o + 13), Ahl, d, Rt);
     }
   }

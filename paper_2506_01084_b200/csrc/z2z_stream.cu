@@ -215,7 +215,7 @@ __device__ __forceinline__ void setup_barriers(Ctrl* ctrl) {
 // =================================================================================================
 // GEMM kernel: weights as the M operand, activation rows (hi | lo) as the N operand
 // =================================================================================================
-struct GemmJob { int g, wrow, kb0, kb1; };
+struct GemmJob { int g, wrow, half, kb0, kb1; };
 struct GemmWalk {
   const StreamGemmParams& p;
   long long u, u1;
@@ -229,7 +229,9 @@ struct GemmWalk {
     const long long tile = u / p.ksteps;
     j.kb0 = (int)(u - tile * p.ksteps);
     const long long left = u1 - u;
-    j.kb1 = (int)((p.ksteps - j.kb0) < left ? p.ksteps : j.kb0 + left);
+    const int mid = p.half_stride ? p.ksteps / 2 : 0, end = j.kb0 < mid ? mid : p.ksteps;
+    j.half = p.half_stride && j.kb0 >= mid;
+    j.kb1 = (int)((end - j.kb0) < left ? end : j.kb0 + left);
     j.g = (int)tile / p.tiles_per_group;
     j.wrow = ((int)tile - j.g * p.tiles_per_group) * kGemmNT;
     u += j.kb1 - j.kb0;
@@ -372,7 +374,7 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
       const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
       if (!mbar_wait(smem_u32(&ctrl->acc_full[buf]), aph, &ctrl->abort)) break;
       tc_fence_after();
-      float* dst = p.out + (size_t)j.g * p.Rt * p.J + j.wrow + feature;
+      float* dst = p.out + (j.half ? p.half_stride : 0) + (size_t)j.g * p.Rt * p.J + j.wrow + feature;
       const uint32_t t0 = tmem_base + ((uint32_t)(q * 32) << 16) + buf * (uint32_t)p.a_box_rows;
 #pragma unroll 1
       for (int r0 = 0; r0 < rows; r0 += 8) {
@@ -690,8 +692,9 @@ cudaError_t launch_stream_gemm(StreamGemmParams p, const StreamGemmMaps& maps, i
   p.box_step = gemm_box_step(p.R);
   p.a_box_rows = gemm_box_rows(p.R);
   p.tiles_per_group = p.J / kGemmNT;
-  const long long units = (long long)p.groups * p.tiles_per_group * p.ksteps;
-  const int grid = units < n_sm ? (int)units : n_sm;           // every CTA owns >= 1 unit
+  const long long tiles = (long long)p.groups * p.tiles_per_group, units = tiles * p.ksteps;
+  const int most = p.half_stride ? halves_workers(tiles, n_sm) : n_sm;
+  const int grid = units < most ? (int)units : most;           // every CTA owns >= 1 unit
   return stream_gemm_ksb(p.R) == 2 ? launch_stream_gemm_k<2>(p, maps, grid, s) : launch_stream_gemm_k<1>(p, maps, grid, s);
 }
 

@@ -61,12 +61,18 @@ cudaError_t run_logits_decode(const CbView& cb, const LogitsArgs& a, int* counte
 // reductions grow with the number of rows that exist, not with the capacity of the pass.  The
 // epilogue adds the hi and lo columns of a row in registers and reduces the sums into the fp32
 // result matrix out[group][Rt][J] (lanes = consecutive features = consecutive addresses).
+//
+// Three or more sums that meet in one word of the result are added in the order in which they arrive, and
+// their rounding depends on it.  With half_stride > 0 the two halves of K have a result matrix each and the
+// work is cut so that at most two sums meet in a word (0 + a + b = 0 + b + a): the same call then
+// gives the same bits.  The kernel that reads the results adds the two matrices.
 // The caller fills the first block of fields, the launch the second.
 struct StreamGemmParams {
   int groups, ksteps;    // ksteps = K / (64 * ksb), ksb = 64-column k-blocks per stage and TMA box
   int R;                 // row capacity of the pass
   float* out;            // [groups][Rt][J] fp32, zero before the first add
   int J, Rt;
+  size_t half_stride;    // floats from the result matrix of K's first half to that of its second, or 0
   const int* rows_dev;   // device word: packed rows that carry data (<= R)
   int* err;
 
@@ -77,6 +83,13 @@ struct StreamGemmMaps {
   CUtensorMap a[2][8];   // activation operand of each group, boxes of 1 .. 8 steps
   CUtensorMap w[2];      // weights of each group, 128 rows
 };
+// Workers (CTAs or clusters, `most` at most) for `tiles` tiles so that no half of a tile's K range is cut
+// more than once: pieces of half a tile or more, or two to four equal ones per tile.
+inline int halves_workers(long long tiles, int most) {
+  if (2 * tiles >= most) return most;
+  const long long per = most / tiles < 4 ? most / tiles : 4;
+  return (int)(tiles * per);
+}
 int stream_gemm_ksb(int R);
 bool stream_gemm_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int R);
 // At most 128 rows, one CTA per tile of 128 weight rows.
@@ -89,6 +102,7 @@ struct StreamPairParams {
   int R;
   float* out;
   int J, Rt;
+  size_t half_stride;
   const int* rows_dev;
   int* err;
 

@@ -204,12 +204,13 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
     int live = *p.rows_dev;
     live = live < p.R ? live : p.R;
     const int n_blocks = sp_live_blocks(p, live);
+    const int chain = p.half_stride ? p.ksteps / 2 : kSpChain / KSB;       // (K is a multiple of 128: the k-steps are even in number)
     if (warp == 1) {
       if (lane == 0 && rank == 0) {
         // ---------------- MMA issuer (leader only): D[256 weight rows][n] += W tile x activation rows -----
         int stage = 0; uint32_t phase = 0, job_i = 0;
         bool ok = true;
-        SpWalk walk(p, n_blocks, kSpChain / KSB);
+        SpWalk walk(p, n_blocks, chain);
         SpJob j;
         while (ok && walk.next(j)) {
           const uint32_t aph = job_i & 1u;
@@ -253,7 +254,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
       const int group = (warp - 2) >> 2;               // takes every other 32 columns
       const uint32_t acc_empty_leader = map_to_cta(smem_u32(&ctrl->acc_empty), 0);
       uint32_t job_i = 0;
-      SpWalk walk(p, n_blocks, kSpChain / KSB);
+      SpWalk walk(p, n_blocks, chain);
       SpJob j;
       while (walk.next(j)) {
         const uint32_t aph = job_i & 1u;
@@ -261,10 +262,11 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
         tc_fence_after();
         const int feature0 = j.wrow + (int)rank * 128;
         if (feature0 < p.J) {                          // the last tile may be half outside (J is a multiple of 128)
+          const size_t half = j.kb0 >= chain ? p.half_stride : 0;
           const int row0 = j.block * kSpBlockRows;
           const int rows = live - row0 < kSpBlockRows ? live - row0 : kSpBlockRows;
           // this lane's row of every four, and the first of the four features it adds
-          float* dst = p.out + ((size_t)j.g * p.Rt + row0 + (lane & 3)) * p.J + feature0 + q * 32 + (lane & ~3);
+          float* dst = p.out + half + ((size_t)j.g * p.Rt + row0 + (lane & 3)) * p.J + feature0 + q * 32 + (lane & ~3);
           const uint32_t t0 = tmem_base + ((uint32_t)(q * 32) << 16);
           auto add4 = [&](float (&f)[4], int r) {      // rows r .. r + 3
             transpose4(f, lane);
@@ -334,7 +336,8 @@ cudaError_t launch_stream_pair(StreamPairParams p, const StreamPairMaps& maps, i
   // epilogue instead of two; worth up to a seventh of the clusters (217 rows, d = 3072: 859 -> 750 us a
   // request start with 72 of 74).
   const int tiles = p.groups * p.tiles_per_group, whole = clusters / tiles * tiles;
-  if (7 * whole >= 6 * clusters) clusters = whole;
+  if (p.half_stride) clusters = halves_workers(tiles, clusters);
+  else if (7 * whole >= 6 * clusters) clusters = whole;
   auto kern = ksb == 2 ? k_stream_pair<2> : k_stream_pair<1>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

@@ -99,6 +99,23 @@ def test_whole_prompts_in_passes_cut_by_rows(M, d, dff):
         assert torch.all(p.E_f32[b, n[b]:] == 0)
 
 
+@pytest.mark.parametrize("d,dff", [(1024, 4096), (384, 1152)])
+@pytest.mark.parametrize("total", [16, 40, 43, 85, 86, 200])
+def test_a_bounded_call_gives_the_same_bits_every_time(d, dff, total):
+    """Sessions whose passes hold 1024 rows or more: on one CTA per tile, on pairs, in several row blocks."""
+    w, p = _pair(d, dff, 3, B=2, T=900, cap=600, seed=total)
+    i32 = lambda x: torch.tensor(x, dtype=torch.int32, device=p.dev)
+    count = [total // 2, total - total // 2]
+    assert all(p.oracle.books[b].n() >= count[b] for b in range(2))
+    first = None
+    for _ in range(10):
+        f32 = torch.full((2, w.cap, d), -5.0, dtype=torch.float32, device=p.dev)
+        zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, i32([0, 0]), i32(count), total, p.E_h, f32)
+        first = f32 if first is None else first
+        assert torch.equal(f32, first)
+    _check(w, p, first, [0, 0], count)
+
+
 def test_entries_beyond_the_bound_stay_due():
     w, p = _pair(256, 512, 3, B=3, T=500, cap=400, seed=8)
     n = [p.oracle.books[b].n() for b in range(w.B)]
