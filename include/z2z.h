@@ -132,10 +132,11 @@ int32_t z2z_lzw_step(z2z_codebook* cb, const int32_t* d_new_codes, const uint8_t
  *   d_table  [V, d]; enc: that side's encoder.
  *   d_first / d_count [B] or both NULL = every entry created since the last such call.
  *   max_entries  host upper bound on sum_b count_b (<= 0: B * cap).  It bounds the launch count
- *            and sizes the passes (entries beyond it stay due for the next call): entries are processed in
- *            passes of at most 1024, the last one sized for the rest, and a pass is about ten launches per layer
- *            whether or not it finds entries (the counts are device state).  After z2z_lzw_encode
- *            pass the number of prompt tokens (or the sum of the code lengths, if known on the
+ *            and sizes the passes: entries are processed in passes of at most 1024, the last one sized
+ *            for the rest.  Entries beyond it are not computed: with d_first == NULL they stay due for the next
+ *            such call, also through decode steps in between; those of a given range are the caller's to
+ *            give again.  A pass is about ten launches per layer whether or not it finds entries (the
+ *            counts are device state).  After z2z_lzw_encode pass the number of prompt tokens (or the sum of the code lengths, if known on the
  *            host): a prompt of T tokens creates fewer than T entries.  With 0 a large session
  *            (B * cap = 524288) would enqueue 512 passes.
  *            max_entries < 0: exact.  The call reads the number of entries it has to embed back

@@ -26,7 +26,7 @@ constexpr float kLnEps = 1e-5f;
 // n     [B]          i32   hypertokens so far
 // prev  [B]          i32   last code seen by the online update (-1: none)
 // status[B]          i32   Z2Z_ST_* bits
-// n_emb [2, B]       i32   entries already embedded into E_h (row 0) / U_h (row 1)
+// n_emb [2, B]       i32   entries already embedded into E_h (row 0) / U_h (row 1); ~n while a bounded call has left some out
 // ---------------------------------------------------------------------------------------------
 struct CbView {
   int V, M, cap, B, n_slots;

@@ -93,10 +93,12 @@ __global__ void __launch_bounds__(kUpdateThreads) k_decode_update(CbView cb, Dec
   // low half, rows in the high half (at most 128 entries of at most 8 rows).
   const StepRecord* mine_rec = reinterpret_cast<const StepRecord*>(reinterpret_cast<const char*>(a.records) + (size_t)tid * 64);
   int4 head = make_int4(0, 0, 0, 0);
+  int emb[2] = {0, 0};
   int tok[kMaxM];
 #pragma unroll
   for (int i = 0; i < kMaxM; ++i) tok[i] = -1;
   if (tid < cb.B) {
+    emb[0] = cb.n_emb[tid]; emb[1] = cb.n_emb[cb.B + tid];
     head = __ldcg(reinterpret_cast<const int4*>(mine_rec));
     const int4 t0 = __ldcg(reinterpret_cast<const int4*>(mine_rec) + 1), t1 = __ldcg(reinterpret_cast<const int4*>(mine_rec) + 2);
     tok[0] = t0.x; tok[1] = t0.y; tok[2] = t0.z; tok[3] = t0.w;
@@ -141,11 +143,12 @@ __global__ void __launch_bounds__(kUpdateThreads) k_decode_update(CbView cb, Dec
     el.seq[e] = -1; el.idx[e] = 0; el.len[e] = 0; el.row_off[e] = total_rows;
     for (int i = 0; i < cb.M; ++i) el.tok[(size_t)e * cb.M + i] = -1;
   }
-  // both caches will hold every entry once the encoder pass that follows has run
+  // both caches will hold every entry once the encoder pass that follows has run, unless a bounded call left some out
   int full = 1;
   if (tid < cb.B) {
     const int n = head.z;
-    cb.n_emb[tid] = n; cb.n_emb[cb.B + tid] = n;
+    if (emb[0] >= 0) cb.n_emb[tid] = n;
+    if (emb[1] >= 0) cb.n_emb[cb.B + tid] = n;
     full = n >= cb.cap && mine == 0;             // full already when this step began: it created nothing
   }
   // Once every codebook is full no step creates an entry any more.  The host learns it through a

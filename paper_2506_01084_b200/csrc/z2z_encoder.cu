@@ -30,7 +30,13 @@ __device__ __forceinline__ void block_exclusive_scan_1024(int v, int* smem, int&
   __syncthreads();
 }
 
-// mode 0: ranges from first/count (NULL: n_emb[which] .. n);  mode 1: from new_entry (0/1 each)
+// First entry of sequence b that is due on a side.
+__device__ __forceinline__ int due_from(const CbView& cb, int which, int b) {
+  const int e = cb.n_emb[which * cb.B + b];
+  return e < 0 ? ~e : e;
+}
+
+// mode 0: ranges from first/count (NULL: the entries due on side `which`);  mode 1: from new_entry (0/1 each)
 __global__ void __launch_bounds__(1024) k_entry_offsets(CbView cb, int which, int mode,
                                                         const int32_t* __restrict__ first,
                                                         const int32_t* __restrict__ count,
@@ -44,7 +50,7 @@ __global__ void __launch_bounds__(1024) k_entry_offsets(CbView cb, int which, in
     if (mode == 1) {
       c = (new_entry[b] >= 0 && new_entry[b] < n) ? 1 : 0;
     } else {
-      int f = first ? first[b] : cb.n_emb[which * cb.B + b];
+      int f = first ? first[b] : due_from(cb, which, b);
       f = f < 0 ? 0 : (f > n ? n : f);
       c = count ? count[b] : n - f;
       c = c < 0 ? 0 : (c > n - f ? n - f : c);
@@ -68,7 +74,7 @@ __device__ __forceinline__ void entry_of(const CbView& cb, int which, int mode, 
   int f;
   if (mode == 1) f = new_entry[b];
   else {
-    f = first ? first[b] : cb.n_emb[which * cb.B + b];
+    f = first ? first[b] : due_from(cb, which, b);
     const int n = cb.n[b];
     f = f < 0 ? 0 : (f > n ? n : f);
   }
@@ -109,7 +115,7 @@ __global__ void k_entry_fill(CbView cb, int which, int mode, const int32_t* __re
 __global__ void __launch_bounds__(256) k_entry_rows(CbView cb, int which, const int32_t* __restrict__ first, EntryList el) {
   const int b = blockIdx.x;
   const int count = el.off[b + 1] - el.off[b];
-  int f = first ? first[b] : cb.n_emb[which * cb.B + b];
+  int f = first ? first[b] : due_from(cb, which, b);
   const int n = cb.n[b];
   f = f < 0 ? 0 : (f > n ? n : f);
   int sum = 0;
@@ -147,18 +153,21 @@ __global__ void __launch_bounds__(1024) k_entry_passes(CbView cb, int which, con
   }
 }
 
-// off == NULL: every entry is embedded; else those among the first `bound` of the call (off: offsets of the
-// sequences' entries in it), so that what a bound left out is still due for the next call.
+// After a call (off: offsets of the sequences' entries in it): the entries among its first `bound` are embedded;
+// what the bound left out is due for the next call and stays so through decode steps.  After a decode step
+// (off == NULL): every entry is embedded, unless a call left some out.
 __global__ void k_mark_embedded(CbView cb, int which, const int32_t* off, long long bound) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= cb.B) return;
-  int left_out = 0;
-  if (off) {
-    const long long beyond = (long long)off[b + 1] - bound;
-    const int count = off[b + 1] - off[b];
-    left_out = beyond <= 0 ? 0 : (beyond < count ? (int)beyond : count);
+  int32_t* emb = cb.n_emb + which * cb.B + b;
+  if (!off) {
+    if (*emb >= 0) *emb = cb.n[b];
+    return;
   }
-  cb.n_emb[which * cb.B + b] = cb.n[b] - left_out;
+  const long long beyond = (long long)off[b + 1] - bound;
+  const int count = off[b + 1] - off[b];
+  const int left_out = beyond <= 0 ? 0 : (beyond < count ? (int)beyond : count);
+  *emb = left_out ? ~(cb.n[b] - left_out) : cb.n[b];
 }
 
 __device__ __forceinline__ int entry_len(const CbView& cb, const EntryList& el, int e) {

@@ -188,3 +188,49 @@ def test_sums_of_a_decode_pass_of_some_hundred_rows(d, M, B, tied, bound):
             err.append(f32[side][b, M - 2].double() - want)
         err, ref = torch.stack(err), torch.stack(ref)
         assert float(err.pow(2).mean().sqrt() / ref.pow(2).mean().sqrt()) <= bound
+
+
+@pytest.mark.parametrize("B,tied", [(3, 0), (130, 0), (3, 1)])
+def test_entries_left_out_by_a_bound_stay_due_through_decode_steps(B, tied):
+    """The decode step's own launch (up to 128 sequences) and its separate ones, per side."""
+    w, p = _pair(128, 256, 3, B=B, T=120, cap=200, seed=B + tied, tied=tied)
+    n = [p.oracle.books[b].n() for b in range(w.B)]
+    assert min(n) > 8
+    sides = ((zb.CACHE_EMBED, p.g_WE, p.g_encE, p.E_h, p.E_f32, p.enc_E, p.W_E),
+             (zb.CACHE_UNEMBED, p.g_WU, p.g_encU, p.U_h, p.U_f32, p.enc_U, p.W_U))[:1 if tied else 2]
+    for which, table, enc, cache, f32, _, _ in sides:          # cut inside the second sequence; the other side later
+        zb.z2z_hyper_embed(p.cb, which, table, enc, None, None, n[0] + 4 + which, cache, f32)
+    nxt, new = (torch.zeros(B, dtype=torch.int32, device=p.dev) for _ in range(2))
+    lse = torch.zeros(B, device=p.dev)
+    for t in range(2):
+        forced = torch.tensor([(37 * b + 911 * t + 5) % w.V for b in range(B)], dtype=torch.int32, device=p.dev)
+        zb.z2z_decode_step(p.cb, si.make_hidden(w, B, t).to(p.dev), p.g_WE, p.g_WU, p.g_encE, p.g_encU, p.E_h, p.U_h,
+                           zb.SELECT_ARGMAX, 1.0, 0, t, forced, nxt, None, lse, new, p.E_f32, p.U_f32)
+        for b in range(B):
+            p.oracle.books[b].step(int(forced[b]))
+    for which, table, enc, cache, f32, host, W in sides:
+        zb.z2z_hyper_embed(p.cb, which, table, enc, None, None, -1, cache, f32)
+        for b in range(0, B, max(1, B // 8)):
+            want = ohe.hyper_embed(p.oracle.books[b].entries, f64(W), [f64(x) for x in host], w.heads)
+            assert np.abs(f32[b, :len(want)].double().cpu().numpy() - want).max() <= TOL
+        f32.fill_(-5)                                          # nothing is due any more
+        zb.z2z_hyper_embed(p.cb, which, table, enc, None, None, -1, cache, f32)
+        assert torch.all(f32 == -5)
+
+
+def test_decode_steps_settle_what_was_embedded_by_range():
+    """A program that embeds its prompts by given ranges: after a decode step only newer entries are due."""
+    w, p = _pair(128, 256, 3, B=3, T=120, cap=200, seed=5)
+    n = [p.oracle.books[b].n() for b in range(w.B)]
+    i32 = lambda x: torch.tensor(x, dtype=torch.int32, device=p.dev)
+    zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, i32([0] * 3), i32(n), sum(n), p.E_h, p.E_f32)
+    nxt, new = (torch.zeros(3, dtype=torch.int32, device=p.dev) for _ in range(2))
+    zb.z2z_decode_step(p.cb, si.make_hidden(w, 3, 1).to(p.dev), p.g_WE, p.g_WU, p.g_encE, p.g_encU, p.E_h, p.U_h,
+                       zb.SELECT_ARGMAX, 1.0, 0, 0, i32([7, 8, 9]), nxt, None, torch.zeros(3, device=p.dev), new, p.E_f32, p.U_f32)
+    _, m = zb.z2z_status(p.cb)
+    zb.z2z_lzw_step(p.cb, i32([1007, 1008, 1009]), None, new)
+    assert new.cpu().tolist() == m.tolist()
+    p.E_f32.fill_(-5)
+    zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, None, None, 3, p.E_h, p.E_f32)
+    for b in range(3):
+        assert torch.all(p.E_f32[b, int(m[b])] != -5) and torch.all(p.E_f32[b, :int(m[b])] == -5)
