@@ -382,7 +382,7 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
     a.entries = left < el.chunk ? (int)left : el.chunk;
     {
       z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 1, s);
-      Z2Z_CUDA(z2z::launch_entry_fill(cb->view, which, d_first, nullptr, el, c, s), "hyper_embed");
+      Z2Z_CUDA(z2z::launch_entry_fill(cb->view, which, d_first, nullptr, el, c, a.entries, s), "hyper_embed");
     }
     if (tc) Z2Z_CUDA(z2z::run_encoder_pass_tc(cb->view, &a, 1, el, false, &cb->prof, s), "hyper_embed (tensor cores)");
     else if (entry) Z2Z_CUDA(z2z::run_encoder_entries(cb->view, &a, 1, el, &cb->prof, s), "hyper_embed");
@@ -491,7 +491,7 @@ int32_t z2z_decode_step(z2z_codebook* cb, const void* d_hidden, const void* d_WE
     if (cb->cfg.cap > 0) {
       z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 4, s);
       Z2Z_CUDA(z2z::launch_entry_offsets_from_new(cb->view, w_new, el, s), "decode_step");
-      Z2Z_CUDA(z2z::launch_entry_fill(cb->view, 0, nullptr, w_new, el, 0, s), "decode_step");
+      Z2Z_CUDA(z2z::launch_entry_fill(cb->view, 0, nullptr, w_new, el, 0, B, s), "decode_step");
       Z2Z_CUDA(z2z::launch_mark_embedded(cb->view, 0, nullptr, 0, s), "decode_step");
       Z2Z_CUDA(z2z::launch_mark_embedded(cb->view, 1, nullptr, 0, s), "decode_step");
     }

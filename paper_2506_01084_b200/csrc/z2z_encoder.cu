@@ -357,10 +357,10 @@ cudaError_t launch_entry_offsets_from_new(const CbView& cb, const int32_t* new_e
   return cudaGetLastError();
 }
 cudaError_t launch_entry_fill(const CbView& cb, int which, const int32_t* first,
-                              const int32_t* new_entry, const EntryList& el, int chunk_index,
+                              const int32_t* new_entry, const EntryList& el, int chunk_index, int slots,
                               cudaStream_t s) {
-  return launch_pdl(k_entry_fill, dim3((el.chunk + 255) / 256), dim3(256), 0, s, cb, which, new_entry ? 1 : 0, first, new_entry,
-                    el, (long long)chunk_index * el.chunk, el.chunk, nullptr);
+  return launch_pdl(k_entry_fill, dim3((slots + 255) / 256), dim3(256), 0, s, cb, which, new_entry ? 1 : 0, first, new_entry,
+                    el, (long long)chunk_index * el.chunk, slots, nullptr);
 }
 cudaError_t launch_entry_rows(const CbView& cb, int which, const int32_t* first, const EntryList& el, cudaStream_t s) {
   k_entry_rows<<<cb.B, 256, 0, s>>>(cb, which, first, el);
@@ -385,7 +385,7 @@ template <typename T>
 static cudaError_t encoder_pass_simt(const CbView& cb, const EncoderArgs& a, const EntryList& el,
                                      Prof* prof, cudaStream_t s) {
   const int d = a.d, dff = a.dff, M = cb.M;
-  const int E = el.chunk, R = E * M;
+  const int E = a.entries, R = E * M;
   const int32_t* n_live = el.off + cb.B + 1;
   auto W = [&](int i) { return reinterpret_cast<const T*>(a.w[i]); };
   { ProfScope ps(prof, kProfEncOther, 1, s);

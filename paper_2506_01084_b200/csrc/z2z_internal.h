@@ -90,7 +90,7 @@ cudaError_t launch_entry_offsets(const CbView& cb, int which, const int32_t* fir
 cudaError_t launch_entry_offsets_from_new(const CbView& cb, const int32_t* new_entry,
                                           const EntryList& el, cudaStream_t s);
 cudaError_t launch_entry_fill(const CbView& cb, int which, const int32_t* first,
-                              const int32_t* new_entry, const EntryList& el, int chunk_index,
+                              const int32_t* new_entry, const EntryList& el, int chunk_index, int slots,
                               cudaStream_t s);
 // Passes cut by packed rows instead of entries.  launch_entry_rows leaves the rows of all entries of the
 // call in el.off[B + 1] (behind their number in el.off[B]); launch_entry_passes writes the first entry of

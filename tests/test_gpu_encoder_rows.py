@@ -15,10 +15,10 @@ from tests._harness import Pair, TOL, f64
 pytestmark = pytest.mark.gpu
 
 
-def _pair(d, dff, M, B, T, cap, seed, tied=0):
-    w = si.Workload("rows", V=2000, d=d, dtype="bf16", B=B, T=T, M=M, cap=cap, zipf_s=1.0, copy_p=0.5, seg_min=4,
-                    seg_max=14, steps=2, tied=tied, enc_layers=2, enc_heads=d // 128, enc_dff=dff)
-    p = Pair(w, seed)
+def _pair(d, dff, M, B, T, cap, seed, tied=0, dtype="bf16", tensor_cores=1):
+    w = si.Workload("rows", V=2000, d=d, dtype=dtype, B=B, T=T, M=M, cap=cap, zipf_s=1.0, copy_p=0.5, seg_min=4,
+                    seg_max=14, steps=2, tied=tied, enc_layers=2, enc_heads=max(d // 128, 1), enc_dff=dff)
+    p = Pair(w, seed, tensor_cores=tensor_cores)
     p.gpu_encode()
     for b in range(w.B):
         p.oracle.books[b].encode(p.tokens[b].tolist())
@@ -116,11 +116,19 @@ def test_a_bounded_call_gives_the_same_bits_every_time(d, dff, total):
     _check(w, p, first, [0, 0], count)
 
 
-def test_entries_beyond_the_bound_stay_due():
-    w, p = _pair(256, 512, 3, B=3, T=500, cap=400, seed=8)
+@pytest.mark.parametrize("d,dff,dtype,tensor_cores", [(256, 512, "bf16", 1), (384, 512, "bf16", 0), (320, 640, "fp32", 1),
+                                                      (64, 128, "fp32", 1)])
+def test_entries_beyond_the_bound_stay_due(d, dff, dtype, tensor_cores):
+    """On the tensor cores, on the tiled CUDA-core kernels (bf16, fp32) and with narrow models."""
+    w, p = _pair(d, dff, 3, B=3, T=500, cap=400, seed=8, dtype=dtype, tensor_cores=tensor_cores)
     n = [p.oracle.books[b].n() for b in range(w.B)]
+    p.E_f32.fill_(-5)
+    done = 0
     for bound in (20, n[0] + n[1] // 2 - 20, sum(n)):          # inside the first and second sequence, then the rest
         zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, None, None, bound, p.E_h, p.E_f32)
+        done = min(done + bound, sum(n))
+        assert [int((p.E_f32[b, :, 0] != -5).sum()) for b in range(3)] == [
+            max(0, min(n[b], done - sum(n[:b]))) for b in range(3)]
     enc = [f64(t) for t in p.enc_E]
     for b in range(w.B):
         want = ohe.hyper_embed(p.oracle.books[b].entries, f64(p.W_E), enc, w.heads)
