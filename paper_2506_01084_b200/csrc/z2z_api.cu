@@ -351,11 +351,11 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
   }
   // The rows of all entries are known (exact mode, tensor cores): passes are cut by rows, so that the tiles
   // of the linear layers fill their waves, and the rest is sized by what is left.
-  int32_t* pass_first = reinterpret_cast<int32_t*>(cb->ws + cb->plan.off_plan);
+  int32_t* pass_first = reinterpret_cast<int32_t*>(cb->ws + cb->plan.off_pass);
   const int pass_rows = rows > 0 ? z2z::encoder_pass_rows(rows, cb->plan.enc_rows < 256 ? 256 : cb->plan.enc_rows, cb->cfg.M, cb->cfg.d, cb->dff) : 0;
   const int per = pass_rows - (cb->cfg.M - 1);
   const long long n_passes = rows > 0 ? (rows + per - 1) / per : 0;
-  if (n_passes > 0 && pass_rows <= cb->plan.enc_rows && (size_t)(n_passes + 1) * 4 <= cb->plan.plan_bytes) {
+  if (n_passes > 0 && pass_rows <= cb->plan.enc_rows && (size_t)(n_passes + 1) * 4 <= cb->plan.pass_bytes) {
     if (n_passes == 1) {
       pass_first = nullptr;                            // all entries of the call
     } else {

@@ -79,12 +79,15 @@ struct WsPlan {
   size_t off_lpart, lpart_bytes;                  // logits partial reductions
   size_t off_plan, plan_bytes;                    // per-row-tile plan of the prompt-scoring logits kernel
   size_t off_step_out;                            // small per-step outputs
+  size_t off_pass, pass_bytes;                    // first entry of every hyper-encoder pass (apart from the plan:
+                                                  // a call may run beside the joint logits on another stream)
   size_t total;
 };
 
 constexpr int kLogitRowChunk = 8192;              // rows per logits launch (larger N loops)
 constexpr int kLogitPartRows = 1 << 20;           // partial-reduction slots (rows x groups), 32 bytes each
 constexpr int kPrefillPlanTiles = 1 << 14;        // 256-row tiles one prompt-scoring launch may have
+constexpr int kPassTable = 3 << 14;               // passes an exact hyper-embedding call may be cut into by rows, and one
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -146,6 +149,8 @@ inline WsPlan plan_workspace(const z2z_config& c) {
   p.plan_bytes = (size_t)kPrefillPlanTiles * 3 * 4;
   p.off_plan = take(p.plan_bytes);
   p.off_step_out = take((size_t)c.B * 64);
+  p.pass_bytes = (size_t)kPassTable * 4;
+  p.off_pass = take(p.pass_bytes);
   p.total = o;
   return p;
 }

@@ -242,3 +242,36 @@ def test_decode_steps_settle_what_was_embedded_by_range():
     zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, None, None, 3, p.E_h, p.E_f32)
     for b in range(3):
         assert torch.all(p.E_f32[b, int(m[b])] != -5) and torch.all(p.E_f32[b, :int(m[b])] == -5)
+
+
+def test_exact_call_beside_joint_logits_on_another_stream():
+    """The two calls share no scratch: the input side of a prompt may be embedded while positions are scored."""
+    w, p = _pair(256, 512, 3, B=4, T=3000, cap=1200, seed=3)
+    n = sum(p.oracle.books[b].n() for b in range(w.B))
+    assert n * 2 > 2048                                        # more than one pass
+    zb.z2z_hyper_embed(p.cb, zb.CACHE_UNEMBED, p.g_WU, p.g_encU, None, None, -1, p.U_h, None)
+    N = 20000
+    hid = torch.randn(N, w.d, device=p.dev).to(torch.bfloat16)
+    seq = (torch.arange(N, device=p.dev) % w.B).sort().values.to(torch.int32)
+    first = torch.zeros(w.B, dtype=torch.int32, device=p.dev)
+    count = torch.full((w.B,), w.cap, dtype=torch.int32, device=p.dev)       # clipped to what there is
+
+    def logits():
+        lse = torch.zeros(N, device=p.dev)
+        zb.z2z_dynamic_logits(p.cb, hid, seq, None, p.g_WU, p.U_h, zb.SELECT_ARGMAX, 1.0, 0, 0, None, lse, None, None)
+        return lse
+
+    def embed():
+        f32 = torch.zeros_like(p.E_f32)
+        zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, first, count, -1, p.E_h, f32)
+        return f32
+
+    want_lse, want_rows = logits(), embed()
+    torch.cuda.synchronize()
+    other = torch.cuda.Stream()
+    for _ in range(5):
+        with torch.cuda.stream(other):
+            lse = [logits() for _ in range(3)]
+        rows = [embed() for _ in range(3)]
+        torch.cuda.synchronize()
+        assert all(torch.equal(x, want_lse) for x in lse) and all(torch.equal(x, want_rows) for x in rows)
