@@ -122,10 +122,12 @@ int logits_call(z2z_codebook* cb, z2z::LogitsArgs a, cudaStream_t s, z2z::Logits
   const bool tc = cb->use_tensor_cores && z2z::logits_tc_supported(cb->cfg.d, cb->cfg.dtype);
   // By rows: up to 32 the decode kernel; up to 128 rows of a batch (every row another sequence) the
   // single-CTA stream, whose 128-row tiles and narrow hypertoken granules waste less than pairs with 256
-  // (V = 12000, d = 2176, 128 sequences: 54 against 69 us); more rows, or positions of few sequences, the
-  // CTA pairs (V = 32064, d = 3072, 128 positions of 5 sequences: 82 against 115 us).
+  // (V = 12000, d = 2176, 128 sequences: 50 against 71 us); more rows, or positions of few sequences, the
+  // CTA pairs (V = 32064, d = 3072, 128 positions of 5 sequences: 82 against 115 us).  Whose rows they are
+  // only the device knows when d_row_seq is given: as many rows as sequences or fewer are taken for a batch
+  // in another order, or part of one, more rows than sequences for positions.
   const bool decode = tc && z2z::decode_logits_applies(a);
-  const bool batch = info != nullptr || (N <= 128 && a.row_seq == nullptr);
+  const bool batch = info != nullptr || (N <= 128 && (a.row_seq == nullptr || N <= cb->cfg.B));
   const bool prefill = tc && info == nullptr && (cb->use_tensor_cores == 2 || !(decode || batch));
   long long chunk = z2z::kLogitRowChunk;
   int prefill_strips = cb->prefill_strips;

@@ -100,6 +100,32 @@ def test_joint_logits_against_fp64(V, d, N):
             assert torch.isnan(out["tl"][r])
 
 
+@pytest.mark.parametrize("N", [33, 100, 128])
+def test_a_batch_given_with_its_sequences_takes_the_batch_kernel(N):
+    """In order, in another order, a part of the batch, several rows of one sequence: the same kernels as without
+    d_row_seq (counted by their launches), and the right logits."""
+    V, d, B, cap = 1003, 256, 128, 80
+    counts = [(7 * b) % 70 for b in range(B)]
+    cb = _session(V, d, B, cap, counts, 6)
+    g = torch.Generator(device=DEV)
+    g.manual_seed(N)
+    rnd = lambda *s, std: (torch.randn(*s, generator=g, device=DEV) * std).to(torch.bfloat16)
+    hid, WU, Uh = rnd(N, d, std=1.0), rnd(V, d, std=0.05), rnd(B, cap, d, std=0.05)
+    order = torch.randperm(B, generator=g, device=DEV)[:N].to(torch.int32)
+    seqs = [None, torch.arange(N, device=DEV, dtype=torch.int32), order, order // 3]
+    launches = []
+    for seq in seqs:
+        lse = torch.zeros(N, device=DEV)
+        zb.z2z_profile_read(cb)
+        zb.z2z_dynamic_logits(cb, hid, seq, None, WU, Uh, zb.SELECT_ARGMAX, 1.0, 0, 0, None, lse, None, None)
+        launches.append(zb.z2z_profile_read(cb)[1])
+        own = list(range(N)) if seq is None else seq.tolist()
+        for r in range(0, N, 5):
+            l = torch.cat([WU.double() @ hid[r].double(), Uh[own[r], :counts[own[r]]].double() @ hid[r].double()])
+            assert abs(float(lse[r]) - float(torch.logsumexp(l, 0))) < 2e-5 * (1 + float(l.abs().max()))
+    assert all(x == launches[0] for x in launches)
+
+
 def test_overflowed_logit_keeps_its_row_a_number():
     N = 100
     cb = _session(300, 256, N, 8, [1] * N, 5)
