@@ -234,12 +234,20 @@ int32_t z2z_codebook_init(z2z_codebook** cb, const z2z_config* cfg, void* d_ws, 
   v.n_emb = reinterpret_cast<int32_t*>(h->ws + plan.off_n_emb);
   *cb = h;
   Z2Z_CUDA(cudaMemsetAsync(h->ws + plan.off_words, 0, 256, reinterpret_cast<cudaStream_t>(stream)), "codebook_init");
-  // the stream GEMM's result matrix is all zero between GEMMs; the first pass of the session that needs
-  // it clears what it needs (the whole matrix is 280-440 MB at d = 3072 / 4096 and took 28-70 us to clear
-  // here, a decode step uses 1-10 MB of it and a prompt-sized pass none)
-  h->part_clean = 0;
+  // The stream GEMM's result matrix is all zero between GEMMs.  What a decode step uses of it (1-10 MB) is
+  // cleared here together with the codebooks, so that a graph captured from the session's first steps holds
+  // no clear; a pass that needs more clears the rest itself.  (The whole matrix is 280-440 MB at d = 3072 /
+  // 4096, which took 28-70 us, and a prompt-sized pass uses none.)
+  size_t zero = 0;
+  if (c.enc_layers > 0 && c.cap > 0 && z2z::encoder_tc_supported(c.d, c.enc_dff, c.dtype, c.enc_heads, c.M)) {
+    zero = z2z::encoder_result_bytes(c.B * c.M, c.d, c.enc_dff, 2);
+    if (zero > plan.part_bytes) zero = plan.part_bytes;
+  }
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;        // (a captured clear has not happened yet)
+  Z2Z_CUDA(cudaStreamIsCapturing(reinterpret_cast<cudaStream_t>(stream), &cap), "codebook_init");
+  h->part_clean = cap == cudaStreamCaptureStatusNone ? zero : 0;
   z2z::ProfScope ps(&h->prof, z2z::kProfLzw, 1, reinterpret_cast<cudaStream_t>(stream));
-  Z2Z_CUDA(z2z::launch_codebook_clear(v, reinterpret_cast<cudaStream_t>(stream)), "codebook_init");
+  Z2Z_CUDA(z2z::launch_codebook_clear(v, h->ws + plan.off_part, zero, reinterpret_cast<cudaStream_t>(stream)), "codebook_init");
   return Z2Z_OK;
 }
 

@@ -817,6 +817,10 @@ size_t encoder_half_bytes(int d, int dff, int layers) {
 
 bool encoder_rows_are_prompt_sized(int rows) { return rows >= kPromptPassRows; }
 
+size_t encoder_result_bytes(int R, int d, int dff, int matrices) {
+  return (size_t)matrices * ((R + 7) / 8 * 8) * (size_t)(3 * d > dff ? 3 * d : dff) * sizeof(float);
+}
+
 // Makes fp16 copies of the linear-layer weights of one encoder in `scratch` and fills
 // half_ptrs[i] (host array, ABI tensor order) with their device addresses (nullptr elsewhere).
 cudaError_t convert_encoder_weights_to_half(const void* const* w, int d, int dff, int layers, void* scratch,
@@ -884,7 +888,7 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   float* Y = a0.part;                                  // GEMM results, all zero between GEMMs
   const size_t wide = (size_t)(3 * d > dff ? 3 * d : dff);
   const size_t hs = halves ? (size_t)ng * Rt * wide : 0;
-  const size_t y_bytes = (size_t)(halves ? 2 : 1) * ng * Rt * wide * sizeof(float);
+  const size_t y_bytes = encoder_result_bytes(R, d, dff, ng * (halves ? 2 : 1));
   if (y_bytes > a0.part_bytes) return cudaErrorMemoryAllocation;
   if (a0.layers > 0 && y_bytes > *a0.part_clean) {
     // a clear that is only captured into a graph leaves nothing cleared for calls outside of it

@@ -27,7 +27,7 @@ inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
 void set_last_error(const char* msg);      // text returned by z2z_last_error on this thread
 
 // ---- z2z_lzw.cu ------------------------------------------------------------------------------
-cudaError_t launch_codebook_clear(const CbView& cb, cudaStream_t s);
+cudaError_t launch_codebook_clear(const CbView& cb, void* zero, size_t zero_bytes, cudaStream_t s);
 cudaError_t launch_lzw_encode(const CbView& cb, const int32_t* tokens, const int32_t* lens,
                               int T_max, int32_t* codes, int32_t* code_lens,
                               int32_t* entries_after, cudaStream_t s);
@@ -76,6 +76,8 @@ struct EncoderArgs {
 bool encoder_tc_supported(int d, int dff, int dtype, int heads, int M);
 size_t encoder_half_bytes(int d, int dff, int layers);
 bool encoder_rows_are_prompt_sized(int rows);
+// Bytes of `matrices` GEMM result matrices of a pass of R rows.
+size_t encoder_result_bytes(int R, int d, int dff, int matrices);
 cudaError_t convert_encoder_weights_to_half(const void* const* w, int d, int dff, int layers, void* scratch,
                                             const void** half_ptrs, int* err_word, Prof* prof, cudaStream_t s);
 bool logits_tc_supported(int d, int dtype);

@@ -13,19 +13,23 @@
 
 namespace z2z {
 
-__global__ void k_codebook_clear(CbView cb) {
-  size_t n_hash = (size_t)cb.B * cb.n_slots;
-  size_t n_cons = (size_t)cb.B * cb.cap * cb.M;
-  size_t n_len = (size_t)cb.B * cb.cap;
-  size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  size_t stride = (size_t)gridDim.x * blockDim.x;
-  for (size_t i = tid; i < n_hash; i += stride) cb.hash[i] = kEmptySlot;
-  for (size_t i = tid; i < n_cons; i += stride) cb.cons[i] = -1;
-  for (size_t i = tid; i < n_len; i += stride) cb.len[i] = 0;
+// Session reset.  An empty slot and an absent constituent are all ones, and the workspace plan puts the two
+// tables behind one another and the lengths behind them, each from a 256-byte boundary: 16-byte stores.
+// zero / n_zero: words of the hyper-encoder's result matrix that have to be zero before its first pass.
+__global__ void k_codebook_clear(CbView cb, uint4* zero, size_t n_zero) {
+  uint4* const ones = reinterpret_cast<uint4*>(cb.hash);
+  uint4* const lens = reinterpret_cast<uint4*>(cb.len);
+  const size_t n_ones = (size_t)(lens - ones), n_lens = (size_t)(reinterpret_cast<uint4*>(cb.n) - lens);
+  const size_t tid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const size_t stride = (size_t)gridDim.x * blockDim.x;
+  for (size_t i = tid; i < n_ones; i += stride) ones[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+  for (size_t i = tid; i < n_zero; i += stride) zero[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (size_t i = tid; i < n_lens; i += stride) lens[i] = make_uint4(0u, 0u, 0u, 0u);
   for (size_t i = tid; i < (size_t)cb.B; i += stride) {
     cb.n[i] = 0; cb.prev[i] = -1; cb.status[i] = 0; cb.n_emb[i] = 0; cb.n_emb[cb.B + i] = 0;
   }
 }
+static_assert(kEmptySlot == ~0ull, "an empty slot is all ones");
 
 // Prompt compression (Section 2.1; Section 2.3 step 2).  One block per sequence; a window of
 // kParseLanes input positions at a time (z2z_lzw_dev.cuh).
@@ -204,12 +208,13 @@ __global__ void __launch_bounds__(128) k_lzw_step(CbView cb, const int32_t* __re
   if (lane == 0 && new_entry) new_entry[b] = created;
 }
 
-cudaError_t launch_codebook_clear(const CbView& cb, cudaStream_t s) {
-  size_t work = (size_t)cb.B * cb.n_slots;
+cudaError_t launch_codebook_clear(const CbView& cb, void* zero, size_t zero_bytes, cudaStream_t s) {
+  size_t work = (size_t)(reinterpret_cast<char*>(cb.len) - reinterpret_cast<char*>(cb.hash)) / 16;
+  if (work < zero_bytes / 16) work = zero_bytes / 16;
   int blocks = (int)((work + 255) / 256);
   if (blocks > 148 * 8) blocks = 148 * 8;
   if (blocks < 1) blocks = 1;
-  k_codebook_clear<<<blocks, 256, 0, s>>>(cb);
+  k_codebook_clear<<<blocks, 256, 0, s>>>(cb, reinterpret_cast<uint4*>(zero), zero_bytes / 16);
   return cudaGetLastError();
 }
 

@@ -3,6 +3,8 @@ change: one entry, capacities around 128, 256 and 512 packed rows (also with few
 to whole output tiles, a rest behind full passes; odd multiples of 128 as width (half a tile of 256 weight
 rows); a session whose very first pass is captured into a graph.  Against the fp64 oracle.  Full-size decode
 passes of some hundred rows are held to the rounding of their sums, against fp64 on the GPU."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -83,6 +85,66 @@ def test_decode_step_of_a_large_batch_captured_first(B, tied):
         if want >= 0 and b % 7 < 2:
             row = ohe.hyper_embed([p.oracle.books[b].entries[want]], table, enc, w.heads)[0]
             assert np.abs(p.E_f32[b, want].double().cpu().numpy() - row).max() <= TOL
+
+
+def _node_types(graph):
+    """Types of the nodes of a captured graph (0: kernel, 1: copy, 2: set)."""
+    rt = ctypes.CDLL("libcudart.so.12")
+    n = ctypes.c_size_t(0)
+    g = ctypes.c_void_p(graph.raw_cuda_graph())
+    assert rt.cudaGraphGetNodes(g, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert rt.cudaGraphGetNodes(g, nodes, ctypes.byref(n)) == 0
+    types = []
+    for x in nodes:
+        t = ctypes.c_int(-1)
+        assert rt.cudaGraphNodeGetType(ctypes.c_void_p(x), ctypes.byref(t)) == 0
+        types.append(t.value)
+    return types
+
+
+@pytest.mark.parametrize("B,tied", [(2, 0), (43, 1), (90, 0), (150, 0)])
+def test_steps_captured_first_hold_no_clear(B, tied):
+    """Neither the first step of a new session nor of one that starts again, nor a bounded call of one entry per
+    sequence, captures anything but kernels; what the session start itself captures clears when it runs."""
+    w, p = _pair(256, 512, 3, B, T=64, cap=64, seed=B, tied=tied)
+    hid = si.make_hidden(w, B, 3).to(p.dev)
+    nxt = torch.zeros(B, dtype=torch.int32, device=p.dev)
+
+    def step():
+        zb.z2z_decode_step(p.cb, hid, p.g_WE, p.g_WU, p.g_encE, p.g_encU, p.E_h, p.U_h, zb.SELECT_ARGMAX, 1.0, 0, 0,
+                           None, nxt, None, None, None, p.E_f32, p.U_f32)
+        zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, None, None, B, p.E_h, p.E_f32)
+
+    for again in (False, True):
+        if again:
+            zb.z2z_codebook_init(p.cb)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph(keep_graph=True)
+        with torch.cuda.graph(graph):
+            step()
+        assert set(_node_types(graph)) == {0}
+        step()
+
+
+def test_a_captured_session_start_clears_when_it_runs():
+    w, p = _pair(256, 512, 3, 3, T=64, cap=64, seed=3)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        zb.z2z_codebook_init(p.cb)
+    # the graph has not run: the words of the result matrix may hold anything a failed pass left there
+    p.cb.workspace.fill_(0xff)
+    hid = si.make_hidden(w, 3, 3).to(p.dev)
+    nxt, new = (torch.zeros(3, dtype=torch.int32, device=p.dev) for _ in range(2))
+    graph.replay()
+    for t, codes in enumerate(([5, 6, 7], [8, 9, 10])):
+        zb.z2z_decode_step(p.cb, hid, p.g_WE, p.g_WU, p.g_encE, p.g_encU, p.E_h, p.U_h, zb.SELECT_ARGMAX, 1.0, 0, t,
+                           torch.tensor(codes, dtype=torch.int32, device=p.dev), nxt, None, torch.zeros(3, device=p.dev), new,
+                           p.E_f32, p.U_f32)
+    assert new.cpu().tolist() == [0, 0, 0]
+    want = ohe.hyper_embed([(5, 8), (6, 9), (7, 10)], f64(p.W_E), [f64(t) for t in p.enc_E], w.heads)
+    assert np.abs(p.E_f32[:, 0].double().cpu().numpy() - want).max() <= TOL
 
 
 @pytest.mark.parametrize("M,d,dff", [(2, 128, 256), (3, 384, 384), (5, 128, 128)])
