@@ -324,7 +324,6 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
   const bool tc = cb->use_tensor_cores && cb->cfg.enc_layers >= 0 &&
                   z2z::encoder_tc_supported(cb->cfg.d, cb->dff, cb->cfg.dtype, cb->heads, cb->cfg.M);
   a.prompt = z2z::encoder_rows_are_prompt_sized(el.chunk * cb->cfg.M);
-  const bool entry = z2z::encoder_entry_applies(cb->cfg.d, cb->dff, cb->cfg.enc_layers);
   {
     z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 1, s);
     Z2Z_CUDA(z2z::launch_entry_offsets(cb->view, which, d_first, d_count, el, s), "hyper_embed");
@@ -395,7 +394,7 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
       Z2Z_CUDA(z2z::launch_entry_fill(cb->view, which, d_first, nullptr, el, c, a.entries, s), "hyper_embed");
     }
     if (tc) Z2Z_CUDA(z2z::run_encoder_pass_tc(cb->view, &a, 1, el, false, &cb->prof, s), "hyper_embed (tensor cores)");
-    else if (entry) Z2Z_CUDA(z2z::run_encoder_entries(cb->view, &a, 1, el, &cb->prof, s), "hyper_embed");
+    else if (z2z::encoder_entry_applies(cb->cfg.d, cb->dff, cb->cfg.enc_layers, a.entries)) Z2Z_CUDA(z2z::run_encoder_entries(cb->view, &a, 1, el, &cb->prof, s), "hyper_embed");
     else Z2Z_CUDA(z2z::run_encoder_pass(cb->view, a, el, false, &cb->prof, s), "hyper_embed");
   }
   if (!d_first) {
@@ -515,7 +514,7 @@ int32_t z2z_decode_step(z2z_codebook* cb, const void* d_hidden, const void* d_WE
     if (!tied) g[1] = encoder_args(cb, d_WU, enc_U, d_Uh, d_Uh_f32, B, 1);
     if (tc) {
       Z2Z_CUDA(z2z::run_encoder_pass_tc(cb->view, g, tied ? 1 : 2, el, fused, &cb->prof, s), "decode_step (tensor cores)");
-    } else if (z2z::encoder_entry_applies(cb->cfg.d, cb->dff, cb->cfg.enc_layers)) {
+    } else if (z2z::encoder_entry_applies(cb->cfg.d, cb->dff, cb->cfg.enc_layers, B)) {
       Z2Z_CUDA(z2z::run_encoder_entries(cb->view, g, tied ? 1 : 2, el, &cb->prof, s), "decode_step");
     } else {
       Z2Z_CUDA(z2z::run_encoder_pass(cb->view, g[0], el, false, &cb->prof, s), "decode_step");

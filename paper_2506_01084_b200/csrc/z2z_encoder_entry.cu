@@ -215,9 +215,13 @@ size_t entry_smem_bytes(int M, int d, int dff) { return (size_t)M * (5 * d + dff
 }  // namespace
 
 // Narrow models: at d = 256 a layer set is 6 MB, which four SMs still read in about 13 us; wider ones
-// are a stream that needs all SMs (z2z_encoder.cu, z2z_encoder_tc.cu).
-bool encoder_entry_applies(int d, int dff, int layers) {
-  return d <= kEntryMaxD && dff <= kEntryMaxDff && layers <= kEntryMaxLayers;
+// are a stream that needs all SMs (z2z_encoder.cu, z2z_encoder_tc.cu).  And few entries: every one reads all
+// weights again, so that the time grows with each wave of some 36 clusters, while the tiled kernels of
+// z2z_encoder.cu take about as long for 200 entries as for one (us for 64 / 96 / 128 / 1024 entries of one
+// fp32 encoder of two layers, dff = 4 d, here and there: d = 64 66 93 119 828 / 134 134 134 172, d = 128 95 138 178
+// 1291 / 179 179 179 241, d = 192 156 230 301 2224 / 234 234 234 337, d = 256 195 290 380 2851 / 281 281 282 552).
+bool encoder_entry_applies(int d, int dff, int layers, int entries) {
+  return d <= kEntryMaxD && dff <= kEntryMaxDff && layers <= kEntryMaxLayers && entries <= (d <= 192 ? 96 : 72);
 }
 
 cudaError_t run_encoder_entries(const CbView& cb, const EncoderArgs* grp, int ng, const EntryList& el, Prof* prof,

@@ -111,8 +111,8 @@ cudaError_t run_encoder_pass(const CbView& cb, const EncoderArgs& a, const Entry
                              bool use_tensor_cores, Prof* prof, cudaStream_t s);
 
 // ---- z2z_encoder_entry.cu --------------------------------------------------------------------
-// Narrow models on the CUDA cores: the whole pass of one or two encoders in one launch.
-bool encoder_entry_applies(int d, int dff, int layers);
+// Few entries of narrow models on the CUDA cores: the whole pass of one or two encoders in one launch.
+bool encoder_entry_applies(int d, int dff, int layers, int entries);
 cudaError_t run_encoder_entries(const CbView& cb, const EncoderArgs* groups, int n_groups, const EntryList& el,
                                 Prof* prof, cudaStream_t s);
 
