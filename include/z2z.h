@@ -143,7 +143,9 @@ int32_t z2z_lzw_step(z2z_codebook* cb, const int32_t* d_new_codes, const uint8_t
  *            from the device - it waits for the stream once, the only enqueueing call that does,
  *            and therefore cannot be captured into a graph - and launches no pass without work.
  *            In prompt-sized bf16 sessions (min(max(B * cap, B), 1024) * M >= 1024) the rows are then the same
- *            bits whatever else is in the call; with max_entries >= 0 they are the same bits for the same call.
+ *            bits whatever else is in the call, unless fp16 scratch is lent (z2z_set_encoder_half_scratch: how
+ *            many entries a call has decides whether it uses the copies); with max_entries >= 0 they are the
+ *            same bits for the same call.
  *            Meant for whole prompts, where hundreds of empty passes would cost more than the wait.
  *   d_cache  [B, cap, d] in the configured dtype (row k of sequence b = hypertoken V + k).
  *   d_cache_f32 [B, cap, d] fp32 or NULL: the same rows before rounding to the cache dtype.    */
@@ -272,13 +274,14 @@ int32_t z2z_set_tensor_cores(z2z_codebook* cb, int32_t enable);
  * 2.3 steps 3-4; the number format is this library's choice, the paper fixes none).  By default
  * the tensor-core passes keep activations as two bf16 parts (about 16 mantissa bits), two
  * tensor-core instructions per k-step.  When the caller lends device memory for fp16 copies of one
- * encoder's linear-layer weights, z2z_hyper_embed calls that span at least four prompt-sized passes
- * (bf16 sessions, passes of >= 1024 rows) remake the copies at the start of the call - a bf16
+ * encoder's linear-layer weights, z2z_hyper_embed calls of more than 3072 entries (known from
+ * max_entries or, with max_entries < 0, read back; bf16 sessions of prompt size) remake the copies at the start of the call - a bf16
  * value inside fp16's range converts exactly - and round each activation once to fp16 (11 mantissa
  * bits): one instruction per k-step, half the tensor-core work.  Measured against the fp64
  * definition with randomly drawn gains and biases, the largest error of a hyper-embedding grows
  * from 9e-5 to 7.3e-3 at d = 4096 (tolerance 2e-2); sessions that need the wider margin leave the
- * scratch unset.  Decode steps are not affected.
+ * scratch unset.  Decode steps are not affected, nor are shorter calls, whose rows then differ from
+ * those of a longer call by that rounding.
  *   d_scratch: 256-byte aligned, bytes >= 2 * enc_layers * (4 d^2 + 2 d enc_dff) * 2, valid until
  *   replaced; NULL or 0 bytes returns to the two-part form.  A weight beyond fp16's range
  *   (|w| > 65504) cannot be copied exactly: Z2Z_ST_HALF_RANGE is then reported by z2z_status.   */

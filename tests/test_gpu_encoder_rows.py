@@ -337,3 +337,19 @@ def test_exact_call_beside_joint_logits_on_another_stream():
         rows = [embed() for _ in range(3)]
         torch.cuda.synchronize()
         assert all(torch.equal(x, want_lse) for x in lse) and all(torch.equal(x, want_rows) for x in rows)
+
+
+def test_exact_rows_do_not_depend_on_the_rest_of_the_call():
+    """A few entries alone, in a call of one pass and in a call of several: the same bits."""
+    w, p = _pair(256, 512, 3, B=3, T=3000, cap=1400, seed=12)
+    n = [p.oracle.books[b].n() for b in range(w.B)]
+    assert sum(n) > 1100
+    rows = []
+    for count in ([5, 0, 9], [200, 30, 100], n):
+        f32 = torch.full((3, w.cap, 256), -5.0, device=p.dev)
+        i32 = lambda x: torch.tensor(x, dtype=torch.int32, device=p.dev)
+        zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, i32([0] * 3), i32(count), -1, p.E_h, f32)
+        rows.append(f32)
+    assert torch.equal(rows[0][0, :5], rows[2][0, :5]) and torch.equal(rows[0][2, :9], rows[2][2, :9])
+    for b, c in enumerate([200, 30, 100]):
+        assert torch.equal(rows[1][b, :c], rows[2][b, :c])
