@@ -22,7 +22,8 @@
 //
 // Bound by the passes' barriers and dependent round trips, not by bytes.  (16 rows of 128 k columns, k = 50,
 // p = 0.9: 100 us when every pass read its columns from L2, took two cluster barriers and the nucleus was
-// always looked for; a whole step of 16 sequences went from 716 to 679 us.)
+// always looked for; a whole step of 16 sequences went from 716 to 679 us.)  Rows that are not kept: 96 rows of
+// 129 k columns, k = 50 64 us, p = 0.9 171, without a filter 82.
 #include <cooperative_groups.h>
 
 #include "z2z_common.cuh"
@@ -88,17 +89,27 @@ __device__ __forceinline__ float block_sum_f(float v, SfShared* sh) {
   return t;
 }
 
-// Calls f(logit, column) for the n columns from c0 on that lie at l (shared or global memory), each
-// thread its share: 16-byte loads when l starts on a 16-byte boundary.
-template <typename F>
-__device__ __forceinline__ void for_each_logit(const float* l, int c0, int n, F f) {
-  const int t = threadIdx.x;
+// Calls f(logit, column) for the n columns from c0 (a multiple of 4) on that lie at l, each thread its share:
+// 16-byte loads when l starts on a 16-byte boundary, from global memory two of them in flight.  The columns of
+// a load are written as 4 q + 0 .. 3, which lets the compiler see that they share one Philox block.
+template <bool GLOBAL, typename F>
+__device__ __forceinline__ void for_each_logit(const float* __restrict__ l, int c0, int n, F f) {
+  const int t = threadIdx.x, q0 = c0 >> 2;
   if ((reinterpret_cast<uintptr_t>(l) & 15u) == 0) {
     const float4* l4 = reinterpret_cast<const float4*>(l);
     const int n4 = n >> 2;
-    for (int i = t; i < n4; i += kSfThreads) {
+    int i = t;
+    if (GLOBAL) {
+      for (; i + kSfThreads < n4; i += 2 * kSfThreads) {
+        const float4 a = l4[i], b = l4[i + kSfThreads];
+        const int c = 4 * (q0 + i), e = 4 * (q0 + i + kSfThreads);
+        f(a.x, c); f(a.y, c + 1); f(a.z, c + 2); f(a.w, c + 3);
+        f(b.x, e); f(b.y, e + 1); f(b.z, e + 2); f(b.w, e + 3);
+      }
+    }
+    for (; i < n4; i += kSfThreads) {
       const float4 a = l4[i];
-      const int c = c0 + 4 * i;
+      const int c = 4 * (q0 + i);
       f(a.x, c); f(a.y, c + 1); f(a.z, c + 2); f(a.w, c + 3);
     }
     for (int i = (n4 << 2) + t; i < n; i += kSfThreads) f(l[i], c0 + i);
@@ -128,17 +139,16 @@ __global__ void __launch_bounds__(kSfThreads) k_sample_filtered(const float* __r
   const int c0 = rank * share < C ? rank * share : C;
   const int n = C - c0 < share ? C - c0 : share;
   const bool held = share <= hold;
-  const float* mine = held ? s_hold : l + c0;
   float m = -INFINITY;
   if (held) {
-    for_each_logit(l + c0, 0, n, [&](float x, int i) { s_hold[i] = x; m = fmaxf(m, x); });
+    for_each_logit<true>(l + c0, 0, n, [&](float x, int i) { s_hold[i] = x; m = fmaxf(m, x); });
     __syncthreads();
   } else if (top_p < 1.0f) {
-    for_each_logit(mine, c0, n, [&](float x, int) { m = fmaxf(m, x); });
+    for_each_logit<true>(l + c0, c0, n, [&](float x, int) { m = fmaxf(m, x); });
   }
   auto each = [&](auto f) {
-    if (held) for_each_logit(static_cast<const float*>(s_hold), c0, n, f);
-    else for_each_logit(mine, c0, n, f);
+    if (held) for_each_logit<false>(static_cast<const float*>(s_hold), c0, n, f);
+    else for_each_logit<true>(l + c0, c0, n, f);
   };
   // ---- 1. max and partition sum; only the nucleus filter needs them
   float mx = 0.f, z = 0.f;
@@ -367,7 +377,8 @@ extern "C" int32_t z2z_sample_filtered(const float* d_logits, int32_t N, int64_t
   int G = 1;
   while (G < 8 && (long long)N * (2 * G) <= 148) G *= 2;
   const long long share = ((ld + G - 1) / G + 3) & ~3ll;
-  const int hold = share <= z2z::kSfHold ? (int)share : 0;
+  // (without a filter there is a single pass, which gains nothing from a copy)
+  const int hold = share <= z2z::kSfHold && (top_k > 0 || top_p < 1.0f) ? (int)share : 0;
   cudaError_t e = cudaFuncSetAttribute(z2z::k_sample_filtered, cudaFuncAttributeMaxDynamicSharedMemorySize, z2z::kSfHold * 4);
   if (e != cudaSuccess) { z2z::set_last_error(cudaGetErrorString(e)); return Z2Z_ERR_CUDA; }
   cudaLaunchConfig_t lc = {};

@@ -105,6 +105,26 @@ def test_filtered_sampling_with_every_cluster_size(N):
             assert gap < GAP or band[got[r]] or band[a]
 
 
+@pytest.mark.parametrize("C", [41004, 45057, 49156])
+@pytest.mark.parametrize("top_k,top_p", [(30, 0.9), (0, 0.7), (12, 1.0), (0, 1.0)])
+def test_filtered_sampling_of_rows_too_long_to_be_kept(C, top_k, top_p):
+    # one CTA per row and more columns than its shared memory takes: every pass reads them from L2, two
+    # 16-byte loads at a time (C a multiple of 4: whole rounds, a single load and a scalar tail) or one by one
+    rng = np.random.default_rng(C)
+    N = 75
+    l32 = (rng.standard_normal((N, C)) * 2.0).astype(np.float32)
+    n_cols = [C - (r % 5) * 1023 for r in range(N)]
+    got, kept = _run(l32, n_cols, top_k, top_p, 0.9, 21, 4, row_base=3)
+    for r in list(range(5)) + [40, 74]:
+        l = l32[r, :n_cols[r]].astype(np.float64)
+        a, keep, gap = olg.select_filtered(l, 0.9, top_k, top_p, 21, 4, 3 + r)
+        band = _band(l, 0.9, top_p)
+        assert abs(int(kept[r]) - int(keep.sum())) <= int(band.sum())
+        assert keep[got[r]] or band[got[r]]
+        if got[r] != a:
+            assert gap < GAP or band[got[r]] or band[a]
+
+
 def test_filtered_sampling_small_rows_and_frequencies():
     # tiny rows, exhaustively comparable; and frequencies over many steps against the renormalised distribution
     p = np.array([0.4, 0.25, 0.2, 0.1, 0.05])
