@@ -32,7 +32,7 @@ __global__ void k_codebook_clear(CbView cb, uint4* zero, size_t n_zero) {
 static_assert(kEmptySlot == ~0ull, "an empty slot is all ones");
 
 // Prompt compression (Section 2.1; Section 2.3 step 2).  One block per sequence; a window of
-// kParseLanes input positions at a time (z2z_lzw_dev.cuh).
+// LANES input positions at a time (z2z_lzw_dev.cuh).
 //
 // Each lane follows the longest match from its own position (at most M - 1 dependent lookups).
 // Which positions start a phrase is a walk position -> position + match length: inside a warp by
@@ -43,20 +43,18 @@ static_assert(kEmptySlot == ~0ull, "an empty slot is all ones");
 // Bound by the latency of one window (a few dependent shared-memory lookups, ten shuffles, four
 // barriers).  The chain used to be walked token by token by one thread: 180 ns per token with the
 // table in shared memory, 220 with it in global memory.  Four texts of 32768 tokens (cap 16384), to
-// codes and back with both session resets: 9.62 ms before, 1.00 ms with windows here and in the replay.
-constexpr int kTokRing = 512;
-static_assert(kTokRing >= kParseLanes + kMaxM, "a window's tokens fit the ring");
-
-template <bool SMEM>
-__global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const int32_t* __restrict__ tokens,
+// codes and back with both session resets: 9.62 ms before, 0.65 ms with windows here and in the replay.
+template <int LANES, bool SMEM>
+__global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_encode(CbView cb, const int32_t* __restrict__ tokens,
                                                               const int32_t* __restrict__ lens, int T_max,
                                                               int32_t* __restrict__ codes,
                                                               int32_t* __restrict__ code_lens,
                                                               int32_t* __restrict__ entries_after) {
+  constexpr int WARPS = LANES / 32, kTokRing = 2 * LANES;      // (a window's tokens and a match behind it fit the ring)
   extern __shared__ __align__(16) unsigned char s_parse[];
   __shared__ int s_tok[kTokRing];                    // token of position p at p mod kTokRing
-  __shared__ int2 s_walk[kParseWarps][kMaxM];        // per warp and entry lane: lanes visited, exit
-  __shared__ ParseVotes s_votes;
+  __shared__ int2 s_walk[WARPS][kMaxM];        // per warp and entry lane: lanes visited, exit
+  __shared__ ParseVotes<WARPS> s_votes;
   __shared__ int s_prev, s_n1, s_st;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
@@ -69,22 +67,22 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const i
   table.open(cb, b, n0, s_parse);
   if (tid == 0) { s_prev = -1; s_st = 0; s_n1 = n0; }
   __syncthreads();
-  if (tid < kParseLanes) {
+  if (tid < LANES) {
     int32_t* out = codes + (size_t)b * T_max;
     int32_t* aft = entries_after ? entries_after + (size_t)b * T_max : nullptr;
     int n = n0, n_out = 0, st = 0;
     int loaded = 0;                                  // tokens already in s_tok
     int ahead = tid < T ? x[tid] : 0;                // token loaded + tid
     for (int p0 = 0; p0 < T;) {                      // p0: a phrase starts here
-      // Positions below p0 + kParseLanes + kMaxM are looked at; the ring is filled as far as it goes, so
+      // Positions below p0 + LANES + kMaxM are looked at; the ring is filled as far as it goes, so
       // that a token has been on its way for a window before it is stored.  (A window moves p0 by 257 on
       // average where no phrase repeats in it: with nothing in reserve every other window would wait for
       // the last few tokens.  s_tok is only read ahead of a window's second barrier, so that the tokens
       // of the last window may be overwritten here.)
-      const int need = p0 + kParseLanes + kMaxM < T ? p0 + kParseLanes + kMaxM : T;
+      const int need = p0 + LANES + kMaxM < T ? p0 + LANES + kMaxM : T;
       const int room_end = p0 + kTokRing < T ? p0 + kTokRing : T;
       do {
-        const int cnt = room_end - loaded < kParseLanes ? room_end - loaded : kParseLanes;
+        const int cnt = room_end - loaded < LANES ? room_end - loaded : LANES;
         if (tid < cnt) {
           int c = ahead;
           if ((unsigned)c >= (unsigned)V) { st |= Z2Z_ST_BAD_TOKEN; c = 0; }     // not a base token
@@ -93,7 +91,7 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const i
         loaded += cnt;
         ahead = loaded + tid < T ? x[loaded + tid] : 0;
       } while (loaded < need);
-      parse_sync();
+      parse_sync<LANES>();
       // ---- longest match from every position of the window
       const int q = p0 + tid;
       const bool live = q < T;
@@ -118,11 +116,11 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const i
         if (to < 32) { visited |= v2; to = t2; }
       }
       if (lane < kMaxM) s_walk[warp][lane] = make_int2((int)visited, warp * 32 + to);
-      parse_sync();
+      parse_sync<LANES>();
       uint32_t mine = 0;
       int at = 0;                                    // entry into warp k, then the window's exit
 #pragma unroll
-      for (int k = 0; k < kParseWarps; ++k) {
+      for (int k = 0; k < WARPS; ++k) {
         if ((at >> 5) == k) {                        // (a walk that reached the end of the input stays where it is)
           const int2 wk = s_walk[k][at & 31];
           if (k == warp) mine = (uint32_t)wk.x;
@@ -134,18 +132,18 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const i
       const bool ins = on && miss && n < cap && slot >= 0;
       if (on && miss && n < cap && slot < 0) st |= Z2Z_ST_TABLE_FULL;
       if (ins) table.bid(slot, tid);
-      parse_sync();
+      parse_sync<LANES>();
       const bool own = ins && table.owns(slot, tid);
       const uint32_t v_on = __ballot_sync(0xffffffffu, on), v_ins = __ballot_sync(0xffffffffu, ins);
       const uint32_t v_lost = __ballot_sync(0xffffffffu, ins && !own);
       if (lane == 0) { s_votes.on[warp] = v_on; s_votes.ins[warp] = v_ins; s_votes.lost[warp] = v_lost; }
-      parse_sync();
-      const ParseVotes votes = s_votes;
+      parse_sync<LANES>();
+      const ParseVotes<WARPS> votes = s_votes;
       const int stop = parse_first_lost(votes.lost); // lanes below it are final
       const int room = cap - n;
       int made, emitted;
       const int new_before = parse_rank(votes.ins, warp, lane, made), on_before = parse_rank(votes.on, warp, lane, emitted);
-      if (stop < kParseLanes) { made = parse_count_below(votes.ins, stop); emitted = parse_count_below(votes.on, stop); }
+      if (stop < LANES) { made = parse_count_below(votes.ins, stop); emitted = parse_count_below(votes.on, stop); }
       if (own) {
         const int entry = tid < stop && new_before < room ? n + new_before : -1;
         table.settle(slot, (uint32_t)w, (uint32_t)c, entry);
@@ -166,7 +164,7 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_encode(CbView cb, const i
         if (n >= cap) st |= Z2Z_ST_CAP_FROZEN;
       }
       n_out += emitted;
-      p0 += stop < kParseLanes ? stop : at;
+      p0 += stop < LANES ? stop : at;
       // (the barrier at the head of the next window orders these writes before its lookups; s_votes
       // and s_walk are rewritten behind further barriers)
     }
@@ -218,19 +216,38 @@ cudaError_t launch_codebook_clear(const CbView& cb, void* zero, size_t zero_byte
   return cudaGetLastError();
 }
 
+// The wide window while at most two sequences share an SM: with 1024 sequences its blocks ran in two waves (cap
+// 1024, 200 tokens: 106 us, narrow 29; 49 with a warp or a thread per sequence).  The table goes to shared
+// memory when it fits for all sequences of an SM at once - in waves, 1024 sequences of cap 16384 took 173 us and
+// 263 for a second call, which brings the codebooks in, from global memory 43 and 13 - and when the call is long
+// enough to repay bringing it in: 16 tokens of one sequence, cap 16384, second call 19 against 10 us.
+ParseLaunch parse_launch(const CbView& cb, int T) {
+  static int n_sm = 0;
+  if (!n_sm) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    if (n_sm <= 0) n_sm = 148;
+  }
+  const int per_sm = (cb.B + n_sm - 1) / n_sm;
+  ParseLaunch p{per_sm > 2 ? kParseLanesMany : kParseLanes, 0};
+  const size_t bytes = parse_smem_bytes(cb.n_slots, cb.cap), fixed = 4096;      // fixed: the kernels' own arrays and the block's reserve
+  const bool fits = cb.cap <= kParseSmemMaxCap && (per_sm == 1 || per_sm * (bytes + fixed) <= (size_t)227 * 1024);
+  if (fits && (long long)T * 512 >= cb.n_slots) p.smem_bytes = bytes;
+  return p;
+}
+
 cudaError_t launch_lzw_encode(const CbView& cb, const int32_t* tokens, const int32_t* lens,
                               int T_max, int32_t* codes, int32_t* code_lens,
                               int32_t* entries_after, cudaStream_t s) {
-  // Shared memory holds codebooks of up to 16384 entries (224 KB); a larger table stays in global
-  // memory and every lookup of a window costs a round trip to L2 instead.
-  if (cb.cap <= kParseSmemMaxCap) {
-    const size_t smem = parse_smem_bytes(cb.n_slots, cb.cap);
-    cudaError_t e = cudaFuncSetAttribute(k_lzw_encode<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const ParseLaunch pl = parse_launch(cb, T_max);
+  auto kern = pl.lanes == kParseLanes ? (pl.smem_bytes ? k_lzw_encode<kParseLanes, true> : k_lzw_encode<kParseLanes, false>)
+                                      : (pl.smem_bytes ? k_lzw_encode<kParseLanesMany, true> : k_lzw_encode<kParseLanesMany, false>);
+  if (pl.smem_bytes) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem_bytes);
     if (e != cudaSuccess) return e;
-    k_lzw_encode<true><<<cb.B, kParseThreads, smem, s>>>(cb, tokens, lens, T_max, codes, code_lens, entries_after);
-  } else {
-    k_lzw_encode<false><<<cb.B, kParseThreads, 0, s>>>(cb, tokens, lens, T_max, codes, code_lens, entries_after);
   }
+  kern<<<cb.B, parse_threads(pl.lanes), pl.smem_bytes, s>>>(cb, tokens, lens, T_max, codes, code_lens, entries_after);
   return cudaGetLastError();
 }
 

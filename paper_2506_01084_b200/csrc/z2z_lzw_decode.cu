@@ -33,7 +33,7 @@ __device__ __forceinline__ int entry_len(const CbView& cb, int b, int code) {
 // n_valid[b] = number of codes accepted; replay of a sequence stops at the first code that names
 // no hypertoken (BAD_TOKEN; the state is the one after the last accepted code).
 //
-// One block per sequence; a window of kParseLanes codes at a time (z2z_lzw_dev.cuh).  Code i asks
+// One block per sequence; a window of LANES codes at a time (z2z_lzw_dev.cuh).  Code i asks
 // for the entry (code i - 1, first token of code i), which depends on no other code of the window
 // as long as both name entries from before it: the window ends before the first code that does not
 // (the entry it names is known once the codes before it are in), and before the first lane whose bid
@@ -42,15 +42,16 @@ __device__ __forceinline__ int entry_len(const CbView& cb, int b, int code) {
 // Bound by the latency of one window (the codes' first tokens and lengths from L2, one lookup, three
 // barriers); one thread that replayed code by code took 170 ns per code with the table in shared
 // memory and 260 with it in global memory.
-template <bool SMEM>
-__global__ void __launch_bounds__(kParseThreads) k_lzw_replay(CbView cb, const int32_t* __restrict__ codes,
+template <int LANES, bool SMEM>
+__global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_replay(CbView cb, const int32_t* __restrict__ codes,
                                                               const int32_t* __restrict__ code_lens, int Tc_max,
                                                               int32_t* __restrict__ n_valid) {
+  constexpr int WARPS = LANES / 32;
   extern __shared__ __align__(16) unsigned char s_parse[];
-  __shared__ int s_code[kParseLanes + 1], s_first[kParseLanes + 1];   // [0]: the code before the window
-  __shared__ uint8_t s_len[kParseLanes + 4];
-  __shared__ uint32_t s_known[kParseWarps];
-  __shared__ ParseVotes s_votes;
+  __shared__ int s_code[LANES + 1], s_first[LANES + 1];   // [0]: the code before the window
+  __shared__ uint8_t s_len[LANES + 4];
+  __shared__ uint32_t s_known[WARPS];
+  __shared__ ParseVotes<WARPS> s_votes;
   __shared__ int s_n1, s_bad0;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
@@ -72,11 +73,11 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_replay(CbView cb, const i
     s_bad0 = 0;
   }
   __syncthreads();
-  if (tid < kParseLanes) {
+  if (tid < LANES) {
     int n = n0, st = 0, base = 0;
     int z = tid < Tc ? zs[tid] : -1;
     while (base < Tc) {
-      const int z_ahead = base + kParseLanes + tid < Tc ? zs[base + kParseLanes + tid] : -1;
+      const int z_ahead = base + LANES + tid < Tc ? zs[base + LANES + tid] : -1;
       const int i = base + tid;
       // ---- first token and length of every code, as far as known
       bool known = i < Tc && z >= 0 && z < V + n;
@@ -88,10 +89,10 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_replay(CbView cb, const i
       s_code[tid + 1] = z; s_first[tid + 1] = f; s_len[tid + 1] = (uint8_t)l;
       const uint32_t v_known = __ballot_sync(0xffffffffu, known);
       if (lane == 0) s_known[warp] = v_known;
-      parse_sync();
-      int limit = kParseLanes;                       // first lane that is not known
+      parse_sync<LANES>();
+      int limit = LANES;                       // first lane that is not known
 #pragma unroll
-      for (int k = kParseWarps - 1; k >= 0; --k)
+      for (int k = WARPS - 1; k >= 0; --k)
         if (~s_known[k]) limit = k * 32 + __ffs((int)~s_known[k]) - 1;
       // the table in global memory keeps no keys to rebuild a row from later: a row is written at once,
       // which needs the previous code's row to be there
@@ -105,21 +106,21 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_replay(CbView cb, const i
         if (!found && slot < 0) st |= Z2Z_ST_TABLE_FULL;
         want = !found && slot >= 0;
       }
-      parse_sync();
+      parse_sync<LANES>();
       if (want) table.bid(slot, tid);
-      parse_sync();
+      parse_sync<LANES>();
       const bool own = want && table.owns(slot, tid);
       const uint32_t v_ins = __ballot_sync(0xffffffffu, want), v_lost = __ballot_sync(0xffffffffu, want && !own);
       if (lane == 0) { s_votes.ins[warp] = v_ins; s_votes.lost[warp] = v_lost; }
-      parse_sync();
-      const ParseVotes votes = s_votes;
+      parse_sync<LANES>();
+      const ParseVotes<WARPS> votes = s_votes;
       int stop = parse_first_lost(votes.lost);
       if (stop > limit) stop = limit;
       if (s_bad0) stop = 0;
       const int room = cap - n;
       int made;
       const int new_before = parse_rank(votes.ins, warp, lane, made);
-      if (stop < kParseLanes) made = parse_count_below(votes.ins, stop);
+      if (stop < LANES) made = parse_count_below(votes.ins, stop);
       if (own) {
         const int entry = tid < stop && new_before < room ? n + new_before : -1;
         table.settle(slot, (uint32_t)pz, (uint32_t)f, entry);
@@ -140,10 +141,10 @@ __global__ void __launch_bounds__(kParseThreads) k_lzw_replay(CbView cb, const i
       if (stop == 0) { st |= Z2Z_ST_BAD_TOKEN; break; }        // the window's first code names no hypertoken
       const int lz = s_code[stop], lf = s_first[stop], ll = s_len[stop];
       base += stop;
-      z = stop == kParseLanes ? z_ahead : (base + tid < Tc ? zs[base + tid] : -1);
-      parse_sync();                                  // everybody has read the window's last code
+      z = stop == LANES ? z_ahead : (base + tid < Tc ? zs[base + tid] : -1);
+      parse_sync<LANES>();                                  // everybody has read the window's last code
       if (tid == 0) { s_code[0] = lz; s_first[0] = lf; s_len[0] = (uint8_t)ll; }
-      parse_sync();
+      parse_sync<LANES>();
     }
     if (tid == 0) {
       s_n1 = n;
@@ -290,16 +291,15 @@ cudaError_t launch_lzw_decode(const CbView& cb, const int32_t* codes, const int3
                               int Tc_max, int replay, int32_t* n_valid, int32_t* tokens,
                               int32_t* token_lens, int T_out_max, cudaStream_t s) {
   if (replay) {
-    cudaError_t e;
-    if (cb.cap <= kParseSmemMaxCap) {                // as for prompt compression
-      const size_t smem = parse_smem_bytes(cb.n_slots, cb.cap);
-      e = cudaFuncSetAttribute(k_lzw_replay<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const ParseLaunch pl = parse_launch(cb, Tc_max);             // as for prompt compression
+    auto kern = pl.lanes == kParseLanes ? (pl.smem_bytes ? k_lzw_replay<kParseLanes, true> : k_lzw_replay<kParseLanes, false>)
+                                        : (pl.smem_bytes ? k_lzw_replay<kParseLanesMany, true> : k_lzw_replay<kParseLanesMany, false>);
+    if (pl.smem_bytes) {
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem_bytes);
       if (e != cudaSuccess) return e;
-      k_lzw_replay<true><<<cb.B, kParseThreads, smem, s>>>(cb, codes, code_lens, Tc_max, n_valid);
-    } else {
-      k_lzw_replay<false><<<cb.B, kParseThreads, 0, s>>>(cb, codes, code_lens, Tc_max, n_valid);
     }
-    e = cudaGetLastError();
+    kern<<<cb.B, parse_threads(pl.lanes), pl.smem_bytes, s>>>(cb, codes, code_lens, Tc_max, n_valid);
+    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   dim3 grid(Tc_max / kExpandChunk + 1, cb.B);

@@ -151,7 +151,7 @@ __device__ __forceinline__ int warp_lzw_step(const CbView& cb, int b, int z) {
 // Windowed parsing, shared by prompt compression and by replay of a code stream.
 //
 // Both are defined as a chain of one dictionary lookup per token or code, but the dictionary
-// changes little while 256 of them are looked at: kParseLanes threads look up kParseLanes starting
+// changes little while a window of them is looked at: LANES threads look up LANES starting
 // points at once in the dictionary as it was before the window, the results that lie on the chain
 // are picked out, and only the new phrases of the chain are inserted.  A lookup is invalid only if
 // an earlier phrase of the same window inserted exactly the key that it missed; such a lane shares
@@ -169,16 +169,18 @@ __device__ __forceinline__ int warp_lzw_step(const CbView& cb, int b, int z) {
 // ---------------------------------------------------------------------------------------------
 // A window of 256 costs little more than one of 128 (two warps per scheduler hide each other's latencies)
 // and moves 216 tokens on in long repetitive text where 128 moved 122; 512 would gain there and lose
-// where phrases repeat sooner (vocabulary 32064: 93 tokens either way).
+// where phrases repeat sooner (vocabulary 32064: 93 tokens either way).  Where more than two sequences share an
+// SM, its warps have other sequences to turn to and narrow windows leave room for all blocks at once.
 constexpr int kParseLanes = 256;          // starting points looked up at once
-constexpr int kParseWarps = kParseLanes / 32;
-constexpr int kParseThreads = 512;        // the other warps only help to fill and to write back
+constexpr int kParseLanesMany = 64;       // ... with many sequences
 constexpr int kParseSmemMaxCap = 16384;
+constexpr int parse_threads(int lanes) { return 2 * lanes; }      // the other warps only help to fill and to write back
 
 inline size_t parse_smem_bytes(int n_slots, int cap) { return (size_t)n_slots * 4 + (size_t)(cap + (cap & 1)) * 6; }
 
-// Barrier among the kParseLanes parsing threads only.
-__device__ __forceinline__ void parse_sync() { asm volatile("bar.sync 1, %0;" ::"n"(kParseLanes) : "memory"); }
+// Barrier among the parsing threads only.
+template <int LANES>
+__device__ __forceinline__ void parse_sync() { asm volatile("bar.sync 1, %0;" ::"n"(LANES) : "memory"); }
 
 template <bool SMEM>
 struct ParseTable {
@@ -291,23 +293,30 @@ struct ParseTable {
   }
 };
 
+// How a call of B sequences of at most T tokens or codes is launched (z2z_lzw.cu); smem_bytes 0: SMEM false.
+struct ParseLaunch { int lanes; size_t smem_bytes; };
+ParseLaunch parse_launch(const CbView& cb, int T);
+
 // What the parsing warps tell each other inside a window: per warp a mask of lanes on the chain, of
 // those that want a new entry, and of those whose bid lost.
-struct ParseVotes { uint32_t on[kParseWarps], ins[kParseWarps], lost[kParseWarps]; };
+template <int WARPS>
+struct ParseVotes { uint32_t on[WARPS], ins[WARPS], lost[WARPS]; };
 
-// First losing lane of the window (kParseLanes if none).
-__device__ __forceinline__ int parse_first_lost(const uint32_t (&lost)[kParseWarps]) {
-  int f = kParseLanes;
+// First losing lane of the window (all lanes if none).
+template <int WARPS>
+__device__ __forceinline__ int parse_first_lost(const uint32_t (&lost)[WARPS]) {
+  int f = 32 * WARPS;
 #pragma unroll
-  for (int k = kParseWarps - 1; k >= 0; --k)
+  for (int k = WARPS - 1; k >= 0; --k)
     if (lost[k]) f = k * 32 + __ffs((int)lost[k]) - 1;
   return f;
 }
 // Bits of m below lane `at` of the window.
-__device__ __forceinline__ int parse_count_below(const uint32_t (&m)[kParseWarps], int at) {
+template <int WARPS>
+__device__ __forceinline__ int parse_count_below(const uint32_t (&m)[WARPS], int at) {
   int c = 0;
 #pragma unroll
-  for (int k = 0; k < kParseWarps; ++k) {
+  for (int k = 0; k < WARPS; ++k) {
     const int left = at - k * 32;
     const uint32_t keep = left >= 32 ? 0xffffffffu : (left <= 0 ? 0u : (1u << left) - 1u);
     c += __popc(m[k] & keep);
@@ -315,11 +324,12 @@ __device__ __forceinline__ int parse_count_below(const uint32_t (&m)[kParseWarps
   return c;
 }
 // The same for this thread's own lane, and the number of all bits.
-__device__ __forceinline__ int parse_rank(const uint32_t (&m)[kParseWarps], int warp, int lane, int& total) {
+template <int WARPS>
+__device__ __forceinline__ int parse_rank(const uint32_t (&m)[WARPS], int warp, int lane, int& total) {
   int below = 0;
   total = 0;
 #pragma unroll
-  for (int k = 0; k < kParseWarps; ++k) {
+  for (int k = 0; k < WARPS; ++k) {
     if (k == warp) below = total + __popc(m[k] & ((1u << lane) - 1u));
     total += __popc(m[k]);
   }
