@@ -166,7 +166,7 @@ int logits_call(z2z_codebook* cb, z2z::LogitsArgs a, cudaStream_t s, z2z::Logits
     } else if (decode) {
       Z2Z_CUDA(z2z::run_logits_decode(cb->view, c, words + 2, words, info, &cb->prof, s), "logits (decode batch)");
     } else if (tc) {
-      Z2Z_CUDA(z2z::run_logits_stream(cb->view, c, words + 1, words, info, &cb->prof, s), "logits (batch)");
+      Z2Z_CUDA(z2z::run_logits_stream(cb->view, c, words, info, &cb->prof, s), "logits (batch)");
     } else {
       Z2Z_CUDA(z2z::run_logits_simt(cb->view, c, info, &cb->prof, s), "logits");
     }

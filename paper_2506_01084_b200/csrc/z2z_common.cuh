@@ -55,11 +55,6 @@ __host__ __device__ inline uint32_t hash_pair(uint32_t prefix, uint32_t token) {
   return hash_join(prefix, hash_token_part(token));
 }
 
-// CTA that owns unit u when U units are dealt to G CTAs as [floor(c U / G), floor((c+1) U / G)).
-__host__ __device__ inline long long owner_of(long long u, long long U, long long G) {
-  return ((u + 1) * G - 1) / U;
-}
-
 // ---------------------------------------------------------------------------------------------
 // Workspace plan: byte offsets of every region inside the caller's workspace.
 // ---------------------------------------------------------------------------------------------
@@ -74,7 +69,7 @@ struct WsPlan {
   size_t off_X, off_A, off_QKV, off_H;            // fp32 encoder activations
   size_t off_Ahl, off_Hhl;                        // bf16 hi/lo activations (tensor-core path)
   size_t off_g1_X, off_g1_QKV, off_g1_Ahl, off_g1_Hhl;   // second encoder of the decode step
-  size_t off_words;                               // device words: [0] kernel error, [1] logits tiles
+  size_t off_words;                               // device words: [0] kernel error, [2], [3] decode logits, [4] decode update
   size_t off_part, part_bytes;                    // fp32 GEMM results of the hyper-encoder passes
   size_t off_lpart, lpart_bytes;                  // logits partial reductions
   size_t off_plan, plan_bytes;                    // per-row-tile plan of the prompt-scoring logits kernel

@@ -912,7 +912,7 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   // one GEMM: activations (hi/lo of packed row r in operand rows 2r, 2r + 1; K columns) x weight
   // [J, K], added into Y[group][Rt][J]
   const bool paired = R > kStreamSingleRows;
-  const int ksb = paired ? stream_pair_ksb(R) : stream_gemm_ksb(R);
+  const int ksb = paired ? 1 : stream_gemm_ksb(R);
   StreamGemmMaps maps;
   StreamPairMaps pair_maps;
   auto gemm = [&](const MPtr2& act, int K, int widx, int J) -> cudaError_t {
@@ -929,7 +929,7 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
     };
     ProfScope ps(prof, kProfEncGemm, 1, s);
     if (paired) {
-      if (!make(pair_maps, [&](int g) { return stream_pair_act_maps(pair_maps.a[g], act.p[g], Rt, K, R); })) return cudaErrorInvalidValue;
+      if (!make(pair_maps, [&](int g) { return stream_pair_act_maps(pair_maps.a[g], act.p[g], Rt, K); })) return cudaErrorInvalidValue;
       return launch_stream_pair(fill(StreamPairParams{}), pair_maps, n_sm, s);
     }
     if (!make(maps, [&](int g) { return stream_gemm_act_maps(maps.a[g], act.p[g], Rt, K, R); })) return cudaErrorInvalidValue;

@@ -41,13 +41,14 @@ cudaError_t launch_lzw_step(const CbView& cb, const int32_t* new_codes, const ui
                             int none_sits_out, int32_t* new_entry, cudaStream_t s);
 
 // ---- z2z_encoder.cu --------------------------------------------------------------------------
-// Work list of one encoder pass: up to `chunk` entries, entry e -> (sequence, entry number).
+// Work list of one encoder pass: up to `list` entries of together at most chunk * M rows, entry e ->
+// (sequence, entry number).
 struct EntryList {
-  int32_t* seq;       // [chunk]  sequence of entry e, -1 = unused slot
-  int32_t* idx;       // [chunk]  entry number within the sequence
-  int32_t* len;       // [chunk]  base tokens of the entry, 0 for an unused slot
-  int32_t* tok;       // [chunk * M]  base token of each row of the entry, -1 for padding rows
-  int32_t* row_off;   // [chunk + 1]  tensor-core passes: first packed row of each entry; the row total sits
+  int32_t* seq;       // [list]  sequence of entry e, -1 = unused slot
+  int32_t* idx;       // [list]  entry number within the sequence
+  int32_t* len;       // [list]  base tokens of the entry, 0 for an unused slot
+  int32_t* tok;       // [list * M]  base token of each row of the entry, -1 for padding rows
+  int32_t* row_off;   // [list + 1]  tensor-core passes: first packed row of each entry; the row total sits
                       //              behind the last entry slot of the pass
   int32_t* row_src;   // [chunk * M]  tensor-core passes: packed row -> entry * M + position
   int32_t* row_tok;   // [chunk * M]  tensor-core passes: base token of each packed row
@@ -145,8 +146,8 @@ struct LogitsPartInfo { int stride, count; };
 cudaError_t run_logits_simt(const CbView& cb, const LogitsArgs& a, LogitsPartInfo* info, Prof* prof,
                             cudaStream_t s);
 // Batches of 33 .. 128 rows of different sequences (bf16, d % 64 == 0).
-cudaError_t run_logits_stream(const CbView& cb, const LogitsArgs& a, int* vt_word, int* err_word,
-                              LogitsPartInfo* info, Prof* prof, cudaStream_t s);
+cudaError_t run_logits_stream(const CbView& cb, const LogitsArgs& a, int* err_word, LogitsPartInfo* info, Prof* prof,
+                              cudaStream_t s);
 
 // ---- z2z_prefill_logits.cu -------------------------------------------------------------------
 // Many hidden rows, or positions of few sequences (bf16, d % 64 == 0).  `plan` is scratch for 3 int32 per 256-row tile.

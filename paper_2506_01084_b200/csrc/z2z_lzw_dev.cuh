@@ -42,20 +42,6 @@ __device__ __forceinline__ Probe warp_probe(const unsigned long long* __restrict
   return r;
 }
 
-// Write entry k = phrase(w) ++ c.  Lanes 0..M-1 each write one constituent.
-__device__ __forceinline__ void warp_write_entry(const CbView& cb, int b, int k, int w, int wlen,
-                                                 int c) {
-  const int lane = threadIdx.x & 31;
-  int32_t* dst = cb.cons + ((size_t)b * cb.cap + k) * cb.M;
-  if (lane < cb.M) {
-    int v = -1;
-    if (lane < wlen) v = (w < cb.V) ? w : cb.cons[((size_t)b * cb.cap + (w - cb.V)) * cb.M + lane];
-    else if (lane == wlen) v = c;
-    dst[lane] = v;
-  }
-  if (lane == 0) cb.len[(size_t)b * cb.cap + k] = (uint8_t)(wlen + 1);
-}
-
 // The part of a sequence's state that the update needs and that does not depend on the new code;
 // a caller that still has to compute the code can load it ahead.  ptok: base token `lane` of the
 // previous phrase (-1 beyond its length), so that writing a new entry needs no further load.

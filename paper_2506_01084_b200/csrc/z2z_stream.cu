@@ -44,16 +44,11 @@ __host__ __device__ constexpr int tmem_cols(int nt) {
   return 2 * nt <= 32 ? 32 : (2 * nt <= 64 ? 64 : (2 * nt <= 128 ? 128 : (2 * nt <= 256 ? 256 : 512)));
 }
 
+// A job of the logits kernel: weight rows [wrow, wrow + nrows) of tensor wmap (0: W_U, 1: U_h).
 struct Job {
-  int amap, wmap;        // tensor map indices
-  int arow, wrow;        // first row in A / W tensors
-  int kb0, kb1;          // k-step range
-  long long slot;        // GEMM: partial slot
-  int col0, nvalid, owner, k0;   // logits: first column id, valid rows, owning sequence, first entry
-  int rt;                // hidden-row tile
-  int nrows;             // weight rows in this job (the MMA's N), multiple of 16
-  int wbox_min;          // smallest TMA box of W in rows; boxes are powers of two times this, up
-  int wbox_classes;      // to wbox_min << (wbox_classes - 1); tensor map = wmap * classes + class
+  int wmap, wrow;
+  int col0, nvalid, owner, k0;           // first column id, valid rows, owning sequence, first entry
+  int nrows;                             // the MMA's N, a multiple of kLogitGran
 };
 
 // ---- logits schedule ----------------------------------------------------------------------------
@@ -64,22 +59,16 @@ struct LogitSched {
   const StreamLogitsParams& p;
   const int* pref;       // shared: prefix of per-sequence granule counts, [B + 1]
   long long u, u1;
-  int n_static, vt, ksteps;
-  __device__ LogitSched(const StreamLogitsParams& pp, const int* s_pref, int vt_, int NT) : p(pp), pref(s_pref) {
+  int n_static;
+  __device__ LogitSched(const StreamLogitsParams& pp, const int* s_pref, int vt) : p(pp), pref(s_pref) {
     n_static = (p.cb.V + kLogitGran - 1) / kLogitGran;
-    vt = vt_;
-    ksteps = p.ksteps;
-    const long long U = (long long)p.row_tiles * vt, G = gridDim.x, c = blockIdx.x;
+    const long long U = vt, G = gridDim.x, c = blockIdx.x;
     u = c * U / G;
     u1 = (c + 1) * U / G;
-    (void)NT;
   }
-  __device__ bool next(Job& j, int NT) {
+  __device__ bool next(Job& j) {
     if (u >= u1) return false;
-    j.rt = (int)(u / vt);
-    const int v = (int)(u - (long long)j.rt * vt);
-    j.amap = 0; j.arow = j.rt * 128; j.kb0 = 0; j.kb1 = ksteps; j.slot = 0;
-    j.wbox_min = kLogitGran; j.wbox_classes = kLogitBoxClasses;
+    const int v = (int)u;
     int remaining, total_rows, g0;
     if (v < n_static) {
       g0 = v; remaining = n_static - v; total_rows = p.cb.V;
@@ -92,7 +81,7 @@ struct LogitSched {
       j.owner = lo; j.k0 = g0 * kLogitGran;
       j.wmap = 1; j.wrow = lo * p.cb.cap + j.k0; j.col0 = p.cb.V + j.k0;
     }
-    int ng = NT / kLogitGran;
+    int ng = kLogitNT / kLogitGran;
     if (remaining < ng) ng = remaining;
     if (u1 - u < ng) ng = (int)(u1 - u);
     j.nrows = ng * kLogitGran;
@@ -102,91 +91,57 @@ struct LogitSched {
   }
 };
 
-// ---- roles shared by both kernels -----------------------------------------------------------------
-template <int NT, int KSB, int STAGES, class Sched>
-__device__ __forceinline__ void producer_role(Sched& sched, Ctrl* ctrl, uint32_t stage_base,
-                                              int a_parts, int a_box_rows, int a_part_row,
-                                              const CUtensorMap* const* amaps,
-                                              const CUtensorMap* const* wmaps) {
-  const uint32_t a_part_bytes = (uint32_t)KSB * a_box_rows * 128;
-  const uint32_t stage_bytes = a_parts * a_part_bytes + (uint32_t)KSB * NT * 128;   // smem stride of a stage
+// ---- producer and MMA role of the logits kernel -----------------------------------------------------
+template <int STAGES>
+__device__ __forceinline__ void logits_producer(LogitSched& sched, int ksteps, Ctrl* ctrl, uint32_t stage_base, int a_box_rows,
+                                                const LogitMaps& tm) {
+  const uint32_t a_bytes = (uint32_t)a_box_rows * 128;
+  const uint32_t stage_bytes = a_bytes + kLogitNT * 128;           // smem stride of a stage
   const uint64_t pol_w = policy_evict_first(), pol_a = policy_evict_last();
   int stage = 0; uint32_t phase = 0;
-  // The weight tiles depend on no earlier kernel, the activation tiles do.  During the first
-  // pass over the ring only the weight boxes are issued and the activation boxes are noted; once
-  // the ring is full (or the work ends) the producer waits for the preceding kernel and issues
-  // them.  With an ordinary launch the wait returns at once.
-  struct Deferred { uint32_t dst, bar; int map, row, kb; };
-  Deferred def[kMaxStages * 2];
-  int n_def = 0, issued = 0;
-  bool deps = false;
-  auto need_deps = [&]() {
-    if (deps) return;
-    pdl_wait();
-    for (int i = 0; i < n_def; ++i) tma_load_3d(def[i].dst, amaps[def[i].map], 0, def[i].row, def[i].kb, def[i].bar, pol_a);
-    deps = true;
-  };
   Job j;
-  while (sched.next(j, NT)) {
-    for (int ks = j.kb0; ks < j.kb1; ++ks) {
-      if (issued == STAGES) need_deps();
+  while (sched.next(j)) {
+    for (int ks = 0; ks < ksteps; ++ks) {
       if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) return;
       const uint32_t full = smem_u32(&ctrl->full[stage]);
-      mbar_expect_tx(full, a_parts * a_part_bytes + (uint32_t)KSB * j.nrows * 128);
+      mbar_expect_tx(full, a_bytes + (uint32_t)j.nrows * 128);
       const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
-      // one box per operand part: KSB k-blocks of the rows, laid out k-block after k-block
-      for (int part = 0; part < a_parts; ++part) {
-        const uint32_t dst = sb + part * a_part_bytes;
-        const int row = j.arow + part * a_part_row;
-        if (deps) tma_load_3d(dst, amaps[j.amap], 0, row, ks * KSB, full, pol_a);
-        else { def[n_def].dst = dst; def[n_def].bar = full; def[n_def].map = j.amap; def[n_def].row = row; def[n_def].kb = ks * KSB; ++n_def; }
-      }
+      tma_load_3d(sb, &tm.h, 0, 0, ks, full, pol_a);
       // the W rows of the job go out as few boxes as possible: largest power-of-two box first
-      // (several boxes only with KSB == 1: a box's k-blocks lie one box height apart)
       for (int r0 = 0; r0 < j.nrows;) {
-        int cls = j.wbox_classes - 1;
-        while (cls > 0 && (j.wbox_min << cls) > j.nrows - r0) --cls;
-        tma_load_3d(sb + a_parts * a_part_bytes + r0 * 128, wmaps[j.wmap * j.wbox_classes + cls], 0, j.wrow + r0,
-                    ks * KSB, full, pol_w);
-        r0 += j.wbox_min << cls;
+        int cls = kLogitBoxClasses - 1;
+        while (cls > 0 && (kLogitGran << cls) > j.nrows - r0) --cls;
+        tma_load_3d(sb + a_bytes + r0 * 128, &tm.w[j.wmap * kLogitBoxClasses + cls], 0, j.wrow + r0, ks, full, pol_w);
+        r0 += kLogitGran << cls;
       }
-      ++issued;
       if (++stage == STAGES) { stage = 0; phase ^= 1u; }
     }
   }
-  need_deps();
 }
 
-template <int NT, int KSB, int STAGES, class Sched>
-__device__ __forceinline__ void mma_role(Sched& sched, Ctrl* ctrl, uint32_t stage_base, int a_parts,
-                                         int a_box_rows, uint32_t tmem_base) {
-  const uint32_t a_part_bytes = (uint32_t)KSB * a_box_rows * 128;
-  const uint32_t stage_bytes = a_parts * a_part_bytes + (uint32_t)KSB * NT * 128;
+template <int STAGES>
+__device__ __forceinline__ void logits_mma(LogitSched& sched, int ksteps, Ctrl* ctrl, uint32_t stage_base, int a_box_rows,
+                                           uint32_t tmem_base) {
+  const uint32_t a_bytes = (uint32_t)a_box_rows * 128;
+  const uint32_t stage_bytes = a_bytes + kLogitNT * 128;
   int stage = 0; uint32_t phase = 0;
   uint32_t job_i = 0;
   Job j;
-  while (sched.next(j, NT)) {
+  while (sched.next(j)) {
     const uint32_t idesc = idesc_bf16_f32(128, j.nrows);
     const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
     if (!mbar_wait(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) return;
     tc_fence_after();
-    const uint32_t d = tmem_base + buf * NT;
+    const uint32_t d = tmem_base + buf * kLogitNT;
     uint32_t acc = 0;
-    for (int ks = j.kb0; ks < j.kb1; ++ks) {
+    for (int ks = 0; ks < ksteps; ++ks) {
       if (!mbar_wait(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) return;
       tc_fence_after();
       const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
 #pragma unroll
-      for (int i = 0; i < KSB; ++i) {
-        const uint32_t wb = sb + a_parts * a_part_bytes + i * NT * 128;
-        for (int part = 0; part < a_parts; ++part) {
-          const uint32_t ab = sb + part * a_part_bytes + i * a_box_rows * 128;
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            umma_bf16(d, smem_desc_sw128(ab + k * 32), smem_desc_sw128(wb + k * 32), idesc, acc);
-            acc = 1;
-          }
-        }
+      for (int k = 0; k < 4; ++k) {
+        umma_bf16(d, smem_desc_sw128(sb + k * 32), smem_desc_sw128(sb + a_bytes + k * 32), idesc, acc);
+        acc = 1;
       }
       umma_commit(smem_u32(&ctrl->empty[stage]));          // frees the stage when the MMAs are done
       if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -400,9 +355,10 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
 // =================================================================================================
 // Logits kernel: fused reductions
 // =================================================================================================
-template <int NT, int KSB, int STAGES>
+template <int STAGES>
 __global__ void __launch_bounds__(kThreads, 1)
 k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm) {
+  constexpr int NT = kLogitNT;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   Ctrl* ctrl = reinterpret_cast<Ctrl*>(sm);
@@ -418,70 +374,45 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
     s_pref[0] = 0;
     for (int b = 0; b < p.cb.B; ++b) s_pref[b + 1] += s_pref[b];
     ctrl->vt = (p.cb.V + kLogitGran - 1) / kLogitGran + s_pref[p.cb.B];
-    if (blockIdx.x == 0) *p.vt_out = ctrl->vt;
   }
   if (warp == 2) { tmem_alloc(smem_u32(&ctrl->tmem_base), tmem_cols(NT)); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = ctrl->tmem_base;
-  const int vt = ctrl->vt;
+  LogitSched sched(p, s_pref, ctrl->vt);
 
   if (warp == 0) {
-    if (lane == 0) {
-      const CUtensorMap* amaps[1] = {&tm.h};
-      const CUtensorMap* wmaps[2 * kLogitBoxClasses];
-      for (int i = 0; i < 2 * kLogitBoxClasses; ++i) wmaps[i] = &tm.w[i];
-      LogitSched sched(p, s_pref, vt, NT);
-      producer_role<NT, KSB, STAGES>(sched, ctrl, stage_base, 1, p.a_box_rows, 0, amaps, wmaps);
-    }
+    if (lane == 0) logits_producer<STAGES>(sched, p.ksteps, ctrl, stage_base, p.a_box_rows, tm);
   } else if (warp == 1) {
-    if (lane == 0) {
-      LogitSched sched(p, s_pref, vt, NT);
-      mma_role<NT, KSB, STAGES>(sched, ctrl, stage_base, 1, p.a_box_rows, tmem_base);
-    }
+    if (lane == 0) logits_mma<STAGES>(sched, p.ksteps, ctrl, stage_base, p.a_box_rows, tmem_base);
   } else {
     const int q = warp & 3;
     const LogitsArgs& a = p.la;
-    LogitSched sched(p, s_pref, vt, NT);
-    const long long U = (long long)p.row_tiles * vt, G = gridDim.x;
     const uint32_t k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32);
     const uint32_t c2 = (uint32_t)a.step, c3 = (uint32_t)(a.step >> 32);
     const size_t ldbg = (size_t)p.cb.V + p.cb.cap;
     RowRed red; red.init();
-    int cur_rt = -1, r = -1, my_seq = -1, my_nvis = 0, my_tgt = -1;
+    const int r = q * 32 + lane;
+    int my_seq = -1, my_nvis = 0, my_tgt = -1;
+    if (r < a.N) {
+      my_seq = a.row_seq ? a.row_seq[r] : r;
+      if (my_seq < 0 || my_seq >= p.cb.B) my_seq = -1;
+      if (my_seq >= 0) {
+        my_nvis = p.cb.n[my_seq];
+        if (a.row_nvis) { const int x = a.row_nvis[r]; my_nvis = x < my_nvis ? (x < 0 ? 0 : x) : my_nvis; }
+      }
+      if (a.targets) my_tgt = a.targets[r];
+    }
     uint32_t job_i = 0;
     Job j;
-    auto flush = [&]() {
-      if (cur_rt >= 0 && r < a.N) {
-        const long long first = owner_of((long long)cur_rt * vt, U, G);
-        LogitPartial* lp = reinterpret_cast<LogitPartial*>(a.lpart) + (size_t)r * p.part_stride + (blockIdx.x - first);
-        lp->m = red.m; lp->s = red.s; lp->idx = red.idx; lp->gm = red.gm; lp->gidx = red.gidx;
-      }
-    };
-    while (sched.next(j, NT)) {
-      if (j.rt != cur_rt) {
-        flush();
-        cur_rt = j.rt; red.init();
-        r = cur_rt * 128 + q * 32 + lane;
-        my_seq = -1; my_nvis = 0; my_tgt = -1;
-        if (r < a.N) {
-          my_seq = a.row_seq ? a.row_seq[r] : r;
-          if (my_seq < 0 || my_seq >= p.cb.B) my_seq = -1;
-          if (my_seq >= 0) {
-            my_nvis = p.cb.n[my_seq];
-            if (a.row_nvis) { const int x = a.row_nvis[r]; my_nvis = x < my_nvis ? (x < 0 ? 0 : x) : my_nvis; }
-          }
-          if (a.targets) my_tgt = a.targets[r];
-        }
-      }
+    while (sched.next(j)) {
       const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
       if (!mbar_wait(smem_u32(&ctrl->acc_full[buf]), aph, &ctrl->abort)) break;
       tc_fence_after();
       int limit = 0;
       if (my_seq >= 0) limit = j.owner < 0 ? j.nvalid : (my_seq == j.owner ? min(j.nvalid, my_nvis - j.k0) : 0);
-      const int rows_here = a.N - cur_rt * 128;
-      if (q * 32 < rows_here && __any_sync(0xffffffffu, limit > 0)) {
+      if (__any_sync(0xffffffffu, limit > 0)) {
 #pragma unroll 1
         for (int c0 = 0; c0 < j.nrows; c0 += 32) {
           if (!__any_sync(0xffffffffu, limit > c0)) break;
@@ -505,7 +436,10 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
       if (lane == 0) mbar_arrive(smem_u32(&ctrl->acc_empty[buf]));
       ++job_i;
     }
-    flush();
+    if (r < a.N) {
+      LogitPartial* lp = reinterpret_cast<LogitPartial*>(a.lpart) + (size_t)r * p.part_stride + blockIdx.x;
+      lp->m = red.m; lp->s = red.s; lp->idx = red.idx; lp->gm = red.gm; lp->gidx = red.gidx;
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -513,20 +447,15 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
   if (warp == 2) tmem_dealloc(tmem_base, tmem_cols(NT));
 }
 
-// One warp per row: merge the partial reductions of the CTAs that touched the row's tile.
+// One warp per row: merge the partial reductions of the G CTAs.
 __global__ void __launch_bounds__(128) k_stream_logits_merge(StreamLogitsParams p, int G) {
   const LogitsArgs& a = p.la;
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= a.N) return;
-  const long long vt = *p.vt_out, U = (long long)p.row_tiles * vt;
-  const int rt = r >> 7;
-  const long long first = owner_of((long long)rt * vt, U, G), last = owner_of((long long)(rt + 1) * vt - 1, U, G);
   const LogitPartial* lp = reinterpret_cast<const LogitPartial*>(a.lpart) + (size_t)r * p.part_stride;
   RowRed red; red.init();
-  for (int g = lane; g <= (int)(last - first); g += 32) {
-    red.merge(load_partial(lp + g));
-  }
+  for (int g = lane; g < G; g += 32) red.merge(load_partial(lp + g));
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     RowRed o;
@@ -637,13 +566,6 @@ bool make_tmap_bf16_kblocks(CUtensorMap* m, const void* base, long long rows, lo
   g_tmap_cache.emplace(key, *m);
   return true;
 }
-template <int NT, int KSB>
-static int pick_stages(int a_parts, int a_box_rows, int extra) {
-  const int stage = a_parts * KSB * a_box_rows * 128 + KSB * NT * 128;
-  int s = (227 * 1024 - 2048 - extra - kTailPad) / stage;
-  return s > kMaxStages ? kMaxStages : s;
-}
-
 // Capacity of the activation box (hi and lo rows of R packed rows) and the step of its heights: eight
 // heights cover it.
 static int gemm_box_step(int R) { return 2 * R <= 128 ? 16 : 32; }
@@ -698,19 +620,19 @@ cudaError_t launch_stream_gemm(StreamGemmParams p, const StreamGemmMaps& maps, i
   return stream_gemm_ksb(p.R) == 2 ? launch_stream_gemm_k<2>(p, maps, grid, s) : launch_stream_gemm_k<1>(p, maps, grid, s);
 }
 
-template <int NT, int KSB, int STAGES>
-static cudaError_t launch_logits_t(const StreamLogitsParams& p, const LogitMaps* maps, int grid, cudaStream_t s) {
-  const size_t stage = (size_t)KSB * p.a_box_rows * 128 + (size_t)KSB * NT * 128;
-  const size_t smem = 1024 + 1024 + 5120 + STAGES * stage + kTailPad;
-  auto kern = k_stream_logits<NT, KSB, STAGES>;
+template <int STAGES>
+static cudaError_t launch_logits_t(const StreamLogitsParams& p, const LogitMaps& maps, int grid, cudaStream_t s) {
+  const size_t smem = 1024 + 1024 + 5120 + STAGES * ((size_t)p.a_box_rows + kLogitNT) * 128 + kTailPad;
+  auto kern = k_stream_logits<STAGES>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<grid, kThreads, smem, s>>>(p, *maps);
+  kern<<<grid, kThreads, smem, s>>>(p, maps);
   return cudaGetLastError();
 }
 
-cudaError_t run_logits_stream(const CbView& cb, const LogitsArgs& a, int* vt_word, int* err_word,
-                              LogitsPartInfo* info, Prof* prof, cudaStream_t s) {
+cudaError_t run_logits_stream(const CbView& cb, const LogitsArgs& a, int* err_word, LogitsPartInfo* info, Prof* prof,
+                              cudaStream_t s) {
+  if (a.N > 128) return cudaErrorInvalidValue;
   static int n_sm = 0;
   if (!n_sm) {
     int dev = 0;
@@ -720,38 +642,26 @@ cudaError_t run_logits_stream(const CbView& cb, const LogitsArgs& a, int* vt_wor
   }
   StreamLogitsParams p{};
   p.cb = cb; p.la = a;
-  p.ksteps = (a.d / 64 + kLogitKSB - 1) / kLogitKSB;
-  p.row_tiles = (a.N + 127) / 128;
-  p.a_box_rows = a.N >= 128 ? 128 : (a.N + 7) / 8 * 8;
-  p.part_stride = (n_sm + p.row_tiles - 1) / p.row_tiles + 2;
-  p.vt_out = vt_word; p.err = err_word;
-  if ((size_t)a.N * p.part_stride * sizeof(LogitPartial) > a.lpart_bytes) return cudaErrorMemoryAllocation;
+  p.ksteps = a.d / 64;
+  p.a_box_rows = (a.N + 7) / 8 * 8;
+  p.err = err_word;
   LogitMaps maps;
-  if (!make_tmap_bf16_kblocks(&maps.h, a.hidden, a.N, a.d, p.a_box_rows, kLogitKSB)) return cudaErrorInvalidValue;
+  if (!make_tmap_bf16_kblocks(&maps.h, a.hidden, a.N, a.d, p.a_box_rows, 1)) return cudaErrorInvalidValue;
   for (int c = 0; c < kLogitBoxClasses; ++c) {
-    if (!make_tmap_bf16_kblocks(&maps.w[c], a.WU, cb.V, a.d, kLogitGran << c, kLogitKSB)) return cudaErrorInvalidValue;
+    if (!make_tmap_bf16_kblocks(&maps.w[c], a.WU, cb.V, a.d, kLogitGran << c, 1)) return cudaErrorInvalidValue;
     if (cb.cap > 0) {
-      if (!make_tmap_bf16_kblocks(&maps.w[kLogitBoxClasses + c], a.Uh, (long long)cb.B * cb.cap, a.d, kLogitGran << c, kLogitKSB))
+      if (!make_tmap_bf16_kblocks(&maps.w[kLogitBoxClasses + c], a.Uh, (long long)cb.B * cb.cap, a.d, kLogitGran << c, 1))
         return cudaErrorInvalidValue;
     } else {
       maps.w[kLogitBoxClasses + c] = maps.w[c];
     }
   }
-  // every CTA must own at least one unit: the static tiles alone give a lower bound on the units
-  long long units_lb = (long long)p.row_tiles * ((cb.V + kLogitGran - 1) / kLogitGran);
-  const int grid = units_lb < n_sm ? (int)units_lb : n_sm;
-  p.part_stride = (grid + p.row_tiles - 1) / p.row_tiles + 2;
-  if (info) {
-    if (p.row_tiles != 1) return cudaErrorInvalidValue;
-    info->stride = p.part_stride; info->count = grid;
-  }
-  return launch_stream_logits(p, &maps, grid, info == nullptr, prof, s);
-}
-
-cudaError_t launch_stream_logits(const StreamLogitsParams& p, const LogitMaps* maps, int grid, bool merge,
-                                 Prof* prof, cudaStream_t s) {
-  constexpr int NT = kLogitNT, KSB = kLogitKSB;
-  const LogitsArgs& a = p.la;
+  // every CTA must own at least one unit: the granules of W_U alone are a lower bound on the units
+  const int units_lb = (cb.V + kLogitGran - 1) / kLogitGran;
+  const int grid = units_lb < n_sm ? units_lb : n_sm;
+  p.part_stride = grid + 2;
+  if ((size_t)a.N * p.part_stride * sizeof(LogitPartial) > a.lpart_bytes) return cudaErrorMemoryAllocation;
+  if (info) { info->stride = p.part_stride; info->count = grid; }
   if (a.target_logit) {
     ProfScope ps(prof, kProfLogitsMerge, 1, s);
     k_fill_nan_f32<<<(a.N + 255) / 256, 256, 0, s>>>(a.target_logit, a.N);
@@ -759,13 +669,10 @@ cudaError_t launch_stream_logits(const StreamLogitsParams& p, const LogitMaps* m
   cudaError_t e;
   {
     ProfScope ps(prof, kProfLogits, 1, s);
-    const int st = pick_stages<NT, KSB>(1, p.a_box_rows, 5120);
-    if (st >= 8) e = launch_logits_t<NT, KSB, 8>(p, maps, grid, s);
-    else if (st >= 6) e = launch_logits_t<NT, KSB, 6>(p, maps, grid, s);
-    else if (st >= 4) e = launch_logits_t<NT, KSB, 4>(p, maps, grid, s);
-    else e = cudaErrorInvalidConfiguration;
+    const int st = (227 * 1024 - 2048 - 5120 - kTailPad) / ((p.a_box_rows + kLogitNT) * 128);      // stages that fit, 6 or more
+    e = st >= 8 ? launch_logits_t<8>(p, maps, grid, s) : launch_logits_t<6>(p, maps, grid, s);
   }
-  if (e != cudaSuccess || !merge) return e;
+  if (e != cudaSuccess || info) return e;
   ProfScope ps(prof, kProfLogitsMerge, 1, s);
   k_stream_logits_merge<<<(a.N + 3) / 4, 128, 0, s>>>(p, grid);
   return cudaGetLastError();

@@ -11,7 +11,7 @@ namespace z2z {
 constexpr int kMaxStages = 8;
 constexpr int kGemmNT = 128;                    // weight rows per tile of the stream-K GEMM
 
-constexpr int kLogitNT = 128, kLogitKSB = 1;
+constexpr int kLogitNT = 128;                   // weight rows per job of the logits kernel at most
 constexpr int kLogitGran = 32;                  // scheduling granule of the logits kernel, in weight rows (TMA boxes of
                                                 // fewer rows stream several times slower)
 constexpr int kLogitBoxClasses = 3;             // TMA boxes of 32, 64 and 128 weight rows
@@ -98,7 +98,7 @@ cudaError_t launch_stream_gemm(StreamGemmParams p, const StreamGemmMaps& maps, i
 // The same product for more than 128 rows on CTA pairs (z2z_stream_pair.cu): up to 256 packed rows ride on one stream of the
 // weights, and more run as blocks of 256.
 struct StreamPairParams {
-  int groups, ksteps;
+  int groups, ksteps;    // ksteps = K / 64
   int R;
   float* out;
   int J, Rt;
@@ -115,8 +115,7 @@ struct StreamPairMaps {
   CUtensorMap a[2][8];   // activation operand of each group, boxes of 16, 32, .. 128 rows
   CUtensorMap w[2];      // weights of each group, 128 rows
 };
-int stream_pair_ksb(int R);
-bool stream_pair_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int R);
+bool stream_pair_act_maps(CUtensorMap* maps, const void* act, int Rt, int K);
 cudaError_t launch_stream_pair(StreamPairParams p, const StreamPairMaps& maps, int n_sm, cudaStream_t s);
 
 struct StreamLogitsParams {
@@ -124,9 +123,7 @@ struct StreamLogitsParams {
   LogitsArgs la;
   int ksteps;
   int a_box_rows;
-  int row_tiles;         // ceil(N / 128)
   int part_stride;       // partial slots per row
-  int* vt_out;           // device word: number of virtual column tiles
   int* err;
 };
 
@@ -166,7 +163,5 @@ cudaError_t launch_pair_gemm(const PairGemmParams& p, const void* act, const voi
                              cudaStream_t s);
 
 bool make_tmap_bf16(CUtensorMap* m, const void* base, long long rows, long long cols, int box_rows);
-cudaError_t launch_stream_logits(const StreamLogitsParams& p, const LogitMaps* maps, int grid, bool merge,
-                                 Prof* prof, cudaStream_t s);
 
 }  // namespace z2z

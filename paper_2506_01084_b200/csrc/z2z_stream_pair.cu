@@ -91,7 +91,7 @@ __device__ __forceinline__ int sp_cols(int live, int block, int h) {
   if (rows > kSpHalfRows) rows = kSpHalfRows;
   return (2 * rows + 31) & ~31;
 }
-// Bytes per CTA and k-block of the activation box for n columns: half of the operand rows.
+// Bytes per CTA of the activation box for n columns: half of the operand rows.
 __device__ __forceinline__ uint32_t sp_box_bytes(int n) { return (uint32_t)n * 64u; }
 // Row blocks with a live row (at least one).  A pass whose capacity is one block does not need the count.
 __device__ __forceinline__ int sp_live_blocks(const StreamPairParams& p, int live) {
@@ -110,7 +110,6 @@ __device__ __forceinline__ void transpose4(float (&f)[4], int lane) {
   if (lane & 2) { f[0] = s0; f[1] = s1; } else { f[2] = s0; f[3] = s1; }
 }
 
-template <int KSB>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps tm) {
   extern __shared__ unsigned char smem_raw[];
@@ -119,7 +118,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
   const uint32_t stage_base = smem_u32(sm + 1024);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();          // 0: leader (issues the MMAs), 1: peer
-  const uint32_t stage_bytes = (uint32_t)p.act_bytes + KSB * 16384u;
+  const uint32_t stage_bytes = (uint32_t)p.act_bytes + 16384u;
   const int STAGES = p.stages;
   pdl_trigger();                                    // the next kernel may get resident behind this one
   if (threadIdx.x == 0) {
@@ -154,15 +153,15 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
       SpJob def[kSpMaxStages];                        // load i of the first pass uses stage i; kb0 = its k-step
       int n_def = 0, issued = 0, live = 0;
       bool deps = false, ok = true;
-      auto act_bytes = [&](int block) { return KSB * sp_box_bytes(sp_cols(live, block, 0) + sp_cols(live, block, 1)); };
+      auto act_bytes = [&](int block) { return sp_box_bytes(sp_cols(live, block, 0) + sp_cols(live, block, 1)); };
       auto load_act = [&](int st, const SpJob& j, int ks) {
         const uint32_t sb = stage_base + (uint32_t)st * stage_bytes;
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const int n = sp_cols(live, j.block, h);
           if (n == 0) continue;
-          tma_load_3d_pair(sb + h * (KSB * 16384u), &tm.a[j.g][(n >> 5) - 1], 0,
-                           2 * (j.block * kSpBlockRows + h * kSpHalfRows) + (int)rank * (n >> 1), ks * KSB, full_leader[st], pol_a);
+          tma_load_3d_pair(sb + h * 16384u, &tm.a[j.g][(n >> 5) - 1], 0,
+                           2 * (j.block * kSpBlockRows + h * kSpHalfRows) + (int)rank * (n >> 1), ks, full_leader[st], pol_a);
         }
       };
       auto need_deps = [&]() {
@@ -186,11 +185,11 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
           if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) { ok = false; break; }
           if (rank == 0) {
             const uint32_t full = smem_u32(&ctrl->full[stage]);
-            if (deps) mbar_expect_tx(full, 2 * (KSB * 16384u + act_bytes(j.block)));
-            else mbar_expect_only(full, 2 * KSB * 16384u);
+            if (deps) mbar_expect_tx(full, 2 * (16384u + act_bytes(j.block)));
+            else mbar_expect_only(full, 2 * 16384u);
           }
           const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
-          tma_load_3d_pair(sb + p.act_bytes, &tm.w[j.g], 0, j.wrow + (int)rank * 128, ks * KSB, full_leader[stage], pol_w);
+          tma_load_3d_pair(sb + p.act_bytes, &tm.w[j.g], 0, j.wrow + (int)rank * 128, ks, full_leader[stage], pol_w);
           if (deps) load_act(stage, j, ks);
           else { def[n_def] = j; def[n_def].kb0 = ks; ++n_def; }
           ++issued;
@@ -204,7 +203,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
     int live = *p.rows_dev;
     live = live < p.R ? live : p.R;
     const int n_blocks = sp_live_blocks(p, live);
-    const int chain = p.half_stride ? p.ksteps / 2 : kSpChain / KSB;       // (K is a multiple of 128: the k-steps are even in number)
+    const int chain = p.half_stride ? p.ksteps / 2 : kSpChain;       // (K is a multiple of 128: the k-steps are even in number)
     if (warp == 1) {
       if (lane == 0 && rank == 0) {
         // ---------------- MMA issuer (leader only): D[256 weight rows][n] += W tile x activation rows -----
@@ -219,22 +218,17 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
           const int n0 = sp_cols(live, j.block, 0), n1 = sp_cols(live, j.block, 1);
           const uint32_t id0 = idesc_bf16_f32(256, n0), id1 = idesc_bf16_f32(256, n1 ? n1 : 32);
           const uint32_t d = tmem_base;
-          const uint32_t kb0 = sp_box_bytes(n0), kb1 = sp_box_bytes(n1);                    // one k-block of a half's box
           uint32_t acc = 0;
           for (int ks = j.kb0; ks < j.kb1; ++ks) {
             if (!mbar_wait(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
             tc_fence_after();
             const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
+            const uint32_t wb = sb + p.act_bytes;
 #pragma unroll
-            for (int i = 0; i < KSB; ++i) {
-              const uint32_t wb = sb + p.act_bytes + i * 16384u;
-              const uint32_t a0 = sb + (uint32_t)i * kb0, a1 = sb + KSB * 16384u + (uint32_t)i * kb1;
-#pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                umma_bf16_pair(d, smem_desc_sw128(wb + k * 32), smem_desc_sw128(a0 + k * 32), id0, acc);
-                if (n1) umma_bf16_pair(d + 256, smem_desc_sw128(wb + k * 32), smem_desc_sw128(a1 + k * 32), id1, acc);
-                acc = 1;
-              }
+            for (int k = 0; k < 4; ++k) {
+              umma_bf16_pair(d, smem_desc_sw128(wb + k * 32), smem_desc_sw128(sb + k * 32), id0, acc);
+              if (n1) umma_bf16_pair(d + 256, smem_desc_sw128(wb + k * 32), smem_desc_sw128(sb + 16384u + k * 32), id1, acc);
+              acc = 1;
             }
             umma_commit_pair(smem_u32(&ctrl->empty[stage]));      // frees the stage in both CTAs
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -302,31 +296,26 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
 
 int round32(int n) { return (n + 31) / 32 * 32; }
 
-// Shared memory of one stage's activation boxes per CTA and k-block, for a pass of at most R > 128 rows.
+// Shared memory of one stage's activation boxes per CTA, for a pass of at most R > 128 rows.
 int pair_act_bytes(int R) {
   return 16384 + (R < kSpBlockRows ? round32(2 * (R - kSpHalfRows)) * 64 : 16384);
 }
 
 }  // namespace
 
-// Two k-blocks per stage (fewer TMA operations per byte) while at least four stages still fit.
-int stream_pair_ksb(int R) { return (kSpSmem - 2048) / (2 * (16384 + pair_act_bytes(R))) >= 4 ? 2 : 1; }
-
 // Tensor maps of one activation operand ([2 Rt, K], hi and lo rows interleaved): one per box height.
-bool stream_pair_act_maps(CUtensorMap* maps, const void* act, int Rt, int K, int R) {
-  const int ksb = stream_pair_ksb(R);
+bool stream_pair_act_maps(CUtensorMap* maps, const void* act, int Rt, int K) {
   for (int i = 0; i < 8; ++i)
-    if (!make_tmap_bf16_kblocks(&maps[i], act, 2ll * Rt, K, 16 * (i + 1), ksb)) return false;
+    if (!make_tmap_bf16_kblocks(&maps[i], act, 2ll * Rt, K, 16 * (i + 1), 1)) return false;
   return true;
 }
 
 cudaError_t launch_stream_pair(StreamPairParams p, const StreamPairMaps& maps, int n_sm, cudaStream_t s) {
   if (!p.out || !p.err || !p.rows_dev || p.R <= 128) return cudaErrorInvalidValue;
-  const int ksb = stream_pair_ksb(p.R);
   p.tiles_per_group = (p.J + 255) / 256;
   p.blocks = (p.R + kSpBlockRows - 1) / kSpBlockRows;
-  p.act_bytes = ksb * pair_act_bytes(p.R);
-  const int stage = p.act_bytes + ksb * 16384;
+  p.act_bytes = pair_act_bytes(p.R);
+  const int stage = p.act_bytes + 16384;
   p.stages = (kSpSmem - 2048) / stage;
   if (p.stages > kSpMaxStages) p.stages = kSpMaxStages;
   const size_t smem = 2048 + (size_t)p.stages * stage;
@@ -338,10 +327,9 @@ cudaError_t launch_stream_pair(StreamPairParams p, const StreamPairMaps& maps, i
   const int tiles = p.groups * p.tiles_per_group, whole = clusters / tiles * tiles;
   if (p.half_stride) clusters = halves_workers(tiles, clusters);
   else if (7 * whole >= 6 * clusters) clusters = whole;
-  auto kern = ksb == 2 ? k_stream_pair<2> : k_stream_pair<1>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(k_stream_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(2 * clusters), dim3(kThreads), smem, s, p, maps);
+  return launch_pdl(k_stream_pair, dim3(2 * clusters), dim3(kThreads), smem, s, p, maps);
 }
 
 }  // namespace z2z
