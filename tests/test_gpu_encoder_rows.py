@@ -147,6 +147,50 @@ def test_a_captured_session_start_clears_when_it_runs():
     assert np.abs(p.E_f32[:, 0].double().cpu().numpy() - want).max() <= TOL
 
 
+@pytest.mark.parametrize("captured", [False, True])
+@pytest.mark.parametrize("B,tied", [(8, 0), (60, 0), (100, 1)])
+def test_steps_without_an_entry_between_steps_that_create_some(B, tied, captured):
+    """A pass without a row leaves the result matrix and the caches alone: all sequences sit out, or feed a code
+    that makes no entry, then some create one, in the middle of the batch or everywhere."""
+    w, p = _pair(256, 512, 3, B, T=64, cap=96, seed=B, tied=tied)
+    i32 = lambda x: torch.tensor(x, dtype=torch.int32, device=p.dev)
+    hid = si.make_hidden(w, B, 3).to(p.dev)
+    nxt, new, forced = (torch.zeros(B, dtype=torch.int32, device=p.dev) for _ in range(3))
+    lse = torch.zeros(B, device=p.dev)
+    none = [zb.CODE_NONE] * B
+    some = [(41 * b + 3) % w.V if b % 3 == 1 else zb.CODE_NONE for b in range(B)]
+    every = [(57 * b + 9) % w.V for b in range(B)]
+    plan = [none, some, none, none, every, some, every]           # (the second `some` and `every` repeat codes)
+
+    def step():
+        zb.z2z_decode_step(p.cb, hid, p.g_WE, p.g_WU, p.g_encE, p.g_encU, p.E_h, p.U_h, zb.SELECT_ARGMAX, 1.0, 0, 0,
+                           forced, nxt, None, lse, new, p.E_f32, p.U_f32)
+
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    if captured:
+        forced.copy_(i32(none))
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph):
+            step()
+    sides = [(p.E_f32, p.W_E, p.enc_E), (p.U_f32, p.W_U, p.enc_U)][:1 if tied else 2]
+    for codes in plan:
+        forced.copy_(i32(codes))
+        before = [f32.clone() for f32, _, _ in sides]
+        graph.replay() if captured else step()
+        want = [-1 if z == zb.CODE_NONE else p.oracle.books[b].step(z) for b, z in enumerate(codes)]
+        assert new.cpu().tolist() == want
+        for (f32, W, enc), old in zip(sides, before):
+            made = [b for b in range(B) if want[b] >= 0]
+            mask = torch.ones(B, w.cap, dtype=torch.bool, device=p.dev)
+            for b in made:
+                mask[b, want[b]] = False
+            assert torch.equal(f32[mask], old[mask])
+            for b in made[::7]:
+                row = ohe.hyper_embed([p.oracle.books[b].entries[want[b]]], f64(W), [f64(t) for t in enc], w.heads)[0]
+                assert np.abs(f32[b, want[b]].double().cpu().numpy() - row).max() <= TOL
+
+
 @pytest.mark.parametrize("M,d,dff", [(2, 128, 256), (3, 384, 384), (5, 128, 128)])
 def test_whole_prompts_in_passes_cut_by_rows(M, d, dff):
     """Every entry of a call of several passes, so that those on both sides of a cut are among them."""
