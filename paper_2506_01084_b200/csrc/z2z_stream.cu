@@ -170,11 +170,12 @@ __device__ __forceinline__ void setup_barriers(Ctrl* ctrl) {
 // =================================================================================================
 // GEMM kernel: weights as the M operand, activation rows (hi | lo) as the N operand
 // =================================================================================================
-struct GemmJob { int g, wrow, half, kb0, kb1; };
+struct GemmJob { int g, wrow, kb0, kb1; };
 struct GemmWalk {
   const StreamGemmParams& p;
+  int mid;                               // > 0: a job ends there
   long long u, u1;
-  __device__ GemmWalk(const StreamGemmParams& pp) : p(pp) {
+  __device__ GemmWalk(const StreamGemmParams& pp) : p(pp), mid(pp.half_stride ? pp.ksteps / 2 : 0) {
     const long long U = (long long)p.groups * p.tiles_per_group * p.ksteps, G = gridDim.x, c = blockIdx.x;
     u = c * U / G;
     u1 = (c + 1) * U / G;
@@ -184,8 +185,7 @@ struct GemmWalk {
     const long long tile = u / p.ksteps;
     j.kb0 = (int)(u - tile * p.ksteps);
     const long long left = u1 - u;
-    const int mid = p.half_stride ? p.ksteps / 2 : 0, end = j.kb0 < mid ? mid : p.ksteps;
-    j.half = p.half_stride && j.kb0 >= mid;
+    const int end = j.kb0 < mid ? mid : p.ksteps;
     j.kb1 = (int)((end - j.kb0) < left ? end : j.kb0 + left);
     j.g = (int)tile / p.tiles_per_group;
     j.wrow = ((int)tile - j.g * p.tiles_per_group) * kGemmNT;
@@ -329,7 +329,7 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
       const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
       if (!mbar_wait(smem_u32(&ctrl->acc_full[buf]), aph, &ctrl->abort)) break;
       tc_fence_after();
-      float* dst = p.out + (j.half ? p.half_stride : 0) + (size_t)j.g * p.Rt * p.J + j.wrow + feature;
+      float* dst = p.out + (j.kb0 >= walk.mid ? p.half_stride : 0) + (size_t)j.g * p.Rt * p.J + j.wrow + feature;
       const uint32_t t0 = tmem_base + ((uint32_t)(q * 32) << 16) + buf * (uint32_t)p.a_box_rows;
 #pragma unroll 1
       for (int r0 = 0; r0 < rows; r0 += 8) {
