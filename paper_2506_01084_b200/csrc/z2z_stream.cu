@@ -10,7 +10,8 @@
 //     operand, the packed activation rows (hi and lo part of a row in adjacent operand rows) its
 //     N operand, as wide as the rows that exist; work is cut stream-K style, every CTA gets the
 //     same number of (tile, k-step) units and adds its accumulators into one fp32 result matrix
-//     with reductions in global memory (sums of two or three partial tiles in arrival order);
+//     with reductions in global memory (sums of a few partial tiles in arrival order; where the bits
+//     must not depend on it, two matrices of at most two partials each);
 //   * joint logits for 33 .. 128 hidden rows of a batch (k_stream_logits; paper Section 2.3 steps 7-9):
 //     the hidden rows are the 128-row M operand, tiles run over W_U and then over the visible
 //     rows of each sequence's U_h; the epilogue keeps max / sum-exp / argmax / best perturbed

@@ -1,5 +1,5 @@
 // Weight-streaming skinny GEMM on CTA pairs, for hyper-encoder passes of a large decode batch or of a call
-// bounded to some hundred activation rows:
+// bounded to some hundred activation rows (more than 128, fewer than a prompt-sized pass has):
 //
 //   out[group][r][j] += sum_k A[group][r][k] * W[group][j][k]
 //
@@ -242,8 +242,9 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
       // ---------------- epilogue (both CTAs): thread = output feature -----------------------------------
       // Nothing overlaps the epilogue, as both accumulators are in use, and one reduction instruction per
       // row and feature is what it costs: four lanes transpose four rows x four features among
-      // themselves and add 16 bytes each.  (217 rows, d = 3072, both encoders: 859 us a request start
-      // with single words on four warps, 805 with 16 bytes, 714 with the split below, 654 on eight warps.)
+      // themselves and add 16 bytes each.  (Two passes of 217 rows, one per encoder, d = 3072, with the parse
+      // and the logits around them: 859 us with single words on four warps, 805 with 16 bytes, 714 with
+      // whole clusters per tile, 654 on eight warps.)
       const int q = warp & 3;                          // TMEM lane quarter this warp may read
       const int group = (warp - 2) >> 2;               // takes every other 32 columns
       const uint32_t acc_empty_leader = map_to_cta(smem_u32(&ctrl->acc_empty), 0);
@@ -322,8 +323,9 @@ cudaError_t launch_stream_pair(StreamPairParams p, const StreamPairMaps& maps, i
   const long long units = (long long)p.groups * p.tiles_per_group * p.ksteps;      // every cluster owns >= 1 unit
   int clusters = units < n_sm / 2 ? (int)units : n_sm / 2;
   // A whole number of clusters per tile leaves every cluster with one piece of one tile, and so with one
-  // epilogue instead of two; worth up to a seventh of the clusters (217 rows, d = 3072: 859 -> 750 us a
-  // request start with 72 of 74).
+  // epilogue instead of two; worth up to a seventh of the clusters (decode steps with all rows live, 74 -> whole:
+  // d = 3072 180 rows of both encoders 426 -> 405 us, 384 811 -> 789, d = 1024 640 rows 343 -> 311; d = 2048 640 rows
+  // lose, 664 -> 678).
   const int tiles = p.groups * p.tiles_per_group, whole = clusters / tiles * tiles;
   if (p.half_stride) clusters = halves_workers(tiles, clusters);
   else if (7 * whole >= 6 * clusters) clusters = whole;
