@@ -190,13 +190,14 @@ __device__ __forceinline__ uint32_t philox_word(const Philox4& p, int i) {
 }
 
 // Running reduction over logit columns: max / sum-exp / argmax (lowest index on ties) and the
-// same for Gumbel-perturbed scores.
+// same for Gumbel-perturbed scores.  A logit that equals the maximum counts 1 without a difference being
+// taken, so that overflowed logits (+inf, or nothing but -inf so far) leave the sum a number.
 struct RowRed {
   float m, s; int idx; float gm; int gidx;
   __device__ __forceinline__ void init() { m = -INFINITY; s = 0.f; idx = 0x7fffffff; gm = -INFINITY; gidx = 0x7fffffff; }
   __device__ __forceinline__ void add(float l, int col) {
     if (l > m) { s = s * __expf(m - l) + 1.f; m = l; idx = col; }
-    else { s += __expf(l - m); if (l == m && col < idx) idx = col; }
+    else { s += l == m ? 1.f : __expf(l - m); if (l == m && col < idx) idx = col; }
   }
   __device__ __forceinline__ void add_score(float sc, int col) {
     if (sc > gm || (sc == gm && col < gidx)) { gm = sc; gidx = col; }
@@ -223,7 +224,7 @@ __device__ __forceinline__ void fold_row32(uint32_t (&v)[32], int limit, int col
   float cm = __uint_as_float(v[0]);
 #pragma unroll
   for (int x = 1; x < 32; ++x) cm = fmaxf(cm, __uint_as_float(v[x]));
-  if (cm == INFINITY || red.m == INFINITY) {      // an overflowed logit: differences to it are not numbers
+  if (fabsf(cm) == INFINITY || red.m == INFINITY) {      // overflowed logits: differences of two are not numbers
 #pragma unroll
     for (int x = 0; x < 32; ++x) if (x < limit) red.add(__uint_as_float(v[x]), col + x);
     return;

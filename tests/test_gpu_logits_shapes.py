@@ -137,3 +137,33 @@ def test_overflowed_logit_keeps_its_row_a_number():
     am = torch.zeros(N, dtype=torch.int32, device=DEV)
     zb.z2z_dynamic_logits(cb, hid, None, None, WU, Uh, zb.SELECT_ARGMAX, 1.0, 0, 0, None, lse, am, mx)
     assert torch.all(torch.isposinf(lse)) and torch.all(torch.isposinf(mx)) and torch.all(am == 77)
+
+
+@pytest.mark.parametrize("N,B", [(33, 33), (100, 100), (40, 5), (200, 200), (300, 5), (2100, 5)])
+@pytest.mark.parametrize("select", [0, 1])
+@pytest.mark.parametrize("which", ["two_inf", "first_neg_inf", "many_neg_inf", "all_neg_inf"])
+def test_overflowed_logits_leave_the_sum_a_number(N, B, select, which):
+    """Overflowed columns anywhere, beyond the decode kernel's 32 rows: several of +inf give +inf, those of -inf add
+    nothing, a row of nothing else is -inf, however the columns are split."""
+    V, d = 1000, 128
+    cb = _session(V, d, B, 8, [1] * B, 5)
+    hid = torch.ones(N, d, dtype=torch.bfloat16, device=DEV)
+    WU = torch.zeros(V, d, dtype=torch.bfloat16, device=DEV)
+    WU[:, 0] = torch.arange(V, device=DEV).fmod(7).to(torch.bfloat16)
+    Uh = torch.zeros(B, 8, d, dtype=torch.bfloat16, device=DEV)
+    cols = {"two_inf": [77, 500], "first_neg_inf": [0, 1, 2], "many_neg_inf": list(range(250, 420)) + list(range(900, V)),
+            "all_neg_inf": list(range(V))}[which]
+    WU[cols] = 3e38 if which == "two_inf" else -3e38
+    if which == "all_neg_inf":
+        Uh[:] = -3e38
+    seq = None if N == B else (torch.arange(N, device=DEV) * B // N).to(torch.int32)
+    lse, mx = torch.zeros(N, device=DEV), torch.zeros(N, device=DEV)
+    am, sm = torch.zeros(N, dtype=torch.int32, device=DEV), torch.zeros(N, dtype=torch.int32, device=DEV)
+    zb.z2z_dynamic_logits(cb, hid, seq, None, WU, Uh, select, 1.0, 1, 2, None, lse, am, mx, sm if select else None)
+    l = torch.cat([WU[:, 0].double(), torch.zeros(1, dtype=torch.float64, device=DEV)])
+    l[cols] = float("inf") if which == "two_inf" else float("-inf")
+    if which == "all_neg_inf":
+        l[-1] = float("-inf")
+    want = float(torch.logsumexp(l, 0))
+    assert torch.all(mx == float(l.max())) and torch.all(am == int(l.argmax()))
+    assert torch.all(lse == want) if abs(want) == float("inf") else torch.all((lse - want).abs() < 1e-5 * (1 + abs(want)))
