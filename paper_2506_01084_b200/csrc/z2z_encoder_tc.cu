@@ -29,7 +29,7 @@
 // of the pass (the GEMM adds nothing to rows beyond them), which restores the invariant for the
 // next GEMM.  The first pass of a session that needs it clears Y.  Sums of three or more partials depend on
 // the order in which they arrive: calls whose bits must not (z2z_hyper_embed in a session of prompt size)
-// use a matrix for each half of K (StreamGemmParams::half_stride), and the kernel after the GEMM adds the two.
+// use a matrix for each half or quarter of K (StreamPairParams::parts), and the kernel after the GEMM adds them.
 //
 // Launches per layer: GEMM(qkv) -> [+ bias, attention] -> GEMM(o) -> [+ bias + residual,
 // LayerNorm 2] -> GEMM(1) -> [+ bias, GELU] -> GEMM(2) -> [+ bias + residual, LayerNorm 1 of the
@@ -113,8 +113,8 @@ __device__ __forceinline__ float4 unpack_bf16x4(uint2 u) {
   return make_float4(bf_lo(u.x), bf_hi(u.x), bf_lo(u.y), bf_hi(u.y));
 }
 
-// A result that lies in two matrices (StreamGemmParams::half_stride): always first half + second half.
-__device__ __forceinline__ void add_half(float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; }
+// A result that lies in several matrices (StreamPairParams::parts): always added in the order of the parts.
+__device__ __forceinline__ void add_part(float4& a, const float4& b) { a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w; }
 
 __device__ __forceinline__ float block_sum(float v, float* sm) {
 #pragma unroll
@@ -204,8 +204,8 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_gather_ln(CbView cb, EntryLi
 // x = X[r] + Y[r] + bias for a live packed row (Y consumed and cleared); then LayerNorm -> hi/lo
 // for the next GEMM.  grid (rows, groups).  All loads (row count, Y, X, bias, gamma, beta) are
 // issued together; whether the row is live only decides what is stored.
-template <int NV, bool HALVES>
-__global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_ln(const int* total, float* Y, size_t half_stride, Ptr2 bias,
+template <int NV, int PARTS>
+__global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_ln(const int* total, float* Y, size_t part_stride, Ptr2 bias,
                                                                     MPtr2 X, Ptr2 ln_w, Ptr2 ln_b, MPtr2 Ahl,
                                                                     int d, int Rt) {
   __shared__ float sm[32];
@@ -219,14 +219,15 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_ln(const int* t
   const uint2* lw = reinterpret_cast<const uint2*>(ln_w.p[g]);
   const uint2* lb = reinterpret_cast<const uint2*>(ln_b.p[g]);
   const int nvec = d / 4;
-  float4 xv[NV], yv[NV], zv[HALVES ? NV : 1];
+  float4 xv[NV], yv[NV], zv[PARTS][NV];            // (zv[0] is not used)
   uint2 bv[NV], gw[NV], gb[NV];
 #pragma unroll
   for (int v = 0; v < NV; ++v) {
     const int idx = (int)threadIdx.x + v * kRowThreads;
     if (idx < nvec) {
       yv[v] = *reinterpret_cast<const float4*>(y + idx * 4);
-      if (HALVES) zv[HALVES ? v : 0] = *reinterpret_cast<const float4*>(y + half_stride + idx * 4);
+#pragma unroll
+      for (int k = 1; k < PARTS; ++k) zv[k][v] = *reinterpret_cast<const float4*>(y + k * part_stride + idx * 4);
       xv[v] = *reinterpret_cast<const float4*>(x + idx * 4);
       bv[v] = bs[idx]; gw[v] = lw[idx]; gb[v] = lb[idx];
     }
@@ -237,9 +238,10 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_ln(const int* t
     const int idx = (int)threadIdx.x + v * kRowThreads;
     if (idx < nvec) {
       *reinterpret_cast<float4*>(y + idx * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (HALVES) {
-        *reinterpret_cast<float4*>(y + half_stride + idx * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
-        add_half(yv[v], zv[HALVES ? v : 0]);
+#pragma unroll
+      for (int k = 1; k < PARTS; ++k) {
+        *reinterpret_cast<float4*>(y + k * part_stride + idx * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
+        add_part(yv[v], zv[k][v]);
       }
       const float4 b = unpack_bf16x4(bv[v]);
       xv[v] = make_float4(xv[v].x + yv[v].x + b.x, xv[v].y + yv[v].y + b.y, xv[v].z + yv[v].z + b.z,
@@ -254,8 +256,8 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_ln(const int* t
 // Last layer: x_i = X[r_i] + Y[r_i] + bias for the entry's rows, cache row = mean_i x_i.
 // grid (entries, groups, ceil(d / (4 * kRowThreads))): a thread owns 4 columns of the entry and
 // issues the loads of all its rows before it adds.
-template <bool HALVES>
-__global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_pool(CbView cb, EntryList el, float* Y, size_t half_stride,
+template <int PARTS>
+__global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_pool(CbView cb, EntryList el, float* Y, size_t part_stride,
                                                                       Ptr2 bias, MPtr2 X, MPtr2 cache, MPtr2 cache_f32,
                                                                       int d, int Rt) {
   sm100::pdl_trigger();
@@ -268,13 +270,14 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_pool(CbView cb,
   const int seq = el.seq[e], idx = el.idx[e];
   const float4 b = load_bf16x4(reinterpret_cast<const bf16*>(bias.p[g]) + col);
   if (L <= 0) return;
-  float4 yv[kMaxM], xv[kMaxM], zv[HALVES ? kMaxM : 1];
+  float4 yv[kMaxM], xv[kMaxM], zv[PARTS][kMaxM];
 #pragma unroll
   for (int i = 0; i < kMaxM; ++i)
     if (i < L) {
       const size_t r = (size_t)r0 + i;
       yv[i] = *reinterpret_cast<const float4*>(Y + ((size_t)g * Rt + r) * d + col);
-      if (HALVES) zv[HALVES ? i : 0] = *reinterpret_cast<const float4*>(Y + half_stride + ((size_t)g * Rt + r) * d + col);
+#pragma unroll
+      for (int k = 1; k < PARTS; ++k) zv[k][i] = *reinterpret_cast<const float4*>(Y + k * part_stride + ((size_t)g * Rt + r) * d + col);
       xv[i] = *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(X.p[g]) + r * d + col);
     }
   float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -283,9 +286,10 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_reduce_resid_pool(CbView cb,
     if (i < L) {
       const size_t r = (size_t)r0 + i;
       *reinterpret_cast<float4*>(Y + ((size_t)g * Rt + r) * d + col) = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (HALVES) {
-        *reinterpret_cast<float4*>(Y + half_stride + ((size_t)g * Rt + r) * d + col) = make_float4(0.f, 0.f, 0.f, 0.f);
-        add_half(yv[i], zv[HALVES ? i : 0]);
+#pragma unroll
+      for (int k = 1; k < PARTS; ++k) {
+        *reinterpret_cast<float4*>(Y + k * part_stride + ((size_t)g * Rt + r) * d + col) = make_float4(0.f, 0.f, 0.f, 0.f);
+        add_part(yv[i], zv[k][i]);
       }
       acc.x += xv[i].x + yv[i].x + b.x; acc.y += xv[i].y + yv[i].y + b.y;
       acc.z += xv[i].z + yv[i].z + b.z; acc.w += xv[i].w + yv[i].w + b.w;
@@ -327,7 +331,7 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_pool(CbView cb, EntryList el
 // grid = ceil(groups * R * J / 4 / (kGeluThreads * kGeluPerThread)), R = row capacity of the pass.
 constexpr int kGeluThreads = 256, kGeluPerThread = 4;
 template <bool HALVES>
-__global__ void __launch_bounds__(kGeluThreads) k_tc_reduce_gelu(const int* total_rows, float* Y, size_t half_stride, Ptr2 bias,
+__global__ void __launch_bounds__(kGeluThreads) k_tc_reduce_gelu(const int* total_rows, float* Y, size_t part_stride, Ptr2 bias,
                                                                  MPtr2 Hhl, int J, int R, int Rt, int ng) {
   sm100::pdl_trigger();
   sm100::pdl_wait();
@@ -346,7 +350,7 @@ __global__ void __launch_bounds__(kGeluThreads) k_tc_reduce_gelu(const int* tota
       jj[k] = (int)(f - (long long)row[k] * J4) * 4;
       const int g = row[k] / R, r = row[k] - g * R;
       q[k] = *reinterpret_cast<const float4*>(Y + ((size_t)g * Rt + r) * J + jj[k]);
-      if (HALVES) q2[HALVES ? k : 0] = *reinterpret_cast<const float4*>(Y + half_stride + ((size_t)g * Rt + r) * J + jj[k]);
+      if (HALVES) q2[HALVES ? k : 0] = *reinterpret_cast<const float4*>(Y + part_stride + ((size_t)g * Rt + r) * J + jj[k]);
       bs[k] = load_bf16x4(reinterpret_cast<const bf16*>(bias.p[g]) + jj[k]);
     }
   }
@@ -357,8 +361,8 @@ __global__ void __launch_bounds__(kGeluThreads) k_tc_reduce_gelu(const int* tota
     if (r >= live) continue;                       // no row there: Y is still zero, nothing reads the operand row
     *reinterpret_cast<float4*>(Y + ((size_t)g * Rt + r) * J + jj[k]) = make_float4(0.f, 0.f, 0.f, 0.f);
     if (HALVES) {
-      *reinterpret_cast<float4*>(Y + half_stride + ((size_t)g * Rt + r) * J + jj[k]) = make_float4(0.f, 0.f, 0.f, 0.f);
-      add_half(q[k], q2[HALVES ? k : 0]);
+      *reinterpret_cast<float4*>(Y + part_stride + ((size_t)g * Rt + r) * J + jj[k]) = make_float4(0.f, 0.f, 0.f, 0.f);
+      add_part(q[k], q2[HALVES ? k : 0]);
     }
     float4 v = make_float4(q[k].x + bs[k].x, q[k].y + bs[k].y, q[k].z + bs[k].z, q[k].w + bs[k].w);
     v.x = 0.5f * v.x * (1.0f + erff(v.x * 0.70710678118654752440f));
@@ -374,7 +378,7 @@ __global__ void __launch_bounds__(kGeluThreads) k_tc_reduce_gelu(const int* tota
 // bidirectional attention over the entry's rows; output as hi/lo.
 // grid (entries, heads, groups), block (32, M), dynamic smem M * 3 * dh floats; dh % 4 == 0.
 template <bool HALVES>
-__global__ void k_tc_qkv_attention(CbView cb, EntryList el, float* Y, size_t half_stride, Ptr2 bias, MPtr2 Ohl, int d,
+__global__ void k_tc_qkv_attention(CbView cb, EntryList el, float* Y, size_t part_stride, Ptr2 bias, MPtr2 Ohl, int d,
                                    int heads, int Rt) {
   extern __shared__ float s_qkv[];
   sm100::pdl_trigger();
@@ -392,15 +396,15 @@ __global__ void k_tc_qkv_attention(CbView cb, EntryList el, float* Y, size_t hal
       for (int w = 0; w < 3; ++w) {                // the loads are independent of one another
         const int col = w * d + h * dh + c;
         p[w] = *reinterpret_cast<const float4*>(y + col);
-        if (HALVES) p2[HALVES ? w : 0] = *reinterpret_cast<const float4*>(y + half_stride + col);
+        if (HALVES) p2[HALVES ? w : 0] = *reinterpret_cast<const float4*>(y + part_stride + col);
         b[w] = load_bf16x4(bs + col);
       }
 #pragma unroll
       for (int w = 0; w < 3; ++w) {
         *reinterpret_cast<float4*>(y + w * d + h * dh + c) = make_float4(0.f, 0.f, 0.f, 0.f);
         if (HALVES) {
-          *reinterpret_cast<float4*>(y + half_stride + w * d + h * dh + c) = make_float4(0.f, 0.f, 0.f, 0.f);
-          add_half(p[w], p2[HALVES ? w : 0]);
+          *reinterpret_cast<float4*>(y + part_stride + w * d + h * dh + c) = make_float4(0.f, 0.f, 0.f, 0.f);
+          add_part(p[w], p2[HALVES ? w : 0]);
         }
         *reinterpret_cast<float4*>(&s_qkv[(i * 3 + w) * dh + c]) =
             make_float4(p[w].x + b[w].x, p[w].y + b[w].y, p[w].z + b[w].z, p[w].w + b[w].w);
@@ -883,11 +887,17 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   const int n_sm = sm_count();
   const bool narrow = d <= 4 * kRowThreads * kNarrowVec4;      // a row fits four float4 per thread
   const bool halves = a0.prompt;                       // the call's bits must not depend on who adds first
-  auto rlk = halves ? (narrow ? k_tc_reduce_resid_ln<kNarrowVec4, true> : k_tc_reduce_resid_ln<kMaxVec4, true>)
-                    : (narrow ? k_tc_reduce_resid_ln<kNarrowVec4, false> : k_tc_reduce_resid_ln<kMaxVec4, false>);
+  const int parts2 = halves ? 2 : 1;
+  // (results in four parts have at most 14 tiles of 256 columns: d <= 3584, a narrow row)
+  auto rlk = [&](int parts) {
+    return parts == 4 ? k_tc_reduce_resid_ln<kNarrowVec4, 4>
+           : parts == 2 ? (narrow ? k_tc_reduce_resid_ln<kNarrowVec4, 2> : k_tc_reduce_resid_ln<kMaxVec4, 2>)
+                        : (narrow ? k_tc_reduce_resid_ln<kNarrowVec4, 1> : k_tc_reduce_resid_ln<kMaxVec4, 1>);
+  };
   float* Y = a0.part;                                  // GEMM results, all zero between GEMMs
   const size_t wide = (size_t)(3 * d > dff ? 3 * d : dff);
   const size_t hs = halves ? (size_t)ng * Rt * wide : 0;
+  auto stride = [&](int parts) { return parts == 4 ? hs / 2 : hs; };       // (four matrices of d <= wide / 3 columns)
   const size_t y_bytes = encoder_result_bytes(R, d, dff, ng * (halves ? 2 : 1));
   if (y_bytes > a0.part_bytes) return cudaErrorMemoryAllocation;
   if (a0.layers > 0 && y_bytes > *a0.part_clean) {
@@ -915,9 +925,9 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   const int ksb = paired ? 1 : stream_gemm_ksb(R);
   StreamGemmMaps maps;
   StreamPairMaps pair_maps;
-  auto gemm = [&](const MPtr2& act, int K, int widx, int J) -> cudaError_t {
+  auto gemm = [&](const MPtr2& act, int K, int widx, int J, int parts) -> cudaError_t {
     auto fill = [&](auto p) {
-      p.groups = ng; p.ksteps = K / (64 * ksb); p.R = R; p.out = Y; p.J = J; p.Rt = Rt; p.half_stride = hs;
+      p.groups = ng; p.ksteps = K / (64 * ksb); p.R = R; p.out = Y; p.J = J; p.Rt = Rt;
       p.rows_dev = total; p.err = a0.err;
       return p;
     };
@@ -930,10 +940,19 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
     ProfScope ps(prof, kProfEncGemm, 1, s);
     if (paired) {
       if (!make(pair_maps, [&](int g) { return stream_pair_act_maps(pair_maps.a[g], act.p[g], Rt, K); })) return cudaErrorInvalidValue;
-      return launch_stream_pair(fill(StreamPairParams{}), pair_maps, n_sm, s);
+      StreamPairParams p = fill(StreamPairParams{});
+      p.parts = parts; p.part_stride = stride(parts);
+      return launch_stream_pair(p, pair_maps, n_sm, s);
     }
     if (!make(maps, [&](int g) { return stream_gemm_act_maps(maps.a[g], act.p[g], Rt, K, R); })) return cudaErrorInvalidValue;
-    return launch_stream_gemm(fill(StreamGemmParams{}), maps, n_sm, s);
+    StreamGemmParams p = fill(StreamGemmParams{});
+    p.half_stride = hs;
+    return launch_stream_gemm(p, maps, n_sm, s);
+  };
+
+  // parts of the results of d columns, which the two linear maps that end a half layer have
+  auto parts_d = [&](int K) {
+    return halves && paired ? stream_pair_parts((long long)ng * ((d + 255) / 256), n_sm / 2, K / 64, R) : parts2;
   };
 
   if (!rows_mapped) {
@@ -954,21 +973,22 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   for (int l = 0; l < a0.layers; ++l) {
     const int o = 1 + 12 * l;
     const bool last = l + 1 == a0.layers;
-    if ((e = gemm(Ahl, d, o + 2, 3 * d)) != cudaSuccess) return e;
+    if ((e = gemm(Ahl, d, o + 2, 3 * d, parts2)) != cudaSuccess) return e;
     {
       ProfScope ps(prof, kProfEncOther, 1, s);
       launch_pdl(halves ? k_tc_qkv_attention<true> : k_tc_qkv_attention<false>, dim3(E, a0.heads, ng), dim3(32, M),
                  (size_t)M * 3 * dh * 4, s, cb, el, Y, hs, W(o + 3), Ahl, d, a0.heads, Rt);
     }
-    if ((e = gemm(Ahl, d, o + 4, d)) != cudaSuccess) return e;
+    int parts = parts_d(d);
+    if ((e = gemm(Ahl, d, o + 4, d, parts)) != cudaSuccess) return e;
     int last_bias = o + 5;                             // bias of the layer's last linear map
     if (dff > 0) {                                     // dff == 0: attention-only layer
       {
         ProfScope ps(prof, kProfEncOther, 1, s);
-        launch_pdl(rlk, dim3(R, ng), dim3(kRowThreads), 0, s, total, Y, hs, W(o + 5), X, W(o + 6),
+        launch_pdl(rlk(parts), dim3(R, ng), dim3(kRowThreads), 0, s, total, Y, stride(parts), W(o + 5), X, W(o + 6),
                    W(o + 7), Ahl, d, Rt);
       }
-      if ((e = gemm(Ahl, d, o + 8, dff)) != cudaSuccess) return e;
+      if ((e = gemm(Ahl, d, o + 8, dff, parts2)) != cudaSuccess) return e;
       {
         ProfScope ps(prof, kProfEncOther, 1, s);
         const long long f4 = (long long)ng * R * (dff / 4);
@@ -976,16 +996,17 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
         launch_pdl(halves ? k_tc_reduce_gelu<true> : k_tc_reduce_gelu<false>, dim3((unsigned)((f4 + per_cta - 1) / per_cta)),
                    dim3(kGeluThreads), 0, s, total, Y, hs, W(o + 9), Hhl, dff, R, Rt, ng);
       }
-      if ((e = gemm(Hhl, dff, o + 10, d)) != cudaSuccess) return e;
+      parts = parts_d(dff);
+      if ((e = gemm(Hhl, dff, o + 10, d, parts)) != cudaSuccess) return e;
       last_bias = o + 11;
     }
     {
       ProfScope ps(prof, kProfEncOther, 1, s);
       if (last)
-        launch_pdl(halves ? k_tc_reduce_resid_pool<true> : k_tc_reduce_resid_pool<false>,
-                   dim3(E, ng, (d / 4 + kRowThreads - 1) / kRowThreads), dim3(kRowThreads), 0, s, cb, el, Y, hs, W(last_bias), X, cache, c32, d, Rt);
+        launch_pdl(parts == 4 ? k_tc_reduce_resid_pool<4> : parts == 2 ? k_tc_reduce_resid_pool<2> : k_tc_reduce_resid_pool<1>,
+                   dim3(E, ng, (d / 4 + kRowThreads - 1) / kRowThreads), dim3(kRowThreads), 0, s, cb, el, Y, stride(parts), W(last_bias), X, cache, c32, d, Rt);
       else
-        launch_pdl(rlk, dim3(R, ng), dim3(kRowThreads), 0, s, total, Y, hs, W(last_bias), X, W(o + 12),
+        launch_pdl(rlk(parts), dim3(R, ng), dim3(kRowThreads), 0, s, total, Y, stride(parts), W(last_bias), X, W(o + 12),
                    W(o + 13), Ahl, d, Rt);
     }
   }

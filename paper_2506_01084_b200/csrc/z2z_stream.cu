@@ -616,7 +616,7 @@ cudaError_t launch_stream_gemm(StreamGemmParams p, const StreamGemmMaps& maps, i
   p.a_box_rows = gemm_box_rows(p.R);
   p.tiles_per_group = p.J / kGemmNT;
   const long long tiles = (long long)p.groups * p.tiles_per_group, units = tiles * p.ksteps;
-  const int most = p.half_stride ? halves_workers(tiles, n_sm) : n_sm;
+  const int most = p.half_stride ? fixed_order_workers(tiles, n_sm, 2) : n_sm;
   const int grid = units < most ? (int)units : most;           // every CTA owns >= 1 unit
   return stream_gemm_ksb(p.R) == 2 ? launch_stream_gemm_k<2>(p, maps, grid, s) : launch_stream_gemm_k<1>(p, maps, grid, s);
 }

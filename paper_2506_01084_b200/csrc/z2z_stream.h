@@ -83,11 +83,13 @@ struct StreamGemmMaps {
   CUtensorMap a[2][8];   // activation operand of each group, boxes of 1 .. 8 steps
   CUtensorMap w[2];      // weights of each group, 128 rows
 };
-// Workers (CTAs or clusters, `most` at most) for `tiles` tiles so that no half of a tile's K range is cut
-// more than once: pieces of half a tile or more, or two to four equal ones per tile.
-inline int halves_workers(long long tiles, int most) {
-  if (2 * tiles >= most) return most;
-  const long long per = most / tiles < 4 ? most / tiles : 4;
+// Workers (CTAs or clusters, `most` at most) for `tiles` tiles so that no part of a tile's K range is cut
+// more than once: pieces no shorter than a part, or equal ones whose cuts fall into different parts (of two
+// parts: 2, 3, 4 per tile; of four: 5, 6 and 8, but not 7).
+inline int fixed_order_workers(long long tiles, int most, int parts) {
+  if (parts * tiles >= most) return most;
+  long long per = most / tiles < 2 * parts ? most / tiles : 2 * parts;
+  if (parts == 4 && per == 7) per = 6;
   return (int)(tiles * per);
 }
 int stream_gemm_ksb(int R);
@@ -102,7 +104,8 @@ struct StreamPairParams {
   int R;
   float* out;
   int J, Rt;
-  size_t half_stride;
+  int parts;             // result matrices: 1, or 2 or 4 for as many equal parts of K
+  size_t part_stride;    // floats from one of them to the next
   const int* rows_dev;
   int* err;
 
@@ -115,6 +118,15 @@ struct StreamPairMaps {
   CUtensorMap a[2][8];   // activation operand of each group, boxes of 16, 32, .. 128 rows
   CUtensorMap w[2];      // weights of each group, 128 rows
 };
+// Parts of K for a pass of R rows whose bits must not depend on who adds first.  Two parts keep four clusters per
+// tile busy at most and four keep eight, but the kernel after the GEMM then reads and clears four matrices.
+// z2z_hyper_embed bounded to R rows, us with two parts -> with four: eight clusters per tile, d = 1024 192 / 384 /
+// 639 rows 138 -> 131, 198 -> 178, 288 -> 260, d = 2048 197 -> 178, 329 -> 297, 466 -> 414; six per tile, d = 3072
+// 300 / 384 / 639 rows 325 -> 333, 466 -> 458, 703 -> 654.
+inline int stream_pair_parts(long long tiles, int most, int ksteps, int R) {
+  const int pays = R >= 384 ? 5 : 8;                             // clusters per tile from which four parts pay
+  return pays * tiles <= most && ksteps % 4 == 0 ? 4 : 2;
+}
 bool stream_pair_act_maps(CUtensorMap* maps, const void* act, int Rt, int K);
 cudaError_t launch_stream_pair(StreamPairParams p, const StreamPairMaps& maps, int n_sm, cudaStream_t s);
 

@@ -203,7 +203,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
     int live = *p.rows_dev;
     live = live < p.R ? live : p.R;
     const int n_blocks = sp_live_blocks(p, live);
-    const int chain = p.half_stride ? p.ksteps / 2 : kSpChain;       // (K is a multiple of 128: the k-steps are even in number)
+    const int chain = p.parts > 1 ? p.ksteps / p.parts : kSpChain;
     if (warp == 1) {
       if (lane == 0 && rank == 0) {
         // ---------------- MMA issuer (leader only): D[256 weight rows][n] += W tile x activation rows -----
@@ -257,11 +257,11 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
         tc_fence_after();
         const int feature0 = j.wrow + (int)rank * 128;
         if (feature0 < p.J) {                          // the last tile may be half outside (J is a multiple of 128)
-          const size_t half = j.kb0 >= chain ? p.half_stride : 0;
+          const size_t part = p.parts > 1 ? (j.kb0 / chain) * p.part_stride : 0;
           const int row0 = j.block * kSpBlockRows;
           const int rows = live - row0 < kSpBlockRows ? live - row0 : kSpBlockRows;
           // this lane's row of every four, and the first of the four features it adds
-          float* dst = p.out + half + ((size_t)j.g * p.Rt + row0 + (lane & 3)) * p.J + feature0 + q * 32 + (lane & ~3);
+          float* dst = p.out + part + ((size_t)j.g * p.Rt + row0 + (lane & 3)) * p.J + feature0 + q * 32 + (lane & ~3);
           const uint32_t t0 = tmem_base + ((uint32_t)(q * 32) << 16);
           auto add4 = [&](float (&f)[4], int r) {      // rows r .. r + 3
             transpose4(f, lane);
@@ -312,7 +312,7 @@ bool stream_pair_act_maps(CUtensorMap* maps, const void* act, int Rt, int K) {
 }
 
 cudaError_t launch_stream_pair(StreamPairParams p, const StreamPairMaps& maps, int n_sm, cudaStream_t s) {
-  if (!p.out || !p.err || !p.rows_dev || p.R <= 128) return cudaErrorInvalidValue;
+  if (!p.out || !p.err || !p.rows_dev || p.R <= 128 || p.parts < 1 || p.ksteps % p.parts) return cudaErrorInvalidValue;
   p.tiles_per_group = (p.J + 255) / 256;
   p.blocks = (p.R + kSpBlockRows - 1) / kSpBlockRows;
   p.act_bytes = pair_act_bytes(p.R);
@@ -327,7 +327,7 @@ cudaError_t launch_stream_pair(StreamPairParams p, const StreamPairMaps& maps, i
   // d = 3072 180 rows of both encoders 426 -> 405 us, 384 811 -> 789, d = 1024 640 rows 343 -> 311; d = 2048 640 rows
   // lose, 664 -> 678).
   const int tiles = p.groups * p.tiles_per_group, whole = clusters / tiles * tiles;
-  if (p.half_stride) clusters = halves_workers(tiles, clusters);
+  if (p.parts > 1) clusters = fixed_order_workers(tiles, clusters, p.parts);
   else if (7 * whole >= 6 * clusters) clusters = whole;
   cudaError_t e = cudaFuncSetAttribute(k_stream_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;

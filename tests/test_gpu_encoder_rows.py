@@ -205,10 +205,11 @@ def test_whole_prompts_in_passes_cut_by_rows(M, d, dff):
         assert torch.all(p.E_f32[b, n[b]:] == 0)
 
 
-@pytest.mark.parametrize("d,dff", [(1024, 4096), (384, 1152)])
+@pytest.mark.parametrize("d,dff", [(1024, 4096), (384, 1152), (2560, 768)])
 @pytest.mark.parametrize("total", [16, 40, 43, 85, 86, 200])
 def test_a_bounded_call_gives_the_same_bits_every_time(d, dff, total):
-    """Sessions whose passes hold 1024 rows or more: on one CTA per tile, on pairs, in several row blocks."""
+    """Sessions whose passes hold 1024 rows or more: on one CTA per tile, on pairs, in several row blocks; the
+    pairs with eight (d = 1024) and six (2560) clusters per tile."""
     w, p = _pair(d, dff, 3, B=2, T=900, cap=600, seed=total)
     i32 = lambda x: torch.tensor(x, dtype=torch.int32, device=p.dev)
     count = [total // 2, total - total // 2]
