@@ -10,6 +10,7 @@ import pytest
 import torch
 
 from oracle import hyper_encoder as ohe
+from oracle import lzw as olzw
 from paper_2506_01084_b200 import binding as zb
 from paper_2506_01084_b200 import synth_inputs as si
 from tests._harness import Pair, TOL, f64
@@ -125,6 +126,42 @@ def test_steps_captured_first_hold_no_clear(B, tied):
             step()
         assert set(_node_types(graph)) == {0}
         step()
+
+
+@pytest.mark.parametrize("after_eager_steps", [False, True])
+def test_a_graph_replays_over_a_session_that_starts_again(after_eager_steps):
+    """The workspace holds anything when the session starts, and other rows exist in every replay."""
+    B = 40
+    w, p = _pair(256, 512, 3, B, T=64, cap=96, seed=B)
+    hid = si.make_hidden(w, B, 3).to(p.dev)
+    nxt, new, forced = (torch.zeros(B, dtype=torch.int32, device=p.dev) for _ in range(3))
+    lse = torch.zeros(B, device=p.dev)
+
+    def step():
+        zb.z2z_decode_step(p.cb, hid, p.g_WE, p.g_WU, p.g_encE, p.g_encU, p.E_h, p.U_h, zb.SELECT_ARGMAX, 1.0, 0, 0,
+                           forced, nxt, None, lse, new, p.E_f32, p.U_f32)
+
+    if after_eager_steps:
+        step()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        step()
+    p.cb.workspace.fill_(0x42)                                  # (48.6 as fp32)
+    zb.z2z_codebook_init(p.cb)
+    books = [olzw.Codebook(w.V, w.M, w.cap) for _ in range(B)]
+    for t in range(5):
+        codes = [(b + 31 * t) % w.V if t == 0 or (b + t) % (5 - t) == 0 else zb.CODE_NONE for b in range(B)]
+        forced.copy_(torch.tensor(codes, dtype=torch.int32))
+        graph.replay()
+        want = [-1 if z == zb.CODE_NONE else books[b].step(z) for b, z in enumerate(codes)]
+        assert new.cpu().tolist() == want
+        made = [b for b in range(B) if want[b] >= 0][::3]
+        for f32, W, enc in ((p.E_f32, p.W_E, p.enc_E), (p.U_f32, p.W_U, p.enc_U)):
+            if made:
+                rows = ohe.hyper_embed([books[b].entries[want[b]] for b in made], f64(W), [f64(x) for x in enc], w.heads)
+                got = torch.stack([f32[b, want[b]] for b in made]).double().cpu().numpy()
+                assert np.abs(got - rows).max() <= TOL
 
 
 def test_a_captured_session_start_clears_when_it_runs():
