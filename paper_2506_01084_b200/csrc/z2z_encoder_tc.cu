@@ -925,6 +925,7 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   const int ksb = paired ? 1 : stream_gemm_ksb(R);
   StreamGemmMaps maps;
   StreamPairMaps pair_maps;
+  int gemms = 0;
   auto gemm = [&](const MPtr2& act, int K, int widx, int J, int parts) -> cudaError_t {
     auto fill = [&](auto p) {
       p.groups = ng; p.ksteps = K / (64 * ksb); p.R = R; p.out = Y; p.J = J; p.Rt = Rt;
@@ -947,6 +948,7 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
     if (!make(maps, [&](int g) { return stream_gemm_act_maps(maps.a[g], act.p[g], Rt, K, R); })) return cudaErrorInvalidValue;
     StreamGemmParams p = fill(StreamGemmParams{});
     p.half_stride = hs;
+    p.peek = gemms++ > 0;              // (the first one starts before the count of its pass is there)
     return launch_stream_gemm(p, maps, n_sm, s);
   };
 

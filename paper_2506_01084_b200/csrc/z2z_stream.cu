@@ -199,9 +199,9 @@ __host__ __device__ constexpr uint32_t gemm_tmem_cols(int n_act) {
   return 2 * n_act <= 32 ? 32u : (2 * n_act <= 64 ? 64u : (2 * n_act <= 128 ? 128u : (2 * n_act <= 256 ? 256u : 512u)));
 }
 
-// Operand rows (hi and lo) of `live` packed rows, up to a multiple of `step`; at least one step.
+// Operand rows (hi and lo) of `live` > 0 packed rows, up to a multiple of `step`.
 __device__ __forceinline__ int gemm_op_rows(const StreamGemmParams& p, int live, int step) {
-  const int n = ((live < 1 ? 2 : 2 * live) + step - 1) / step * step;
+  const int n = (2 * live + step - 1) / step * step;
   return n < p.a_box_rows ? n : p.a_box_rows;
 }
 
@@ -217,6 +217,8 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
   const uint32_t a_bytes = (uint32_t)KSB * p.a_box_rows * 128;
   const uint32_t stage_bytes = a_bytes + (uint32_t)KSB * NT * 128;
   pdl_trigger();                                   // the next kernel may get resident behind this one
+  // (the word may still be that of the pass before: it only decides whether weights are loaded ahead)
+  const int hint = threadIdx.x == 0 && p.peek ? __ldcg(p.rows_dev) : 1;
   setup_barriers<STAGES>(ctrl);
   if (warp == 0 && lane == 0) { prefetch_tmap(&tm.w[0]); if (p.groups > 1) prefetch_tmap(&tm.w[1]); }
   __syncthreads();
@@ -235,7 +237,10 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
       // capacity brought 1.5 bytes of activations per byte of weights at 96 rows of which 55 were live,
       // and what an SM takes in from L2 bounds a batch of this size, not HBM: 546 -> 511 us per step of
       // 32 sequences at d = 4096, 251 -> 244 of 8 at d = 3072.)  With an ordinary launch the wait
-      // returns at once.
+      // returns at once.  A pass without a live row (a step that created no entry) streams nothing: the
+      // producer takes in what it loaded ahead, and the other roles have no work.  Such a step of one or 8
+      // sequences at d = 3072 went from 224 / 232 to 94 / 90 us (109 / 111 when every GEMM of it still filled
+      // its ring), of 32 at d = 4096 from 563 to 295; steps that create entries take what they took (245, 261, 580).
       const uint64_t pol_w = policy_evict_first(), pol_a = policy_evict_last();
       struct Deferred { int g, kb; };
       Deferred def[kMaxStages];                       // load i of the first pass uses stage i
@@ -245,7 +250,15 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
       auto need_deps = [&]() {
         if (deps) return;
         pdl_wait();
-        const int rows = gemm_op_rows(p, *p.rows_dev, p.box_step);
+        deps = true;
+        const int live = *p.rows_dev;
+        if (live < 1) {
+          ok = false;
+          for (int i = 0; i < n_def; ++i) mbar_arrive(smem_u32(&ctrl->full[i]));
+          for (int i = 0; i < n_def; ++i) mbar_wait(smem_u32(&ctrl->full[i]), 0, &ctrl->abort);
+          return;
+        }
+        const int rows = gemm_op_rows(p, live, p.box_step);
         box = rows / p.box_step - 1;
         box_bytes = (uint32_t)KSB * rows * 128;
         for (int i = 0; i < n_def; ++i) {
@@ -253,14 +266,15 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
           mbar_expect_tx(full, box_bytes);
           tma_load_3d(stage_base + (uint32_t)i * stage_bytes, &tm.a[def[i].g][box], 0, 0, def[i].kb, full, pol_a);
         }
-        deps = true;
       };
+      if (hint < 1) need_deps();
       int stage = 0; uint32_t phase = 0;
       GemmWalk walk(p);
       GemmJob j;
       while (ok && walk.next(j)) {
         for (int ks = j.kb0; ks < j.kb1; ++ks) {
           if (issued == STAGES) need_deps();
+          if (!ok) break;
           if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) { ok = false; break; }
           const uint32_t full = smem_u32(&ctrl->full[stage]);
           const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
@@ -283,7 +297,7 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
       const uint32_t box_kb = (uint32_t)gemm_op_rows(p, live, p.box_step) * 128;    // one k-block of the activation box
       const uint32_t idesc = idesc_bf16_f32(128, gemm_op_rows(p, live, 16));
       int stage = 0; uint32_t phase = 0, job_i = 0;
-      bool ok = true;
+      bool ok = live > 0;
       GemmWalk walk(p);
       GemmJob j;
       while (ok && walk.next(j)) {
@@ -326,7 +340,7 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
     uint32_t job_i = 0;
     GemmWalk walk(p);
     GemmJob j;
-    while (walk.next(j)) {
+    while (rows > 0 && walk.next(j)) {
       const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
       if (!mbar_wait(smem_u32(&ctrl->acc_full[buf]), aph, &ctrl->abort)) break;
       tc_fence_after();

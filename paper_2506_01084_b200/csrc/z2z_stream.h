@@ -74,6 +74,7 @@ struct StreamGemmParams {
   int J, Rt;
   size_t half_stride;    // floats from the result matrix of K's first half to that of its second, or 0
   const int* rows_dev;   // device word: packed rows that carry data (<= R)
+  int peek;              // look at it before the preceding kernel is done: no weights ahead when it holds 0
   int* err;
 
   int tiles_per_group;

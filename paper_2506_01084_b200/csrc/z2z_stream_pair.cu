@@ -84,10 +84,10 @@ struct SpWalk {
 };
 
 // Columns of tensor memory (the MMA's N, a multiple of 32) that half `h` of a row block takes, 0 if it has
-// no live row; the first half of a block always counts as having one.
+// no live row.
 __device__ __forceinline__ int sp_cols(int live, int block, int h) {
   int rows = live - block * kSpBlockRows - h * kSpHalfRows;
-  if (rows < 1) rows = (h == 0) ? 1 : 0;
+  if (rows < 1) return 0;
   if (rows > kSpHalfRows) rows = kSpHalfRows;
   return (2 * rows + 31) & ~31;
 }
@@ -169,11 +169,21 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
         pdl_wait();
         live = *p.rows_dev;
         live = live < p.R ? live : p.R;
+        deps = true;
+        if (live < 1) {
+          // a pass without a row: the leader takes in what both CTAs loaded ahead, and the peer stays until then
+          // (the cluster leaves together).  Such a step of 90 sequences, d = 3072, one encoder: 270 -> 145 us.
+          ok = false;
+          if (rank == 0) {
+            for (int i = 0; i < n_def; ++i) mbar_arrive(smem_u32(&ctrl->full[i]));
+            for (int i = 0; i < n_def; ++i) mbar_wait(smem_u32(&ctrl->full[i]), 0, &ctrl->abort);
+          }
+          return;
+        }
         for (int i = 0; i < n_def; ++i) {
           if (rank == 0) mbar_expect_tx(smem_u32(&ctrl->full[i]), 2 * act_bytes(def[i].block));
           load_act(i, def[i], def[i].kb0);
         }
-        deps = true;
       };
       if (p.blocks > 1) need_deps();                   // the walk itself depends on the row count
       int stage = 0; uint32_t phase = 0;
@@ -182,6 +192,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
       while (ok && walk.next(j)) {
         for (int ks = j.kb0; ks < j.kb1; ++ks) {
           if (issued == STAGES) need_deps();
+          if (!ok) break;
           if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) { ok = false; break; }
           if (rank == 0) {
             const uint32_t full = smem_u32(&ctrl->full[stage]);
@@ -208,7 +219,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
       if (lane == 0 && rank == 0) {
         // ---------------- MMA issuer (leader only): D[256 weight rows][n] += W tile x activation rows -----
         int stage = 0; uint32_t phase = 0, job_i = 0;
-        bool ok = true;
+        bool ok = live > 0;
         SpWalk walk(p, n_blocks, chain);
         SpJob j;
         while (ok && walk.next(j)) {
@@ -251,7 +262,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
       uint32_t job_i = 0;
       SpWalk walk(p, n_blocks, chain);
       SpJob j;
-      while (walk.next(j)) {
+      while (live > 0 && walk.next(j)) {
         const uint32_t aph = job_i & 1u;
         if (!mbar_wait(smem_u32(&ctrl->acc_full), aph, &ctrl->abort)) break;
         tc_fence_after();

@@ -388,6 +388,28 @@ def test_decode_steps_settle_what_was_embedded_by_range():
         assert torch.all(p.E_f32[b, int(m[b])] != -5) and torch.all(p.E_f32[b, :int(m[b])] == -5)
 
 
+@pytest.mark.parametrize("d,dff,total", [(2560, 768, 40), (2560, 768, 80), (384, 512, 200)])
+def test_a_bounded_call_without_an_entry_streams_nothing(d, dff, total):
+    """Calls whose ranges are empty between calls that embed some: on one CTA per tile and on pairs, with weights
+    for more than the load ring (d = 2560), in several row blocks."""
+    w, p = _pair(d, dff, 3, B=2, T=900, cap=600, seed=total)
+    i32 = lambda x: torch.tensor(x, dtype=torch.int32, device=p.dev)
+    some = [total // 2 - 3, total - total // 2]
+    assert all(p.oracle.books[b].n() >= total - total // 2 for b in range(2))
+    want = None
+    for count in ([0, 0], some, [0, 0], [0, 0], some):
+        f32 = torch.full((2, w.cap, d), -5.0, dtype=torch.float32, device=p.dev)
+        zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, i32([3, 0]), i32(count), total, p.E_h, f32)
+        if count == some:
+            want = f32 if want is None else want
+            assert torch.equal(f32, want)
+        else:
+            assert torch.all(f32 == -5)
+    _check(w, p, want, [3, 0], some)
+    st, _ = zb.z2z_status(p.cb)
+    assert all(int(x) & zb.ST_WAIT_TIMEOUT == 0 for x in st)
+
+
 def test_exact_call_beside_joint_logits_on_another_stream():
     """The two calls share no scratch: the input side of a prompt may be embedded while positions are scored."""
     w, p = _pair(256, 512, 3, B=4, T=3000, cap=1200, seed=3)
