@@ -71,6 +71,7 @@ z2z::EntryList entry_list(z2z_codebook* cb) {
   el.row_off = reinterpret_cast<int32_t*>(cb->ws + cb->plan.off_row_off);
   el.row_src = reinterpret_cast<int32_t*>(cb->ws + cb->plan.off_row_src);
   el.row_tok = reinterpret_cast<int32_t*>(cb->ws + cb->plan.off_row_tok);
+  el.row_uniq = reinterpret_cast<int32_t*>(cb->ws + cb->plan.off_row_uniq);
   el.off = reinterpret_cast<int32_t*>(cb->ws + cb->plan.off_entry_off);
   el.chunk = cb->plan.enc_chunk_entries;
   el.list = cb->plan.enc_list;

@@ -65,7 +65,7 @@ struct WsPlan {
   int enc_list;               // entries the work list of a pass can hold: passes cut by rows may hold more
                               // entries than enc_chunk_entries, at two rows or more each
   size_t off_hash, off_cons, off_len, off_n, off_prev, off_status, off_n_emb, state_end;
-  size_t off_entry_seq, off_entry_idx, off_entry_len, off_entry_tok, off_row_off, off_row_src, off_row_tok, off_entry_off, off_new_entry, off_sel;
+  size_t off_entry_seq, off_entry_idx, off_entry_len, off_entry_tok, off_row_off, off_row_src, off_row_tok, off_row_uniq, off_entry_off, off_new_entry, off_sel;
   size_t off_X, off_A, off_QKV, off_H;            // fp32 encoder activations
   size_t off_Ahl, off_Hhl;                        // bf16 hi/lo activations (tensor-core path)
   size_t off_g1_X, off_g1_QKV, off_g1_Ahl, off_g1_Hhl;   // second encoder of the decode step
@@ -116,6 +116,7 @@ inline WsPlan plan_workspace(const z2z_config& c) {
   p.off_row_off = take((list + 1) * 4);
   p.off_row_src = take((size_t)chunk * c.M * 4);
   p.off_row_tok = take((size_t)chunk * c.M * 4);
+  p.off_row_uniq = take(((size_t)chunk * c.M + 1) * 4);
   p.off_entry_off = take((size_t)(c.B + 2) * 4);
   p.off_new_entry = take((size_t)c.B * 4);
   p.off_sel = take((size_t)c.B * 4 * 4);
@@ -162,6 +163,32 @@ template <typename T> __device__ __forceinline__ T from_f32(float x);
 template <> __device__ __forceinline__ float from_f32<float>(float x) { return x; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(float x) {
   return __float2bfloat16_rn(x);
+}
+
+// Exclusive sum over the 1024 threads of a block; warp_sums: 32 words of shared memory.
+__device__ __forceinline__ int block_scan_1024(int v, int* warp_sums, int& total) {       // exclusive
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += x;
+  }
+  __syncthreads();                                 // (the sums may still be read by an earlier scan)
+  if (lane == 31) warp_sums[warp] = inc;
+  __syncthreads();
+  if (warp == 0) {
+    int w = warp_sums[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += x;
+    }
+    warp_sums[lane] = w;
+  }
+  __syncthreads();
+  total = warp_sums[31];
+  return inc - v + (warp > 0 ? warp_sums[warp - 1] : 0);
 }
 
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw: "Parallel random numbers: as easy as 1, 2, 3",

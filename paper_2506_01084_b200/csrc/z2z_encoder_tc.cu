@@ -455,12 +455,20 @@ __global__ void k_tc_qkv_attention(CbView cb, EntryList el, float* Y, size_t par
 // last entry slot, the way back from a packed row to (entry, position) and the row's base token.
 // E <= 1024 * kMapPerThread entries, neighbouring ones per thread.  (The decode step's update kernel
 // writes the same map itself.)
+//
+// UNIQ: also finds the rows that are alike.  Up to the first attention a row depends on its base token and its place in
+// the entry only, and the rows of a pass repeat them (of 3072 rows of prompts with vocabulary 32064 a third are
+// distinct, of 2304 with 128256 a quarter): LayerNorm and the q, k, v products run on the distinct ones, numbered by
+// first appearance.  Dynamic shared memory: uniq_slots words of a hash table of first rows, then the rows' keys.
 constexpr int kMapPerThread = kMaxM / 2;
-__global__ void __launch_bounds__(1024) k_tc_row_map(CbView cb, EntryList el, int E) {
+template <bool UNIQ>
+__global__ void __launch_bounds__(1024) k_tc_row_map(CbView cb, EntryList el, int E, int uniq_slots, int R) {
   __shared__ int warp_sums[32];
+  extern __shared__ uint32_t s_first[];
+  uint32_t* s_key = s_first + uniq_slots;
   sm100::pdl_trigger();
   sm100::pdl_wait();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   const int per = (E + 1023) / 1024, e0 = tid * per;
   int len[kMapPerThread], mine = 0;
 #pragma unroll
@@ -468,41 +476,61 @@ __global__ void __launch_bounds__(1024) k_tc_row_map(CbView cb, EntryList el, in
     len[q] = q < per && e0 + q < E ? entry_len_tc(cb, el, e0 + q) : 0;
     mine += len[q];
   }
-  int inc = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int x = __shfl_up_sync(0xffffffffu, inc, o);
-    if (lane >= o) inc += x;
-  }
-  if (lane == 31) warp_sums[warp] = inc;
-  __syncthreads();
-  if (warp == 0) {
-    int w = warp_sums[lane];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int x = __shfl_up_sync(0xffffffffu, w, o);
-      if (lane >= o) w += x;
-    }
-    warp_sums[lane] = w;
-  }
-  __syncthreads();
-  int row = inc - mine + (warp > 0 ? warp_sums[warp - 1] : 0);
+  int rows;
+  int row = block_scan_1024(mine, warp_sums, rows);
 #pragma unroll
   for (int q = 0; q < kMapPerThread; ++q) {
     if (q >= per || e0 + q >= E) break;
     el.row_off[e0 + q] = row;
     for (int i = 0; i < len[q]; ++i) {
+      const int tok = el.tok[(size_t)(e0 + q) * cb.M + i];
       el.row_src[row + i] = (e0 + q) * cb.M + i;
-      el.row_tok[row + i] = el.tok[(size_t)(e0 + q) * cb.M + i];
+      el.row_tok[row + i] = tok;
+      if (UNIQ && row + i < R) s_key[row + i] = (uint32_t)tok * kMaxM + i;
     }
     row += len[q];
   }
-  if (tid == 0) el.row_off[E] = warp_sums[31];
+  if (tid == 0) el.row_off[E] = rows;
+  if (!UNIQ) return;
+  rows = rows < R ? rows : R;
+  for (int i = tid; i < uniq_slots; i += 1024) s_first[i] = ~0u;
+  __syncthreads();
+  // every row bids for the slot of its key: the lowest row of a kind keeps it
+  const int rper = (rows + 1023) / 1024, r0 = tid * rper;      // at most kMaxM rows per thread, neighbouring ones
+  int slot[kMaxM], fresh = 0;
+#pragma unroll
+  for (int q = 0; q < kMaxM; ++q) {
+    slot[q] = -1;
+    if (q >= rper || r0 + q >= rows) continue;
+    const uint32_t key = s_key[r0 + q];
+    uint32_t at = (key * 0x9E3779B1u >> 8) & (uint32_t)(uniq_slots - 1);
+    for (int it = 0; it < uniq_slots; ++it) {                  // bounded; half of the slots stay empty
+      const uint32_t old = atomicCAS(s_first + at, ~0u, (uint32_t)(r0 + q));
+      if (old == ~0u) break;
+      if (s_key[old] == key) { atomicMin(s_first + at, (uint32_t)(r0 + q)); break; }
+      at = (at + 1) & (uint32_t)(uniq_slots - 1);
+    }
+    slot[q] = (int)at;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < kMaxM; ++q)
+    if (slot[q] >= 0 && s_first[slot[q]] == (uint32_t)(r0 + q)) ++fresh;
+  int kinds;
+  int u = block_scan_1024(fresh, warp_sums, kinds);
+#pragma unroll
+  for (int q = 0; q < kMaxM; ++q)
+    if (slot[q] >= 0 && s_first[slot[q]] == (uint32_t)(r0 + q)) { s_key[r0 + q] = u; el.row_uniq[r0 + q] = u | kFirstOfKind; ++u; }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < kMaxM; ++q)
+    if (slot[q] >= 0 && s_first[slot[q]] != (uint32_t)(r0 + q)) el.row_uniq[r0 + q] = (int)s_key[s_first[slot[q]]];
+  if (tid == 0) el.row_uniq[el.chunk * cb.M] = kinds;
 }
 
-// X = table[y] + pos for every packed row, then LN1 of layer 0 -> hi/lo.  grid (row capacity).
+// X = table[y] + pos for every packed row, then LN1 of layer 0 -> hi/lo (uniq: of the distinct rows).  grid (row capacity).
 template <int NV, bool HALF>
-__global__ void __launch_bounds__(kRowThreads) k_tc_gather_ln_packed(CbView cb, EntryList el, const int* total,
+__global__ void __launch_bounds__(kRowThreads) k_tc_gather_ln_packed(CbView cb, EntryList el, const int* total, const int* uniq,
                                                                      const bf16* table, const bf16* pos, const bf16* ln_w,
                                                                      const bf16* ln_b, float* X, bf16* Ahl, int d, int Rt,
                                                                      int has_ln) {
@@ -512,9 +540,10 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_gather_ln_packed(CbView cb, 
   const int r = blockIdx.x;
   if (r >= *total) return;
   const int src = el.row_src[r];
+  const int u = uniq ? uniq[r] : r | kFirstOfKind;
   const int y = el.tok[src], i = src % cb.M;
   float* x = X + (size_t)r * d;
-  bf16* hi = Ahl + (size_t)r * d;
+  bf16* hi = Ahl + (size_t)(u & ~kFirstOfKind) * d;
   const bf16* row = table + (size_t)y * d;
   const bf16* pp = pos + (size_t)i * d;
   const int nvec = d / 4;
@@ -531,7 +560,7 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_gather_ln_packed(CbView cb, 
       *reinterpret_cast<float4*>(x + idx * 4) = xv[v];
     }
   }
-  if (has_ln) layernorm_split_regs<NV, HALF>(xv, nvec, gw, gb, hi, hi + (size_t)Rt * d, d, sm);
+  if (has_ln && u < 0) layernorm_split_regs<NV, HALF>(xv, nvec, gw, gb, hi, hi + (size_t)Rt * d, d, sm);
 }
 
 // Mean-pool on packed rows: cache row = mean of the entry's rows of X.  grid (entries,
@@ -595,8 +624,8 @@ __global__ void __launch_bounds__(kRowThreads) k_tc_ln_rows(const int* total, co
 // warp reductions, no shared memory and no block barrier.  MM = compile-time bound on the merge
 // size; dh <= 128 (larger heads take the kernel below).  grid = ceil(entries * heads / 8), block 256.
 template <int MM, bool HALF>
-__global__ void __launch_bounds__(256) k_tc_attention_rows_warp(CbView cb, EntryList el, const float* QKV, bf16* Ohl,
-                                                                int E, int d, int heads, int Rt) {
+__global__ void __launch_bounds__(256) k_tc_attention_rows_warp(CbView cb, EntryList el, const float* QKV,
+                                                                const int* uniq, bf16* Ohl, int E, int d, int heads, int Rt) {
   sm100::pdl_trigger();
   sm100::pdl_wait();
   const int lane = threadIdx.x & 31;
@@ -608,13 +637,16 @@ __global__ void __launch_bounds__(256) k_tc_attention_rows_warp(CbView cb, Entry
   const int dh = d / heads, c = lane * 4;
   const bool on = c < dh;                      // lanes beyond the head's width hold zeros
   const size_t r0 = el.row_off[e];
-  const float* y = QKV + r0 * 3 * d + (size_t)h * dh + c;
+  const float* y = QKV + (size_t)h * dh + c;
+  size_t at[MM];
+#pragma unroll
+  for (int i = 0; i < MM; ++i) at[i] = i < L && uniq ? uniq[r0 + i] & ~kFirstOfKind : r0 + i;
   float4 q[MM], k[MM], v[MM];
 #pragma unroll
   for (int i = 0; i < MM; ++i) {
     q[i] = k[i] = v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     if (i < L && on) {
-      const float* yi = y + (size_t)i * 3 * d;
+      const float* yi = y + at[i] * 3 * d;
       q[i] = *reinterpret_cast<const float4*>(yi);
       k[i] = *reinterpret_cast<const float4*>(yi + d);
       v[i] = *reinterpret_cast<const float4*>(yi + 2 * d);
@@ -655,8 +687,8 @@ __global__ void __launch_bounds__(256) k_tc_attention_rows_warp(CbView cb, Entry
 
 // The same for heads wider than 128 columns or merge sizes above 4: staged in shared memory.
 // grid (entries, heads), block (32, M), dynamic smem M * 3 * dh floats.
-__global__ void k_tc_attention_rows(CbView cb, EntryList el, const float* QKV, bf16* Ohl, int d, int heads, int Rt,
-                                    int half) {
+__global__ void k_tc_attention_rows(CbView cb, EntryList el, const float* QKV, const int* uniq, bf16* Ohl, int d, int heads,
+                                    int Rt, int half) {
   extern __shared__ float s_qkv[];
   sm100::pdl_trigger();
   sm100::pdl_wait();
@@ -666,7 +698,7 @@ __global__ void k_tc_attention_rows(CbView cb, EntryList el, const float* QKV, b
   const int dh = d / heads;
   const int r = el.row_off[e] + i;
   if (i < L) {
-    const float* y = QKV + (size_t)r * 3 * d;
+    const float* y = QKV + (size_t)(uniq ? uniq[r] & ~kFirstOfKind : r) * 3 * d;
     for (int w = 0; w < 3; ++w)
       for (int c = lane * 4; c < dh; c += 128)
         *reinterpret_cast<float4*>(&s_qkv[(i * 3 + w) * dh + c]) = *reinterpret_cast<const float4*>(y + w * d + h * dh + c);
@@ -771,26 +803,43 @@ static cudaError_t run_encoder_pass_pair(const CbView& cb, const EncoderArgs& a,
     return launch_pair_gemm(p, act, half ? a.w_half[widx] : a.w[widx], K, epi, half, s);
   };
   cudaError_t e;
+  // The q, k, v of the first layer on the distinct rows, where that can save row tiles: two of them take the
+  // clusters one wave, as one does.  (The map takes 9 us instead of 3.5; 8 prompts of 2048 tokens, d = 3072,
+  // 19.8 -> 18.4 ms, 16 of 8192 with their positions scored, d = 4096, single operand, 145 -> 137 ms.)
+  const bool uniq = a.layers > 0 && R > 512;
+  const int* row_uniq = uniq ? el.row_uniq : nullptr;
   {
     ProfScope ps(prof, kProfEncOther, 2, s);
-    if ((e = launch_pdl(k_tc_row_map, dim3(1), dim3(1024), 0, s, cb, el, E)) != cudaSuccess) return e;
+    if (uniq) {
+      int slots = 2048;
+      while (slots < 2 * R) slots *= 2;
+      const size_t smem = (size_t)(slots + R) * 4;
+      if ((e = cudaFuncSetAttribute(k_tc_row_map<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+      e = launch_pdl(k_tc_row_map<true>, dim3(1), dim3(1024), smem, s, cb, el, E, slots, R);
+    } else {
+      e = launch_pdl(k_tc_row_map<false>, dim3(1), dim3(1024), 0, s, cb, el, E, 0, 0);
+    }
+    if (e != cudaSuccess) return e;
     auto gk = half ? (narrow ? k_tc_gather_ln_packed<kNarrowVec4, true> : k_tc_gather_ln_packed<kMaxVec4, true>)
                    : (narrow ? k_tc_gather_ln_packed<kNarrowVec4, false> : k_tc_gather_ln_packed<kMaxVec4, false>);
-    e = launch_pdl(gk, dim3(R), dim3(kRowThreads), 0, s, cb, el, total, reinterpret_cast<const bf16*>(a.table), Wp(0),
+    e = launch_pdl(gk, dim3(R), dim3(kRowThreads), 0, s, cb, el, total, row_uniq, reinterpret_cast<const bf16*>(a.table), Wp(0),
                    a.layers ? Wp(1) : Wp(0), a.layers ? Wp(2) : Wp(0), a.X, a.Ahl, d, Rt, a.layers > 0 ? 1 : 0);
     if (e != cudaSuccess) return e;
   }
   const int dh = d / a.heads;
   for (int l = 0; l < a.layers; ++l) {
     const int o = 1 + 12 * l;
+    const int* at = l == 0 ? row_uniq : nullptr;
+    g.live_rows = at ? at + (size_t)el.chunk * M : total;
     if ((e = gemm(a.Ahl, d, o + 2, 3 * d, kEpiStore, a.QKV, nullptr)) != cudaSuccess) return e;
+    g.live_rows = total;
     {
       ProfScope ps(prof, kProfEncOther, 1, s);
       if (dh <= 128 && M <= 4) {
         auto ak = half ? k_tc_attention_rows_warp<4, true> : k_tc_attention_rows_warp<4, false>;
-        e = launch_pdl(ak, dim3((E * a.heads + 7) / 8), dim3(256), 0, s, cb, el, a.QKV, a.Ahl, E, d, a.heads, Rt);
+        e = launch_pdl(ak, dim3((E * a.heads + 7) / 8), dim3(256), 0, s, cb, el, a.QKV, at, a.Ahl, E, d, a.heads, Rt);
       } else {
-        e = launch_pdl(k_tc_attention_rows, dim3(E, a.heads), dim3(32, M), (size_t)M * 3 * dh * 4, s, cb, el, a.QKV, a.Ahl, d,
+        e = launch_pdl(k_tc_attention_rows, dim3(E, a.heads), dim3(32, M), (size_t)M * 3 * dh * 4, s, cb, el, a.QKV, at, a.Ahl, d,
                        a.heads, Rt, half ? 1 : 0);
       }
       if (e != cudaSuccess) return e;
@@ -959,7 +1008,7 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
 
   if (!rows_mapped) {
     ProfScope ps(prof, kProfEncOther, 1, s);
-    launch_pdl(k_tc_row_map, dim3(1), dim3(1024), 0, s, cb, el, E);
+    launch_pdl(k_tc_row_map<false>, dim3(1), dim3(1024), 0, s, cb, el, E, 0, 0);
   }
   cudaError_t e;
   {

@@ -52,10 +52,13 @@ struct EntryList {
                       //              behind the last entry slot of the pass
   int32_t* row_src;   // [chunk * M]  tensor-core passes: packed row -> entry * M + position
   int32_t* row_tok;   // [chunk * M]  tensor-core passes: base token of each packed row
+  int32_t* row_uniq;  // [chunk * M + 1]  prompt-sized passes: packed row -> row of its (base token, position) among the
+                      //              distinct ones, | kFirstOfKind in the first such row; their number behind the last
   int32_t* off;       // [B + 2]  exclusive prefix sum of per-sequence counts, then the total
   int chunk;          // entries of a pass cut by entries
   int list;           // entries the work list can hold
 };
+constexpr int32_t kFirstOfKind = (int32_t)0x80000000;
 struct EncoderArgs {
   int d, dff, heads, layers, M;
   int dtype;

@@ -443,6 +443,27 @@ def test_exact_call_beside_joint_logits_on_another_stream():
         assert all(torch.equal(x, want_lse) for x in lse) and all(torch.equal(x, want_rows) for x in rows)
 
 
+@pytest.mark.parametrize("M,heads", [(2, 2), (4, 2), (7, 2), (3, 1)])
+def test_rows_that_are_alike_share_the_first_layers_products(M, heads):
+    """A pass of more than 512 rows computes q, k, v once per (base token, position); a short one does not.  The same
+    bits, on both attention kernels (merge sizes up to 4 with heads of up to 128 columns, and others)."""
+    w = si.Workload("alike", V=40, d=256, dtype="bf16", B=3, T=2500, M=M, cap=900, zipf_s=1.0, copy_p=0.5, seg_min=4, seg_max=14,
+                    steps=2, enc_layers=2, enc_heads=heads, enc_dff=512)
+    p = Pair(w, 5)
+    p.gpu_encode()
+    n = zb.z2z_status(p.cb)[1].tolist()
+    assert 512 < int(sum(n)) and min(n) > 40
+    i32 = lambda x: torch.tensor(x, dtype=torch.int32, device=p.dev)
+    f32 = torch.full((3, w.cap, 256), -5.0, device=p.dev)
+    zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, i32([0] * 3), i32(n), -1, p.E_h, f32)
+    part = torch.full((3, w.cap, 256), -5.0, device=p.dev)
+    last = [k - 17 for k in n]
+    zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, i32(last), i32([17] * 3), -1, p.E_h, part)
+    for b in range(3):
+        assert torch.equal(f32[b, last[b]:n[b]], part[b, last[b]:n[b]])
+        assert torch.all(f32[b, n[b]:] == -5)
+
+
 def test_exact_rows_do_not_depend_on_the_rest_of_the_call():
     """A few entries alone, in a call of one pass and in a call of several: the same bits."""
     w, p = _pair(256, 512, 3, B=3, T=3000, cap=1400, seed=12)
