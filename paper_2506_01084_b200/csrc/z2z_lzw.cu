@@ -38,12 +38,14 @@ static_assert(kEmptySlot == ~0ull, "an empty slot is all ones");
 // Which positions start a phrase is a walk position -> position + match length: inside a warp by
 // pointer doubling (five rounds carry the set of visited lanes and the exit), across the
 // warps by looking up the exit of one as the entry of the next (a match is at most kMaxM long, so
-// only the first kMaxM lanes of a warp can be entered).
+// only the first kMaxM lanes of a warp can be entered: a warp's exits fit one word, four bits each).
 //
-// Bound by the latency of one window (a few dependent shared-memory lookups, ten shuffles, four
+// Bound by the latency of one window (a few dependent shared-memory lookups, ten shuffles, three
 // barriers).  The chain used to be walked token by token by one thread: 180 ns per token with the
 // table in shared memory, 220 with it in global memory.  Four texts of 32768 tokens (cap 16384), to
-// codes and back with both session resets: 9.62 ms before, 0.65 ms with windows here and in the replay.
+// codes and back with both session resets: 9.62 ms before, 0.65 ms with windows here and in the replay, 0.56 with
+// three barriers a window instead of four (four instead of six there), exits in one word and entries written back
+// four at a time.
 template <int LANES, bool SMEM>
 __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_encode(CbView cb, const int32_t* __restrict__ tokens,
                                                               const int32_t* __restrict__ lens, int T_max,
@@ -53,9 +55,11 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_encode(CbView cb, 
   constexpr int WARPS = LANES / 32, kTokRing = 2 * LANES;      // (a window's tokens and a match behind it fit the ring)
   extern __shared__ __align__(16) unsigned char s_parse[];
   __shared__ int s_tok[kTokRing];                    // token of position p at p mod kTokRing
-  __shared__ int2 s_walk[WARPS][kMaxM];        // per warp and entry lane: lanes visited, exit
+  __shared__ uint32_t s_exit[WARPS];           // per warp, four bits per entry lane: the next warp's entry lane
   __shared__ ParseVotes<WARPS> s_votes;
-  __shared__ int s_prev, s_n1, s_st;
+  __shared__ int s_prev, s_n1, s_st, s_lost[2];      // first loser of this window, of the next one
+  static_assert(kMaxM * 4 <= 32, "a warp's exits fit one word");
+  constexpr uint32_t kInputEnd = 15;           // instead of an entry lane
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
   const int V = cb.V, M = cb.M, cap = cb.cap;
@@ -65,7 +69,7 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_encode(CbView cb, 
   const int32_t* x = tokens + (size_t)b * T_max;
   ParseTable<SMEM> table;
   table.open(cb, b, n0, s_parse);
-  if (tid == 0) { s_prev = -1; s_st = 0; s_n1 = n0; }
+  if (tid == 0) { s_prev = -1; s_st = 0; s_n1 = n0; s_lost[0] = s_lost[1] = LANES; }
   __syncthreads();
   if (tid < LANES) {
     int32_t* out = codes + (size_t)b * T_max;
@@ -73,7 +77,7 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_encode(CbView cb, 
     int n = n0, n_out = 0, st = 0;
     int loaded = 0;                                  // tokens already in s_tok
     int ahead = tid < T ? x[tid] : 0;                // token loaded + tid
-    for (int p0 = 0; p0 < T;) {                      // p0: a phrase starts here
+    for (int p0 = 0, par = 0; p0 < T; par ^= 1) {    // p0: a phrase starts here
       // Positions below p0 + LANES + kMaxM are looked at; the ring is filled as far as it goes, so
       // that a token has been on its way for a window before it is stored.  (A window moves p0 by 257 on
       // average where no phrase repeats in it: with nothing in reserve every other window would wait for
@@ -99,8 +103,10 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_encode(CbView cb, 
       bool miss = false;
       if (live) {
         w = s_tok[q & (kTokRing - 1)];
+        int next = s_tok[(q + 1) & (kTokRing - 1)];            // (the ring's slot is there whether or not its token is)
         while (len < M && q + len < T) {
-          c = s_tok[(q + len) & (kTokRing - 1)];
+          c = next;
+          next = s_tok[(q + len + 1) & (kTokRing - 1)];
           const int e = table.probe((uint32_t)w, (uint32_t)c, slot);
           if (e < 0) { miss = true; break; }
           w = V + e; ++len;
@@ -115,41 +121,42 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_encode(CbView cb, 
         const int t2 = __shfl_sync(0xffffffffu, to, to & 31);
         if (to < 32) { visited |= v2; to = t2; }
       }
-      if (lane < kMaxM) s_walk[warp][lane] = make_int2((int)visited, warp * 32 + to);
+      const uint32_t exits = __reduce_or_sync(0xffffffffu, lane < kMaxM ? (to >= 32 ? (uint32_t)(to - 32) : kInputEnd) << (4 * lane) : 0u);
+      if (lane == 0) s_exit[warp] = exits;
       parse_sync<LANES>();
-      uint32_t mine = 0;
-      int at = 0;                                    // entry into warp k, then the window's exit
+      if (tid == 0) s_lost[par ^ 1] = LANES;         // (read ahead of this window's first barrier)
+      uint32_t at = 0, entered = kInputEnd;          // entry lane of warp k, and of this thread's
 #pragma unroll
       for (int k = 0; k < WARPS; ++k) {
-        if ((at >> 5) == k) {                        // (a walk that reached the end of the input stays where it is)
-          const int2 wk = s_walk[k][at & 31];
-          if (k == warp) mine = (uint32_t)wk.x;
-          at = wk.y;
-        }
+        if (k == warp) entered = at;
+        if (at != kInputEnd) at = (s_exit[k] >> (4 * at)) & 15u;
       }
-      const bool on = (mine >> lane) & 1u;
+      const uint32_t chain = __shfl_sync(0xffffffffu, visited, (int)entered);
+      const bool on = entered != kInputEnd && ((chain >> lane) & 1u);
       // ---- new phrases of the chain bid for their slots
       const bool ins = on && miss && n < cap && slot >= 0;
       if (on && miss && n < cap && slot < 0) st |= Z2Z_ST_TABLE_FULL;
-      if (ins) table.bid(slot, tid);
-      parse_sync<LANES>();
-      const bool own = ins && table.owns(slot, tid);
+      if (ins) {
+        const int loser = table.bid(slot, tid, LANES);
+        if (loser < LANES) atomicMin(&s_lost[par], loser);
+      }
       const uint32_t v_on = __ballot_sync(0xffffffffu, on), v_ins = __ballot_sync(0xffffffffu, ins);
-      const uint32_t v_lost = __ballot_sync(0xffffffffu, ins && !own);
-      if (lane == 0) { s_votes.on[warp] = v_on; s_votes.ins[warp] = v_ins; s_votes.lost[warp] = v_lost; }
+      if (lane == 0) { s_votes.on[warp] = v_on; s_votes.ins[warp] = v_ins; }
       parse_sync<LANES>();
       const ParseVotes<WARPS> votes = s_votes;
-      const int stop = parse_first_lost(votes.lost); // lanes below it are final
+      const int stop = s_lost[par];                  // lanes below it are final
       const int room = cap - n;
       int made, emitted;
       const int new_before = parse_rank(votes.ins, warp, lane, made), on_before = parse_rank(votes.on, warp, lane, emitted);
       if (stop < LANES) { made = parse_count_below(votes.ins, stop); emitted = parse_count_below(votes.on, stop); }
-      if (own) {
-        const int entry = tid < stop && new_before < room ? n + new_before : -1;
-        table.settle(slot, (uint32_t)w, (uint32_t)c, entry);
-        if (entry >= 0) {                            // the phrase and its next token: input from q on (expanded below)
+      if (ins) {
+        if (tid < stop && new_before < room) {       // the phrase and its next token: input from q on (expanded below)
+          const int entry = n + new_before;
+          table.settle(slot, (uint32_t)w, (uint32_t)c, entry);
           cb.cons[((size_t)b * cap + entry) * M] = q;
           cb.len[(size_t)b * cap + entry] = (uint8_t)(len + 1);
+        } else {
+          table.withdraw(slot, tid);
         }
       }
       if (on && tid < stop) {
@@ -164,9 +171,9 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_encode(CbView cb, 
         if (n >= cap) st |= Z2Z_ST_CAP_FROZEN;
       }
       n_out += emitted;
-      p0 += stop < LANES ? stop : at;
+      p0 = stop < LANES ? p0 + stop : at == kInputEnd ? T : p0 + LANES + (int)at;
       // (the barrier at the head of the next window orders these writes before its lookups; s_votes
-      // and s_walk are rewritten behind further barriers)
+      // and s_exit are rewritten behind further barriers)
     }
     if (st) atomicOr(&s_st, st);
     if (tid == 0) { code_lens[b] = n_out; s_n1 = n; }
@@ -178,14 +185,28 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_encode(CbView cb, 
     if (s_st) atomicOr(&cb.status[b], s_st);
   }
   table.close(n0, s_n1);
-  // constituent rows of the entries created here: tokens [start, start + len), -1 padded
-  for (int e = n0 + tid; e < s_n1; e += blockDim.x) {
-    int32_t* row = cb.cons + ((size_t)b * cap + e) * M;
-    const int start = row[0], L = cb.len[(size_t)b * cap + e];
-    for (int j = 0; j < M; ++j) {
-      int v = -1;
-      if (j < L) { v = x[start + j]; if ((unsigned)v >= (unsigned)V) v = 0; }
-      row[j] = v;
+  // constituent rows of the entries created here: tokens [start, start + len), -1 padded; four entries of a
+  // thread at a time, so that their loads do not wait for one another
+  for (int e0 = n0 + tid; e0 < s_n1; e0 += 4 * (int)blockDim.x) {
+    int start[4], L[4], tok[4][kMaxM];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = e0 + u * (int)blockDim.x;
+      start[u] = L[u] = 0;
+      if (e < s_n1) { start[u] = cb.cons[((size_t)b * cap + e) * M]; L[u] = cb.len[(size_t)b * cap + e]; }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int j = 0; j < kMaxM; ++j) tok[u][j] = j < L[u] ? x[start[u] + j] : -1;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int e = e0 + u * (int)blockDim.x;
+      if (e >= s_n1) break;
+      int32_t* row = cb.cons + ((size_t)b * cap + e) * M;
+#pragma unroll
+      for (int j = 0; j < kMaxM; ++j)
+        if (j < M) row[j] = j < L[u] && (unsigned)tok[u][j] >= (unsigned)V ? 0 : tok[u][j];
     }
   }
 }

@@ -39,7 +39,7 @@ __device__ __forceinline__ int entry_len(const CbView& cb, int b, int code) {
 // (the entry it names is known once the codes before it are in), and before the first lane whose bid
 // for a slot lost.  The code that names the very entry it creates can only be the window's first.
 //
-// Bound by the latency of one window (the codes' first tokens and lengths from L2, one lookup, three
+// Bound by the latency of one window (the codes' first tokens and lengths from L2, one lookup, four
 // barriers); one thread that replayed code by code took 170 ns per code with the table in shared
 // memory and 260 with it in global memory.
 template <int LANES, bool SMEM>
@@ -50,9 +50,8 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_replay(CbView cb, 
   extern __shared__ __align__(16) unsigned char s_parse[];
   __shared__ int s_code[LANES + 1], s_first[LANES + 1];   // [0]: the code before the window
   __shared__ uint8_t s_len[LANES + 4];
-  __shared__ uint32_t s_known[WARPS];
-  __shared__ ParseVotes<WARPS> s_votes;
-  __shared__ int s_n1, s_bad0;
+  __shared__ uint32_t s_known[WARPS], s_ins[WARPS];
+  __shared__ int s_n1, s_bad0, s_prev0[3], s_lost[2];      // first loser of this window, of the next one
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int b = blockIdx.x;
   const int V = cb.V, M = cb.M, cap = cb.cap;
@@ -66,27 +65,29 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_replay(CbView cb, 
   table.open(cb, b, n0, s_parse);
   if (tid == 0) {
     const int prev = cb.prev[b];
-    s_code[0] = prev;
-    s_first[0] = prev >= 0 ? entry_first(cb, b, prev) : -1;
-    s_len[0] = (uint8_t)(prev >= 0 ? entry_len(cb, b, prev) : 0);
+    s_prev0[0] = prev;
+    s_prev0[1] = prev >= 0 ? entry_first(cb, b, prev) : -1;
+    s_prev0[2] = prev >= 0 ? entry_len(cb, b, prev) : 0;
     s_n1 = n0;
     s_bad0 = 0;
+    s_lost[0] = s_lost[1] = LANES;
   }
   __syncthreads();
   if (tid < LANES) {
     int n = n0, st = 0, base = 0;
     int z = tid < Tc ? zs[tid] : -1;
-    while (base < Tc) {
+    int prev0 = s_prev0[0], first0 = s_prev0[1], plen0 = s_prev0[2];       // the code before the window
+    for (int par = 0; base < Tc; par ^= 1) {
       const int z_ahead = base + LANES + tid < Tc ? zs[base + LANES + tid] : -1;
       const int i = base + tid;
       // ---- first token and length of every code, as far as known
       bool known = i < Tc && z >= 0 && z < V + n;
       int f = -1, l = 0;
       if (known) { f = entry_first(cb, b, z); l = entry_len(cb, b, z); }
-      const int prev0 = s_code[0], plen0 = s_len[0];
       const bool self_ref = tid == 0 && z == V + n && prev0 >= 0 && plen0 < M && n < cap;   // the entry this code creates
-      if (self_ref) { known = true; f = s_first[0]; l = plen0 + 1; }
+      if (self_ref) { known = true; f = first0; l = plen0 + 1; }
       s_code[tid + 1] = z; s_first[tid + 1] = f; s_len[tid + 1] = (uint8_t)l;
+      if (tid == 0) { s_code[0] = prev0; s_first[0] = first0; s_len[0] = (uint8_t)plen0; }
       const uint32_t v_known = __ballot_sync(0xffffffffu, known);
       if (lane == 0) s_known[warp] = v_known;
       parse_sync<LANES>();
@@ -107,24 +108,28 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_replay(CbView cb, 
         want = !found && slot >= 0;
       }
       parse_sync<LANES>();
-      if (want) table.bid(slot, tid);
+      if (tid == 0) s_lost[par ^ 1] = LANES;           // (read ahead of this window's first barrier)
+      if (want) {
+        const int loser = table.bid(slot, tid, LANES);
+        if (loser < LANES) atomicMin(&s_lost[par], loser);
+      }
+      const uint32_t v_ins = __ballot_sync(0xffffffffu, want);
+      if (lane == 0) s_ins[warp] = v_ins;
       parse_sync<LANES>();
-      const bool own = want && table.owns(slot, tid);
-      const uint32_t v_ins = __ballot_sync(0xffffffffu, want), v_lost = __ballot_sync(0xffffffffu, want && !own);
-      if (lane == 0) { s_votes.ins[warp] = v_ins; s_votes.lost[warp] = v_lost; }
-      parse_sync<LANES>();
-      const ParseVotes<WARPS> votes = s_votes;
-      int stop = parse_first_lost(votes.lost);
+      uint32_t ins[WARPS];
+#pragma unroll
+      for (int k = 0; k < WARPS; ++k) ins[k] = s_ins[k];
+      int stop = s_lost[par];
       if (stop > limit) stop = limit;
       if (s_bad0) stop = 0;
       const int room = cap - n;
       int made;
-      const int new_before = parse_rank(votes.ins, warp, lane, made);
-      if (stop < LANES) made = parse_count_below(votes.ins, stop);
-      if (own) {
-        const int entry = tid < stop && new_before < room ? n + new_before : -1;
-        table.settle(slot, (uint32_t)pz, (uint32_t)f, entry);
-        if (entry >= 0) {
+      const int new_before = parse_rank(ins, warp, lane, made);
+      if (stop < LANES) made = parse_count_below(ins, stop);
+      if (want) {
+        if (tid < stop && new_before < room) {
+          const int entry = n + new_before;
+          table.settle(slot, (uint32_t)pz, (uint32_t)f, entry);
           int32_t* row = cons + (size_t)entry * M;
           row[0] = pf;                               // what later windows ask for; SMEM: the rest follows below
           if (!SMEM) {
@@ -132,6 +137,8 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_replay(CbView cb, 
             for (int j = 1; j < M; ++j) row[j] = j < pl ? from[j] : (j == pl ? f : -1);
           }
           elen[entry] = (uint8_t)(pl + 1);
+        } else {
+          table.withdraw(slot, tid);
         }
       }
       if (made > 0) {
@@ -139,17 +146,15 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_replay(CbView cb, 
         if (n >= cap) st |= Z2Z_ST_CAP_FROZEN;
       }
       if (stop == 0) { st |= Z2Z_ST_BAD_TOKEN; break; }        // the window's first code names no hypertoken
-      const int lz = s_code[stop], lf = s_first[stop], ll = s_len[stop];
+      prev0 = s_code[stop]; first0 = s_first[stop]; plen0 = s_len[stop];
       base += stop;
       z = stop == LANES ? z_ahead : (base + tid < Tc ? zs[base + tid] : -1);
-      parse_sync<LANES>();                                  // everybody has read the window's last code
-      if (tid == 0) { s_code[0] = lz; s_first[0] = lf; s_len[0] = (uint8_t)ll; }
-      parse_sync<LANES>();
+      parse_sync<LANES>();                             // rows, lengths and slots are there for the next window
     }
     if (tid == 0) {
       s_n1 = n;
       cb.n[b] = n;
-      if (base > 0) cb.prev[b] = s_code[0];
+      if (base > 0) cb.prev[b] = prev0;
       n_valid[b] = base;
     }
     if (st) atomicOr(&cb.status[b], st);
@@ -233,10 +238,19 @@ __global__ void __launch_bounds__(kExpandThreads) k_lzw_expand(
   __syncthreads();
   // codes before this chunk: total length and validity
   int before = 0;
-  for (int i = tid; i < lo; i += kExpandThreads) {
-    const int z = zs[i];
-    if (z < 0 || z >= cb.V + n) atomicMin(&s_first_bad, i);
-    else before += entry_len(cb, b, z);
+  constexpr int kAhead = 8;                      // codes a thread looks at together: their lengths are a second round of loads
+  for (int i0 = tid; i0 < lo; i0 += kAhead * kExpandThreads) {
+    int z[kAhead], l[kAhead];
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) z[u] = i0 + u * kExpandThreads < lo ? zs[i0 + u * kExpandThreads] : 0;
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u)
+      l[u] = i0 + u * kExpandThreads < lo && z[u] >= 0 && z[u] < cb.V + n ? entry_len(cb, b, z[u]) : 0;
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      before += l[u];
+      if (z[u] < 0 || z[u] >= cb.V + n) atomicMin(&s_first_bad, i0 + u * kExpandThreads);
+    }
   }
   int total = 0;
   block_exclusive_scan(before, warp_sums, &total);

@@ -144,7 +144,9 @@ __device__ __forceinline__ int warp_lzw_step(const CbView& cb, int b, int z) {
 // its first empty slot with the earlier lane, so one atomicMin of the lane number per new phrase on
 // that slot finds it (a loser may also be a different key whose probe sequence ends in the same
 // slot; it is treated the same).  The window then ends before the first loser, which is looked up
-// again; the lowest lane never loses, so every window makes progress.
+// again; the lowest lane never loses, so every window makes progress.  Whoever of two bidders comes
+// second learns of the other from the atomic and reports the higher lane of both: the lowest lane
+// reported is the second lowest bidder of some slot, that is the first loser, known one barrier after the bids.
 //
 // ParseTable holds the dictionary during the parse.
 //   SMEM  (codebooks of at most kParseSmemMaxCap entries): the slot array lies in shared memory as
@@ -198,7 +200,7 @@ struct ParseTable {
         while (hit) {
           const uint32_t v = (hit & 1u) ? g.x : (hit & 2u) ? g.y : (hit & 4u) ? g.z : g.w;
           const int e = (int)(v & 0xffffu);
-          if (key0[e] == k0 && key1[e] == (uint16_t)k1) return e;
+          if ((key0[e] == k0) & (key1[e] == (uint16_t)k1)) return e;      // (both loads under way)
           hit &= hit - 1;
         }
         if (gap) { slot = (int)at + __ffs((int)gap) - 1; return -1; }
@@ -218,23 +220,30 @@ struct ParseTable {
     }
     return -1;
   }
-  // A lane bids for its empty slot; after a barrier the lowest lane among the bidders owns it.
-  __device__ __forceinline__ void bid(int slot, int lane) {
-    if (SMEM) atomicMin(tab + slot, (uint32_t)lane);
-    else atomicMin(hash + slot, (unsigned long long)lane);
+  // A bid is above every entry's word (tags have 15 bits; no code is 2^24 - 1) and below the empty slot.
+  static constexpr uint32_t kBid = 0xffff0000u;
+  // A lane bids for its empty slot.  Returns the higher lane when another one has bid before, `none` otherwise.
+  __device__ __forceinline__ int bid(int slot, int lane, int none) {
+    uint32_t old;
+    if (SMEM) old = atomicMin(tab + slot, kBid | (uint32_t)lane);
+    else old = (uint32_t)atomicMin(hash + slot, (unsigned long long)0xffffffffu << 32 | (kBid | (uint32_t)lane));
+    const int other = (int)(old & 0xffffu);
+    return old == ~0u ? none : (other > lane ? other : lane);
   }
-  __device__ __forceinline__ bool owns(int slot, int lane) const {
-    if (SMEM) return *reinterpret_cast<volatile uint32_t*>(tab + slot) == (uint32_t)lane;
-    return __ldcg(hash + slot) == (unsigned long long)lane;
-  }
-  // The owner turns its bid into the entry, or back into an empty slot.
+  // After a barrier: the owner of a slot (a bidder ahead of all losers) turns its bid into the entry.
   __device__ __forceinline__ void settle(int slot, uint32_t prefix, uint32_t token, int entry) {
     if (SMEM) {
-      tab[slot] = entry < 0 ? 0xffffffffu : (tag_of(mix(prefix, token)) << 16) | (uint32_t)entry;
-      if (entry >= 0) { key0[entry] = prefix | (token << 24); key1[entry] = (uint16_t)(token >> 8); }
+      tab[slot] = (tag_of(mix(prefix, token)) << 16) | (uint32_t)entry;
+      key0[entry] = prefix | (token << 24);
+      key1[entry] = (uint16_t)(token >> 8);
     } else {
-      hash[slot] = entry < 0 ? kEmptySlot : pack_slot(prefix, token, (uint32_t)entry);
+      hash[slot] = pack_slot(prefix, token, (uint32_t)entry);
     }
+  }
+  // A bidder that gets no entry empties the slot if its bid is the one that stands there.
+  __device__ __forceinline__ void withdraw(int slot, int lane) {
+    if (SMEM) atomicCAS(tab + slot, kBid | (uint32_t)lane, ~0u);
+    else atomicCAS(hash + slot, (unsigned long long)0xffffffffu << 32 | (kBid | (uint32_t)lane), (unsigned long long)kEmptySlot);
   }
   __device__ __forceinline__ uint32_t prefix_of(int e) const { return key0[e] & 0xffffffu; }
   __device__ __forceinline__ uint32_t token_of(int e) const { return (key0[e] >> 24) | ((uint32_t)key1[e] << 8); }
@@ -268,12 +277,30 @@ struct ParseTable {
   // All threads of the block: entries [n0, n1) go to the codebook's hash table.
   __device__ void close(int n0, int n1) {
     if (!SMEM) return;
-    for (int e = n0 + (int)threadIdx.x; e < n1; e += blockDim.x) {
-      const uint32_t prefix = prefix_of(e), token = token_of(e);
-      int at = probe_start(n_slots, prefix, token);
+    // (four entries of a thread at a time: their insertions do not wait for one another)
+    for (int e0 = n0 + (int)threadIdx.x; e0 < n1; e0 += 4 * (int)blockDim.x) {
+      unsigned long long word[4];
+      int at[4];
+      bool open[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = e0 + u * (int)blockDim.x;
+        open[u] = e < n1;
+        const uint32_t prefix = open[u] ? prefix_of(e) : 0u, token = open[u] ? token_of(e) : 0u;
+        at[u] = probe_start(n_slots, prefix, token);
+        word[u] = pack_slot(prefix, token, (uint32_t)e);
+      }
       for (int it = 0; it < n_slots; ++it) {
-        if (atomicCAS(hash + at, kEmptySlot, pack_slot(prefix, token, (uint32_t)e)) == kEmptySlot) break;
-        at = (at + 1) & (n_slots - 1);
+        unsigned long long old[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) old[u] = open[u] ? atomicCAS(hash + at[u], (unsigned long long)kEmptySlot, word[u]) : kEmptySlot;
+        bool more = false;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          open[u] = open[u] && old[u] != kEmptySlot;
+          if (open[u]) { at[u] = (at[u] + 1) & (n_slots - 1); more = true; }
+        }
+        if (!more) break;
       }
     }
   }
@@ -283,20 +310,11 @@ struct ParseTable {
 struct ParseLaunch { int lanes; size_t smem_bytes; };
 ParseLaunch parse_launch(const CbView& cb, int T);
 
-// What the parsing warps tell each other inside a window: per warp a mask of lanes on the chain, of
-// those that want a new entry, and of those whose bid lost.
+// What the parsing warps tell each other inside a window: per warp a mask of lanes on the chain, and of
+// those that want a new entry.
 template <int WARPS>
-struct ParseVotes { uint32_t on[WARPS], ins[WARPS], lost[WARPS]; };
+struct ParseVotes { uint32_t on[WARPS], ins[WARPS]; };
 
-// First losing lane of the window (all lanes if none).
-template <int WARPS>
-__device__ __forceinline__ int parse_first_lost(const uint32_t (&lost)[WARPS]) {
-  int f = 32 * WARPS;
-#pragma unroll
-  for (int k = WARPS - 1; k >= 0; --k)
-    if (lost[k]) f = k * 32 + __ffs((int)lost[k]) - 1;
-  return f;
-}
 // Bits of m below lane `at` of the window.
 template <int WARPS>
 __device__ __forceinline__ int parse_count_below(const uint32_t (&m)[WARPS], int at) {
