@@ -401,6 +401,8 @@ k_decode_logits(const DecodeLogitsParams p, const __grid_constant__ DecodeLogitM
 
 // One warp per hidden row: merge the partials of all CTAs, write the outputs.
 __global__ void __launch_bounds__(128) k_decode_logits_merge(LogitsArgs a, int stride, int count) {
+  pdl_trigger();
+  pdl_wait();
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= a.N) return;
@@ -508,8 +510,7 @@ cudaError_t run_logits_decode(const CbView& cb, const LogitsArgs& a, int* counte
   }
   if (e != cudaSuccess || info) return e;
   ProfScope ps(prof, kProfLogitsMerge, 1, s);
-  k_decode_logits_merge<<<(a.N + 3) / 4, 128, 0, s>>>(a, p.part_stride, grid);
-  return cudaGetLastError();
+  return launch_pdl(k_decode_logits_merge, dim3((a.N + 3) / 4), dim3(128), 0, s, a, p.part_stride, grid);
 }
 
 }  // namespace z2z

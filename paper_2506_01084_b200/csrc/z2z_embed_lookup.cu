@@ -7,6 +7,7 @@
 // the rows with a grid sized to the machine.
 #include "z2z_common.cuh"
 #include "z2z_internal.h"
+#include "z2z_sm100.cuh"
 
 namespace z2z {
 
@@ -16,9 +17,10 @@ constexpr int kLookupUnroll = 4;
 }
 
 __global__ void __launch_bounds__(kLookupThreads) k_embed_lookup(
-    CbView cb, const int32_t* __restrict__ codes, int N, const int32_t* __restrict__ row_seq,
-    const uint4* __restrict__ WE, const uint4* __restrict__ Eh, uint4* __restrict__ out,
+    CbView cb, const int32_t* codes, int N, const int32_t* row_seq, const uint4* WE, const uint4* Eh, uint4* out,
     int row_vecs /* 16-byte vectors per row */) {
+  sm100::pdl_trigger();
+  sm100::pdl_wait();                              // codes, codebook state and cache rows come from earlier kernels
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < N; r += warps) {
@@ -39,11 +41,11 @@ __global__ void __launch_bounds__(kLookupThreads) k_embed_lookup(
     for (; i + 32 * (kLookupUnroll - 1) < row_vecs; i += 32 * kLookupUnroll) {
       uint4 v[kLookupUnroll];
 #pragma unroll
-      for (int u = 0; u < kLookupUnroll; ++u) v[u] = __ldg(src + i + 32 * u);
+      for (int u = 0; u < kLookupUnroll; ++u) v[u] = __ldcg(src + i + 32 * u);
 #pragma unroll
       for (int u = 0; u < kLookupUnroll; ++u) __stcs(dst + i + 32 * u, v[u]);
     }
-    for (; i < row_vecs; i += 32) __stcs(dst + i, __ldg(src + i));
+    for (; i < row_vecs; i += 32) __stcs(dst + i, __ldcg(src + i));
   }
 }
 
@@ -55,10 +57,8 @@ cudaError_t launch_embed_lookup(const CbView& cb, const int32_t* codes, int N,
   int blocks = (N + warps_per_block - 1) / warps_per_block;
   const int full = 148 * 8;                       // 8 resident blocks of 256 threads per SM
   if (blocks > full) blocks = full;
-  k_embed_lookup<<<blocks, kLookupThreads, 0, s>>>(
-      cb, codes, N, row_seq, reinterpret_cast<const uint4*>(WE), reinterpret_cast<const uint4*>(Eh),
-      reinterpret_cast<uint4*>(out), row_vecs);
-  return cudaGetLastError();
+  return launch_pdl(k_embed_lookup, dim3(blocks), dim3(kLookupThreads), 0, s, cb, codes, N, row_seq,
+                    reinterpret_cast<const uint4*>(WE), reinterpret_cast<const uint4*>(Eh), reinterpret_cast<uint4*>(out), row_vecs);
 }
 
 }  // namespace z2z

@@ -15,21 +15,6 @@ namespace z2z {
 // ---------------------------------------------------------------------------------------------
 // Work list
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ void block_exclusive_scan_1024(int v, int* smem, int& excl, int& total) {
-  const int t = threadIdx.x;
-  smem[t] = v;
-  __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {
-    int x = t >= o ? smem[t - o] : 0;
-    __syncthreads();
-    smem[t] += x;
-    __syncthreads();
-  }
-  excl = smem[t] - v;
-  total = smem[1023];
-  __syncthreads();
-}
-
 // First entry of sequence b that is due on a side.
 __device__ __forceinline__ int due_from(const CbView& cb, int which, int b) {
   const int e = cb.n_emb[which * cb.B + b];
@@ -38,11 +23,11 @@ __device__ __forceinline__ int due_from(const CbView& cb, int which, int b) {
 
 // mode 0: ranges from first/count (NULL: the entries due on side `which`);  mode 1: from new_entry (0/1 each)
 __global__ void __launch_bounds__(1024) k_entry_offsets(CbView cb, int which, int mode,
-                                                        const int32_t* __restrict__ first,
-                                                        const int32_t* __restrict__ count,
-                                                        const int32_t* __restrict__ new_entry,
-                                                        int32_t* __restrict__ off) {
-  __shared__ int sm[1024];
+                                                        const int32_t* first, const int32_t* count,
+                                                        const int32_t* new_entry, int32_t* off) {
+  __shared__ int sm[32];
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   const int b = threadIdx.x;
   int c = 0;
   if (b < cb.B) {
@@ -56,8 +41,8 @@ __global__ void __launch_bounds__(1024) k_entry_offsets(CbView cb, int which, in
       c = c < 0 ? 0 : (c > n - f ? n - f : c);
     }
   }
-  int excl, total;
-  block_exclusive_scan_1024(c, sm, excl, total);
+  int total;
+  const int excl = block_scan_1024(c, sm, total);
   if (b < cb.B) off[b] = excl;
   if (b == 0) { off[cb.B] = total; off[cb.B + 1] = 0; }
 }
@@ -82,9 +67,8 @@ __device__ __forceinline__ void entry_of(const CbView& cb, int which, int mode, 
 }
 
 // Work list of a pass: entries [g0, g0 + slots) of the call, or those of one pass of pass_first.
-__global__ void k_entry_fill(CbView cb, int which, int mode, const int32_t* __restrict__ first,
-                             const int32_t* __restrict__ new_entry, EntryList el, long long g0, int slots,
-                             const int32_t* __restrict__ pass_first) {
+__global__ void k_entry_fill(CbView cb, int which, int mode, const int32_t* first, const int32_t* new_entry, EntryList el,
+                             long long g0, int slots, const int32_t* pass_first) {
   sm100::pdl_trigger();
   sm100::pdl_wait();
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
@@ -112,7 +96,9 @@ __global__ void k_entry_fill(CbView cb, int which, int mode, const int32_t* __re
 }
 
 // Packed rows (base tokens) of all entries of the call, added up in el.off[B + 1] (zero before).
-__global__ void __launch_bounds__(256) k_entry_rows(CbView cb, int which, const int32_t* __restrict__ first, EntryList el) {
+__global__ void __launch_bounds__(256) k_entry_rows(CbView cb, int which, const int32_t* first, EntryList el) {
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   const int b = blockIdx.x;
   const int count = el.off[b + 1] - el.off[b];
   int f = first ? first[b] : due_from(cb, which, b);
@@ -126,9 +112,11 @@ __global__ void __launch_bounds__(256) k_entry_rows(CbView cb, int which, const 
 
 // First entry of every pass: the entry whose first row is row r of the call belongs to pass r / rows_per, so
 // that a pass holds at most rows_per + M - 1 rows.  One block walks the entries 1024 at a time.
-__global__ void __launch_bounds__(1024) k_entry_passes(CbView cb, int which, const int32_t* __restrict__ first, EntryList el,
-                                                       int rows_per, int n_passes, int32_t* __restrict__ pass_first) {
-  __shared__ int sm[1024];
+__global__ void __launch_bounds__(1024) k_entry_passes(CbView cb, int which, const int32_t* first, EntryList el, int rows_per,
+                                                       int n_passes, int32_t* pass_first) {
+  __shared__ int sm[32];
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   const int total = el.off[cb.B];
   long long before = 0;                          // rows ahead of this batch of entries
   for (int g0 = 0; g0 < total; g0 += 1024) {
@@ -139,8 +127,8 @@ __global__ void __launch_bounds__(1024) k_entry_passes(CbView cb, int which, con
       entry_of(cb, which, 0, first, nullptr, el, g, b, k);
       if (k < cb.cap) len = (int)cb.len[(size_t)b * cb.cap + k];
     }
-    int excl, rows;
-    block_exclusive_scan_1024(len, sm, excl, rows);
+    int rows;
+    const int excl = block_scan_1024(len, sm, rows);
     if (g < total) {
       const long long r0 = before + excl;
       const int pass = (int)(r0 / rows_per);
@@ -157,6 +145,8 @@ __global__ void __launch_bounds__(1024) k_entry_passes(CbView cb, int which, con
 // what the bound left out is due for the next call and stays so through decode steps.  After a decode step
 // (off == NULL): every entry is embedded, unless a call left some out.
 __global__ void k_mark_embedded(CbView cb, int which, const int32_t* off, long long bound) {
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= cb.B) return;
   int32_t* emb = cb.n_emb + which * cb.B + b;
@@ -348,13 +338,11 @@ __global__ void __launch_bounds__(256) k_enc_pool(CbView cb, EntryList el,
 // ---------------------------------------------------------------------------------------------
 cudaError_t launch_entry_offsets(const CbView& cb, int which, const int32_t* first,
                                  const int32_t* count, const EntryList& el, cudaStream_t s) {
-  k_entry_offsets<<<1, 1024, 0, s>>>(cb, which, 0, first, count, nullptr, el.off);
-  return cudaGetLastError();
+  return launch_pdl(k_entry_offsets, dim3(1), dim3(1024), 0, s, cb, which, 0, first, count, nullptr, el.off);
 }
 cudaError_t launch_entry_offsets_from_new(const CbView& cb, const int32_t* new_entry,
                                           const EntryList& el, cudaStream_t s) {
-  k_entry_offsets<<<1, 1024, 0, s>>>(cb, 0, 1, nullptr, nullptr, new_entry, el.off);
-  return cudaGetLastError();
+  return launch_pdl(k_entry_offsets, dim3(1), dim3(1024), 0, s, cb, 0, 1, nullptr, nullptr, new_entry, el.off);
 }
 cudaError_t launch_entry_fill(const CbView& cb, int which, const int32_t* first,
                               const int32_t* new_entry, const EntryList& el, int chunk_index, int slots,
@@ -363,13 +351,11 @@ cudaError_t launch_entry_fill(const CbView& cb, int which, const int32_t* first,
                     el, (long long)chunk_index * el.chunk, slots, nullptr);
 }
 cudaError_t launch_entry_rows(const CbView& cb, int which, const int32_t* first, const EntryList& el, cudaStream_t s) {
-  k_entry_rows<<<cb.B, 256, 0, s>>>(cb, which, first, el);
-  return cudaGetLastError();
+  return launch_pdl(k_entry_rows, dim3(cb.B), dim3(256), 0, s, cb, which, first, el);
 }
 cudaError_t launch_entry_passes(const CbView& cb, int which, const int32_t* first, const EntryList& el, int rows,
                                 int n_passes, int32_t* pass_first, cudaStream_t s) {
-  k_entry_passes<<<1, 1024, 0, s>>>(cb, which, first, el, rows - (cb.M - 1), n_passes, pass_first);
-  return cudaGetLastError();
+  return launch_pdl(k_entry_passes, dim3(1), dim3(1024), 0, s, cb, which, first, el, rows - (cb.M - 1), n_passes, pass_first);
 }
 cudaError_t launch_entry_fill_pass(const CbView& cb, int which, const int32_t* first, const EntryList& el, int pass,
                                    const int32_t* pass_first, int slots, cudaStream_t s) {
@@ -377,8 +363,7 @@ cudaError_t launch_entry_fill_pass(const CbView& cb, int which, const int32_t* f
                     pass_first ? pass_first + pass : nullptr);
 }
 cudaError_t launch_mark_embedded(const CbView& cb, int which, const int32_t* off, long long bound, cudaStream_t s) {
-  k_mark_embedded<<<(cb.B + 255) / 256, 256, 0, s>>>(cb, which, off, bound);
-  return cudaGetLastError();
+  return launch_pdl(k_mark_embedded, dim3((cb.B + 255) / 256), dim3(256), 0, s, cb, which, off, bound);
 }
 
 template <typename T>

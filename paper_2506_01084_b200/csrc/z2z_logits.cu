@@ -9,6 +9,7 @@
 #include "z2z_common.cuh"
 #include "z2z_internal.h"
 #include "z2z_simt_tile.cuh"
+#include "z2z_sm100.cuh"
 
 namespace z2z {
 
@@ -44,6 +45,8 @@ __global__ void __launch_bounds__(256) k_logits_simt(CbView cb, LogitsArgs a, in
   const int r0 = blockIdx.y * kTR;
   const int G = gridDim.x, g = blockIdx.x;
   const int t = threadIdx.x;
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   if (t < kTR) {
     const int r = r0 + t;
     int sq = -1, nv = 0, tg = -1;
@@ -124,6 +127,8 @@ __global__ void __launch_bounds__(256) k_logits_simt(CbView cb, LogitsArgs a, in
 
 // One warp per row: merge G partials, write the outputs.
 __global__ void __launch_bounds__(128) k_logits_merge(LogitsArgs a, int G) {
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= a.N) return;
@@ -179,15 +184,13 @@ cudaError_t run_logits_simt(const CbView& cb, const LogitsArgs& a, LogitsPartInf
   }
   {
     ProfScope ps(prof, kProfLogits, 1, s);
-    if (a.dtype == Z2Z_DTYPE_FP32)
-      k_logits_simt<float><<<dim3(G, row_tiles), 256, 0, s>>>(cb, a, n_static, tiles_per_seq, n_tiles);
-    else
-      k_logits_simt<__nv_bfloat16><<<dim3(G, row_tiles), 256, 0, s>>>(cb, a, n_static, tiles_per_seq, n_tiles);
+    const cudaError_t e = launch_pdl(a.dtype == Z2Z_DTYPE_FP32 ? k_logits_simt<float> : k_logits_simt<__nv_bfloat16>,
+                                     dim3(G, row_tiles), dim3(256), 0, s, cb, a, n_static, tiles_per_seq, n_tiles);
+    if (e != cudaSuccess) return e;
   }
-  if (info) { info->stride = G; info->count = G; return cudaGetLastError(); }
+  if (info) { info->stride = G; info->count = G; return cudaSuccess; }
   ProfScope ps(prof, kProfLogitsMerge, 1, s);
-  k_logits_merge<<<(a.N + 3) / 4, 128, 0, s>>>(a, G);
-  return cudaGetLastError();
+  return launch_pdl(k_logits_merge, dim3((a.N + 3) / 4), dim3(128), 0, s, a, G);
 }
 
 __global__ void k_pick_codes(int B, const int32_t* __restrict__ argmax,

@@ -10,6 +10,7 @@
 #include "z2z_common.cuh"
 #include "z2z_internal.h"
 #include "z2z_lzw_dev.cuh"
+#include "z2z_sm100.cuh"
 
 namespace z2z {
 
@@ -213,9 +214,10 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_encode(CbView cb, 
 
 // Online update with one new code per sequence (Figure 1; Section 2.3 step 10).
 // none_sits_out: a code equal to Z2Z_CODE_NONE marks a sequence that takes no part in this step.
-__global__ void __launch_bounds__(128) k_lzw_step(CbView cb, const int32_t* __restrict__ new_codes,
-                                                  const uint8_t* __restrict__ active, int none_sits_out,
-                                                  int32_t* __restrict__ new_entry) {
+__global__ void __launch_bounds__(128) k_lzw_step(CbView cb, const int32_t* new_codes, const uint8_t* active,
+                                                  int none_sits_out, int32_t* new_entry) {
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (b >= cb.B) return;
@@ -275,8 +277,7 @@ cudaError_t launch_lzw_encode(const CbView& cb, const int32_t* tokens, const int
 cudaError_t launch_lzw_step(const CbView& cb, const int32_t* new_codes, const uint8_t* active,
                             int none_sits_out, int32_t* new_entry, cudaStream_t s) {
   int wpb = 4;
-  k_lzw_step<<<(cb.B + wpb - 1) / wpb, wpb * 32, 0, s>>>(cb, new_codes, active, none_sits_out, new_entry);
-  return cudaGetLastError();
+  return launch_pdl(k_lzw_step, dim3((cb.B + wpb - 1) / wpb), dim3(wpb * 32), 0, s, cb, new_codes, active, none_sits_out, new_entry);
 }
 
 }  // namespace z2z

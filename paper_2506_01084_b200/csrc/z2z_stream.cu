@@ -380,8 +380,10 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
   int* s_pref = reinterpret_cast<int*>(sm + 1024);              // [B + 1] <= 4100 bytes
   const uint32_t stage_base = smem_u32(sm + 1024 + 5120);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  pdl_wait();                                      // the prologue already reads codebook state
+  pdl_trigger();                                   // the next kernel may get resident behind this one
   setup_barriers<STAGES>(ctrl);
+  if (warp == 2) { tmem_alloc(smem_u32(&ctrl->tmem_base), tmem_cols(NT)); tmem_relinquish(); }
+  pdl_wait();                                      // codebook counters, row tables and partial slots are dependent
   for (int b = threadIdx.x; b < p.cb.B; b += kThreads) s_pref[b + 1] = (p.cb.n[b] + kLogitGran - 1) / kLogitGran;
   if (warp == 0 && lane < 1 + 2 * kLogitBoxClasses) prefetch_tmap(lane == 0 ? &tm.h : &tm.w[lane - 1]);
   __syncthreads();
@@ -390,7 +392,6 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
     for (int b = 0; b < p.cb.B; ++b) s_pref[b + 1] += s_pref[b];
     ctrl->vt = (p.cb.V + kLogitGran - 1) / kLogitGran + s_pref[p.cb.B];
   }
-  if (warp == 2) { tmem_alloc(smem_u32(&ctrl->tmem_base), tmem_cols(NT)); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -464,6 +465,8 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
 
 // One warp per row: merge the partial reductions of the G CTAs.
 __global__ void __launch_bounds__(128) k_stream_logits_merge(StreamLogitsParams p, int G) {
+  pdl_trigger();
+  pdl_wait();
   const LogitsArgs& a = p.la;
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
@@ -641,8 +644,7 @@ static cudaError_t launch_logits_t(const StreamLogitsParams& p, const LogitMaps&
   auto kern = k_stream_logits<STAGES>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  kern<<<grid, kThreads, smem, s>>>(p, maps);
-  return cudaGetLastError();
+  return launch_pdl(kern, dim3(grid), dim3(kThreads), smem, s, p, maps);
 }
 
 cudaError_t run_logits_stream(const CbView& cb, const LogitsArgs& a, int* err_word, LogitsPartInfo* info, Prof* prof,
@@ -689,8 +691,7 @@ cudaError_t run_logits_stream(const CbView& cb, const LogitsArgs& a, int* err_wo
   }
   if (e != cudaSuccess || info) return e;
   ProfScope ps(prof, kProfLogitsMerge, 1, s);
-  k_stream_logits_merge<<<(a.N + 3) / 4, 128, 0, s>>>(p, grid);
-  return cudaGetLastError();
+  return launch_pdl(k_stream_logits_merge, dim3((a.N + 3) / 4), dim3(128), 0, s, p, grid);
 }
 
 }  // namespace z2z
