@@ -325,12 +325,14 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
   const bool tc = cb->use_tensor_cores && cb->cfg.enc_layers >= 0 &&
                   z2z::encoder_tc_supported(cb->cfg.d, cb->dff, cb->cfg.dtype, cb->heads, cb->cfg.M);
   a.prompt = z2z::encoder_rows_are_prompt_sized(el.chunk * cb->cfg.M);
-  {
+  long long bound = (long long)cb->cfg.B * cb->cfg.cap, rows = 0;
+  if (max_entries > 0 && max_entries < bound) bound = max_entries;
+  // a bounded call of one short pass: list, offsets and row map come from one launch
+  const bool short_list = max_entries >= 0 && bound <= el.chunk && bound <= z2z::kListSlots;
+  if (!short_list) {
     z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 1, s);
     Z2Z_CUDA(z2z::launch_entry_offsets(cb->view, which, d_first, d_count, el, s), "hyper_embed");
   }
-  long long bound = (long long)cb->cfg.B * cb->cfg.cap, rows = 0;
-  if (max_entries > 0 && max_entries < bound) bound = max_entries;
   if (max_entries < 0) {
     // exact: read the number of entries this call has to embed, and of their rows, back from the device
     // (the one place where an enqueueing call waits for the stream), so that no pass is launched for
@@ -379,11 +381,13 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
       a.rows = left < pass_rows ? (int)left : pass_rows;
       a.entries = (a.rows + 1) / 2;
       if (a.entries > bound) a.entries = (int)bound;
+      const bool listed = n_passes == 1 && a.entries <= z2z::kListSlots;
       {
         z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 1, s);
-        Z2Z_CUDA(z2z::launch_entry_fill_pass(cb->view, which, d_first, el, c, pass_first, a.entries, s), "hyper_embed");
+        if (listed) Z2Z_CUDA(z2z::launch_entry_list(cb->view, which, d_first, d_count, el, a.entries, true, s), "hyper_embed");
+        else Z2Z_CUDA(z2z::launch_entry_fill_pass(cb->view, which, d_first, el, c, pass_first, a.entries, s), "hyper_embed");
       }
-      Z2Z_CUDA(z2z::run_encoder_pass_tc(cb->view, &a, 1, el, false, &cb->prof, s), "hyper_embed (tensor cores)");
+      Z2Z_CUDA(z2z::run_encoder_pass_tc(cb->view, &a, 1, el, listed, &cb->prof, s), "hyper_embed (tensor cores)");
     }
   } else for (int c = 0; c < n_chunks; ++c) {
     // a short call, and the rest of a long one, is sized for what it can hold: 16 entries at d = 4096 took
@@ -392,9 +396,10 @@ int32_t z2z_hyper_embed(z2z_codebook* cb, int32_t which, const void* d_table,
     a.entries = left < el.chunk ? (int)left : el.chunk;
     {
       z2z::ProfScope ps(&cb->prof, z2z::kProfEncOther, 1, s);
-      Z2Z_CUDA(z2z::launch_entry_fill(cb->view, which, d_first, nullptr, el, c, a.entries, s), "hyper_embed");
+      if (short_list) Z2Z_CUDA(z2z::launch_entry_list(cb->view, which, d_first, d_count, el, a.entries, false, s), "hyper_embed");
+      else Z2Z_CUDA(z2z::launch_entry_fill(cb->view, which, d_first, nullptr, el, c, a.entries, s), "hyper_embed");
     }
-    if (tc) Z2Z_CUDA(z2z::run_encoder_pass_tc(cb->view, &a, 1, el, false, &cb->prof, s), "hyper_embed (tensor cores)");
+    if (tc) Z2Z_CUDA(z2z::run_encoder_pass_tc(cb->view, &a, 1, el, short_list, &cb->prof, s), "hyper_embed (tensor cores)");
     else if (z2z::encoder_entry_applies(cb->cfg.d, cb->dff, cb->cfg.enc_layers, a.entries)) Z2Z_CUDA(z2z::run_encoder_entries(cb->view, &a, 1, el, &cb->prof, s), "hyper_embed");
     else Z2Z_CUDA(z2z::run_encoder_pass(cb->view, a, el, false, &cb->prof, s), "hyper_embed");
   }

@@ -95,6 +95,71 @@ __global__ void k_entry_fill(CbView cb, int which, int mode, const int32_t* firs
     el.tok[(size_t)e * cb.M + i] = in_book ? cb.cons[((size_t)b * cb.cap + k) * cb.M + i] : -1;
 }
 
+// A call of one pass of at most kListSlots entries: offsets of the sequences (unless `have_off`: they are there), the
+// work list and the map of the packed rows, in one block - a launch and the latency of its loads for each of the three
+// were 4 to 5 us apart, with nothing else on the GPU (two such calls, the logits and the sampling of 16 sequences at
+// d = 4096: 628 -> 618 us).  Thread = sequence, then slot of the list.
+__global__ void __launch_bounds__(1024) k_entry_list(CbView cb, int which, const int32_t* first, const int32_t* count, EntryList el,
+                                                     int slots, int have_off) {
+  __shared__ int warp_sums[32], s_off[1024], s_from[1024];
+  sm100::pdl_trigger();
+  sm100::pdl_wait();
+  const int e = threadIdx.x;
+  int f = 0, c = 0, off = 0, total;
+  if (e < cb.B) {
+    const int n = cb.n[e];
+    f = first ? first[e] : due_from(cb, which, e);
+    f = f < 0 ? 0 : (f > n ? n : f);
+    c = count ? count[e] : n - f;
+    c = c < 0 ? 0 : (c > n - f ? n - f : c);
+    if (have_off) off = el.off[e];
+  }
+  if (have_off) {
+    total = el.off[cb.B];
+  } else {
+    off = block_scan_1024(c, warp_sums, total);
+    if (e < cb.B) el.off[e] = off;
+    if (e == 0) el.off[cb.B] = total;
+  }
+  s_off[e] = off; s_from[e] = f;
+  __syncthreads();
+  if (e == 0) el.off[cb.B + 1] = total < slots ? total : slots;
+  int len = 0, tok[kMaxM];
+#pragma unroll
+  for (int i = 0; i < kMaxM; ++i) tok[i] = -1;
+  if (e < slots) {
+    int b = -1, k = 0;
+    if (e < total) {
+      int lo = 0, hi = cb.B - 1;                   // last b with off[b] <= e
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (s_off[mid] <= e) lo = mid; else hi = mid - 1;
+      }
+      b = lo;
+      k = s_from[b] + (e - s_off[b]);
+      if (k >= 0 && k < cb.cap) {
+        len = (int)cb.len[(size_t)b * cb.cap + k];
+#pragma unroll
+        for (int i = 0; i < kMaxM; ++i)            // constituents are -1 padded behind the entry's length
+          if (i < cb.M) tok[i] = cb.cons[((size_t)b * cb.cap + k) * cb.M + i];
+      }
+    }
+    el.seq[e] = b; el.idx[e] = k; el.len[e] = len;
+#pragma unroll
+    for (int i = 0; i < kMaxM; ++i)
+      if (i < cb.M) el.tok[(size_t)e * cb.M + i] = tok[i];
+  }
+  int rows;
+  const int row = block_scan_1024(len, warp_sums, rows);
+  if (e < slots) {
+    el.row_off[e] = row;
+#pragma unroll
+    for (int i = 0; i < kMaxM; ++i)
+      if (i < len) { el.row_src[row + i] = e * cb.M + i; el.row_tok[row + i] = tok[i]; }
+  }
+  if (e == 0) el.row_off[slots] = rows;
+}
+
 // Packed rows (base tokens) of all entries of the call, added up in el.off[B + 1] (zero before).
 __global__ void __launch_bounds__(256) k_entry_rows(CbView cb, int which, const int32_t* first, EntryList el) {
   sm100::pdl_trigger();
@@ -349,6 +414,11 @@ cudaError_t launch_entry_fill(const CbView& cb, int which, const int32_t* first,
                               cudaStream_t s) {
   return launch_pdl(k_entry_fill, dim3((slots + 255) / 256), dim3(256), 0, s, cb, which, new_entry ? 1 : 0, first, new_entry,
                     el, (long long)chunk_index * el.chunk, slots, nullptr);
+}
+cudaError_t launch_entry_list(const CbView& cb, int which, const int32_t* first, const int32_t* count, const EntryList& el,
+                              int slots, bool have_off, cudaStream_t s) {
+  if (slots > kListSlots) return cudaErrorInvalidValue;
+  return launch_pdl(k_entry_list, dim3(1), dim3(1024), 0, s, cb, which, first, count, el, slots, have_off ? 1 : 0);
 }
 cudaError_t launch_entry_rows(const CbView& cb, int which, const int32_t* first, const EntryList& el, cudaStream_t s) {
   return launch_pdl(k_entry_rows, dim3(cb.B), dim3(256), 0, s, cb, which, first, el);

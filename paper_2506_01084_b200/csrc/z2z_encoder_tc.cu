@@ -785,7 +785,7 @@ bool encoder_tc_supported(int d, int dff, int dtype, int heads, int M) {
 // that own whole output tiles, so bias, residual and GELU are applied in their epilogues; only
 // attention, LayerNorm and pooling remain as separate kernels.
 static cudaError_t run_encoder_pass_pair(const CbView& cb, const EncoderArgs& a, const EntryList& el, int E, int R,
-                                         Prof* prof, cudaStream_t s) {
+                                         bool rows_mapped, Prof* prof, cudaStream_t s) {
   const int d = a.d, dff = a.dff, M = cb.M;
   const int Rt = (R + 7) / 8 * 8;
   const bool half = a.w_half != nullptr;               // fp16 copies of the linear-layer weights exist
@@ -802,21 +802,21 @@ static cudaError_t run_encoder_pass_pair(const CbView& cb, const EncoderArgs& a,
     ProfScope ps(prof, kProfEncGemm, 1, s);
     return launch_pair_gemm(p, act, half ? a.w_half[widx] : a.w[widx], K, epi, half, s);
   };
-  cudaError_t e;
+  cudaError_t e = cudaSuccess;
   // The q, k, v of the first layer on the distinct rows, where that can save row tiles: two of them take the
   // clusters one wave, as one does.  (The map takes 9 us instead of 3.5; 8 prompts of 2048 tokens, d = 3072,
   // 19.8 -> 18.4 ms, 16 of 8192 with their positions scored, d = 4096, single operand, 145 -> 137 ms.)
   const bool uniq = a.layers > 0 && R > 512;
   const int* row_uniq = uniq ? el.row_uniq : nullptr;
   {
-    ProfScope ps(prof, kProfEncOther, 2, s);
+    ProfScope ps(prof, kProfEncOther, uniq || !rows_mapped ? 2 : 1, s);
     if (uniq) {
       int slots = 2048;
       while (slots < 2 * R) slots *= 2;
       const size_t smem = (size_t)(slots + R) * 4;
       if ((e = cudaFuncSetAttribute(k_tc_row_map<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
       e = launch_pdl(k_tc_row_map<true>, dim3(1), dim3(1024), smem, s, cb, el, E, slots, R);
-    } else {
+    } else if (!rows_mapped) {
       e = launch_pdl(k_tc_row_map<false>, dim3(1), dim3(1024), 0, s, cb, el, E, 0, 0);
     }
     if (e != cudaSuccess) return e;
@@ -930,7 +930,7 @@ cudaError_t run_encoder_pass_tc(const CbView& cb, const EncoderArgs* grp, int ng
   // Passes of a call that knows its rows (a0.rows) always take whole tiles in a session of prompt size: their
   // results are then the same bits whatever else is in the call, which stream-K sums are not.
   const bool whole_tiles = R >= kPromptPassRows || (a0.prompt && (a0.rows > 0 || R >= prompt_call_min_rows(d)));
-  if (ng == 1 && whole_tiles) return run_encoder_pass_pair(cb, a0, el, E, R, prof, s);
+  if (ng == 1 && whole_tiles) return run_encoder_pass_pair(cb, a0, el, E, R, rows_mapped, prof, s);
   const int Rt = (R + 7) / 8 * 8;                      // rows of the result matrix per group
   const int* total = el.row_off + E;                   // packed rows of this pass (device word)
   const int n_sm = sm_count();

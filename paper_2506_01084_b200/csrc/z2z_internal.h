@@ -98,6 +98,11 @@ cudaError_t launch_entry_offsets_from_new(const CbView& cb, const int32_t* new_e
 cudaError_t launch_entry_fill(const CbView& cb, int which, const int32_t* first,
                               const int32_t* new_entry, const EntryList& el, int chunk_index, int slots,
                               cudaStream_t s);
+// Offsets (unless they are there), work list and packed-row map of a call of one pass of at most
+// kListSlots entries.
+constexpr int kListSlots = 1024;
+cudaError_t launch_entry_list(const CbView& cb, int which, const int32_t* first, const int32_t* count, const EntryList& el,
+                              int slots, bool have_off, cudaStream_t s);
 // Passes cut by packed rows instead of entries.  launch_entry_rows leaves the rows of all entries of the
 // call in el.off[B + 1] (behind their number in el.off[B]); launch_entry_passes writes the first entry of
 // every pass of at most `rows` rows to pass_first[0 .. n_passes]; launch_entry_fill_pass fills the work

@@ -388,6 +388,32 @@ def test_decode_steps_settle_what_was_embedded_by_range():
         assert torch.all(p.E_f32[b, int(m[b])] != -5) and torch.all(p.E_f32[b, :int(m[b])] == -5)
 
 
+@pytest.mark.parametrize("B,bound", [(37, 200), (37, 64), (700, 1000), (5, 1)])
+def test_short_list_of_ranges(B, bound):
+    """Calls whose offsets, list and row map come from one launch: ranges that start before the first entry, end behind
+    the last one or are empty, over one and several warps of sequences, and a bound below what they hold."""
+    w, p = _pair(128, 128, 3, B, T=60, cap=40, seed=B)
+    n = [p.oracle.books[b].n() for b in range(B)]
+    first = [(5 * b) % 7 - 2 for b in range(B)]
+    count = [[0, 2, -3, 1, 400][b % 5] if B < 100 else [0, 1, 2, 0, -1][b % 5] for b in range(B)]
+    lo = [min(max(f, 0), k) for f, k in zip(first, n)]
+    size = [min(max(c, 0), k - f) for c, k, f in zip(count, n, lo)]
+    left = bound
+    for b in range(B):
+        size[b] = min(size[b], left)
+        left -= size[b]
+    f32 = torch.full((B, w.cap, 128), -5.0, device=p.dev)
+    i32 = lambda x: torch.tensor(x, dtype=torch.int32, device=p.dev)
+    zb.z2z_hyper_embed(p.cb, zb.CACHE_EMBED, p.g_WE, p.g_encE, i32(first), i32(count), bound, p.E_h, f32)
+    got = f32.double().cpu().numpy()
+    enc, table = [f64(t) for t in p.enc_E], f64(p.W_E)
+    for b in range(B):
+        assert np.all(got[b, :lo[b]] == -5) and np.all(got[b, lo[b] + size[b]:] == -5)
+        if size[b]:
+            want = ohe.hyper_embed(p.oracle.books[b].entries[lo[b]:lo[b] + size[b]], table, enc, w.heads)
+            assert np.abs(got[b, lo[b]:lo[b] + size[b]] - want).max() <= TOL
+
+
 @pytest.mark.parametrize("d,dff,total", [(2560, 768, 40), (2560, 768, 80), (384, 512, 200)])
 def test_a_bounded_call_without_an_entry_streams_nothing(d, dff, total):
     """Calls whose ranges are empty between calls that embed some: on one CTA per tile and on pairs, with weights
