@@ -32,13 +32,11 @@ using namespace sm100;
 namespace {
 
 constexpr int kThreads = 192;
-constexpr int kTailPad = 16384;          // readable shared memory behind the last A tile
 
 struct Ctrl {
-  unsigned long long full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2];
+  unsigned long long full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2], pref_ready;
   uint32_t tmem_base;
   int abort;
-  int vt;                                // logits: number of virtual column tiles
 };
 
 __host__ __device__ constexpr int tmem_cols(int nt) {
@@ -50,99 +48,168 @@ struct Job {
   int wmap, wrow;
   int col0, nvalid, owner, k0;           // first column id, valid rows, owning sequence, first entry
   int nrows;                             // the MMA's N, a multiple of kLogitGran
+  int kb;                                // k-blocks of 64 columns per stage
+  int group;                             // >= 0: only this group of 8 hidden rows is loaded
 };
 
 // ---- logits schedule ----------------------------------------------------------------------------
-// Columns are dealt in granules of kLogitGran rows: first the granules of W_U, then those of the
-// visible rows of each sequence's U_h.  Every CTA owns the same number of granules (+-1); a job
-// is a run of up to NT / kLogitGran granules inside one segment (W_U, or one sequence).
+// Columns are dealt in granules of kLogitGran rows: every CTA takes an even share of the granules of W_U, which it
+// knows without any codebook state, and then one of those of the visible rows of each sequence's U_h.  (One share of
+// both in a row gave some CTAs nothing but hypertokens, whose jobs are short and cost more per granule: V = 128256,
+// d = 4096, 90 sequences of 29 hypertokens 385 us.)  A job is a run of up to kLogitNT / kLogitGran granules inside
+// one segment (W_U, or one sequence).
 struct LogitSched {
   const StreamLogitsParams& p;
   const int* pref;       // shared: prefix of per-sequence granule counts, [B + 1]
-  long long u, u1;
-  int n_static;
-  __device__ LogitSched(const StreamLogitsParams& pp, const int* s_pref, int vt) : p(pp), pref(s_pref) {
-    n_static = (p.cb.V + kLogitGran - 1) / kLogitGran;
-    const long long U = vt, G = gridDim.x, c = blockIdx.x;
-    u = c * U / G;
-    u1 = (c + 1) * U / G;
+  int u, u1;
+  bool hyper;
+  __device__ LogitSched(const StreamLogitsParams& pp, const int* s_pref) : p(pp), pref(s_pref), hyper(false) {
+    share((p.cb.V + kLogitGran - 1) / kLogitGran);
   }
+  __device__ void share(int total) {
+    const int G = gridDim.x, c = blockIdx.x;
+    u = (int)((long long)c * total / G);
+    u1 = (int)((long long)(c + 1) * total / G);
+  }
+  __device__ void begin_hyper() { hyper = true; share(pref[p.cb.B]); }        // (pref is there by now)
   __device__ bool next(Job& j) {
     if (u >= u1) return false;
-    const int v = (int)u;
     int remaining, total_rows, g0;
-    if (v < n_static) {
-      g0 = v; remaining = n_static - v; total_rows = p.cb.V;
+    if (!hyper) {
+      g0 = u; remaining = u1 - u; total_rows = p.cb.V;
       j.wmap = 0; j.wrow = g0 * kLogitGran; j.col0 = g0 * kLogitGran; j.owner = -1; j.k0 = 0;
     } else {
-      const int x = v - n_static;
-      int lo = 0, hi = p.cb.B - 1;                 // last b with pref[b] <= x
-      while (lo < hi) { int mid = (lo + hi + 1) >> 1; if (pref[mid] <= x) lo = mid; else hi = mid - 1; }
-      g0 = x - pref[lo]; remaining = pref[lo + 1] - pref[lo] - g0; total_rows = p.cb.n[lo];
+      int lo = 0, hi = p.cb.B - 1;                 // last b with pref[b] <= u
+      while (lo < hi) { int mid = (lo + hi + 1) >> 1; if (pref[mid] <= u) lo = mid; else hi = mid - 1; }
+      g0 = u - pref[lo]; remaining = pref[lo + 1] - pref[lo] - g0; total_rows = p.cb.n[lo];
       j.owner = lo; j.k0 = g0 * kLogitGran;
       j.wmap = 1; j.wrow = lo * p.cb.cap + j.k0; j.col0 = p.cb.V + j.k0;
     }
     int ng = kLogitNT / kLogitGran;
     if (remaining < ng) ng = remaining;
-    if (u1 - u < ng) ng = (int)(u1 - u);
+    if (u1 - u < ng) ng = u1 - u;
     j.nrows = ng * kLogitGran;
     j.nvalid = total_rows - g0 * kLogitGran < j.nrows ? total_rows - g0 * kLogitGran : j.nrows;
     u += ng;
+    // A sequence's hypertokens meet the hidden row of that sequence only.  Where row r is known to be sequence r's, just
+    // the group of 8 rows around it is loaded, to where all rows would put it (the other rows of the operand are what
+    // is left there, and nobody reads their accumulators), and a job of few rows takes several k-blocks per stage: with
+    // one, a job of 64 rows had 8 KB a stage in flight, and took as long as one of 256 (V = 128256, d = 4096, 90
+    // sequences of 59 hypertokens 301 us, of 256 hypertokens 218).
+    j.kb = 1; j.group = -1;
+    if (j.owner >= 0 && !p.la.row_seq) {
+      j.group = j.owner < p.la.N ? j.owner >> 3 : 0;
+      if (ng <= 4) {                               // up to 128 rows: one box, of 1, 2 or 4 granules
+        if (ng == 3) j.nrows = 4 * kLogitGran;
+        j.kb = logit_short_kb(ng > 2 ? 2 : ng - 1);
+      }
+    }
     return true;
+  }
+  __device__ bool next_of_both(Job& j) {
+    if (next(j)) return true;
+    if (hyper) return false;
+    begin_hyper();
+    return next(j);
   }
 };
 
+// Weight rows of a stage: behind the hidden rows, and behind the further k-blocks of the last group of 8.  (The MMA reads
+// 128 hidden rows from a k-block's start; those that are not there lie in the weight rows.)
+__host__ __device__ constexpr uint32_t logit_w_offset(int a_box_rows) { return (uint32_t)a_box_rows * 128u + 3u * 1024u; }
+
 // ---- producer and MMA role of the logits kernel -----------------------------------------------------
+// W_U depends on no earlier kernel, the hidden rows and the codebooks do: the first pass over the ring issues
+// the weight boxes at once and notes the boxes of hidden rows, which go out behind the dependency wait.
 template <int STAGES>
-__device__ __forceinline__ void logits_producer(LogitSched& sched, int ksteps, Ctrl* ctrl, uint32_t stage_base, int a_box_rows,
+__device__ __forceinline__ void logits_producer(const StreamLogitsParams& p, const int* s_pref, Ctrl* ctrl, uint32_t stage_base,
                                                 const LogitMaps& tm) {
-  const uint32_t a_bytes = (uint32_t)a_box_rows * 128;
-  const uint32_t stage_bytes = a_bytes + kLogitNT * 128;           // smem stride of a stage
+  const uint32_t a_bytes = (uint32_t)p.a_box_rows * 128, w_off = logit_w_offset(p.a_box_rows);
+  const uint32_t stage_bytes = w_off + kLogitNT * 128;             // smem stride of a stage
   const uint64_t pol_w = policy_evict_first(), pol_a = policy_evict_last();
   int stage = 0; uint32_t phase = 0;
+  int noted[STAGES], n_noted = 0;                                  // load i of the first pass uses stage i: its k-block
+  bool deps = false;
+  auto need_deps = [&]() {
+    if (deps) return;
+    pdl_wait();
+    deps = true;
+    for (int i = 0; i < n_noted; ++i) {
+      const uint32_t full = smem_u32(&ctrl->full[i]);
+      mbar_expect_tx(full, a_bytes);
+      tma_load_3d(stage_base + (uint32_t)i * stage_bytes, &tm.h, 0, 0, noted[i], full, pol_a);
+    }
+  };
+  LogitSched sched(p, s_pref);
   Job j;
-  while (sched.next(j)) {
-    for (int ks = 0; ks < ksteps; ++ks) {
-      if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) return;
-      const uint32_t full = smem_u32(&ctrl->full[stage]);
-      mbar_expect_tx(full, a_bytes + (uint32_t)j.nrows * 128);
-      const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
-      tma_load_3d(sb, &tm.h, 0, 0, ks, full, pol_a);
-      // the W rows of the job go out as few boxes as possible: largest power-of-two box first
-      for (int r0 = 0; r0 < j.nrows;) {
-        int cls = kLogitBoxClasses - 1;
-        while (cls > 0 && (kLogitGran << cls) > j.nrows - r0) --cls;
-        tma_load_3d(sb + a_bytes + r0 * 128, &tm.w[j.wmap * kLogitBoxClasses + cls], 0, j.wrow + r0, ks, full, pol_w);
-        r0 += kLogitGran << cls;
+  for (int part = 0; part < 2; ++part) {
+    if (part == 1) {
+      need_deps();
+      if (!mbar_wait(smem_u32(&ctrl->pref_ready), 0, &ctrl->abort)) return;
+      sched.begin_hyper();
+    }
+    while (sched.next(j)) {
+      for (int ks = 0; ks < p.ksteps; ks += j.kb) {
+        if (n_noted == STAGES) need_deps();
+        if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) { need_deps(); return; }
+        const uint32_t full = smem_u32(&ctrl->full[stage]);
+        const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
+        // (k-blocks beyond the last one, and rows outside the tensors, are zero-filled and counted)
+        const uint32_t w_bytes = (uint32_t)(j.kb * j.nrows) * 128u;
+        if (!deps) {
+          mbar_expect_only(full, w_bytes);
+          noted[n_noted++] = ks;
+        } else if (j.group < 0) {
+          mbar_expect_tx(full, a_bytes + w_bytes);
+          tma_load_3d(sb, &tm.h, 0, 0, ks, full, pol_a);
+        } else {
+          mbar_expect_tx(full, (uint32_t)j.kb * 1024u + w_bytes);
+          tma_load_3d(sb + (uint32_t)j.group * 1024u, &tm.h8[j.kb >> 1], 0, 8 * j.group, ks, full, pol_a);
+        }
+        if (j.kb > 1) {
+          tma_load_3d(sb + w_off, &tm.u[j.nrows == kLogitGran ? 0 : j.nrows == 2 * kLogitGran ? 1 : 2], 0, j.wrow, ks, full, pol_w);
+        } else {
+          // the W rows of the job go out as few boxes as possible: largest power-of-two box first
+          for (int r0 = 0; r0 < j.nrows;) {
+            int cls = kLogitBoxClasses - 1;
+            while (cls > 0 && (kLogitGran << cls) > j.nrows - r0) --cls;
+            tma_load_3d(sb + w_off + r0 * 128, &tm.w[j.wmap * kLogitBoxClasses + cls], 0, j.wrow + r0, ks, full, pol_w);
+            r0 += kLogitGran << cls;
+          }
+        }
+        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
       }
-      if (++stage == STAGES) { stage = 0; phase ^= 1u; }
     }
   }
 }
 
 template <int STAGES>
-__device__ __forceinline__ void logits_mma(LogitSched& sched, int ksteps, Ctrl* ctrl, uint32_t stage_base, int a_box_rows,
+__device__ __forceinline__ void logits_mma(const StreamLogitsParams& p, const int* s_pref, Ctrl* ctrl, uint32_t stage_base,
                                            uint32_t tmem_base) {
-  const uint32_t a_bytes = (uint32_t)a_box_rows * 128;
-  const uint32_t stage_bytes = a_bytes + kLogitNT * 128;
+  const uint32_t w_off = logit_w_offset(p.a_box_rows);
+  const uint32_t stage_bytes = w_off + kLogitNT * 128;
   int stage = 0; uint32_t phase = 0;
   uint32_t job_i = 0;
+  LogitSched sched(p, s_pref);
   Job j;
-  while (sched.next(j)) {
+  while (sched.next_of_both(j)) {
     const uint32_t idesc = idesc_bf16_f32(128, j.nrows);
     const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
     if (!mbar_wait(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) return;
     tc_fence_after();
     const uint32_t d = tmem_base + buf * kLogitNT;
     uint32_t acc = 0;
-    for (int ks = 0; ks < ksteps; ++ks) {
+    for (int ks = 0; ks < p.ksteps; ks += j.kb) {
       if (!mbar_wait(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) return;
       tc_fence_after();
       const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
+      for (int i = 0; i < j.kb; ++i) {
+        const uint32_t ab = sb + (uint32_t)i * 1024u, wb = sb + w_off + (uint32_t)(i * j.nrows) * 128u;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        umma_bf16(d, smem_desc_sw128(sb + k * 32), smem_desc_sw128(sb + a_bytes + k * 32), idesc, acc);
-        acc = 1;
+        for (int k = 0; k < 4; ++k) {
+          umma_bf16(d, smem_desc_sw128(ab + k * 32), smem_desc_sw128(wb + k * 32), idesc, acc);
+          acc = 1;
+        }
       }
       umma_commit(smem_u32(&ctrl->empty[stage]));          // frees the stage when the MMAs are done
       if (++stage == STAGES) { stage = 0; phase ^= 1u; }
@@ -163,6 +230,7 @@ __device__ __forceinline__ void setup_barriers(Ctrl* ctrl) {
       mbar_init(smem_u32(&ctrl->acc_full[b]), 1);
       mbar_init(smem_u32(&ctrl->acc_empty[b]), 4);
     }
+    mbar_init(smem_u32(&ctrl->pref_ready), 1);         // logits: the sequences' granules are counted
     ctrl->abort = 0;
     mbar_init_fence();
   }
@@ -382,27 +450,40 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   pdl_trigger();                                   // the next kernel may get resident behind this one
   setup_barriers<STAGES>(ctrl);
-  if (warp == 2) { tmem_alloc(smem_u32(&ctrl->tmem_base), tmem_cols(NT)); tmem_relinquish(); }
-  pdl_wait();                                      // codebook counters, row tables and partial slots are dependent
-  for (int b = threadIdx.x; b < p.cb.B; b += kThreads) s_pref[b + 1] = (p.cb.n[b] + kLogitGran - 1) / kLogitGran;
-  if (warp == 0 && lane < 1 + 2 * kLogitBoxClasses) prefetch_tmap(lane == 0 ? &tm.h : &tm.w[lane - 1]);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    s_pref[0] = 0;
-    for (int b = 0; b < p.cb.B; ++b) s_pref[b + 1] += s_pref[b];
-    ctrl->vt = (p.cb.V + kLogitGran - 1) / kLogitGran + s_pref[p.cb.B];
+  if (warp == 3) {
+    if (lane < 1 + 2 * kLogitBoxClasses) prefetch_tmap(lane == 0 ? &tm.h : &tm.w[lane - 1]);
+    if (lane < 3) { prefetch_tmap(&tm.h8[lane]); prefetch_tmap(&tm.u[lane]); }
   }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = ctrl->tmem_base;
-  LogitSched sched(p, s_pref, ctrl->vt);
+  __syncthreads();                                 // barriers exist; the producer starts at once
 
   if (warp == 0) {
-    if (lane == 0) logits_producer<STAGES>(sched, p.ksteps, ctrl, stage_base, p.a_box_rows, tm);
-  } else if (warp == 1) {
-    if (lane == 0) logits_mma<STAGES>(sched, p.ksteps, ctrl, stage_base, p.a_box_rows, tmem_base);
+    if (lane == 0) logits_producer<STAGES>(p, s_pref, ctrl, stage_base, tm);
   } else {
+    if (warp == 2) { tmem_alloc(smem_u32(&ctrl->tmem_base), tmem_cols(NT)); tmem_relinquish(); }
+    pdl_wait();                                    // codebook counters, row tables and partial slots are dependent
+    if (warp == 1) {                               // prefix of the sequences' granule counts
+      int carry = 0;
+      for (int b0 = 0; b0 < p.cb.B; b0 += 32) {
+        const int b = b0 + lane;
+        int v = b < p.cb.B ? (p.cb.n[b] + kLogitGran - 1) / kLogitGran : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const int x = __shfl_up_sync(0xffffffffu, v, o); if (lane >= o) v += x; }
+        if (b < p.cb.B) s_pref[b + 1] = carry + v;
+        carry += __shfl_sync(0xffffffffu, v, 31);
+      }
+      if (lane == 0) s_pref[0] = 0;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&ctrl->pref_ready));
+    }
+    tc_fence_before();
+    asm volatile("bar.sync 2, %0;" ::"n"(kThreads - 32) : "memory");      // all but the producer warp
+    tc_fence_after();
+  }
+  if (warp == 1) {
+    if (lane == 0) logits_mma<STAGES>(p, s_pref, ctrl, stage_base, ctrl->tmem_base);
+  } else if (warp >= 2) {
+    const uint32_t tmem_base = ctrl->tmem_base;
+    LogitSched sched(p, s_pref);
     const int q = warp & 3;
     const LogitsArgs& a = p.la;
     const uint32_t k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32);
@@ -422,7 +503,7 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
     }
     uint32_t job_i = 0;
     Job j;
-    while (sched.next(j)) {
+    while (sched.next_of_both(j)) {
       const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
       if (!mbar_wait(smem_u32(&ctrl->acc_full[buf]), aph, &ctrl->abort)) break;
       tc_fence_after();
@@ -460,7 +541,7 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
   tc_fence_before();
   __syncthreads();
   if (threadIdx.x == 0 && ctrl->abort) atomicOr(p.err, 1);
-  if (warp == 2) tmem_dealloc(tmem_base, tmem_cols(NT));
+  if (warp == 2) tmem_dealloc(ctrl->tmem_base, tmem_cols(NT));
 }
 
 // One warp per row: merge the partial reductions of the G CTAs.
@@ -638,9 +719,11 @@ cudaError_t launch_stream_gemm(StreamGemmParams p, const StreamGemmMaps& maps, i
   return stream_gemm_ksb(p.R) == 2 ? launch_stream_gemm_k<2>(p, maps, grid, s) : launch_stream_gemm_k<1>(p, maps, grid, s);
 }
 
+constexpr int kLogitSmemFixed = 1024 + 1024 + 5120;
+static int logit_stage_bytes(int a_box_rows) { return (int)logit_w_offset(a_box_rows) + kLogitNT * 128; }
 template <int STAGES>
 static cudaError_t launch_logits_t(const StreamLogitsParams& p, const LogitMaps& maps, int grid, cudaStream_t s) {
-  const size_t smem = 1024 + 1024 + 5120 + STAGES * ((size_t)p.a_box_rows + kLogitNT) * 128 + kTailPad;
+  const size_t smem = kLogitSmemFixed + STAGES * (size_t)logit_stage_bytes(p.a_box_rows);
   auto kern = k_stream_logits<STAGES>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -664,6 +747,13 @@ cudaError_t run_logits_stream(const CbView& cb, const LogitsArgs& a, int* err_wo
   p.err = err_word;
   LogitMaps maps;
   if (!make_tmap_bf16_kblocks(&maps.h, a.hidden, a.N, a.d, p.a_box_rows, 1)) return cudaErrorInvalidValue;
+  for (int c = 0; c < 3; ++c) {
+    const bool hyper = cb.cap > 0;                     // (otherwise no job uses the maps)
+    if (!make_tmap_bf16_kblocks(&maps.h8[c], a.hidden, a.N, a.d, 8, 1 << c)) return cudaErrorInvalidValue;
+    if (!make_tmap_bf16_kblocks(&maps.u[c], hyper ? a.Uh : a.WU, hyper ? (long long)cb.B * cb.cap : cb.V, a.d, kLogitGran << c,
+                                logit_short_kb(c)))
+      return cudaErrorInvalidValue;
+  }
   for (int c = 0; c < kLogitBoxClasses; ++c) {
     if (!make_tmap_bf16_kblocks(&maps.w[c], a.WU, cb.V, a.d, kLogitGran << c, 1)) return cudaErrorInvalidValue;
     if (cb.cap > 0) {
@@ -686,8 +776,8 @@ cudaError_t run_logits_stream(const CbView& cb, const LogitsArgs& a, int* err_wo
   cudaError_t e;
   {
     ProfScope ps(prof, kProfLogits, 1, s);
-    const int st = (227 * 1024 - 2048 - 5120 - kTailPad) / ((p.a_box_rows + kLogitNT) * 128);      // stages that fit, 6 or more
-    e = st >= 8 ? launch_logits_t<8>(p, maps, grid, s) : launch_logits_t<6>(p, maps, grid, s);
+    const int st = (227 * 1024 - kLogitSmemFixed) / logit_stage_bytes(p.a_box_rows);        // stages that fit, 4 or more
+    e = st >= 5 ? launch_logits_t<5>(p, maps, grid, s) : launch_logits_t<4>(p, maps, grid, s);
   }
   if (e != cudaSuccess || info) return e;
   ProfScope ps(prof, kProfLogitsMerge, 1, s);

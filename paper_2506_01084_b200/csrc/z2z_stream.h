@@ -11,15 +11,20 @@ namespace z2z {
 constexpr int kMaxStages = 8;
 constexpr int kGemmNT = 128;                    // weight rows per tile of the stream-K GEMM
 
-constexpr int kLogitNT = 128;                   // weight rows per job of the logits kernel at most
+constexpr int kLogitNT = 256;                   // weight rows per job of the logits kernel at most
 constexpr int kLogitGran = 32;                  // scheduling granule of the logits kernel, in weight rows (TMA boxes of
                                                 // fewer rows stream several times slower)
-constexpr int kLogitBoxClasses = 3;             // TMA boxes of 32, 64 and 128 weight rows
+constexpr int kLogitBoxClasses = 4;             // TMA boxes of 32, 64, 128 and 256 weight rows
 
-// Tensor maps of the logits kernel: hidden rows, then W_U and U_h once per box size.
+// Tensor maps of the logits kernel: hidden rows (all of them), W_U and U_h once per box size, and for the short jobs of
+// a sequence's hypertokens a group of 8 hidden rows and boxes of 32, 64 or 128 rows of U_h with logit_short_kb k-blocks.
+constexpr int kLogitShortClasses = 3;
+__host__ __device__ constexpr int logit_short_kb(int cls) { return cls == 2 ? 2 : 4; }
 struct LogitMaps {
   CUtensorMap h;
   CUtensorMap w[2 * kLogitBoxClasses];
+  CUtensorMap h8[3];     // 1, 2 and 4 k-blocks
+  CUtensorMap u[kLogitShortClasses];
 };
 
 // ---- decode logits kernel (z2z_decode_logits.cu) ---------------------------------------------

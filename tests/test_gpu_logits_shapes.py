@@ -61,6 +61,35 @@ def test_sampled_batch_of_one_row_per_sequence(V, d, B):
         assert abs(float(lse[r]) - (l.max() + np.log(np.exp(l - l.max()).sum()))) < 1e-4
 
 
+@pytest.mark.parametrize("V,d,B", [(257, 192, 33), (1000, 1152, 47), (257, 64, 128)])
+def test_batch_with_hypertokens_of_every_job_size(V, d, B):
+    """Jobs of 1 to 8 granules of 32 hypertokens: boxes of one, two and four k-blocks, of which the last one ends
+    beyond the width, on the group of 8 hidden rows that holds the sequence's; stored logits too."""
+    sizes = [0, 1, 31, 32, 33, 64, 65, 96, 97, 128, 129, 160, 161, 255, 256, 257, 300]
+    counts = [sizes[(5 * b) % len(sizes)] for b in range(B)]
+    cap = 300
+    cb = _session(V, d, B, cap, counts, 8)
+    g = torch.Generator(device=DEV)
+    g.manual_seed(B)
+    rnd = lambda *s, std: (torch.randn(*s, generator=g, device=DEV) * std).to(torch.bfloat16)
+    hid, WU, Uh = rnd(B, d, std=1.0), rnd(V, d, std=0.05), rnd(B, cap, d, std=0.05)
+    for b in range(B):
+        Uh[b, counts[b]:] = float("nan")                     # rows that are no entries are loaded at most
+    lse, mx = torch.zeros(B, device=DEV), torch.zeros(B, device=DEV)
+    am = torch.zeros(B, dtype=torch.int32, device=DEV)
+    out = torch.full((B, V + cap), -7.0, device=DEV)
+    zb.z2z_dynamic_logits(cb, hid, None, None, WU, Uh, zb.SELECT_ARGMAX, 1.0, 0, 0, None, lse, am, mx, logits_debug=out)
+    st, _ = zb.z2z_status(cb)
+    assert all(int(s) & zb.ST_WAIT_TIMEOUT == 0 for s in st)
+    for r in range(B):
+        l = torch.cat([WU.double() @ hid[r].double(), Uh[r, :counts[r]].double() @ hid[r].double()])
+        tol = 2e-5 * (1 + float(l.abs().max()))
+        assert float((out[r, :V + counts[r]].double() - l).abs().max()) < tol
+        assert torch.all(out[r, V + counts[r]:] == -7)
+        assert abs(float(lse[r]) - float(torch.logsumexp(l, 0))) < tol
+        assert float(l.max() - l[int(am[r])]) < 2 * tol and abs(float(mx[r]) - float(l.max())) < tol
+
+
 @pytest.mark.parametrize("N", [1, 31, 32, 33, 64, 65, 96, 128, 129, 192, 193, 256, 257, 511, 700])
 @pytest.mark.parametrize("V,d", [(4097, 192), (1000, 1152), (130, 2176)])
 def test_joint_logits_against_fp64(V, d, N):
