@@ -20,7 +20,7 @@
 //     counter, which evens out the differences in streaming speed between SMs.
 //
 // Roles: warp 0 lane 0 producer (claims work, publishes each job in a shared-memory ring, issues
-// TMA), warp 1 lane 0 MMA issuer, warps 2-5 epilogue.  Every wait is bounded; on a timeout the
+// TMA), warp 1 MMA issuer (an elected lane), warps 2-5 epilogue.  Every wait is bounded; on a timeout the
 // CTA raises an abort flag, all roles leave, tensor memory is freed, an error word is set.
 #include "z2z_common.cuh"
 #include "z2z_internal.h"
@@ -118,7 +118,7 @@ k_decode_logits(const DecodeLogitsParams p, const __grid_constant__ DecodeLogitM
   const uint32_t stage_base = hid_base + ((hid_bytes + 1023u) & ~1023u);
   const uint32_t stage_hid = RESIDENT ? 0u : (uint32_t)((2 * hid_rows * 128 + 1023) & ~1023);
   const uint32_t stage_bytes = NT * 128 + stage_hid;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const LogitsArgs& a = p.la;
   const int STAGES = p.stages;
   if (threadIdx.x == 0) {
@@ -265,43 +265,46 @@ k_decode_logits(const DecodeLogitsParams p, const __grid_constant__ DecodeLogitM
     tc_fence_after();
   }
   if (warp == 1) {
-    if (lane == 0) {
+    {  // the whole warp: elect_one()
       // ---------------- MMA issuer --------------------------------------------------------------------
       const uint32_t tmem_base = ctrl->tmem_base;
       const uint32_t idesc = idesc_bf16_f32(NT, NBP);
       int stage = 0; uint32_t phase = 0, job_i = 0;
-      bool ok = !RESIDENT || mbar_wait(smem_u32(&ctrl->hid_full), 0, &ctrl->abort);
+      bool ok = !RESIDENT || mbar_wait_warp(smem_u32(&ctrl->hid_full), 0, &ctrl->abort);
       while (ok) {
         const uint32_t slot = job_i % kJobRing;
-        if (!mbar_wait(smem_u32(&ctrl->job_ready[slot]), (job_i / kJobRing) & 1u, &ctrl->abort)) break;
-        const DecodeJob j = ds->jobs[slot];
-        if (j.cls < 0) break;
+        if (!mbar_wait_warp(smem_u32(&ctrl->job_ready[slot]), (job_i / kJobRing) & 1u, &ctrl->abort)) break;
+        const int cls = __shfl_sync(0xffffffffu, ds->jobs[slot].cls, 0);
+        if (cls < 0) break;
         const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
-        if (!mbar_wait(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) break;
+        if (!mbar_wait_warp(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) break;
         tc_fence_after();
         const uint32_t d = tmem_base + buf * NBP;
-        const int ksb = j.cls == 2 ? 1 : 2;
-        const uint32_t kb_bytes = (uint32_t)(j.cls == 2 ? NT : kGran) * 128;   // one k-block of the job's rows
+        const int ksb = cls == 2 ? 1 : 2;
+        const uint32_t kb_bytes = (uint32_t)(cls == 2 ? NT : kGran) * 128;   // one k-block of the job's rows
         uint32_t acc = 0;
         for (int ks = 0; ks < p.ksteps; ks += ksb) {
-          if (!mbar_wait(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
+          if (!mbar_wait_warp(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
           tc_fence_after();
           const uint32_t wb = stage_base + (uint32_t)stage * stage_bytes;
-          for (int i = 0; i < ksb; ++i) {
+          const bool issues = elect_one();
+          for (int i = 0; issues && i < ksb; ++i) {
             const uint32_t wi = wb + (uint32_t)i * kb_bytes;
             const uint32_t hb = RESIDENT ? hid_base + (uint32_t)(ks + i) * hid_rows * 128
                                          : wb + NT * 128 + (uint32_t)i * hid_rows * 128;
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-              umma_bf16(d, smem_desc_sw128(wi + k * 32), smem_desc_sw128(hb + k * 32), idesc, acc);
-              acc = 1;
+              umma_bf16(d, smem_desc_sw128(wi + k * 32), smem_desc_sw128(hb + k * 32), idesc, i || k ? 1u : acc);
             }
           }
-          umma_commit(smem_u32(&ctrl->empty[stage]));            // frees the stage once the MMAs have read it
+          if (issues) umma_commit(smem_u32(&ctrl->empty[stage]));      // frees the stage once the MMAs have read it
+          __syncwarp();
+          acc = 1;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        umma_commit(smem_u32(&ctrl->acc_full[buf]));
+        if (elect_one()) umma_commit(smem_u32(&ctrl->acc_full[buf]));
+        __syncwarp();
         ++job_i;
       }
     }

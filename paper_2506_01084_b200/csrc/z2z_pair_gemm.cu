@@ -25,7 +25,7 @@
 // two and a stage holds 32 KB instead of 48: half the tensor-core work of the layer.  kEpiGelu
 // then writes one fp16 matrix.
 //
-// Roles per CTA: warp 0 lane 0 TMA producer, warp 1 lane 0 MMA issuer (leader CTA only), warps
+// Roles per CTA: warp 0 lane 0 TMA producer, warp 1 MMA issuer (an elected lane; leader CTA only), warps
 // 2-5 epilogue (thread = row).  Every mbarrier wait is bounded.
 #include <cuda_fp16.h>
 
@@ -62,7 +62,7 @@ k_pair_gemm(const PairGemmParams p, const __grid_constant__ CUtensorMap tmA, con
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   PgCtrl* ctrl = reinterpret_cast<PgCtrl*>(sm);
   const uint32_t stage_base = smem_u32(sm + 1024);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();          // 0: leader (issues the MMAs), 1: peer
   const int n_clusters = gridDim.x >> 1, cluster_id = blockIdx.x >> 1;
   pdl_trigger();                                    // the next kernel may get resident behind this one
@@ -122,34 +122,37 @@ k_pair_gemm(const PairGemmParams p, const __grid_constant__ CUtensorMap tmA, con
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
-      // ---------------- MMA issuer (leader only) ------------------------------------------------------
+    if (rank == 0) {
+      // ---------------- MMA issuer (leader only, the whole warp: elect_one()) ------------------------------------------------------
       const uint32_t idesc = HALF ? idesc_f16_f32(256, p.tile_cols) : idesc_bf16_f32(256, p.tile_cols);
       int stage = 0; uint32_t phase = 0, job_i = 0;
       bool ok = true;
       for (int t = cluster_id; t < n_tiles && ok; t += n_clusters) {
         const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
-        if (!mbar_wait(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) break;
+        if (!mbar_wait_warp(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) break;
         tc_fence_after();
         const uint32_t d = tmem_base + buf * 256;
         uint32_t acc = 0;
         for (int ks = 0; ks < p.ksteps; ++ks) {
-          if (!mbar_wait(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
+          if (!mbar_wait_warp(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
           tc_fence_after();
           const uint32_t sb = stage_base + (uint32_t)stage * kPgStageBytes;
+          if (elect_one()) {
 #pragma unroll
-          for (int part = 0; part < (HALF ? 1 : 2); ++part)        // hi part, then lo part, into the same accumulator
+            for (int part = 0; part < (HALF ? 1 : 2); ++part)      // hi part, then lo part, into the same accumulator
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              umma_bf16_pair(d, smem_desc_sw128(sb + part * 16384 + k * 32), smem_desc_sw128(sb + kWOff + k * 32),
-                             idesc, acc);
-              acc = 1;
-            }
-          umma_commit_pair(smem_u32(&ctrl->empty[stage]));      // frees the stage in both CTAs
+              for (int k = 0; k < 4; ++k)
+                umma_bf16_pair(d, smem_desc_sw128(sb + part * 16384 + k * 32), smem_desc_sw128(sb + kWOff + k * 32),
+                               idesc, part || k ? 1u : acc);
+            umma_commit_pair(smem_u32(&ctrl->empty[stage]));    // frees the stage in both CTAs
+          }
+          __syncwarp();
+          acc = 1;
           if (++stage == kPgStages) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        umma_commit_pair(smem_u32(&ctrl->acc_full[buf]));       // wakes the epilogues of both CTAs
+        if (elect_one()) umma_commit_pair(smem_u32(&ctrl->acc_full[buf]));       // wakes the epilogues of both CTAs
+        __syncwarp();
         ++job_i;
       }
     }

@@ -22,7 +22,7 @@
 // replaced a kernel of single CTAs that streams all weights once per 128 rows (V = 128256, d = 4096:
 // 343 -> 231 us at 129 rows, 988 -> 570 at 700, 2714 -> 1395 at 2000).
 //
-// Roles per CTA: warp 0 lane 0 TMA producer, warp 1 lane 0 MMA issuer (leader CTA only),
+// Roles per CTA: warp 0 lane 0 TMA producer, warp 1 MMA issuer (an elected lane; leader CTA only),
 // warps 2-5 epilogue.  Every mbarrier wait is bounded; on a timeout the CTA raises an abort flag,
 // all roles leave their loops, tensor memory is released and an error word is set.
 #include "z2z_common.cuh"
@@ -177,7 +177,7 @@ k_prefill_logits(const PrefillLogitsParams p, const __grid_constant__ PrefillMap
   PCtrl* ctrl = reinterpret_cast<PCtrl*>(sm);
   RowRed* s_red = reinterpret_cast<RowRed*>(sm + 1024);
   const uint32_t stage_base = smem_u32(sm + 4096);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();          // 0: leader (issues the MMAs), 1: peer
   const long long n_clusters = gridDim.x >> 1, cluster_id = blockIdx.x >> 1;
   const long long n_units = (long long)p.row_tiles * p.strips;
@@ -240,8 +240,8 @@ k_prefill_logits(const PrefillLogitsParams p, const __grid_constant__ PrefillMap
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {
-      // ---------------- MMA issuer (leader only) ------------------------------------------------------
+    if (rank == 0) {
+      // ---------------- MMA issuer (leader only, the whole warp: elect_one()) ------------------------------------------------------
       UnitWalk w(p);
       int stage = 0; uint32_t phase = 0, job_i = 0;
       bool ok = true;
@@ -250,25 +250,28 @@ k_prefill_logits(const PrefillLogitsParams p, const __grid_constant__ PrefillMap
         TileRef t;
         while (ok && w.next(t)) {
           const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
-          if (!mbar_wait(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) { ok = false; break; }
+          if (!mbar_wait_warp(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) { ok = false; break; }
           tc_fence_after();
           const uint32_t idesc = idesc_bf16_f32(kTileRows, t.ng * kGran);
           const uint32_t d = tmem_base + buf * kTileCols;
           uint32_t acc = 0;
           for (int ks = 0; ks < p.ksteps; ++ks) {
-            if (!mbar_wait(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
+            if (!mbar_wait_warp(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
             tc_fence_after();
             const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
+            if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              umma_bf16_pair(d, smem_desc_sw128(sb + k * 32), smem_desc_sw128(sb + w_off + k * 32), idesc, acc);
-              acc = 1;
+              for (int k = 0; k < 4; ++k)
+                umma_bf16_pair(d, smem_desc_sw128(sb + k * 32), smem_desc_sw128(sb + w_off + k * 32), idesc, k ? 1u : acc);
+              umma_commit_pair(smem_u32(&ctrl->empty[stage]));    // frees the stage in both CTAs
             }
-            umma_commit_pair(smem_u32(&ctrl->empty[stage]));      // frees the stage in both CTAs
+            __syncwarp();
+            acc = 1;
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
           }
           if (!ok) break;
-          umma_commit_pair(smem_u32(&ctrl->acc_full[buf]));       // wakes the epilogues of both CTAs
+          if (elect_one()) umma_commit_pair(smem_u32(&ctrl->acc_full[buf]));       // wakes the epilogues of both CTAs
+          __syncwarp();
           ++job_i;
         }
       }

@@ -195,26 +195,29 @@ __device__ __forceinline__ void logits_mma(const StreamLogitsParams& p, const in
   while (sched.next_of_both(j)) {
     const uint32_t idesc = idesc_bf16_f32(128, j.nrows);
     const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
-    if (!mbar_wait(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) return;
+    if (!mbar_wait_warp(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) return;
     tc_fence_after();
     const uint32_t d = tmem_base + buf * kLogitNT;
     uint32_t acc = 0;
     for (int ks = 0; ks < p.ksteps; ks += j.kb) {
-      if (!mbar_wait(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) return;
+      if (!mbar_wait_warp(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) return;
       tc_fence_after();
       const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
-      for (int i = 0; i < j.kb; ++i) {
-        const uint32_t ab = sb + (uint32_t)i * 1024u, wb = sb + w_off + (uint32_t)(i * j.nrows) * 128u;
+      if (elect_one()) {
+        for (int i = 0; i < j.kb; ++i) {
+          const uint32_t ab = sb + (uint32_t)i * 1024u, wb = sb + w_off + (uint32_t)(i * j.nrows) * 128u;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          umma_bf16(d, smem_desc_sw128(ab + k * 32), smem_desc_sw128(wb + k * 32), idesc, acc);
-          acc = 1;
+          for (int k = 0; k < 4; ++k)
+            umma_bf16(d, smem_desc_sw128(ab + k * 32), smem_desc_sw128(wb + k * 32), idesc, i || k ? 1u : acc);
         }
+        umma_commit(smem_u32(&ctrl->empty[stage]));        // frees the stage when the MMAs are done
       }
-      umma_commit(smem_u32(&ctrl->empty[stage]));          // frees the stage when the MMAs are done
+      __syncwarp();
+      acc = 1;
       if (++stage == STAGES) { stage = 0; phase ^= 1u; }
     }
-    umma_commit(smem_u32(&ctrl->acc_full[buf]));
+    if (elect_one()) umma_commit(smem_u32(&ctrl->acc_full[buf]));
+    __syncwarp();
     ++job_i;
   }
 }
@@ -281,7 +284,7 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   Ctrl* ctrl = reinterpret_cast<Ctrl*>(sm);
   const uint32_t stage_base = smem_u32(sm + 1024);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const uint32_t a_bytes = (uint32_t)KSB * p.a_box_rows * 128;
   const uint32_t stage_bytes = a_bytes + (uint32_t)KSB * NT * 128;
   pdl_trigger();                                   // the next kernel may get resident behind this one
@@ -358,7 +361,7 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
       need_deps();
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {  // the whole warp: elect_one()
       // ---- MMA issue: D[128 weight rows][n] += W tile (M operand) x live activation rows (N operand)
       pdl_wait();                                      // the live-row count comes from an earlier kernel
       const int live = *p.rows_dev;
@@ -370,29 +373,32 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
       GemmJob j;
       while (ok && walk.next(j)) {
         const uint32_t buf = job_i & 1u, aph = (job_i >> 1) & 1u;
-        if (!mbar_wait(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) break;
+        if (!mbar_wait_warp(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) break;
         tc_fence_after();
         const uint32_t d = tmem_base + buf * (uint32_t)p.a_box_rows;
         uint32_t acc = 0;
         for (int ks = j.kb0; ks < j.kb1; ++ks) {
-          if (!mbar_wait(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
+          if (!mbar_wait_warp(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
           tc_fence_after();
           const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
+          if (elect_one()) {
 #pragma unroll
-          for (int i = 0; i < KSB; ++i) {
-            const uint32_t ab = sb + (uint32_t)i * box_kb;
-            const uint32_t wb = sb + a_bytes + (uint32_t)i * NT * 128;
+            for (int i = 0; i < KSB; ++i) {
+              const uint32_t ab = sb + (uint32_t)i * box_kb;
+              const uint32_t wb = sb + a_bytes + (uint32_t)i * NT * 128;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              umma_bf16(d, smem_desc_sw128(wb + k * 32), smem_desc_sw128(ab + k * 32), idesc, acc);
-              acc = 1;
+              for (int k = 0; k < 4; ++k)
+                umma_bf16(d, smem_desc_sw128(wb + k * 32), smem_desc_sw128(ab + k * 32), idesc, i || k ? 1u : acc);
             }
+            umma_commit(smem_u32(&ctrl->empty[stage]));        // frees the stage when the MMAs are done
           }
-          umma_commit(smem_u32(&ctrl->empty[stage]));          // frees the stage when the MMAs are done
+          __syncwarp();
+          acc = 1;
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        umma_commit(smem_u32(&ctrl->acc_full[buf]));
+        if (elect_one()) umma_commit(smem_u32(&ctrl->acc_full[buf]));
+        __syncwarp();
         ++job_i;
       }
     }
@@ -447,7 +453,7 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
   Ctrl* ctrl = reinterpret_cast<Ctrl*>(sm);
   int* s_pref = reinterpret_cast<int*>(sm + 1024);              // [B + 1] <= 4100 bytes
   const uint32_t stage_base = smem_u32(sm + 1024 + 5120);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   pdl_trigger();                                   // the next kernel may get resident behind this one
   setup_barriers<STAGES>(ctrl);
   if (warp == 3) {
@@ -480,7 +486,7 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
     tc_fence_after();
   }
   if (warp == 1) {
-    if (lane == 0) logits_mma<STAGES>(p, s_pref, ctrl, stage_base, ctrl->tmem_base);
+    logits_mma<STAGES>(p, s_pref, ctrl, stage_base, ctrl->tmem_base);
   } else if (warp >= 2) {
     const uint32_t tmem_base = ctrl->tmem_base;
     LogitSched sched(p, s_pref);

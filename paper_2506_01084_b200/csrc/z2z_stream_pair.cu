@@ -30,7 +30,7 @@
 // Operand layout: packed row r of the activations is rows 2 r (bf16 hi) and 2 r + 1 (lo) of
 // [2 Rt, K], seen as [k-block][operand row][64].  An epilogue thread owns one output feature.
 //
-// Roles per CTA: warp 0 lane 0 TMA producer, warp 1 lane 0 MMA issuer (leader CTA only), warps 2-9
+// Roles per CTA: warp 0 lane 0 TMA producer, warp 1 MMA issuer (an elected lane; leader CTA only), warps 2-9
 // epilogue.  Every mbarrier wait is bounded.
 #include "z2z_common.cuh"
 #include "z2z_internal.h"
@@ -116,7 +116,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   SpCtrl* ctrl = reinterpret_cast<SpCtrl*>(sm);
   const uint32_t stage_base = smem_u32(sm + 1024);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = uniform_warp(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();          // 0: leader (issues the MMAs), 1: peer
   const uint32_t stage_bytes = (uint32_t)p.act_bytes + 16384u;
   const int STAGES = p.stages;
@@ -216,7 +216,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
     const int n_blocks = sp_live_blocks(p, live);
     const int chain = p.parts > 1 ? p.ksteps / p.parts : kSpChain;
     if (warp == 1) {
-      if (lane == 0 && rank == 0) {
+      if (rank == 0) {                                 // (the whole warp: elect_one())
         // ---------------- MMA issuer (leader only): D[256 weight rows][n] += W tile x activation rows -----
         int stage = 0; uint32_t phase = 0, job_i = 0;
         bool ok = live > 0;
@@ -224,28 +224,32 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
         SpJob j;
         while (ok && walk.next(j)) {
           const uint32_t aph = job_i & 1u;
-          if (!mbar_wait(smem_u32(&ctrl->acc_empty), aph ^ 1u, &ctrl->abort)) break;
+          if (!mbar_wait_warp(smem_u32(&ctrl->acc_empty), aph ^ 1u, &ctrl->abort)) break;
           tc_fence_after();
           const int n0 = sp_cols(live, j.block, 0), n1 = sp_cols(live, j.block, 1);
           const uint32_t id0 = idesc_bf16_f32(256, n0), id1 = idesc_bf16_f32(256, n1 ? n1 : 32);
           const uint32_t d = tmem_base;
           uint32_t acc = 0;
           for (int ks = j.kb0; ks < j.kb1; ++ks) {
-            if (!mbar_wait(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
+            if (!mbar_wait_warp(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) { ok = false; break; }
             tc_fence_after();
             const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
             const uint32_t wb = sb + p.act_bytes;
+            if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              umma_bf16_pair(d, smem_desc_sw128(wb + k * 32), smem_desc_sw128(sb + k * 32), id0, acc);
-              if (n1) umma_bf16_pair(d + 256, smem_desc_sw128(wb + k * 32), smem_desc_sw128(sb + 16384u + k * 32), id1, acc);
-              acc = 1;
+              for (int k = 0; k < 4; ++k) {
+                umma_bf16_pair(d, smem_desc_sw128(wb + k * 32), smem_desc_sw128(sb + k * 32), id0, k ? 1u : acc);
+                if (n1) umma_bf16_pair(d + 256, smem_desc_sw128(wb + k * 32), smem_desc_sw128(sb + 16384u + k * 32), id1, k ? 1u : acc);
+              }
+              umma_commit_pair(smem_u32(&ctrl->empty[stage]));    // frees the stage in both CTAs
             }
-            umma_commit_pair(smem_u32(&ctrl->empty[stage]));      // frees the stage in both CTAs
+            __syncwarp();
+            acc = 1;
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
           }
           if (!ok) break;
-          umma_commit_pair(smem_u32(&ctrl->acc_full));       // wakes the epilogues of both CTAs
+          if (elect_one()) umma_commit_pair(smem_u32(&ctrl->acc_full));       // wakes the epilogues of both CTAs
+          __syncwarp();
           ++job_i;
         }
       }
