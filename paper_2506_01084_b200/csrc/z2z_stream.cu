@@ -311,7 +311,8 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
       // returns at once.  A pass without a live row (a step that created no entry) streams nothing: the
       // producer takes in what it loaded ahead, and the other roles have no work.  Such a step of one or 8
       // sequences at d = 3072 went from 224 / 232 to 94 / 90 us (109 / 111 when every GEMM of it still filled
-      // its ring), of 32 at d = 4096 from 563 to 295; steps that create entries take what they took (245, 261, 580).
+      // its ring; 76 / 82 since), of 32 at d = 4096 from 563 to 295 (232 since); steps that create entries took
+      // what they had taken (245, 261, 580).
       const uint64_t pol_w = policy_evict_first(), pol_a = policy_evict_last();
       struct Deferred { int g, kb; };
       Deferred def[kMaxStages];                       // load i of the first pass uses stage i
