@@ -56,22 +56,40 @@ struct Job {
 // Columns are dealt in granules of kLogitGran rows: every CTA takes an even share of the granules of W_U, which it
 // knows without any codebook state, and then one of those of the visible rows of each sequence's U_h.  (One share of
 // both in a row gave some CTAs nothing but hypertokens, whose jobs are short and cost more per granule: V = 128256,
-// d = 4096, 90 sequences of 29 hypertokens 385 us.)  A job is a run of up to kLogitNT / kLogitGran granules inside
-// one segment (W_U, or one sequence).
+// d = 4096, 90 sequences of 29 hypertokens 385 us.)  With fewer than kLogitEvenGrans granules of W_U per CTA it is
+// their jobs that would get short, with all hidden rows each: there it is one share of both in a row after all (d =
+// 3072, 149 hypertokens each, even shares -> one: V = 6020, 54 rows 38 -> 33 us, V = 12000 43 -> 37; V = 17000, 128
+// rows 54 -> 61; a sampled step of 54 sequences at V = 6020 440 -> 412).  A job is a run of up to kLogitNT / kLogitGran
+// granules inside one segment (W_U, or one sequence).
+constexpr int kLogitEvenGrans = 3;
 struct LogitSched {
   const StreamLogitsParams& p;
   const int* pref;       // shared: prefix of per-sequence granule counts, [B + 1]
   int u, u1;
   bool hyper;
+  // (pref has to be there unless the shares are even)
   __device__ LogitSched(const StreamLogitsParams& pp, const int* s_pref) : p(pp), pref(s_pref), hyper(false) {
-    share((p.cb.V + kLogitGran - 1) / kLogitGran);
+    const int ns = n_static(p);
+    if (even(p)) { share(ns); return; }
+    share(ns + pref[p.cb.B]);
+    u = u < ns ? u : ns;
+    u1 = u1 < ns ? u1 : ns;
   }
+  static __device__ int n_static(const StreamLogitsParams& p) { return (p.cb.V + kLogitGran - 1) / kLogitGran; }
+  static __device__ bool even(const StreamLogitsParams& p) { return n_static(p) >= kLogitEvenGrans * (int)gridDim.x; }
   __device__ void share(int total) {
     const int G = gridDim.x, c = blockIdx.x;
     u = (int)((long long)c * total / G);
     u1 = (int)((long long)(c + 1) * total / G);
   }
-  __device__ void begin_hyper() { hyper = true; share(pref[p.cb.B]); }        // (pref is there by now)
+  __device__ void begin_hyper() {                    // (pref is there by now)
+    hyper = true;
+    if (even(p)) { share(pref[p.cb.B]); return; }
+    const int ns = n_static(p);
+    share(ns + pref[p.cb.B]);
+    u = u < ns ? 0 : u - ns;
+    u1 = u1 < ns ? 0 : u1 - ns;
+  }
   __device__ bool next(Job& j) {
     if (u >= u1) return false;
     int remaining, total_rows, g0;
@@ -140,6 +158,10 @@ __device__ __forceinline__ void logits_producer(const StreamLogitsParams& p, con
       tma_load_3d(stage_base + (uint32_t)i * stage_bytes, &tm.h, 0, 0, noted[i], full, pol_a);
     }
   };
+  if (!LogitSched::even(p)) {
+    need_deps();
+    if (!mbar_wait(smem_u32(&ctrl->pref_ready), 0, &ctrl->abort)) return;
+  }
   LogitSched sched(p, s_pref);
   Job j;
   for (int part = 0; part < 2; ++part) {

@@ -61,10 +61,11 @@ def test_sampled_batch_of_one_row_per_sequence(V, d, B):
         assert abs(float(lse[r]) - (l.max() + np.log(np.exp(l - l.max()).sum()))) < 1e-4
 
 
-@pytest.mark.parametrize("V,d,B", [(257, 192, 33), (1000, 1152, 47), (257, 64, 128)])
+@pytest.mark.parametrize("V,d,B", [(257, 192, 33), (1000, 1152, 47), (257, 64, 128), (14100, 192, 47), (14300, 64, 70)])
 def test_batch_with_hypertokens_of_every_job_size(V, d, B):
     """Jobs of 1 to 8 granules of 32 hypertokens: boxes of one, two and four k-blocks, of which the last one ends
-    beyond the width, on the group of 8 hidden rows that holds the sequence's; stored logits too."""
+    beyond the width, on the group of 8 hidden rows that holds the sequence's; vocabularies on both sides of
+    three granules of 32 columns per CTA, from which the shares are even; stored logits too."""
     sizes = [0, 1, 31, 32, 33, 64, 65, 96, 97, 128, 129, 160, 161, 255, 256, 257, 300]
     counts = [sizes[(5 * b) % len(sizes)] for b in range(B)]
     cap = 300
