@@ -32,6 +32,11 @@ using namespace sm100;
 namespace {
 
 constexpr int kThreads = 192;
+// The logits kernel drains with eight warps, two per tensor-memory lane quarter that take every other 32 columns: a
+// sampled column costs its row some 30 instructions, and four warps, of which a batch of 43 rows keeps two busy, took
+// longer than the weights (V = 96132, d = 3200, 43 rows 207 us sampled and 104 not; with eight 140).
+constexpr int kLogitEpiWarps = 8;
+constexpr int kLogitThreads = 64 + 32 * kLogitEpiWarps;
 
 struct Ctrl {
   unsigned long long full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2], pref_ready;
@@ -244,7 +249,7 @@ __device__ __forceinline__ void logits_mma(const StreamLogitsParams& p, const in
   }
 }
 
-template <int STAGES>
+template <int STAGES, int EPI_WARPS = 4>
 __device__ __forceinline__ void setup_barriers(Ctrl* ctrl) {
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -253,7 +258,7 @@ __device__ __forceinline__ void setup_barriers(Ctrl* ctrl) {
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&ctrl->acc_full[b]), 1);
-      mbar_init(smem_u32(&ctrl->acc_empty[b]), 4);
+      mbar_init(smem_u32(&ctrl->acc_empty[b]), EPI_WARPS);
     }
     mbar_init(smem_u32(&ctrl->pref_ready), 1);         // logits: the sequences' granules are counted
     ctrl->abort = 0;
@@ -468,7 +473,7 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
 // Logits kernel: fused reductions
 // =================================================================================================
 template <int STAGES>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kLogitThreads, 1)
 k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm) {
   constexpr int NT = kLogitNT;
   extern __shared__ unsigned char smem_raw[];
@@ -478,7 +483,7 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
   const uint32_t stage_base = smem_u32(sm + 1024 + 5120);
   const int warp = uniform_warp(), lane = threadIdx.x & 31;
   pdl_trigger();                                   // the next kernel may get resident behind this one
-  setup_barriers<STAGES>(ctrl);
+  setup_barriers<STAGES, kLogitEpiWarps>(ctrl);
   if (warp == 3) {
     if (lane < 1 + 2 * kLogitBoxClasses) prefetch_tmap(lane == 0 ? &tm.h : &tm.w[lane - 1]);
     if (lane < 3) { prefetch_tmap(&tm.h8[lane]); prefetch_tmap(&tm.u[lane]); }
@@ -505,7 +510,7 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
       if (lane == 0) mbar_arrive(smem_u32(&ctrl->pref_ready));
     }
     tc_fence_before();
-    asm volatile("bar.sync 2, %0;" ::"n"(kThreads - 32) : "memory");      // all but the producer warp
+    asm volatile("bar.sync 2, %0;" ::"n"(kLogitThreads - 32) : "memory");      // all but the producer warp
     tc_fence_after();
   }
   if (warp == 1) {
@@ -513,7 +518,8 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
   } else if (warp >= 2) {
     const uint32_t tmem_base = ctrl->tmem_base;
     LogitSched sched(p, s_pref);
-    const int q = warp & 3;
+    const int q = warp & 3;                        // tensor-memory lane quarter this warp may read
+    const int half = (warp - 2) >> 2;              // which 32-column groups of a job it takes
     const LogitsArgs& a = p.la;
     const uint32_t k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32);
     const uint32_t c2 = (uint32_t)a.step, c3 = (uint32_t)(a.step >> 32);
@@ -540,7 +546,7 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
       if (my_seq >= 0) limit = j.owner < 0 ? j.nvalid : (my_seq == j.owner ? min(j.nvalid, my_nvis - j.k0) : 0);
       if (__any_sync(0xffffffffu, limit > 0)) {
 #pragma unroll 1
-        for (int c0 = 0; c0 < j.nrows; c0 += 32) {
+        for (int c0 = 32 * half; c0 < j.nrows; c0 += 64) {
           if (!__any_sync(0xffffffffu, limit > c0)) break;
           uint32_t v[32];
           tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + buf * NT + c0, v);
@@ -562,7 +568,12 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
       if (lane == 0) mbar_arrive(smem_u32(&ctrl->acc_empty[buf]));
       ++job_i;
     }
-    if (r < a.N) {
+    // every load has been consumed: the ring's first stage takes the second warps' reductions
+    RowRed* other = reinterpret_cast<RowRed*>(sm + 1024 + 5120) + q * 32 + lane;
+    if (half == 1) *other = red;
+    asm volatile("bar.sync 1, %0;" ::"n"(32 * kLogitEpiWarps) : "memory");
+    if (half == 0) red.merge(*other);
+    if (half == 0 && r < a.N) {
       LogitPartial* lp = reinterpret_cast<LogitPartial*>(a.lpart) + (size_t)r * p.part_stride + blockIdx.x;
       lp->m = red.m; lp->s = red.s; lp->idx = red.idx; lp->gm = red.gm; lp->gidx = red.gidx;
     }
@@ -756,7 +767,7 @@ static cudaError_t launch_logits_t(const StreamLogitsParams& p, const LogitMaps&
   auto kern = k_stream_logits<STAGES>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(kern, dim3(grid), dim3(kThreads), smem, s, p, maps);
+  return launch_pdl(kern, dim3(grid), dim3(kLogitThreads), smem, s, p, maps);
 }
 
 cudaError_t run_logits_stream(const CbView& cb, const LogitsArgs& a, int* err_word, LogitsPartInfo* info, Prof* prof,
