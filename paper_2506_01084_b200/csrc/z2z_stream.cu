@@ -32,10 +32,12 @@ using namespace sm100;
 namespace {
 
 constexpr int kThreads = 192;
-// The logits kernel drains with eight warps, two per tensor-memory lane quarter that take every other 32 columns: a
+// The logits kernel drains with twelve warps, three per tensor-memory lane quarter that take every third 32 columns: a
 // sampled column costs its row some 30 instructions, and four warps, of which a batch of 43 rows keeps two busy, took
-// longer than the weights (V = 96132, d = 3200, 43 rows 207 us sampled and 104 not; with eight 140).
-constexpr int kLogitEpiWarps = 8;
+// longer than the weights (sampled with 4 / 8 / 12 warps, argmax: V = 96132, d = 3200, 43 rows 207 / 140 / 142, 104 us;
+// V = 128256, d = 4096, 128 rows 276 / 214 / 199, 180).
+constexpr int kLogitEpiWarps = 12;
+constexpr int kLogitEpiGroups = kLogitEpiWarps / 4;
 constexpr int kLogitThreads = 64 + 32 * kLogitEpiWarps;
 
 struct Ctrl {
@@ -519,7 +521,7 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
     const uint32_t tmem_base = ctrl->tmem_base;
     LogitSched sched(p, s_pref);
     const int q = warp & 3;                        // tensor-memory lane quarter this warp may read
-    const int half = (warp - 2) >> 2;              // which 32-column groups of a job it takes
+    const int group = (warp - 2) >> 2;             // which 32-column groups of a job it takes
     const LogitsArgs& a = p.la;
     const uint32_t k0 = (uint32_t)a.seed, k1 = (uint32_t)(a.seed >> 32);
     const uint32_t c2 = (uint32_t)a.step, c3 = (uint32_t)(a.step >> 32);
@@ -546,7 +548,7 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
       if (my_seq >= 0) limit = j.owner < 0 ? j.nvalid : (my_seq == j.owner ? min(j.nvalid, my_nvis - j.k0) : 0);
       if (__any_sync(0xffffffffu, limit > 0)) {
 #pragma unroll 1
-        for (int c0 = 32 * half; c0 < j.nrows; c0 += 64) {
+        for (int c0 = 32 * group; c0 < j.nrows; c0 += 32 * kLogitEpiGroups) {
           if (!__any_sync(0xffffffffu, limit > c0)) break;
           uint32_t v[32];
           tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + buf * NT + c0, v);
@@ -568,12 +570,13 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
       if (lane == 0) mbar_arrive(smem_u32(&ctrl->acc_empty[buf]));
       ++job_i;
     }
-    // every load has been consumed: the ring's first stage takes the second warps' reductions
-    RowRed* other = reinterpret_cast<RowRed*>(sm + 1024 + 5120) + q * 32 + lane;
-    if (half == 1) *other = red;
+    // every load has been consumed: the ring's first stage takes the other warps' reductions
+    RowRed* others = reinterpret_cast<RowRed*>(sm + 1024 + 5120) + q * 32 + lane;
+    if (group > 0) others[(group - 1) * 128] = red;
     asm volatile("bar.sync 1, %0;" ::"n"(32 * kLogitEpiWarps) : "memory");
-    if (half == 0) red.merge(*other);
-    if (half == 0 && r < a.N) {
+    if (group == 0)
+      for (int g = 1; g < kLogitEpiGroups; ++g) red.merge(others[(g - 1) * 128]);
+    if (group == 0 && r < a.N) {
       LogitPartial* lp = reinterpret_cast<LogitPartial*>(a.lpart) + (size_t)r * p.part_stride + blockIdx.x;
       lp->m = red.m; lp->s = red.s; lp->idx = red.idx; lp->gm = red.gm; lp->gidx = red.gidx;
     }
