@@ -144,8 +144,7 @@ struct LogitSched {
 __host__ __device__ constexpr uint32_t logit_w_offset(int a_box_rows) { return (uint32_t)a_box_rows * 128u + 3u * 1024u; }
 
 // ---- producer and MMA role of the logits kernel -----------------------------------------------------
-// W_U depends on no earlier kernel, the hidden rows and the codebooks do: the first pass over the ring issues
-// the weight boxes at once and notes the boxes of hidden rows, which go out behind the dependency wait.
+// Everything that is loaded, W_U among it, may come from the kernel ahead: nothing is issued before the dependency wait.
 template <int STAGES>
 __device__ __forceinline__ void logits_producer(const StreamLogitsParams& p, const int* s_pref, Ctrl* ctrl, uint32_t stage_base,
                                                 const LogitMaps& tm) {
@@ -153,42 +152,23 @@ __device__ __forceinline__ void logits_producer(const StreamLogitsParams& p, con
   const uint32_t stage_bytes = w_off + kLogitNT * 128;             // smem stride of a stage
   const uint64_t pol_w = policy_evict_first(), pol_a = policy_evict_last();
   int stage = 0; uint32_t phase = 0;
-  int noted[STAGES], n_noted = 0;                                  // load i of the first pass uses stage i: its k-block
-  bool deps = false;
-  auto need_deps = [&]() {
-    if (deps) return;
-    pdl_wait();
-    deps = true;
-    for (int i = 0; i < n_noted; ++i) {
-      const uint32_t full = smem_u32(&ctrl->full[i]);
-      mbar_expect_tx(full, a_bytes);
-      tma_load_3d(stage_base + (uint32_t)i * stage_bytes, &tm.h, 0, 0, noted[i], full, pol_a);
-    }
-  };
-  if (!LogitSched::even(p)) {
-    need_deps();
-    if (!mbar_wait(smem_u32(&ctrl->pref_ready), 0, &ctrl->abort)) return;
-  }
+  pdl_wait();
+  if (!LogitSched::even(p) && !mbar_wait(smem_u32(&ctrl->pref_ready), 0, &ctrl->abort)) return;
   LogitSched sched(p, s_pref);
   Job j;
   for (int part = 0; part < 2; ++part) {
     if (part == 1) {
-      need_deps();
       if (!mbar_wait(smem_u32(&ctrl->pref_ready), 0, &ctrl->abort)) return;
       sched.begin_hyper();
     }
     while (sched.next(j)) {
       for (int ks = 0; ks < p.ksteps; ks += j.kb) {
-        if (n_noted == STAGES) need_deps();
-        if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) { need_deps(); return; }
+        if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) return;
         const uint32_t full = smem_u32(&ctrl->full[stage]);
         const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
         // (k-blocks beyond the last one, and rows outside the tensors, are zero-filled and counted)
         const uint32_t w_bytes = (uint32_t)(j.kb * j.nrows) * 128u;
-        if (!deps) {
-          mbar_expect_only(full, w_bytes);
-          noted[n_noted++] = ks;
-        } else if (j.group < 0) {
+        if (j.group < 0) {
           mbar_expect_tx(full, a_bytes + w_bytes);
           tma_load_3d(sb, &tm.h, 0, 0, ks, full, pol_a);
         } else {
@@ -484,19 +464,19 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
   int* s_pref = reinterpret_cast<int*>(sm + 1024);              // [B + 1] <= 4100 bytes
   const uint32_t stage_base = smem_u32(sm + 1024 + 5120);
   const int warp = uniform_warp(), lane = threadIdx.x & 31;
-  pdl_trigger();                                   // the next kernel may get resident behind this one
   setup_barriers<STAGES, kLogitEpiWarps>(ctrl);
   if (warp == 3) {
     if (lane < 1 + 2 * kLogitBoxClasses) prefetch_tmap(lane == 0 ? &tm.h : &tm.w[lane - 1]);
     if (lane < 3) { prefetch_tmap(&tm.h8[lane]); prefetch_tmap(&tm.u[lane]); }
   }
-  __syncthreads();                                 // barriers exist; the producer starts at once
+  __syncthreads();                                 // barriers exist, which is all that the producer needs
 
   if (warp == 0) {
     if (lane == 0) logits_producer<STAGES>(p, s_pref, ctrl, stage_base, tm);
   } else {
     if (warp == 2) { tmem_alloc(smem_u32(&ctrl->tmem_base), tmem_cols(NT)); tmem_relinquish(); }
     pdl_wait();                                    // codebook counters, row tables and partial slots are dependent
+    pdl_trigger();                                 // (behind the wait: a step's encoder pass loads weights ahead of its own)
     if (warp == 1) {                               // prefix of the sequences' granule counts
       int carry = 0;
       for (int b0 = 0; b0 < p.cb.B; b0 += 32) {
