@@ -21,6 +21,12 @@
  *     into a CUDA graph (arguments passed by value, the sampling step among them, are then fixed
  *     for every replay); capture again after z2z_codebook_init starts a new session, because
  *     z2z_decode_step decides on the host whether the session still needs its hyper-encoder pass.
+ *   - A call sees what the work ahead of it on the stream has written, with one exception.  In bf16
+ *     sessions with d % 128 == 0, z2z_decode_step of B <= 32 sequences reads d_WU and the encoder
+ *     tensors, and z2z_dynamic_logits of N <= 32 rows reads d_WU, before the kernel directly ahead
+ *     is done when that kernel releases its dependents early (programmatic dependent launch:
+ *     z2z_upload_rows does, and library GEMMs may).  Where such a kernel writes those tensors, put
+ *     an ordinary kernel, a copy or an event between it and the call.
  *   - Ids are int32.  Tables are row-major [rows, d] in the configured dtype.
  *   - Hypertoken id = V + k where k is the creation order within the sequence.
  *   - Limits: V + cap < 2^24 - 1, cap <= 65535, 1 <= M <= 8, d % 8 == 0, B <= 1024.
@@ -245,7 +251,8 @@ int32_t z2z_sample_filtered(const float* d_logits, int32_t N, int64_t ld, const 
 /* Host -> device transfer of a small per-step input (the hidden rows of a decode step) by a kernel
  * instead of a copy-engine transfer (no counterpart in the paper; end-to-end latency aid).  The
  * kernel that follows on the stream may start its independent part - z2z_decode_step's logits
- * kernel streams W_U before it needs the hidden rows - while the transfer runs.
+ * kernel streams W_U before it needs the hidden rows - while the transfer runs.  (For rows, not for
+ * tables: see the order of calls on the stream, above.)
  *   h_mapped_src: pinned host memory that is mapped into the device's address space;
  *   d_dst: device memory; bytes: multiple of 16, at most 256 MiB; both pointers 16-byte aligned. */
 int32_t z2z_upload_rows(const void* h_mapped_src, void* d_dst, size_t bytes, z2z_stream stream);

@@ -404,8 +404,8 @@ k_decode_logits(const DecodeLogitsParams p, const __grid_constant__ DecodeLogitM
 
 // One warp per hidden row: merge the partials of all CTAs, write the outputs.
 __global__ void __launch_bounds__(128) k_decode_logits_merge(LogitsArgs a, int stride, int count) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= a.N) return;

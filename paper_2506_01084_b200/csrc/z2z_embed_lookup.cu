@@ -19,8 +19,8 @@ constexpr int kLookupUnroll = 4;
 __global__ void __launch_bounds__(kLookupThreads) k_embed_lookup(
     CbView cb, const int32_t* codes, int N, const int32_t* row_seq, const uint4* WE, const uint4* Eh, uint4* out,
     int row_vecs /* 16-byte vectors per row */) {
-  sm100::pdl_trigger();
   sm100::pdl_wait();                              // codes, codebook state and cache rows come from earlier kernels
+  sm100::pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < N; r += warps) {

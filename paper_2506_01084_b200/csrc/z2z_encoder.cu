@@ -26,8 +26,8 @@ __global__ void __launch_bounds__(1024) k_entry_offsets(CbView cb, int which, in
                                                         const int32_t* first, const int32_t* count,
                                                         const int32_t* new_entry, int32_t* off) {
   __shared__ int sm[32];
-  sm100::pdl_trigger();
   sm100::pdl_wait();
+  sm100::pdl_trigger();
   const int b = threadIdx.x;
   int c = 0;
   if (b < cb.B) {
@@ -102,8 +102,8 @@ __global__ void k_entry_fill(CbView cb, int which, int mode, const int32_t* firs
 __global__ void __launch_bounds__(1024) k_entry_list(CbView cb, int which, const int32_t* first, const int32_t* count, EntryList el,
                                                      int slots, int have_off) {
   __shared__ int warp_sums[32], s_off[1024], s_from[1024];
-  sm100::pdl_trigger();
   sm100::pdl_wait();
+  sm100::pdl_trigger();
   const int e = threadIdx.x;
   int f = 0, c = 0, off = 0, total;
   if (e < cb.B) {
@@ -162,8 +162,8 @@ __global__ void __launch_bounds__(1024) k_entry_list(CbView cb, int which, const
 
 // Packed rows (base tokens) of all entries of the call, added up in el.off[B + 1] (zero before).
 __global__ void __launch_bounds__(256) k_entry_rows(CbView cb, int which, const int32_t* first, EntryList el) {
-  sm100::pdl_trigger();
   sm100::pdl_wait();
+  sm100::pdl_trigger();
   const int b = blockIdx.x;
   const int count = el.off[b + 1] - el.off[b];
   int f = first ? first[b] : due_from(cb, which, b);
@@ -180,8 +180,8 @@ __global__ void __launch_bounds__(256) k_entry_rows(CbView cb, int which, const 
 __global__ void __launch_bounds__(1024) k_entry_passes(CbView cb, int which, const int32_t* first, EntryList el, int rows_per,
                                                        int n_passes, int32_t* pass_first) {
   __shared__ int sm[32];
-  sm100::pdl_trigger();
   sm100::pdl_wait();
+  sm100::pdl_trigger();
   const int total = el.off[cb.B];
   long long before = 0;                          // rows ahead of this batch of entries
   for (int g0 = 0; g0 < total; g0 += 1024) {
@@ -210,8 +210,8 @@ __global__ void __launch_bounds__(1024) k_entry_passes(CbView cb, int which, con
 // what the bound left out is due for the next call and stays so through decode steps.  After a decode step
 // (off == NULL): every entry is embedded, unless a call left some out.
 __global__ void k_mark_embedded(CbView cb, int which, const int32_t* off, long long bound) {
-  sm100::pdl_trigger();
   sm100::pdl_wait();
+  sm100::pdl_trigger();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= cb.B) return;
   int32_t* emb = cb.n_emb + which * cb.B + b;

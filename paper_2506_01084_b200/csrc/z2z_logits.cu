@@ -45,8 +45,8 @@ __global__ void __launch_bounds__(256) k_logits_simt(CbView cb, LogitsArgs a, in
   const int r0 = blockIdx.y * kTR;
   const int G = gridDim.x, g = blockIdx.x;
   const int t = threadIdx.x;
-  sm100::pdl_trigger();
   sm100::pdl_wait();
+  sm100::pdl_trigger();
   if (t < kTR) {
     const int r = r0 + t;
     int sq = -1, nv = 0, tg = -1;
@@ -127,8 +127,8 @@ __global__ void __launch_bounds__(256) k_logits_simt(CbView cb, LogitsArgs a, in
 
 // One warp per row: merge G partials, write the outputs.
 __global__ void __launch_bounds__(128) k_logits_merge(LogitsArgs a, int G) {
-  sm100::pdl_trigger();
   sm100::pdl_wait();
+  sm100::pdl_trigger();
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (r >= a.N) return;

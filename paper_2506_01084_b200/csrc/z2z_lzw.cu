@@ -216,8 +216,8 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_encode(CbView cb, 
 // none_sits_out: a code equal to Z2Z_CODE_NONE marks a sequence that takes no part in this step.
 __global__ void __launch_bounds__(128) k_lzw_step(CbView cb, const int32_t* new_codes, const uint8_t* active,
                                                   int none_sits_out, int32_t* new_entry) {
-  sm100::pdl_trigger();
   sm100::pdl_wait();
+  sm100::pdl_trigger();
   const int lane = threadIdx.x & 31;
   const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (b >= cb.B) return;

@@ -131,8 +131,8 @@ struct UnitWalk {
 // ---- plan: sequence range and cost of the hypertoken tiles of every row tile; target logits start as NaN -----------------------------------
 __global__ void __launch_bounds__(256) k_prefill_plan(PrefillLogitsParams p) {
   __shared__ int s_lo, s_hi, s_nh;
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const int rt = blockIdx.x;
   if (threadIdx.x == 0) { s_lo = 0x7fffffff; s_hi = -1; s_nh = 0; }
   __syncthreads();

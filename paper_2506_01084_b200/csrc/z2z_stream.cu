@@ -569,8 +569,8 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
 
 // One warp per row: merge the partial reductions of the G CTAs.
 __global__ void __launch_bounds__(128) k_stream_logits_merge(StreamLogitsParams p, int G) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const LogitsArgs& a = p.la;
   const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;

@@ -54,3 +54,59 @@ def test_batch_logits_behind_an_upload_of_the_table(V, B, step):
         return lse, best
 
     _uploaded_ahead(WU, call)
+
+
+# max_entries 30: one launch for list, offsets and row map; 1100: offsets, list and map apart; several row blocks
+@pytest.mark.parametrize("bound", [30, 1100])
+def test_bounded_embedding_behind_an_upload_of_the_weights(bound):
+    V, d, dff, cap, B = 500, 256, 512, 600, 2
+    cb = zb.Codebook(zb.make_config(V, d, 2, cap, B, "bf16", 2, 2, dff), DEV)
+    tok = torch.randperm(V, generator=torch.Generator().manual_seed(1))[:2 * 40].to(torch.int32).view(B, 40).to(DEV)
+    codes, lens = torch.zeros_like(tok), torch.zeros(B, dtype=torch.int32, device=DEV)
+    zb.z2z_lzw_encode(cb, tok, None, codes, lens)
+    shapes = [(2, d)] + 2 * [(d,), (d,), (3 * d, d), (3 * d,), (d, d), (d,), (d,), (d,), (dff, d), (dff,), (d, dff), (d,)]
+    sizes = [torch.Size(s).numel() for s in shapes]
+    flat = _rnd(5, sum(sizes), std=0.05)                 # one tensor holds them all
+    enc = zb.encoder_weights([t.view(s) for t, s in zip(flat.split(sizes), shapes)])
+    table = _rnd(6, V, d)
+    first = torch.zeros(B, dtype=torch.int32, device=DEV)
+    count = torch.full((B,), 15, dtype=torch.int32, device=DEV)
+
+    def call():
+        rows = torch.zeros(B, cap, d, dtype=torch.bfloat16, device=DEV)
+        zb.z2z_hyper_embed(cb, zb.CACHE_EMBED, table, enc, first, count, bound, rows)
+        return (rows,)
+
+    _uploaded_ahead(flat, call)
+
+
+# what stands between the upload and the call that may read ahead of the kernel right before it
+@pytest.mark.parametrize("between", ["lookup", "update", "embed", "positions", "batch"])
+def test_decode_logits_behind_another_call_behind_an_upload(between):
+    V, d, cap, B = 14400, 128, 600, 40
+    cb = zb.Codebook(zb.make_config(V, d, 2, cap, B, "bf16", 0, 1, 8), DEV)
+    WE, WU = _rnd(1, V, d), _rnd(2, V, d, std=0.05)
+    Eh, Uh, hid = (_rnd(3 + i, *s) for i, s in enumerate([(B, cap, d), (B, cap, d), (48, d)]))
+    x, lse48, pos = torch.zeros_like(hid), torch.zeros(48, device=DEV), zb.encoder_weights([_rnd(7, 2, d)])
+    code = torch.arange(B, dtype=torch.int32, device=DEV)
+    off = torch.zeros(B, dtype=torch.uint8, device=DEV)
+    zero = torch.zeros(B, dtype=torch.int32, device=DEV)
+    seq = torch.arange(48, dtype=torch.int32, device=DEV) % 3
+    args = (zb.SELECT_ARGMAX, 1.0, 0, 0, None)
+
+    def call():
+        if between == "lookup":
+            zb.z2z_embed_lookup(cb, code, None, WE, Eh, x)
+        elif between == "update":
+            zb.z2z_lzw_step(cb, code, off, None)
+        elif between == "embed":
+            zb.z2z_hyper_embed(cb, zb.CACHE_EMBED, WE, pos, zero, zero, 8, Eh)
+        elif between == "positions":                     # more rows than sequences
+            zb.z2z_dynamic_logits(cb, hid, seq, None, WE, Uh, *args, lse48, None, None)
+        else:
+            zb.z2z_dynamic_logits(cb, hid[:B], None, None, WE, Uh, *args, lse48, None, None)
+        lse, best = torch.zeros(8, device=DEV), torch.zeros(8, dtype=torch.int32, device=DEV)
+        zb.z2z_dynamic_logits(cb, hid[:8], None, None, WU, Uh, *args, lse, best, None)
+        return lse, best
+
+    _uploaded_ahead(WU, call)
