@@ -91,6 +91,62 @@ def test_batch_with_hypertokens_of_every_job_size(V, d, B):
         assert float(l.max() - l[int(am[r])]) < 2 * tol and abs(float(mx[r]) - float(l.max())) < tol
 
 
+@pytest.mark.parametrize("select", [0, 1])
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("N", [33, 70, 128])
+@pytest.mark.parametrize("granules,d", [(3, 448), (8.5, 448), (19.3, 320)])
+def test_batch_with_several_column_jobs_per_cta(granules, d, N, given, select):
+    """Even shares of W_U: three granules of 32 columns per CTA (the fewest that are dealt so), one job of 256 columns
+    and a rest, two of them and a rest; more k-blocks than the ring has stages (five up to 40 rows, four at
+    128); behind them the hypertokens.  Rows in the order of their sequences, or given with them, their limits and targets."""
+    from oracle import logits as olg
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    V = 32 * int(granules * sms) - (5 if granules > 3 else 0)
+    assert (V + 31) // 32 >= 3 * sms
+    sizes = [0, 1, 33, 64, 100, 129, 256, 300]
+    B, cap, T, seed, step = N + 2, 300, 0.9, 77, 5
+    counts = [sizes[(3 * b) % len(sizes)] for b in range(B)]
+    cb = _session(V, d, B, cap, counts, 9)
+    g = torch.Generator(device=DEV)
+    g.manual_seed(N + V)
+    rnd = lambda *s, std: (torch.randn(*s, generator=g, device=DEV) * std).to(torch.bfloat16)
+    hid, WU, Uh = rnd(N, d, std=1.0), rnd(V, d, std=0.05), rnd(B, cap, d, std=0.05)
+    for b in range(B):
+        Uh[b, counts[b]:] = float("nan")                     # rows that are no entries are loaded at most
+    seq = nvis = tgt = tl = None
+    own, vis = list(range(N)), counts[:N]
+    if given:
+        seq = torch.randperm(B, generator=g, device=DEV)[:N].to(torch.int32)
+        nvis = torch.randint(0, cap + 1, (N,), generator=g, device=DEV, dtype=torch.int32)
+        tgt = torch.randint(0, V + cap, (N,), generator=g, device=DEV, dtype=torch.int32)
+        tgt[::3] = V + torch.arange(N, device=DEV, dtype=torch.int32)[::3]
+        tl = torch.zeros(N, device=DEV)
+        own = seq.tolist()
+        vis = [min(v, counts[o]) for v, o in zip(nvis.tolist(), own)]
+    lse, mx = torch.zeros(N, device=DEV), torch.zeros(N, device=DEV)
+    am, sm = (torch.full((N,), -9, dtype=torch.int32, device=DEV) for _ in range(2))
+    out = None if select else torch.full((N, V + cap), -7.0, device=DEV)
+    zb.z2z_dynamic_logits(cb, hid, seq, nvis, WU, Uh, select, T, seed, step, tgt, lse, am, mx, sm if select else None, tl, out)
+    st, _ = zb.z2z_status(cb)
+    assert all(int(s) & zb.ST_WAIT_TIMEOUT == 0 for s in st)
+    base = hid.double() @ WU.double().T
+    for r in range(N):
+        l = torch.cat([base[r], Uh[own[r], :vis[r]].double() @ hid[r].double()])
+        tol = 2e-5 * (1 + float(l.abs().max()))              # fp32 sums of d products, as below
+        assert abs(float(lse[r]) - float(torch.logsumexp(l, 0))) < tol
+        assert abs(float(mx[r]) - float(l.max())) < tol and float(l.max() - l[int(am[r])]) < 2 * tol
+        if given and int(tgt[r]) < len(l):
+            assert abs(float(tl[r]) - float(l[int(tgt[r])])) < tol
+        elif given:
+            assert torch.isnan(tl[r])
+        if out is not None:
+            assert float((out[r, :len(l)].double() - l).abs().max()) < tol and torch.all(out[r, len(l):] == -7)
+        if select and r % 8 in (0, 5):
+            # a score is a logit (error below 1e-4 here) plus noise in fp32 (error below 1e-5 at |g| < 20)
+            choice, scores, _ = olg.select(l.cpu().numpy(), 1, T, seed, step, r)
+            assert scores[int(sm[r])] >= scores[choice] - 5e-4
+
+
 @pytest.mark.parametrize("N", [1, 31, 32, 33, 64, 65, 96, 128, 129, 192, 193, 256, 257, 511, 700])
 @pytest.mark.parametrize("V,d", [(4097, 192), (1000, 1152), (130, 2176)])
 def test_joint_logits_against_fp64(V, d, N):
