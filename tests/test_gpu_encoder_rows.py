@@ -415,9 +415,10 @@ def test_short_list_of_ranges(B, bound):
 
 
 @pytest.mark.parametrize("d,dff,total", [(2560, 768, 40), (2560, 768, 80), (384, 512, 200)])
-def test_a_bounded_call_without_an_entry_streams_nothing(d, dff, total):
-    """Calls whose ranges are empty between calls that embed some: on one CTA per tile and on pairs, with weights
-    for more than the load ring (d = 2560), in several row blocks."""
+def test_bounded_calls_without_an_entry_between_calls_that_embed(d, dff, total):
+    """Calls whose ranges are empty leave nothing behind, in the caches or in the scratch of the calls around them: on one
+    CTA per tile and on pairs, with weights for more than the load ring (d = 2560), in several row blocks.  (That they
+    stream no weights is not seen here; only their time shows it.)"""
     w, p = _pair(d, dff, 3, B=2, T=900, cap=600, seed=total)
     i32 = lambda x: torch.tensor(x, dtype=torch.int32, device=p.dev)
     some = [total // 2 - 3, total - total // 2]
