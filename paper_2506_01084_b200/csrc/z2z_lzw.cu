@@ -32,6 +32,35 @@ __global__ void k_codebook_clear(CbView cb, uint4* zero, size_t n_zero) {
 }
 static_assert(kEmptySlot == ~0ull, "an empty slot is all ones");
 
+// All threads of the block: constituent rows of entries [n0, n1), whose first word is the position of their first token:
+// tokens [start, start + len), -1 padded.  (AT_ONCE entries of a thread at a time: their loads do not wait for one another)
+template <int AT_ONCE>
+__device__ __forceinline__ void write_rows(const CbView& cb, int b, const int32_t* __restrict__ x, int n0, int n1) {
+  const int V = cb.V, M = cb.M, cap = cb.cap;
+  for (int e0 = n0 + (int)threadIdx.x; e0 < n1; e0 += AT_ONCE * (int)blockDim.x) {
+    int start[AT_ONCE], L[AT_ONCE], tok[AT_ONCE][kMaxM];
+#pragma unroll
+    for (int u = 0; u < AT_ONCE; ++u) {
+      const int e = e0 + u * (int)blockDim.x;
+      start[u] = L[u] = 0;
+      if (e < n1) { start[u] = cb.cons[((size_t)b * cap + e) * M]; L[u] = cb.len[(size_t)b * cap + e]; }
+    }
+#pragma unroll
+    for (int u = 0; u < AT_ONCE; ++u)
+#pragma unroll
+      for (int j = 0; j < kMaxM; ++j) tok[u][j] = j < L[u] ? x[start[u] + j] : -1;
+#pragma unroll
+    for (int u = 0; u < AT_ONCE; ++u) {
+      const int e = e0 + u * (int)blockDim.x;
+      if (e >= n1) break;
+      int32_t* row = cb.cons + ((size_t)b * cap + e) * M;
+#pragma unroll
+      for (int j = 0; j < kMaxM; ++j)
+        if (j < M) row[j] = j < L[u] && (unsigned)tok[u][j] >= (unsigned)V ? 0 : tok[u][j];
+    }
+  }
+}
+
 // Prompt compression (Section 2.1; Section 2.3 step 2).  One block per sequence; a window of
 // LANES input positions at a time (z2z_lzw_dev.cuh).
 //
@@ -47,8 +76,9 @@ static_assert(kEmptySlot == ~0ull, "an empty slot is all ones");
 // codes and back with both session resets: 9.62 ms before, 0.65 ms with windows here and in the replay, 0.56 with
 // three barriers a window instead of four (four instead of six there), exits in one word and entries written back
 // four at a time.
+// At most 64 registers: narrow windows are for calls of many sequences, seven per SM at 1024.
 template <int LANES, bool SMEM>
-__global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_encode(CbView cb, const int32_t* __restrict__ tokens,
+__global__ void __launch_bounds__(parse_threads(LANES), 1024 / parse_threads(LANES)) k_lzw_encode(CbView cb, const int32_t* __restrict__ tokens,
                                                               const int32_t* __restrict__ lens, int T_max,
                                                               int32_t* __restrict__ codes,
                                                               int32_t* __restrict__ code_lens,
@@ -186,30 +216,8 @@ __global__ void __launch_bounds__(parse_threads(LANES)) k_lzw_encode(CbView cb, 
     if (s_st) atomicOr(&cb.status[b], s_st);
   }
   table.close(n0, s_n1);
-  // constituent rows of the entries created here: tokens [start, start + len), -1 padded; four entries of a
-  // thread at a time, so that their loads do not wait for one another
-  for (int e0 = n0 + tid; e0 < s_n1; e0 += 4 * (int)blockDim.x) {
-    int start[4], L[4], tok[4][kMaxM];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int e = e0 + u * (int)blockDim.x;
-      start[u] = L[u] = 0;
-      if (e < s_n1) { start[u] = cb.cons[((size_t)b * cap + e) * M]; L[u] = cb.len[(size_t)b * cap + e]; }
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int j = 0; j < kMaxM; ++j) tok[u][j] = j < L[u] ? x[start[u] + j] : -1;
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int e = e0 + u * (int)blockDim.x;
-      if (e >= s_n1) break;
-      int32_t* row = cb.cons + ((size_t)b * cap + e) * M;
-#pragma unroll
-      for (int j = 0; j < kMaxM; ++j)
-        if (j < M) row[j] = j < L[u] && (unsigned)tok[u][j] >= (unsigned)V ? 0 : tok[u][j];
-    }
-  }
+  if (write_back_four(n0, s_n1)) write_rows<4>(cb, b, x, n0, s_n1);
+  else write_rows<1>(cb, b, x, n0, s_n1);
 }
 
 // Online update with one new code per sequence (Figure 1; Section 2.3 step 10).

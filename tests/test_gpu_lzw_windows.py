@@ -111,6 +111,26 @@ def test_windows_match_the_oracle(V, M, cap, copies, kind):
     _check_books(cb2, rb, copies)
 
 
+@pytest.mark.parametrize("copies", [1, 40])             # 9 and 360 sequences: blocks of 512 and 128 threads
+@pytest.mark.parametrize("cap", [1600, 16385])          # table in shared and in global memory
+def test_entries_around_one_per_thread(cap, copies):
+    """What a call has made is written back one entry per thread or four at a time."""
+    sizes, V, M = [1, 127, 128, 129, 511, 512, 513, 514, 1500], 5000, 3
+    rows = [np.random.default_rng(b).permutation(V)[:k + 1].astype(np.int32) for b, k in enumerate(sizes)]
+    cb = _session(V, M, cap, len(rows) * copies)
+    books = [olzw.Codebook(V, M, cap) for _ in rows]
+    codes, clen, _ = _encode(cb, rows * copies, max(sizes) + 1)
+    for b, r in enumerate(rows):
+        assert codes[b, :clen[b]].tolist() == books[b].encode(r.tolist())[0] and books[b].n() == sizes[b]
+    _check_books(cb, books, copies)
+    cb2 = _session(V, M, cap, len(rows) * copies)
+    out, olen = torch.zeros(codes.shape, dtype=torch.int32, device=DEV), torch.zeros(len(codes), dtype=torch.int32, device=DEV)
+    zb.z2z_lzw_decode(cb2, torch.from_numpy(codes).to(DEV), torch.from_numpy(clen).to(DEV), zb.DECODE_REPLAY, out, olen)
+    for b, r in enumerate(rows * copies):
+        assert out[b, :olen[b]].tolist() == r.tolist()
+    _check_books(cb2, books, copies)
+
+
 @pytest.mark.parametrize("B", [3, 400])
 @pytest.mark.parametrize("T", [1, 20, 63, 64, 65])
 def test_short_calls_use_the_table_in_place(T, B):
