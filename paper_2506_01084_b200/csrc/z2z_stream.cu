@@ -4,8 +4,8 @@
 //                                          W: weight rows streamed once from HBM (bf16, K-major)
 //
 // One persistent CTA per SM.  Warp 0 issues TMA loads into a ring of shared-memory stages, warp 1
-// issues tcgen05.mma (fp32 accumulators in tensor memory, double buffered), warps 2-5 drain
-// accumulators.  Two kernels share the ring and its barriers:
+// issues tcgen05.mma (fp32 accumulators in tensor memory, double buffered), warps 2-5 (logits: 2-13)
+// drain accumulators.  Two kernels share the ring and its barriers:
 //   * hyper-encoder linear layers (k_stream_gemm): a tile of 128 weight rows is the MMA's M
 //     operand, the packed activation rows (hi and lo part of a row in adjacent operand rows) its
 //     N operand, as wide as the rows that exist; work is cut stream-K style, every CTA gets the
@@ -40,7 +40,7 @@ constexpr int kLogitEpiWarps = 12;
 constexpr int kLogitEpiGroups = kLogitEpiWarps / 4;
 constexpr int kLogitThreads = 64 + 32 * kLogitEpiWarps;
 
-struct Ctrl {
+struct Ctrl {                            // at most 512 bytes of shared memory
   unsigned long long full[kMaxStages], empty[kMaxStages], acc_full[2], acc_empty[2], pref_ready;
   uint32_t tmem_base;
   int abort;
@@ -69,13 +69,16 @@ struct Job {
 // rows 54 -> 61; a sampled step of 54 sequences at V = 6020 440 -> 412).  A job is a run of up to kLogitNT / kLogitGran
 // granules inside one segment (W_U, or one sequence).
 constexpr int kLogitEvenGrans = 3;
+constexpr int kNoGroup = 254, kManyGroups = 255;       // a sequence without a row; one with rows in several groups of 8
 struct LogitSched {
   const StreamLogitsParams& p;
   const int* pref;       // shared: prefix of per-sequence granule counts, [B + 1]
+  const uint8_t* groups; // shared, with row_seq: the group of 8 hidden rows that holds all rows of a sequence, [B]
   int u, u1;
   bool hyper;
   // (pref has to be there unless the shares are even)
-  __device__ LogitSched(const StreamLogitsParams& pp, const int* s_pref) : p(pp), pref(s_pref), hyper(false) {
+  __device__ LogitSched(const StreamLogitsParams& pp, const int* s_pref) : p(pp), pref(s_pref), groups(nullptr), hyper(false) {
+    if (p.la.row_seq) groups = reinterpret_cast<const uint8_t*>(pref + p.cb.B + 1);
     const int ns = n_static(p);
     if (even(p)) { share(ns); return; }
     share(ns + pref[p.cb.B]);
@@ -116,18 +119,21 @@ struct LogitSched {
     j.nrows = ng * kLogitGran;
     j.nvalid = total_rows - g0 * kLogitGran < j.nrows ? total_rows - g0 * kLogitGran : j.nrows;
     u += ng;
-    // A sequence's hypertokens meet the hidden row of that sequence only.  Where row r is known to be sequence r's, just
-    // the group of 8 rows around it is loaded, to where all rows would put it (the other rows of the operand are what
+    // A sequence's hypertokens meet the hidden rows of that sequence only.  Where those lie in one group of 8 rows, just
+    // that group is loaded, to where all rows would put it (the other rows of the operand are what
     // is left there, and nobody reads their accumulators), and a job of few rows takes several k-blocks per stage: with
     // one, a job of 64 rows had 8 KB a stage in flight, and took as long as one of 256 (V = 128256, d = 4096, 90
     // sequences of 59 hypertokens 301 us, of 256 hypertokens 218).
     j.kb = 1; j.group = -1;
-    if (j.owner >= 0 && !p.la.row_seq) {
-      j.group = j.owner < p.la.N ? j.owner >> 3 : 0;
+    const int group = j.owner < 0 ? kManyGroups : groups ? groups[j.owner] : j.owner < p.la.N ? j.owner >> 3 : kNoGroup;
+    if (group != kManyGroups) {
+      j.group = group == kNoGroup ? 0 : group;
       if (ng <= 4) {                               // up to 128 rows: one box, of 1, 2 or 4 granules
         if (ng == 3) j.nrows = 4 * kLogitGran;
         j.kb = logit_short_kb(ng > 2 ? 2 : ng - 1);
       }
+    } else if (j.owner >= 0 && ng <= 2) {
+      j.kb = 2;         // all hidden rows, two k-blocks of them (V = 32064, d = 3072, 33 rows of 11 sequences, 250 hypertokens: 79 -> 57 us)
     }
     return true;
   }
@@ -142,14 +148,24 @@ struct LogitSched {
 // Weight rows of a stage: behind the hidden rows, and behind the further k-blocks of the last group of 8.  (The MMA reads
 // 128 hidden rows from a k-block's start; those that are not there lie in the weight rows.)
 __host__ __device__ constexpr uint32_t logit_w_offset(int a_box_rows) { return (uint32_t)a_box_rows * 128u + 3u * 1024u; }
+// Where a job's hidden rows and weight rows of k-block i lie in a stage.  (Two k-blocks of all hidden rows push the weight rows
+// back; 64 of them at most then end where 256 would.)
+struct LogitStage {
+  uint32_t w_off, a_step;
+  __device__ LogitStage(const StreamLogitsParams& p, const Job& j) : w_off(logit_w_offset(p.a_box_rows)), a_step(1024u) {
+    if (j.group < 0) a_step = (uint32_t)p.a_box_rows * 128u;
+    if (j.group < 0 && j.kb > 1) w_off = (uint32_t)j.kb * a_step;
+  }
+};
+static_assert(2 * 128 * 128 + 2 * 64 * 128 <= 128 * 128 + 3 * 1024 + kLogitNT * 128, "two k-blocks of 128 hidden and 64 weight rows fit a stage");
 
 // ---- producer and MMA role of the logits kernel -----------------------------------------------------
 // Everything that is loaded, W_U among it, may come from the kernel ahead: nothing is issued before the dependency wait.
 template <int STAGES>
 __device__ __forceinline__ void logits_producer(const StreamLogitsParams& p, const int* s_pref, Ctrl* ctrl, uint32_t stage_base,
                                                 const LogitMaps& tm) {
-  const uint32_t a_bytes = (uint32_t)p.a_box_rows * 128, w_off = logit_w_offset(p.a_box_rows);
-  const uint32_t stage_bytes = w_off + kLogitNT * 128;             // smem stride of a stage
+  const uint32_t a_bytes = (uint32_t)p.a_box_rows * 128;
+  const uint32_t stage_bytes = logit_w_offset(p.a_box_rows) + kLogitNT * 128;      // smem stride of a stage
   const uint64_t pol_w = policy_evict_first(), pol_a = policy_evict_last();
   int stage = 0; uint32_t phase = 0;
   pdl_wait();
@@ -162,6 +178,7 @@ __device__ __forceinline__ void logits_producer(const StreamLogitsParams& p, con
       sched.begin_hyper();
     }
     while (sched.next(j)) {
+      const uint32_t w_off = LogitStage(p, j).w_off;
       for (int ks = 0; ks < p.ksteps; ks += j.kb) {
         if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) return;
         const uint32_t full = smem_u32(&ctrl->full[stage]);
@@ -169,13 +186,15 @@ __device__ __forceinline__ void logits_producer(const StreamLogitsParams& p, con
         // (k-blocks beyond the last one, and rows outside the tensors, are zero-filled and counted)
         const uint32_t w_bytes = (uint32_t)(j.kb * j.nrows) * 128u;
         if (j.group < 0) {
-          mbar_expect_tx(full, a_bytes + w_bytes);
-          tma_load_3d(sb, &tm.h, 0, 0, ks, full, pol_a);
+          mbar_expect_tx(full, (uint32_t)j.kb * a_bytes + w_bytes);
+          tma_load_3d(sb, j.kb > 1 ? &tm.h2 : &tm.h, 0, 0, ks, full, pol_a);
         } else {
           mbar_expect_tx(full, (uint32_t)j.kb * 1024u + w_bytes);
           tma_load_3d(sb + (uint32_t)j.group * 1024u, &tm.h8[j.kb >> 1], 0, 8 * j.group, ks, full, pol_a);
         }
-        if (j.kb > 1) {
+        if (j.kb > 1 && j.group < 0) {
+          tma_load_3d(sb + w_off, &tm.u2[j.nrows == kLogitGran ? 0 : 1], 0, j.wrow, ks, full, pol_w);
+        } else if (j.kb > 1) {
           tma_load_3d(sb + w_off, &tm.u[j.nrows == kLogitGran ? 0 : j.nrows == 2 * kLogitGran ? 1 : 2], 0, j.wrow, ks, full, pol_w);
         } else {
           // the W rows of the job go out as few boxes as possible: largest power-of-two box first
@@ -195,8 +214,7 @@ __device__ __forceinline__ void logits_producer(const StreamLogitsParams& p, con
 template <int STAGES>
 __device__ __forceinline__ void logits_mma(const StreamLogitsParams& p, const int* s_pref, Ctrl* ctrl, uint32_t stage_base,
                                            uint32_t tmem_base) {
-  const uint32_t w_off = logit_w_offset(p.a_box_rows);
-  const uint32_t stage_bytes = w_off + kLogitNT * 128;
+  const uint32_t stage_bytes = logit_w_offset(p.a_box_rows) + kLogitNT * 128;
   int stage = 0; uint32_t phase = 0;
   uint32_t job_i = 0;
   LogitSched sched(p, s_pref);
@@ -207,6 +225,7 @@ __device__ __forceinline__ void logits_mma(const StreamLogitsParams& p, const in
     if (!mbar_wait_warp(smem_u32(&ctrl->acc_empty[buf]), aph ^ 1u, &ctrl->abort)) return;
     tc_fence_after();
     const uint32_t d = tmem_base + buf * kLogitNT;
+    const LogitStage at(p, j);
     uint32_t acc = 0;
     for (int ks = 0; ks < p.ksteps; ks += j.kb) {
       if (!mbar_wait_warp(smem_u32(&ctrl->full[stage]), phase, &ctrl->abort)) return;
@@ -214,7 +233,7 @@ __device__ __forceinline__ void logits_mma(const StreamLogitsParams& p, const in
       const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
       if (elect_one()) {
         for (int i = 0; i < j.kb; ++i) {
-          const uint32_t ab = sb + (uint32_t)i * 1024u, wb = sb + w_off + (uint32_t)(i * j.nrows) * 128u;
+          const uint32_t ab = sb + (uint32_t)i * at.a_step, wb = sb + at.w_off + (uint32_t)(i * j.nrows) * 128u;
 #pragma unroll
           for (int k = 0; k < 4; ++k)
             umma_bf16(d, smem_desc_sw128(ab + k * 32), smem_desc_sw128(wb + k * 32), idesc, i || k ? 1u : acc);
@@ -242,7 +261,7 @@ __device__ __forceinline__ void setup_barriers(Ctrl* ctrl) {
       mbar_init(smem_u32(&ctrl->acc_full[b]), 1);
       mbar_init(smem_u32(&ctrl->acc_empty[b]), EPI_WARPS);
     }
-    mbar_init(smem_u32(&ctrl->pref_ready), 1);         // logits: the sequences' granules are counted
+    mbar_init(smem_u32(&ctrl->pref_ready), 2);         // logits: the sequences' granules are counted, their rows found
     ctrl->abort = 0;
     mbar_init_fence();
   }
@@ -454,6 +473,7 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
 // =================================================================================================
 // Logits kernel: fused reductions
 // =================================================================================================
+static_assert(sizeof(Ctrl) <= 512, "the sequences' tables lie behind it");
 template <int STAGES>
 __global__ void __launch_bounds__(kLogitThreads, 1)
 k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm) {
@@ -461,13 +481,13 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
   extern __shared__ unsigned char smem_raw[];
   unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   Ctrl* ctrl = reinterpret_cast<Ctrl*>(sm);
-  int* s_pref = reinterpret_cast<int*>(sm + 1024);              // [B + 1] <= 4100 bytes
+  int* s_pref = reinterpret_cast<int*>(sm + 512);               // [B + 1], then the groups of the sequences: <= 5124 bytes
   const uint32_t stage_base = smem_u32(sm + 1024 + 5120);
   const int warp = uniform_warp(), lane = threadIdx.x & 31;
   setup_barriers<STAGES, kLogitEpiWarps>(ctrl);
   if (warp == 3) {
     if (lane < 1 + 2 * kLogitBoxClasses) prefetch_tmap(lane == 0 ? &tm.h : &tm.w[lane - 1]);
-    if (lane < 3) { prefetch_tmap(&tm.h8[lane]); prefetch_tmap(&tm.u[lane]); }
+    if (lane < 3) { prefetch_tmap(&tm.h8[lane]); prefetch_tmap(&tm.u[lane]); prefetch_tmap(lane < 2 ? &tm.u2[lane] : &tm.h2); }
   }
   __syncthreads();                                 // barriers exist, which is all that the producer needs
 
@@ -488,6 +508,29 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
         carry += __shfl_sync(0xffffffffu, v, 31);
       }
       if (lane == 0) s_pref[0] = 0;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&ctrl->pref_ready));
+    }
+    if (warp == 3) {                               // the group of each sequence's rows, where they are given
+      if (p.la.row_seq) {
+        uint8_t* s_group = reinterpret_cast<uint8_t*>(s_pref + p.cb.B + 1);
+        for (int b = lane; b < p.cb.B; b += 32) s_group[b] = kNoGroup;
+        int seq[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          seq[i] = 32 * i + lane < p.la.N ? p.la.row_seq[32 * i + lane] : -1;
+          if (seq[i] >= p.cb.B) seq[i] = -1;
+        }
+#pragma unroll
+        for (int g = 0; g < 16; ++g) {             // (rows of one sequence in one group write the same)
+          __syncwarp();
+          const int b = __shfl_sync(0xffffffffu, seq[g / 4], 8 * (g % 4) + (lane & 7));
+          if (b >= 0) {
+            const int was = s_group[b];
+            s_group[b] = (uint8_t)(was == kNoGroup || was == g ? g : kManyGroups);
+          }
+        }
+      }
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&ctrl->pref_ready));
     }
@@ -770,8 +813,12 @@ cudaError_t run_logits_stream(const CbView& cb, const LogitsArgs& a, int* err_wo
   p.err = err_word;
   LogitMaps maps;
   if (!make_tmap_bf16_kblocks(&maps.h, a.hidden, a.N, a.d, p.a_box_rows, 1)) return cudaErrorInvalidValue;
+  const bool hyper = cb.cap > 0;                       // (otherwise no job uses the maps)
+  if (!make_tmap_bf16_kblocks(&maps.h2, a.hidden, a.N, a.d, p.a_box_rows, 2)) return cudaErrorInvalidValue;
+  for (int c = 0; c < 2; ++c)
+    if (!make_tmap_bf16_kblocks(&maps.u2[c], hyper ? a.Uh : a.WU, hyper ? (long long)cb.B * cb.cap : cb.V, a.d, kLogitGran << c, 2))
+      return cudaErrorInvalidValue;
   for (int c = 0; c < 3; ++c) {
-    const bool hyper = cb.cap > 0;                     // (otherwise no job uses the maps)
     if (!make_tmap_bf16_kblocks(&maps.h8[c], a.hidden, a.N, a.d, 8, 1 << c)) return cudaErrorInvalidValue;
     if (!make_tmap_bf16_kblocks(&maps.u[c], hyper ? a.Uh : a.WU, hyper ? (long long)cb.B * cb.cap : cb.V, a.d, kLogitGran << c,
                                 logit_short_kb(c)))

@@ -25,6 +25,7 @@ struct LogitMaps {
   CUtensorMap w[2 * kLogitBoxClasses];
   CUtensorMap h8[3];     // 1, 2 and 4 k-blocks
   CUtensorMap u[kLogitShortClasses];
+  CUtensorMap h2, u2[2]; // two k-blocks of all hidden rows, and of 32 or 64 rows of U_h: for sequences with rows in several groups
 };
 
 // ---- decode logits kernel (z2z_decode_logits.cu) ---------------------------------------------

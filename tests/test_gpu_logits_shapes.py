@@ -92,17 +92,18 @@ def test_batch_with_hypertokens_of_every_job_size(V, d, B):
 
 
 @pytest.mark.parametrize("select", [0, 1])
-@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("given", ["no", "one", "several"])
 @pytest.mark.parametrize("N", [33, 70, 128])
-@pytest.mark.parametrize("granules,d", [(3, 448), (8.5, 448), (19.3, 320)])
+@pytest.mark.parametrize("granules,d", [(0.5, 448), (3, 448), (8.5, 448), (19.3, 320)])
 def test_batch_with_several_column_jobs_per_cta(granules, d, N, given, select):
     """Even shares of W_U: three granules of 32 columns per CTA (the fewest that are dealt so), one job of 256 columns
     and a rest, two of them and a rest; more k-blocks than the ring has stages (five up to 40 rows, four at
-    128); behind them the hypertokens.  Rows in the order of their sequences, or given with them, their limits and targets."""
+    128); behind them the hypertokens.  Below three granules one share of both.  Rows in the order of their sequences, or given
+    with them, their limits and targets: one per sequence, or several, in one group of 8 rows, in several, or of none."""
     from oracle import logits as olg
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     V = 32 * int(granules * sms) - (5 if granules > 3 else 0)
-    assert (V + 31) // 32 >= 3 * sms
+    assert ((V + 31) // 32 >= 3 * sms) == (granules >= 3)
     sizes = [0, 1, 33, 64, 100, 129, 256, 300]
     B, cap, T, seed, step = N + 2, 300, 0.9, 77, 5
     counts = [sizes[(3 * b) % len(sizes)] for b in range(B)]
@@ -115,14 +116,18 @@ def test_batch_with_several_column_jobs_per_cta(granules, d, N, given, select):
         Uh[b, counts[b]:] = float("nan")                     # rows that are no entries are loaded at most
     seq = nvis = tgt = tl = None
     own, vis = list(range(N)), counts[:N]
-    if given:
+    if given != "no":
         seq = torch.randperm(B, generator=g, device=DEV)[:N].to(torch.int32)
+        if given == "several":
+            seq = torch.arange(N, device=DEV, dtype=torch.int32) // 3
+            seq[::7] = seq[::7].flip(0)
+            seq[5], seq[6] = -1, B
         nvis = torch.randint(0, cap + 1, (N,), generator=g, device=DEV, dtype=torch.int32)
         tgt = torch.randint(0, V + cap, (N,), generator=g, device=DEV, dtype=torch.int32)
         tgt[::3] = V + torch.arange(N, device=DEV, dtype=torch.int32)[::3]
         tl = torch.zeros(N, device=DEV)
         own = seq.tolist()
-        vis = [min(v, counts[o]) for v, o in zip(nvis.tolist(), own)]
+        vis = [min(v, counts[o]) if 0 <= o < B else 0 for v, o in zip(nvis.tolist(), own)]
     lse, mx = torch.zeros(N, device=DEV), torch.zeros(N, device=DEV)
     am, sm = (torch.full((N,), -9, dtype=torch.int32, device=DEV) for _ in range(2))
     out = None if select else torch.full((N, V + cap), -7.0, device=DEV)
@@ -131,13 +136,15 @@ def test_batch_with_several_column_jobs_per_cta(granules, d, N, given, select):
     assert all(int(s) & zb.ST_WAIT_TIMEOUT == 0 for s in st)
     base = hid.double() @ WU.double().T
     for r in range(N):
+        if not 0 <= own[r] < B:
+            continue                                         # a row without an owner sees nothing
         l = torch.cat([base[r], Uh[own[r], :vis[r]].double() @ hid[r].double()])
         tol = 2e-5 * (1 + float(l.abs().max()))              # fp32 sums of d products, as below
         assert abs(float(lse[r]) - float(torch.logsumexp(l, 0))) < tol
         assert abs(float(mx[r]) - float(l.max())) < tol and float(l.max() - l[int(am[r])]) < 2 * tol
-        if given and int(tgt[r]) < len(l):
+        if tgt is not None and int(tgt[r]) < len(l):
             assert abs(float(tl[r]) - float(l[int(tgt[r])])) < tol
-        elif given:
+        elif tgt is not None:
             assert torch.isnan(tl[r])
         if out is not None:
             assert float((out[r, :len(l)].double() - l).abs().max()) < tol and torch.all(out[r, len(l):] == -7)
