@@ -12,10 +12,10 @@ namespace z2z {
 // while the previous kernel of the stream is still running.  Every kernel launched this way
 // calls pdl_wait() before it reads what earlier kernels wrote and before it writes anything.
 // Weights are the exception: the GEMMs of an encoder pass load them ahead of the wait, and the decode logits kernel W_U.
-// Therefore a kernel that begins or ends a call, or stands alone, waits BEFORE it triggers: what is launched behind it then
-// starts behind everything ahead of it, as behind an ordinary launch.  (Triggering first let a chain of small kernels and
-// the GEMM at its end start beside a kernel ahead of the call that was still writing the weights.)  The kernels inside
-// a pass trigger first, and so does the decode logits kernel, whose callers are told.
+// Therefore every call has a kernel that waits BEFORE it triggers, ahead of any that loads so in this call or the next: what
+// is launched behind it starts behind everything ahead of it, as behind an ordinary launch.  (Where all triggered first, a
+// chain of small kernels and the GEMM at its end started beside a kernel ahead of the call that was still writing the
+// weights.)  Only a decode step whose logits the decode kernel takes has none; its callers are told.
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                               Args&&... args) {

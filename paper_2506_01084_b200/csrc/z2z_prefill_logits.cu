@@ -131,8 +131,8 @@ struct UnitWalk {
 // ---- plan: sequence range and cost of the hypertoken tiles of every row tile; target logits start as NaN -----------------------------------
 __global__ void __launch_bounds__(256) k_prefill_plan(PrefillLogitsParams p) {
   __shared__ int s_lo, s_hi, s_nh;
-  pdl_wait();
   pdl_trigger();
+  pdl_wait();
   const int rt = blockIdx.x;
   if (threadIdx.x == 0) { s_lo = 0x7fffffff; s_hi = -1; s_nh = 0; }
   __syncthreads();
@@ -361,8 +361,8 @@ k_prefill_logits(const PrefillLogitsParams p, const __grid_constant__ PrefillMap
 
 // Eight lanes per row: merge the partial reductions of the strips, write the outputs.
 __global__ void __launch_bounds__(256) k_prefill_merge(PrefillLogitsParams p) {
-  pdl_trigger();
   pdl_wait();
+  pdl_trigger();
   const LogitsArgs& a = p.la;
   const int r = blockIdx.x * (blockDim.x / 8) + (threadIdx.x >> 3), lane = threadIdx.x & 7;
   RowRed red; red.init();
