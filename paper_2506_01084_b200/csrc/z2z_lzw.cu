@@ -71,11 +71,9 @@ __device__ __forceinline__ void write_rows(const CbView& cb, int b, const int32_
 // only the first kMaxM lanes of a warp can be entered: a warp's exits fit one word, four bits each).
 //
 // Bound by the latency of one window (a few dependent shared-memory lookups, ten shuffles, three
-// barriers).  The chain used to be walked token by token by one thread: 180 ns per token with the
-// table in shared memory, 220 with it in global memory.  Four texts of 32768 tokens (cap 16384), to
-// codes and back with both session resets: 9.62 ms before, 0.65 ms with windows here and in the replay, 0.56 with
-// three barriers a window instead of four (four instead of six there), exits in one word and entries written back
-// four at a time.
+// barriers).  One thread that walks the chain token by token takes 180 ns per token with the table in
+// shared memory, 220 with it in global memory: four texts of 32768 tokens (cap 16384), to codes and back
+// with both session resets, 9.6 ms; in windows, here and in the replay, 0.55.
 // At most 64 registers: narrow windows are for calls of many sequences, seven per SM at 1024.
 template <int LANES, bool SMEM>
 __global__ void __launch_bounds__(parse_threads(LANES), 1024 / parse_threads(LANES)) k_lzw_encode(CbView cb, const int32_t* __restrict__ tokens,

@@ -33,9 +33,8 @@ namespace {
 
 constexpr int kThreads = 192;
 // The logits kernel drains with twelve warps, three per tensor-memory lane quarter that take every third 32 columns: a
-// sampled column costs its row some 30 instructions, and four warps, of which a batch of 43 rows keeps two busy, took
-// longer than the weights (sampled with 4 / 8 / 12 warps, argmax: V = 96132, d = 3200, 43 rows 207 / 140 / 142, 104 us;
-// V = 128256, d = 4096, 128 rows 276 / 214 / 199, 180).
+// sampled column costs its row some 30 instructions, and four warps, of which a batch of 43 rows keeps two busy, take
+// longer than the weights (V = 128256, d = 4096, 128 rows: sampled with 4 / 8 / 12 warps 276 / 214 / 199 us, argmax 180).
 constexpr int kLogitEpiWarps = 12;
 constexpr int kLogitEpiGroups = kLogitEpiWarps / 4;
 constexpr int kLogitThreads = 64 + 32 * kLogitEpiWarps;
@@ -60,14 +59,13 @@ struct Job {
 };
 
 // ---- logits schedule ----------------------------------------------------------------------------
-// Columns are dealt in granules of kLogitGran rows: every CTA takes an even share of the granules of W_U, which it
-// knows without any codebook state, and then one of those of the visible rows of each sequence's U_h.  (One share of
-// both in a row gave some CTAs nothing but hypertokens, whose jobs are short and cost more per granule: V = 128256,
-// d = 4096, 90 sequences of 29 hypertokens 385 us.)  With fewer than kLogitEvenGrans granules of W_U per CTA it is
-// their jobs that would get short, with all hidden rows each: there it is one share of both in a row after all (d =
-// 3072, 149 hypertokens each, even shares -> one: V = 6020, 54 rows 38 -> 33 us, V = 12000 43 -> 37; V = 17000, 128
-// rows 54 -> 61; a sampled step of 54 sequences at V = 6020 440 -> 412).  A job is a run of up to kLogitNT / kLogitGran
-// granules inside one segment (W_U, or one sequence).
+// Columns are dealt in granules of kLogitGran rows: every CTA takes an even share of the granules of W_U, and then one
+// of those of the visible rows of each sequence's U_h.  (One share of both in a row gives some CTAs nothing but
+// hypertokens, whose jobs are short and cost more per granule: V = 128256, d = 4096, 90 sequences of 29 hypertokens
+// 385 us, even shares 190.)  With fewer than kLogitEvenGrans granules of W_U per CTA it is their jobs that would get
+// short, with all hidden rows each: there it is one share of both in a row (d = 3072, 149 hypertokens each, even shares
+// and one: V = 6020, 54 rows 38 and 33 us, V = 12000 43 and 37; V = 17000, 128 rows 54 and 61).  A job is a run of up to
+// kLogitNT / kLogitGran granules inside one segment (W_U, or one sequence).
 constexpr int kLogitEvenGrans = 3;
 constexpr int kNoGroup = 254, kManyGroups = 255;       // a sequence without a row; one with rows in several groups of 8
 struct LogitSched {
@@ -333,14 +331,11 @@ k_stream_gemm(const StreamGemmParams p, const __grid_constant__ StreamGemmMaps t
       // count do: during the first pass over the ring only the weight boxes are issued and the
       // activation boxes are noted; once the ring is full (or the work ends) the producer waits for the
       // preceding kernel, picks the box that covers the live rows and issues them.  (A box of the pass's
-      // capacity brought 1.5 bytes of activations per byte of weights at 96 rows of which 55 were live,
-      // and what an SM takes in from L2 bounds a batch of this size, not HBM: 546 -> 511 us per step of
-      // 32 sequences at d = 4096, 251 -> 244 of 8 at d = 3072.)  With an ordinary launch the wait
-      // returns at once.  A pass without a live row (a step that created no entry) streams nothing: the
-      // producer takes in what it loaded ahead, and the other roles have no work.  Such a step of one or 8
-      // sequences at d = 3072 went from 224 / 232 to 94 / 90 us (109 / 111 when every GEMM of it still filled
-      // its ring; 76 / 82 since), of 32 at d = 4096 from 563 to 295 (232 since); steps that create entries took
-      // what they had taken (245, 261, 580).
+      // capacity would bring 1.5 bytes of activations per byte of weights at 96 rows of which 55 are live,
+      // and what an SM takes in from L2 bounds a batch of this size, not HBM: 546 instead of 511 us per step of
+      // 32 sequences at d = 4096.)  With an ordinary launch the wait returns at once.  A pass without a live row (a
+      // step that created no entry, an empty range) streams nothing: the producer takes in what it loaded ahead,
+      // and the other roles have no work (one sequence, d = 3072: 77 us such a step, 227 with the weights).
       const uint64_t pol_w = policy_evict_first(), pol_a = policy_evict_last();
       struct Deferred { int g, kb; };
       Deferred def[kMaxStages];                       // load i of the first pass uses stage i

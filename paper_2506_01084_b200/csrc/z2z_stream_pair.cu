@@ -20,8 +20,8 @@
 //     in one column would let 512 rows ride on one stream - 384 rows of both encoders, d = 3072: 687
 //     instead of 787 us a step, 640 rows 1392 against 1173 - but the error against fp64, in units of the
 //     rows' rms, is then 2.5e-5 instead of 1.35e-5 at d = 4096 and 2.1e-5 instead of 1.1e-5 at d = 3072.)
-// A decode step of 90 sequences (d = 3072, one encoder, 270 rows of capacity, about 150 live) went from
-// 486 to 291 us against one CTA per weight tile and 128 rows.
+// A decode step of 90 sequences (d = 3072, one encoder, 270 rows of capacity, about 150 live) takes 1.7 times as
+// long with one CTA per weight tile and 128 rows.
 //
 // Work is cut stream-K style: cluster c of C owns units [floor(c U / C), floor((c + 1) U / C)) of the
 // (group, weight tile, row block, k-step) space and adds its accumulators into the fp32 result with
@@ -172,7 +172,7 @@ k_stream_pair(const StreamPairParams p, const __grid_constant__ StreamPairMaps t
         deps = true;
         if (live < 1) {
           // a pass without a row: the leader takes in what both CTAs loaded ahead, and the peer stays until then
-          // (the cluster leaves together).  Such a step of 90 sequences, d = 3072, one encoder: 270 -> 145 us.
+          // (the cluster leaves together).  Such a step of 90 sequences, d = 3072, one encoder: 122 us, 264 with the weights.
           ok = false;
           if (rank == 0) {
             for (int i = 0; i < n_def; ++i) mbar_arrive(smem_u32(&ctrl->full[i]));
