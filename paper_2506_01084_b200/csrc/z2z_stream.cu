@@ -170,41 +170,45 @@ __device__ __forceinline__ void logits_producer(const StreamLogitsParams& p, con
   if (!LogitSched::even(p) && !mbar_wait(smem_u32(&ctrl->pref_ready), 0, &ctrl->abort)) return;
   LogitSched sched(p, s_pref);
   Job j;
-  for (int part = 0; part < 2; ++part) {
-    if (part == 1) {
-      if (!mbar_wait(smem_u32(&ctrl->pref_ready), 0, &ctrl->abort)) return;
-      sched.begin_hyper();
+  auto w_boxes = [&](uint32_t dst, int ks, uint32_t full) {
+    // the rows of the job go out as few boxes as possible: largest power-of-two box first
+    for (int r0 = 0; r0 < j.nrows;) {
+      int cls = kLogitBoxClasses - 1;
+      while (cls > 0 && (kLogitGran << cls) > j.nrows - r0) --cls;
+      tma_load_3d(dst + r0 * 128, &tm.w[j.wmap * kLogitBoxClasses + cls], 0, j.wrow + r0, ks, full, pol_w);
+      r0 += kLogitGran << cls;
     }
-    while (sched.next(j)) {
-      const uint32_t w_off = LogitStage(p, j).w_off;
-      for (int ks = 0; ks < p.ksteps; ks += j.kb) {
-        if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) return;
-        const uint32_t full = smem_u32(&ctrl->full[stage]);
-        const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
-        // (k-blocks beyond the last one, and rows outside the tensors, are zero-filled and counted)
-        const uint32_t w_bytes = (uint32_t)(j.kb * j.nrows) * 128u;
-        if (j.group < 0) {
-          mbar_expect_tx(full, (uint32_t)j.kb * a_bytes + w_bytes);
-          tma_load_3d(sb, j.kb > 1 ? &tm.h2 : &tm.h, 0, 0, ks, full, pol_a);
-        } else {
-          mbar_expect_tx(full, (uint32_t)j.kb * 1024u + w_bytes);
-          tma_load_3d(sb + (uint32_t)j.group * 1024u, &tm.h8[j.kb >> 1], 0, 8 * j.group, ks, full, pol_a);
-        }
-        if (j.kb > 1 && j.group < 0) {
-          tma_load_3d(sb + w_off, &tm.u2[j.nrows == kLogitGran ? 0 : 1], 0, j.wrow, ks, full, pol_w);
-        } else if (j.kb > 1) {
-          tma_load_3d(sb + w_off, &tm.u[j.nrows == kLogitGran ? 0 : j.nrows == 2 * kLogitGran ? 1 : 2], 0, j.wrow, ks, full, pol_w);
-        } else {
-          // the W rows of the job go out as few boxes as possible: largest power-of-two box first
-          for (int r0 = 0; r0 < j.nrows;) {
-            int cls = kLogitBoxClasses - 1;
-            while (cls > 0 && (kLogitGran << cls) > j.nrows - r0) --cls;
-            tma_load_3d(sb + w_off + r0 * 128, &tm.w[j.wmap * kLogitBoxClasses + cls], 0, j.wrow + r0, ks, full, pol_w);
-            r0 += kLogitGran << cls;
-          }
-        }
-        if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-      }
+  };
+  // W_U in a loop of its own: one loop for both kinds of jobs cost it 4 us of 168 (V = 128256, d = 4096, 33 rows)
+  while (sched.next(j)) {
+    const uint32_t w_off = logit_w_offset(p.a_box_rows), bytes = a_bytes + (uint32_t)j.nrows * 128u;
+    for (int ks = 0; ks < p.ksteps; ++ks) {
+      if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) return;
+      const uint32_t full = smem_u32(&ctrl->full[stage]);
+      const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
+      mbar_expect_tx(full, bytes);
+      tma_load_3d(sb, &tm.h, 0, 0, ks, full, pol_a);
+      w_boxes(sb + w_off, ks, full);
+      if (++stage == STAGES) { stage = 0; phase ^= 1u; }
+    }
+  }
+  if (!mbar_wait(smem_u32(&ctrl->pref_ready), 0, &ctrl->abort)) return;
+  sched.begin_hyper();
+  while (sched.next(j)) {                              // the sequences' hypertokens
+    const uint32_t w_off = LogitStage(p, j).w_off;
+    // (k-blocks beyond the last one, and rows outside the tensors, are zero-filled and counted)
+    const uint32_t bytes = (uint32_t)j.kb * ((uint32_t)j.nrows * 128u + (j.group < 0 ? a_bytes : 1024u));
+    for (int ks = 0; ks < p.ksteps; ks += j.kb) {
+      if (!mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, &ctrl->abort)) return;
+      const uint32_t full = smem_u32(&ctrl->full[stage]);
+      const uint32_t sb = stage_base + (uint32_t)stage * stage_bytes;
+      mbar_expect_tx(full, bytes);
+      if (j.group < 0) tma_load_3d(sb, j.kb > 1 ? &tm.h2 : &tm.h, 0, 0, ks, full, pol_a);
+      else tma_load_3d(sb + (uint32_t)j.group * 1024u, &tm.h8[j.kb >> 1], 0, 8 * j.group, ks, full, pol_a);
+      if (j.kb == 1) w_boxes(sb + w_off, ks, full);
+      else if (j.group < 0) tma_load_3d(sb + w_off, &tm.u2[j.nrows == kLogitGran ? 0 : 1], 0, j.wrow, ks, full, pol_w);
+      else tma_load_3d(sb + w_off, &tm.u[j.nrows == kLogitGran ? 0 : j.nrows == 2 * kLogitGran ? 1 : 2], 0, j.wrow, ks, full, pol_w);
+      if (++stage == STAGES) { stage = 0; phase ^= 1u; }
     }
   }
 }
@@ -511,20 +515,24 @@ k_stream_logits(const StreamLogitsParams p, const __grid_constant__ LogitMaps tm
         uint8_t* s_group = reinterpret_cast<uint8_t*>(s_pref + p.cb.B + 1);
         for (int b = lane; b < p.cb.B; b += 32) s_group[b] = kNoGroup;
         int seq[4];
+        bool other[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           seq[i] = 32 * i + lane < p.la.N ? p.la.row_seq[32 * i + lane] : -1;
           if (seq[i] >= p.cb.B) seq[i] = -1;
         }
+        __syncwarp();
 #pragma unroll
-        for (int g = 0; g < 16; ++g) {             // (rows of one sequence in one group write the same)
-          __syncwarp();
-          const int b = __shfl_sync(0xffffffffu, seq[g / 4], 8 * (g % 4) + (lane & 7));
-          if (b >= 0) {
-            const int was = s_group[b];
-            s_group[b] = (uint8_t)(was == kNoGroup || was == g ? g : kManyGroups);
-          }
-        }
+        for (int i = 0; i < 4; ++i)                // one of a sequence's rows has the say,
+          if (seq[i] >= 0) s_group[seq[i]] = (uint8_t)(4 * i + (lane >> 3));
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i)                // and any in another group objects
+          other[i] = seq[i] >= 0 && s_group[seq[i]] != 4 * i + (lane >> 3);
+        __syncwarp();
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          if (other[i]) s_group[seq[i]] = kManyGroups;
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(smem_u32(&ctrl->pref_ready));
